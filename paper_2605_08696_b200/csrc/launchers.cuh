@@ -516,7 +516,10 @@ int launch_lm_head_topk(srm_model& m, int64_t R, const void* a, void* lists, voi
   return SRM_OK;
 }
 
-// From this many prompts per pass the scan kernel (one warp per prompt) is the faster prefill mixer.
+// From this many prompts per pass the scan kernel (one warp per prompt) is the prefill mixer; below it the chunk kernel
+// (a CTA per 16 positions of a prompt), or, for shapes neither is built for, the tile kernel (a CTA per prompt). us per
+// launch, tile / chunk / scan kernel: mid, 1 prompt of 777 positions 2061 / 23.6 / -, 45 ragged prompts of up to 301
+// 717 / 48 / -, 2048 prompts of 256 - / 1844 / 1834; rl, 16 prompts of 200: 760 / 26 / -.
 constexpr int64_t kPrefillScanMinSamples = 384;
 
 template <int NV, typename WT, typename ST>
@@ -541,8 +544,33 @@ int launch_prefill_scan_nv(const PrefillParams& p, int num_sms, cudaStream_t st)
   }
 }
 
+// Whether a pass of np prompts of n positions takes the chunk kernel: widths it is built for, and workspace areas that
+// are free while a layer's tokens are mixed with room for its scratch (the end states of the chunks in the hidden-layer
+// area, the flags in the area of the last-position activations).
+bool prefill_chunk_ok(const srm_model& m, int64_t np, int n) {
+  const srm_config& c = m.cfg;
+  if (c.mixer != SRM_MIXER_MIXED || m.head_proj() || np >= kPrefillScanMinSamples) return false;
+  if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536 && c.d_model != 2048) return false;
+  const int64_t all = np * prefill_chunks(n);
+  return all < ((int64_t)1 << 31) && (size_t)all * c.d_model * 4 <= (size_t)np * n * m.F() * m.act_bytes() &&
+         (size_t)all * 4 <= (size_t)np * c.d_model * m.act_bytes();
+}
+
+template <int NV, typename WT, typename ST>
+int launch_prefill_chunk(const PrefillParams& p, const ChunkScratch& cs, cudaStream_t st) {
+  const size_t smem = prefill_chunk_smem(NV * 128);
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_chunk_kernel<NV, WT, ST>), (int)smem);
+  if (rc != SRM_OK) return rc;
+  const int chunks = (int)prefill_chunks(p.n);
+  SRM_CUDA(launch_kernel(prefill_chunk_kernel<NV, WT, ST>, dim3((unsigned)(p.Bp * chunks)), dim3(NV * 32), smem, st, p, cs, chunks));
+  SRM_CUDA(cudaGetLastError());
+  return SRM_OK;
+}
+
+// cs: scratch of the chunk kernel (prefill_chunk_ok), or nullptr: none.
 int launch_prefill_mixer(const srm_model& m, int layer, int64_t Bp, int n, const int32_t* tok, float* x, void* S,
-                         void* a, uint32_t* status, cudaStream_t st, const int32_t* len = nullptr) {
+                         void* a, uint32_t* status, cudaStream_t st, const int32_t* len = nullptr,
+                         const ChunkScratch* cs = nullptr) {
   if (Bp <= 0) return SRM_OK;
   LaunchScope scope(m, SRM_KERNEL_PREFILL_MIXER, st);
   PrefillParams p;
@@ -554,6 +582,18 @@ int launch_prefill_mixer(const srm_model& m, int layer, int64_t Bp, int n, const
   p.eps = m.cfg.ln_eps; p.status = status; p.len = len;
   const size_t smem = (size_t)kPrefillTile * m.cfg.d_model * 4;
   const int nv = p.d / 128;
+  if (cs != nullptr) {
+    return dispatch_types(m.cfg, [&](auto w, auto c) {
+      using WT = decltype(w);
+      using ST = decltype(c);
+      switch (nv) {
+        case 4: return launch_prefill_chunk<4, WT, ST>(p, *cs, st);
+        case 8: return launch_prefill_chunk<8, WT, ST>(p, *cs, st);
+        case 12: return launch_prefill_chunk<12, WT, ST>(p, *cs, st);
+        default: return launch_prefill_chunk<16, WT, ST>(p, *cs, st);
+      }
+    });
+  }
   const bool scan_shape = p.d % 128 == 0 && (p.d / p.h) % 128 == 0 && p.h <= 8 && (nv == 4 || nv == 8 || nv == 12 || nv == 16);
   if (scan_shape && Bp >= kPrefillScanMinSamples) {        // many prompts: one warp walks each prompt's positions
     return dispatch_types(m.cfg, [&](auto w, auto c) { return launch_prefill_scan_nv<decltype(w), decltype(c)>(p, m.num_sms, st); });

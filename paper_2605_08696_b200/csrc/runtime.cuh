@@ -28,6 +28,7 @@
 #include "mixer_model_variants.cuh"
 #include "prefill.cuh"
 #include "prefill_scan.cuh"
+#include "prefill_chunk.cuh"
 #include "select.cuh"
 #include "select_topp.cuh"
 #include "step_small.cuh"

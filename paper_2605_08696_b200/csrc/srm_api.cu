@@ -239,6 +239,9 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
     const int64_t np = (P - p0 < Bp) ? P - p0 : Bp;
     const int64_t rows = np * n;
     const int64_t b0 = p0 * replicas, nb = np * replicas;          // state rows of this pass
+    const bool chunked = prefill_chunk_ok(*m, np, n);
+    ChunkScratch cs{static_cast<float*>(w.H), static_cast<uint32_t*>(w.a_last), 0};
+    if (chunked) SRM_CUDA(cudaMemsetAsync(cs.flags, 0, (size_t)(np * prefill_chunks(n)) * 4, st));
     for (int l = 0; l < c.n_layers; ++l) {
       uint8_t* Sl = replicas > 1 ? stage + (size_t)l * planes * np * row_bytes
                                  : static_cast<uint8_t*>(s->layer_ptr(l)) + (size_t)b0 * row_bytes;
@@ -255,8 +258,11 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
       } else if (m->head_proj()) {
         if ((rc = launch_mixer_block_proj(*m, l, -1, rows, np, n, l == 0 ? d_tokens + p0 * n : nullptr, w.x, Sl, w.a, w.q, s->status, st,
                                           nullptr, d_len ? d_len + p0 : nullptr))) return rc;
-      } else if ((rc = launch_prefill_mixer(*m, l, np, n, l == 0 ? d_tokens + p0 * n : nullptr, w.x, Sl, w.a, s->status, st,
-                                            d_len ? d_len + p0 : nullptr))) return rc;
+      } else {
+        cs.epoch = (uint32_t)l + 1;
+        if ((rc = launch_prefill_mixer(*m, l, np, n, l == 0 ? d_tokens + p0 * n : nullptr, w.x, Sl, w.a, s->status, st,
+                                       d_len ? d_len + p0 : nullptr, chunked ? &cs : nullptr))) return rc;
+      }
       // The feed-forward block over the rows of the pass: in slabs of kPrefillFfnRows rows, each as ONE kernel
       // (ffn_fused.cuh: a slab's hidden activations are consumed from L2 as they are
       // produced instead of crossing HBM twice), where the model's shape allows and the slab counters fit in the
