@@ -102,8 +102,9 @@ enum {
  *                       dimension, filter i reading the channels shifted by i (zero past the last channel); the
  *                       cache is one sum term per filter, kernel_size * d values; alpha is [kernel_size, n_ctx] and
  *                       lambda [kernel_size] (n_heads is not used by the mixing).
- * The two further mixers run through fused step kernels of their own (warp per row); their sequence form is
- * evaluated through the recurrence, one launch per position over all prompts of a pass. They take the cache in
+ * The two further mixers run through fused step kernels of their own (warp per row); their sequence form goes in
+ * chunks of 16 positions (bf16, d_model 512 or 1024) or through the recurrence, one launch per position over all
+ * prompts of a pass. They take the cache in
  * fp32 or fp16, d_model <= 1024, no head projections and no per-sample positions (srm_prefill_ragged). */
 enum { SRM_MIXER_MIXED = 0, SRM_MIXER_COMBINED = 1, SRM_MIXER_KERNEL = 2 };
 

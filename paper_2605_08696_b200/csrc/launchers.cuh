@@ -104,11 +104,8 @@ int launch_mixer_variant_t(const VariantParams& p, bool kernel_mix, cudaStream_t
   return SRM_OK;
 }
 
-int launch_mixer_variant(const srm_model& m, int layer, int t, int64_t R, const int32_t* tok, int64_t tok_stride, float* x,
-                         void* a, int64_t x_stride, void* S, int64_t plane, uint32_t* status, cudaStream_t st,
-                         const int32_t* ctr = nullptr, int cls = SRM_KERNEL_MIXER) {
-  if (R <= 0) return SRM_OK;
-  LaunchScope scope(m, cls, st);
+VariantParams variant_params(const srm_model& m, int layer, int t, int64_t R, const int32_t* tok, int64_t tok_stride, float* x,
+                             void* a, int64_t x_stride, void* S, int64_t plane, uint32_t* status, const int32_t* ctr) {
   const srm_config& c = m.cfg;
   VariantParams p;
   p.x = x; p.tok = tok; p.E = m.ptr(-1, SRM_T_E); p.S = S; p.a = a;
@@ -122,6 +119,16 @@ int launch_mixer_variant(const srm_model& m, int layer, int t, int64_t R, const 
   p.R = R; p.x_stride = x_stride; p.tok_stride = tok_stride; p.plane = plane;
   p.d = c.d_model; p.h = c.n_heads; p.k = c.kernel_size; p.n_ctx = c.n_ctx; p.t = t; p.vocab = c.vocab;
   p.eps = c.ln_eps; p.status = status; p.ctr = ctr;
+  return p;
+}
+
+int launch_mixer_variant(const srm_model& m, int layer, int t, int64_t R, const int32_t* tok, int64_t tok_stride, float* x,
+                         void* a, int64_t x_stride, void* S, int64_t plane, uint32_t* status, cudaStream_t st,
+                         const int32_t* ctr = nullptr, int cls = SRM_KERNEL_MIXER) {
+  if (R <= 0) return SRM_OK;
+  LaunchScope scope(m, cls, st);
+  const srm_config& c = m.cfg;
+  const VariantParams p = variant_params(m, layer, t, R, tok, tok_stride, x, a, x_stride, S, plane, status, ctr);
   const bool wb = c.dtype == SRM_DTYPE_BF16, half_cache = c.state_dtype == SRM_DTYPE_FP16;
   const bool km = c.mixer == SRM_MIXER_KERNEL;
   if (wb) return half_cache ? launch_mixer_variant_t<bf16, fp16>(p, km, st) : launch_mixer_variant_t<bf16, float>(p, km, st);
@@ -544,15 +551,21 @@ int launch_prefill_scan_nv(const PrefillParams& p, int num_sms, cudaStream_t st)
   }
 }
 
-// Whether a pass of np prompts of n positions takes the chunk kernel: widths it is built for, and workspace areas that
-// are free while a layer's tokens are mixed with room for its scratch (the end states of the chunks in the hidden-layer
-// area, the flags in the area of the last-position activations).
+// Whether a pass of np prompts of n positions takes the chunk kernels: widths and types they are built for, and
+// workspace areas that are free while a layer's tokens are mixed with room for their scratch (the end states of the
+// chunks in the hidden-layer area, the flags in the area of the last-position activations).
 bool prefill_chunk_ok(const srm_model& m, int64_t np, int n) {
   const srm_config& c = m.cfg;
-  if (c.mixer != SRM_MIXER_MIXED || m.head_proj() || np >= kPrefillScanMinSamples) return false;
-  if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536 && c.d_model != 2048) return false;
-  const int64_t all = np * prefill_chunks(n);
-  return all < ((int64_t)1 << 31) && (size_t)all * c.d_model * 4 <= (size_t)np * n * m.F() * m.act_bytes() &&
+  if (m.head_proj()) return false;
+  if (c.mixer == SRM_MIXER_MIXED) {
+    if (np >= kPrefillScanMinSamples) return false;
+    if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536 && c.d_model != 2048) return false;
+  } else if (c.dtype != SRM_DTYPE_BF16 || (c.d_model != 512 && c.d_model != 1024)) {
+    return false;
+  }
+  const int64_t chunks = prefill_chunks(n), all = np * chunks;
+  return all < ((int64_t)1 << 31) &&
+         (size_t)(all - np) * cache_planes(c) * c.d_model * 4 <= (size_t)np * n * m.F() * m.act_bytes() &&
          (size_t)all * 4 <= (size_t)np * c.d_model * m.act_bytes();
 }
 
@@ -605,6 +618,35 @@ int launch_prefill_mixer(const srm_model& m, int layer, int64_t Bp, int n, const
     return SRM_OK;
   };
   return dispatch_types(m.cfg, [&](auto w, auto c) { return go(prefill_mixer_kernel<decltype(w), decltype(c)>); });
+}
+
+// Sequence form of the further mixers in chunks of positions (prefill_chunk_variants.cuh; prefill_chunk_ok).
+template <int NV, typename ST, int KM>
+int launch_variant_chunk_k(const VariantParams& p, const ChunkScratch& cs, int n, cudaStream_t st) {
+  const size_t smem = variant_chunk_smem<NV, KM>();
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(variant_chunk_kernel<NV, bf16, ST, KM>), (int)smem);
+  if (rc != SRM_OK) return rc;
+  const int chunks = (int)prefill_chunks(n);
+  SRM_CUDA(launch_kernel(variant_chunk_kernel<NV, bf16, ST, KM>, dim3((unsigned)(p.R * chunks)), dim3(NV * 32), smem, st, p, cs, n, chunks));
+  SRM_CUDA(cudaGetLastError());
+  return SRM_OK;
+}
+template <int NV, typename ST>
+int launch_variant_chunk_t(const VariantParams& p, bool kernel_mix, const ChunkScratch& cs, int n, cudaStream_t st) {
+  if (!kernel_mix) return launch_variant_chunk_k<NV, ST, 0>(p, cs, n, st);
+  if (p.k <= 2) return launch_variant_chunk_k<NV, ST, 2>(p, cs, n, st);
+  if (p.k <= 4) return launch_variant_chunk_k<NV, ST, 4>(p, cs, n, st);
+  if (p.k <= 8) return launch_variant_chunk_k<NV, ST, 8>(p, cs, n, st);
+  return launch_variant_chunk_k<NV, ST, 16>(p, cs, n, st);
+}
+int launch_variant_chunk(const srm_model& m, int layer, int64_t Bp, int n, const int32_t* tok, float* x, void* a, void* S,
+                         int64_t plane, uint32_t* status, cudaStream_t st, const ChunkScratch& cs) {
+  if (Bp <= 0) return SRM_OK;
+  LaunchScope scope(m, SRM_KERNEL_PREFILL_MIXER, st);
+  const VariantParams p = variant_params(m, layer, 0, Bp, tok, n, x, a, m.cfg.d_model, S, plane, status, nullptr);
+  const bool km = m.cfg.mixer == SRM_MIXER_KERNEL, half = m.cfg.state_dtype == SRM_DTYPE_FP16;
+  if (p.d == 512) return half ? launch_variant_chunk_t<4, fp16>(p, km, cs, n, st) : launch_variant_chunk_t<4, float>(p, km, cs, n, st);
+  return half ? launch_variant_chunk_t<8, fp16>(p, km, cs, n, st) : launch_variant_chunk_t<8, float>(p, km, cs, n, st);
 }
 
 // Token-mixing block with head projections (Eq. 10) on `rows` rows of the residual stream:

@@ -9,9 +9,9 @@
 // The shifted reads of Eq. 11 never leave the warp: channel c + i of a filter's vector sits at most four lanes
 // ahead (k <= 16), so every output float4 is put together from two shuffled float4s of the lanes ahead, the
 // lanes at the end of a vector reading the start of the next one.
-// Rows may be strided (x and a rows `x_stride` elements apart, tokens `tok_stride` apart): the sequence form of
-// these models walks the positions of all prompts of a pass with this kernel, one launch per position, the
-// cache staying in place between launches (it is the recurrence that defines the sequence form's result).
+// Rows may be strided (x and a rows `x_stride` elements apart, tokens `tok_stride` apart): for the
+// shapes variant_chunk_kernel is not built for, the sequence form walks the positions of all prompts of a pass with this
+// kernel, one launch per position, the cache staying in place between launches.
 #pragma once
 
 #include "common.cuh"

@@ -33,7 +33,8 @@ namespace srm {
 constexpr int kChunkRows = 16;
 constexpr long long kChunkWaitLimitCycles = 1ll << 30;
 
-// Scratch of a launch: E of every chunk [Bp * chunks, d] fp32 and one flag per chunk. A flag counts the launches that
+// Scratch of a launch: E of every chunk but a prompt's last [Bp * (chunks - 1), d] fp32 (times the sum terms per
+// channel of the mixer) and one flag per chunk. A flag counts the launches that
 // have published into it (epoch 1, 2, ... of a zeroed array), so the array is cleared once for all layers of a pass.
 struct ChunkScratch {
   float* E = nullptr;
@@ -147,7 +148,7 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
       const float u = is_row ? __ldg(alpha + j) : 1.0f;
       S = make_float4(lam * fmaf(u, z.x, S.x), lam * fmaf(u, z.y, S.y), lam * fmaf(u, z.z, S.z), lam * fmaf(u, z.w, S.w));
     }
-    __stcg(reinterpret_cast<float4*>(cs.E + (b * chunks + ch) * d + c), S);
+    __stcg(reinterpret_cast<float4*>(cs.E + (b * (chunks - 1) + ch) * d + c), S);
     __syncthreads();
     if (tid == 0) {
       __threadfence();
@@ -168,7 +169,7 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
     float lT = lam;                                    // lambda^T by squaring
 #pragma unroll
     for (int k = 1; k < T; k <<= 1) lT *= lT;
-    const float* E = cs.E + b * chunks * (int64_t)d + c;
+    const float* E = cs.E + b * (chunks - 1) * d + c;
 #pragma unroll 8
     for (int i = 0; i < ch; ++i) {
       const float4 e = __ldcg(reinterpret_cast<const float4*>(E + (int64_t)i * d));

@@ -29,6 +29,7 @@
 #include "prefill.cuh"
 #include "prefill_scan.cuh"
 #include "prefill_chunk.cuh"
+#include "prefill_chunk_variants.cuh"
 #include "select.cuh"
 #include "select_topp.cuh"
 #include "step_small.cuh"

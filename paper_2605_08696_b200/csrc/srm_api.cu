@@ -246,12 +246,16 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
       uint8_t* Sl = replicas > 1 ? stage + (size_t)l * planes * np * row_bytes
                                  : static_cast<uint8_t*>(s->layer_ptr(l)) + (size_t)b0 * row_bytes;
       if (c.mixer != SRM_MIXER_MIXED) {
-        // the sequence form of these mixers through their recurrence: one launch per position over all prompts of the
-        // pass, the (zeroed) cache updated in place; rows of one prompt are n apart in x and a
         const int64_t plane = replicas > 1 ? np * (int64_t)d : s->plane_elems();
-        for (int pl = 0; pl < planes; ++pl)          // the recurrence starts from an empty cache
+        // shapes the chunk kernel is not built for: the recurrence with one launch per position over all prompts of
+        // the pass, the (zeroed) cache updated in place; rows of one prompt are n apart in x and a
+        if (chunked) {
+          cs.epoch = (uint32_t)l + 1;
+          if ((rc = launch_variant_chunk(*m, l, np, n, l == 0 ? d_tokens + p0 * n : nullptr, w.x, w.a, Sl, plane, s->status, st, cs))) return rc;
+        }
+        for (int pl = 0; !chunked && pl < planes; ++pl)          // the recurrence starts from an empty cache
           SRM_CUDA(cudaMemsetAsync(Sl + (size_t)pl * plane * m->state_bytes(), 0, (size_t)np * row_bytes, st));
-        for (int t = 0; t < n; ++t)
+        for (int t = 0; !chunked && t < n; ++t)
           if ((rc = launch_mixer_variant(*m, l, t, np, l == 0 ? d_tokens + p0 * n + t : nullptr, n, w.x + (size_t)t * d,
                                          static_cast<uint8_t*>(w.a) + (size_t)t * d * m->act_bytes(), (int64_t)n * d, Sl, plane,
                                          s->status, st, nullptr, SRM_KERNEL_PREFILL_MIXER))) return rc;

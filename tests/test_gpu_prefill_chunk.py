@@ -42,3 +42,26 @@ def test_prefill_in_chunks_matches_the_oracle(d, n, B):
         for l in range(shape.n_layers):
             assert rel_err_rows(c2[l][b:b + 1], sb[l]) < TOL["fp32"]
     assert st.status() == 0 and s2.status() == 0
+
+
+@pytest.mark.parametrize("mixer,k,d,n,B", [("combined", 1, 512, 40, 3), ("combined", 1, 1024, 16, 2), ("kernel", 1, 512, 17, 3),
+                                           ("kernel", 3, 1024, 49, 2), ("kernel", 4, 512, 32, 2), ("kernel", 7, 1024, 18, 3),
+                                           ("kernel", 16, 1024, 33, 2), ("kernel", 16, 512, 1, 2)])
+def test_prefill_in_chunks_of_the_further_mixers_matches_the_oracle(mixer, k, d, n, B):
+    """bf16 models. The cache of layer 0 sees only fp32 arithmetic (embedding, LN1, recurrence): fp32 tolerance. Layer 1
+    and the logits come through the bf16 feed-forward: bf16 tolerance; a wrong y (a wrapped channel, a shift) moves
+    them by far more."""
+    import paper_2605_08696_b200 as P
+    shape = I.SRMShape(n_layers=2, d_model=d, vocab=64, n_ctx=64, dtype="bf16", seed=d + n + k, mixer=mixer, kernel_size=k)
+    W = I.make_weights(shape, alpha_std=0.3)
+    model = P.SRM(shape, W, device=DEV)
+    toks = I.uniform_prompts(B, n, shape.vocab, seed=n)
+    st = model.new_state(B)
+    ws = model.new_workspace(B, n, prefill_samples=B)
+    _, lg = model.prefill(st, torch.from_numpy(toks).to(DEV), P.Sampling("greedy"), ws, want_logits=True)
+    lo, so = oracle_for(shape, W).forward_parallel(toks)
+    cache = st.cache().cpu().numpy()
+    assert rel_err_rows(cache[0], so[0]) < TOL["fp32"]
+    assert rel_err_rows(cache[1], so[1]) < TOL["bf16"]
+    assert rel_err_rows(lg.cpu().numpy(), lo[:, n - 1]) < TOL["bf16"]
+    assert st.status() == 0
