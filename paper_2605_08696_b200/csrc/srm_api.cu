@@ -271,21 +271,22 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
       // (ffn_fused.cuh: a slab's hidden activations are consumed from L2 as they are
       // produced instead of crossing HBM twice), where the model's shape allows and the slab counters fit in the
       // logits area (free until the LM head); else, and for a short last slab, up projection then down projection.
-      const size_t slab_ready = ffn_ready_bytes(kPrefillFfnRows, F);
-      const int64_t n_slabs = (rows + kPrefillFfnRows - 1) / kPrefillFfnRows;
-      bool slabs = !(c.flags & SRM_FLAG_NO_FUSED_FFN) && rows >= kPrefillFfnRows && ffn_fused_shape_ok(*m, kPrefillFfnRows) &&
+      const int64_t slab_rows = rows < kPrefillFfnRows ? rows : kPrefillFfnRows;
+      const size_t slab_ready = ffn_ready_bytes(slab_rows, F);
+      const int64_t n_slabs = (rows + slab_rows - 1) / slab_rows;
+      bool slabs = !(c.flags & SRM_FLAG_NO_FUSED_FFN) && ffn_fused_shape_ok(*m, slab_rows) &&
                    (size_t)n_slabs * slab_ready <= align_up((size_t)np * c.vocab * 4, 256);
       if (slabs) {
         if ((rc = ensure_tc_ready(*m))) return rc;
-        slabs = ffn_fused_worthwhile(*m, kPrefillFfnRows);
+        slabs = ffn_fused_worthwhile(*m, slab_rows);
       }
       if (slabs) SRM_CUDA(cudaMemsetAsync(w.logits, 0, (size_t)n_slabs * slab_ready, st));
-      for (int64_t r0 = 0; slabs && r0 < rows; r0 += kPrefillFfnRows) {
-        const int64_t nr = rows - r0 < kPrefillFfnRows ? rows - r0 : kPrefillFfnRows;
+      for (int64_t r0 = 0; slabs && r0 < rows; r0 += slab_rows) {
+        const int64_t nr = rows - r0 < slab_rows ? rows - r0 : slab_rows;
         uint8_t* a_s = static_cast<uint8_t*>(w.a) + (size_t)r0 * d * m->act_bytes();
         uint8_t* H_s = static_cast<uint8_t*>(w.H) + (size_t)r0 * F * m->act_bytes();
         float* x_s = w.x + (size_t)r0 * d;
-        int32_t* ready = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(w.logits) + (size_t)(r0 / kPrefillFfnRows) * slab_ready);
+        int32_t* ready = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(w.logits) + (size_t)(r0 / slab_rows) * slab_ready);
         rc = ffn_fused_worthwhile(*m, nr) ? launch_ffn_fused(*m, l, nr, a_s, H_s, x_s, ready, s->status, st) : SRM_ERR_UNSUPPORTED;
         if (rc == SRM_ERR_UNSUPPORTED) {
           if ((rc = launch_gemm(*m, kEpiBiasGelu, nr, F, d, a_s, m->ptr(l, SRM_T_W1), m->fptr(l, SRM_T_B1), H_s, s->status, st))) return rc;
