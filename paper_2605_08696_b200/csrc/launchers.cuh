@@ -389,7 +389,7 @@ int launch_select(const srm_model& m, int64_t R, const float* logits, const srm_
   LaunchScope scope(m, SRM_KERNEL_SELECT, st);
   const int V = m.cfg.vocab;
   if (s.mode == SRM_SELECT_GREEDY) {
-    SRM_CUDA(launch_kernel(select_greedy_kernel, dim3((unsigned)R), dim3(kSelThreads), 0, st, logits, R, V, out, status));
+    SRM_CUDA(launch_kernel(select_greedy_kernel, dim3((unsigned)(R / out.row_div)), dim3(kSelThreads), 0, st, logits, R, V, out, status));
   } else if (s.mode == SRM_SELECT_TOPP) {
     const float inv_t = 1.0f / s.temperature;
     const size_t scratch = ((sizeof(ToppScratch) + 15) & ~size_t(15)) + sizeof(ToppHist);
@@ -410,7 +410,7 @@ int launch_select(const srm_model& m, int64_t R, const float* logits, const srm_
   } else {
     const float inv_t = 1.0f / s.temperature;
     const float z0 = topk_z0(s.top_k, V);
-    SRM_CUDA(launch_kernel(select_topk_stream_kernel, dim3((unsigned)R), dim3(kSelThreads), 0, st, logits, R, V, s.top_k,
+    SRM_CUDA(launch_kernel(select_topk_stream_kernel, dim3((unsigned)(R / out.row_div)), dim3(kSelThreads), 0, st, logits, R, V, s.top_k,
                            inv_t, z0, s.seed, sample_base, step, out, status));
     // rows the streaming kernel could not settle (marked -1): the radix selection, reading the row from
     // global memory; every other block exits at once

@@ -57,9 +57,9 @@ __global__ void __launch_bounds__(kSelThreads)
 select_greedy_kernel(const float* __restrict__ logits, int64_t R, int V, SelectOut out, uint32_t* status) {
   pdl_trigger();
   pdl_wait();
-  const int64_t row = blockIdx.x;
+  const int64_t row = blockIdx.x * out.row_div;         // a block per row of logits, for all rows that share it
   if (row >= R) return;
-  const float* lr = logits + (row / out.row_div) * (int64_t)V;
+  const float* lr = logits + (int64_t)blockIdx.x * V;
   float bv = -INFINITY;
   int bi = 0x7fffffff;
   bool bad = false;
@@ -84,8 +84,10 @@ select_greedy_kernel(const float* __restrict__ logits, int64_t R, int V, SelectO
   if (threadIdx.x == 0) {
     for (int w = 1; w < kSelThreads / 32; ++w) argmax_take(sv[w], si[w], bv, bi);
     if (bi < 0 || bi >= V) bi = 0;       // all-NaN row
-    write_token(out, row, bi);
+    si[0] = bi;
   }
+  __syncthreads();
+  for (int64_t j = threadIdx.x; j < out.row_div; j += kSelThreads) write_token(out, row + j, si[0]);
 }
 
 // Second stage of the selection fused into the LM head: reduces the per-slice partial results
@@ -184,25 +186,43 @@ __device__ inline float next_threshold(const unsigned long long* sorted, int c, 
   return t == 0.f ? -0.0f : t;                   // a threshold of zero keeps a bit set
 }
 
-// Thread 0 of a block: inverse-CDF draw over the k first of `sorted` (logit desc, id asc) and the row's outputs.
+// Inverse-CDF draws over the k first of `sorted` (logit desc, id asc) and the outputs of rows row0 .. row0 + reps - 1,
+// which share these logits (replicas of one prompt; else reps = 1). All threads of the block call it, k <= threads.
+// The weights are formed in parallel and added in order by one thread (the sum's order is part of the result); each
+// replica's draw is one warp's search for the first cumulative weight above its target.
 __device__ inline void draw_topk(const unsigned long long* sorted, int c, int k, float inv_temp, uint64_t seed,
-                                 uint64_t sidx, int step, const SelectOut& out, int64_t row, float* cdf) {
+                                 uint64_t sample_base, int step, const SelectOut& out, int64_t row0, int64_t reps, float* cdf) {
+  __shared__ float sh_thr;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, warps = blockDim.x >> 5;
   const float l0 = cand_value(sorted[0]);
-  float acc = 0.f;
-  for (int i = 0; i < k; ++i) {
-    acc += expf((cand_value(sorted[i]) - l0) * inv_temp);
-    cdf[i] = acc;
+  if (tid < k) cdf[tid] = expf((cand_value(sorted[tid]) - l0) * inv_temp);
+  __syncthreads();
+  if (tid == 0) {
+    float acc = 0.f;
+    for (int i = 0; i < k; ++i) {
+      acc += cdf[i];
+      cdf[i] = acc;
+    }
+  } else if (tid == 32 && out.thr_out != nullptr) {
+    sh_thr = next_threshold(sorted, c, k);
   }
-  const uint32_t r = philox4x32_10_word0((uint32_t)sidx, (uint32_t)(out.ctr != nullptr ? out.ctr[kCtrStep] : step), 0u, 0u,
-                                         (uint32_t)seed, (uint32_t)(seed >> 32));
-  const float u = (float)(r >> 8) * (1.0f / 16777216.0f);
-  const float target = u * acc;
-  int pick = k - 1;
-  for (int i = 0; i < k; ++i) {
-    if (cdf[i] > target) { pick = i; break; }
+  __syncthreads();
+  const uint32_t ph_step = (uint32_t)(out.ctr != nullptr ? out.ctr[kCtrStep] : step);
+  for (int64_t j = warp; j < reps; j += warps) {
+    const int64_t row = row0 + j;
+    const uint64_t sidx = sample_base + (uint64_t)row;
+    const uint32_t r = philox4x32_10_word0((uint32_t)sidx, ph_step, 0u, 0u, (uint32_t)seed, (uint32_t)(seed >> 32));
+    const float target = (float)(r >> 8) * (1.0f / 16777216.0f) * cdf[k - 1];
+    int pick = k - 1;
+    for (int i0 = 0; i0 < k; i0 += 32) {
+      const uint32_t above = __ballot_sync(0xffffffffu, i0 + lane < k && cdf[i0 + lane] > target);
+      if (above != 0u) { pick = i0 + __ffs(above) - 1; break; }
+    }
+    if (lane == 0) {
+      if (out.thr_out != nullptr) out.thr_out[row] = sh_thr;
+      write_token(out, row, (int)(uint32_t)(sorted[pick] & 0xffffffffull));
+    }
   }
-  if (out.thr_out != nullptr) out.thr_out[row] = next_threshold(sorted, c, k);
-  write_token(out, row, (int)(uint32_t)(sorted[pick] & 0xffffffffull));
 }
 
 // Sorts cand[0 .. c) of a block's shared memory ascending, i.e. by (logit desc, id asc); c <= the array's
@@ -389,8 +409,10 @@ select_topk_stream_kernel(const float* __restrict__ logits, int64_t R, int V, in
   __shared__ uint32_t sh_count;
   __shared__ float cdf[kTopKMax];
 
+  // one block per row of logits: replicas of one prompt differ in their draws only
+  const int64_t reps = out.row_map != nullptr ? 1 : out.row_div;
   int64_t row, lrow;
-  if (!select_rows(out, blockIdx.x, R, &row, &lrow)) return;
+  if (!select_rows(out, blockIdx.x * reps, R, &row, &lrow)) return;
   const float* lr = logits + lrow * (int64_t)V;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -445,12 +467,12 @@ select_topk_stream_kernel(const float* __restrict__ logits, int64_t R, int V, in
     __syncthreads();
   }
   if (!found) {                                      // block-uniform
-    if (tid == 0) out.last_tok[row] = -1;
+    for (int64_t j = tid; j < reps; j += kSelThreads) out.last_tok[row + j] = -1;
     return;
   }
 
   sort_candidates(cand, (int)c, tid, kSelThreads);
-  if (tid == 0) draw_topk(cand, (int)c, k, inv_temp, seed, sample_base + (uint64_t)row, step, out, row, cdf);
+  draw_topk(cand, (int)c, k, inv_temp, seed, sample_base, step, out, row, reps, cdf);
 }
 
 // ---- top-k fused into the LM head: second stage ------------------------------------------------------
@@ -494,7 +516,7 @@ topk_merge_kernel(const unsigned long long* __restrict__ lists, const uint32_t* 
   for (int i = tid; i < (int)c; i += kSelThreads) cand[i] = lr[i];
   __syncthreads();
   sort_candidates(cand, (int)c, tid, kSelThreads);
-  if (tid == 0) draw_topk(cand, (int)c, k, inv_temp, seed, sample_base + (uint64_t)row, step, out, row, cdf);
+  draw_topk(cand, (int)c, k, inv_temp, seed, sample_base, step, out, row, 1, cdf);
 }
 
 // Cache rows of `replicas` consecutive samples = the row of their prompt:
