@@ -789,52 +789,63 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
 }
 
 // ---- small batches: the whole step in one cooperative kernel (step_small.cuh) ----------------------
-struct SmallPlan { sb::Params p; int grid; size_t smem; };
+struct SmallPlan { sb::Params p; size_t smem; };
 
-// Whether a batch of B samples takes the single-kernel step, and its slab plan. Mixed heads, bf16 weights, at most
-// 64 samples and 1024 channels; everything else takes the kernel-per-operation path.
-bool small_step_plan(const srm_model& m, const srm_state& s, SmallPlan* P) {
-  const srm_config& c = m.cfg;
-  if (c.dtype != SRM_DTYPE_BF16 || (c.flags & (SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_HEAD_PROJ))) return false;
-  if (c.mixer != SRM_MIXER_MIXED || s.ragged || s.B > sb::kMaxRows || c.d_model > 1024 || m.num_sms < 16 || m.num_sms > 256) return false;
-  const int d = c.d_model, F = (int)m.F(), V = c.vocab, G = m.num_sms;
-  if (F % 32 || d % 64) return false;
-  sb::Params& p = P->p;
-  p.up_cols = ((F + G - 1) / G + 15) / 16 * 16;
-  p.up_ctas = (F + p.up_cols - 1) / p.up_cols;
-  p.dn_cols = 64;
-  p.dn_nslabs = d / 64;
-  int ks = G / p.dn_nslabs;
-  ks = ks > 8 ? 8 : ks;
-  if (ks < 1) return false;
-  p.dn_klen = ((F + ks - 1) / ks + 31) / 32 * 32;
-  p.dn_kslabs = (F + p.dn_klen - 1) / p.dn_klen;
-  p.lm_cols = ((V + G - 1) / G + sb::kLmChunkCols - 1) / sb::kLmChunkCols * sb::kLmChunkCols;
-  p.lm_ctas = (V + p.lm_cols - 1) / p.lm_cols;
-  P->grid = G;
-  P->smem = 128 + (size_t)sb::act_region_bytes(d, p.dn_klen) + (size_t)sb::weight_region_bytes(d, p.up_cols, p.dn_cols, p.dn_klen);
-  return P->smem <= (size_t)sb::kSmemBytes;
+// f(kernel) for the instance of the step kernel that the configuration takes.
+template <int d, typename Fn>
+int with_small_kernel_d(const srm_config& c, Fn&& f) {
+  if (c.state_dtype == SRM_DTYPE_FP16) return f(sb::step_small_kernel<d, fp16>);
+  if (c.state_dtype == SRM_DTYPE_BF16) return f(sb::step_small_kernel<d, bf16>);
+  return f(sb::step_small_kernel<d, float>);
+}
+template <typename Fn>
+int with_small_kernel(const srm_config& c, Fn&& f) {
+  switch (c.d_model) {
+    case 256: return with_small_kernel_d<256>(c, f);
+    case 512: return with_small_kernel_d<512>(c, f);
+    case 768: return with_small_kernel_d<768>(c, f);
+    default: return with_small_kernel_d<1024>(c, f);
+  }
 }
 
-template <typename ST>
-int launch_step_small_t(const SmallPlan& P, cudaStream_t st) {
-  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(sb::step_small_kernel<ST>), sb::kSmemBytes);
-  if (rc != SRM_OK) return rc;
-  int per_sm = 0;
-  SRM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sb::step_small_kernel<ST>, sb::kThreads, P.smem));
-  if (per_sm < 1) return SRM_ERR_UNSUPPORTED;
+// Both launch attributes of the kernel: all CTAs resident at once (it has grid-wide barriers), in clusters.
+struct SmallLaunch {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)P.grid);
-  cfg.blockDim = dim3(sb::kThreads);
-  cfg.dynamicSmemBytes = P.smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeCooperative;           // all CTAs resident at once: the kernel has grid-wide barriers
-  attr.val.cooperative = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  SRM_CUDA(cudaLaunchKernelEx(&cfg, sb::step_small_kernel<ST>, P.p));
-  return SRM_OK;
+  cudaLaunchAttribute attr[2];
+  SmallLaunch(size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3(sb::kGrid);
+    cfg.blockDim = dim3(sb::kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = sb::kCluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
+// Whether a batch of B samples takes the single-kernel step, and its shared-memory plan. Mixed heads, bf16 weights, at
+// most 64 samples and 1024 channels (a multiple of 256), a device that holds all clusters at once; everything
+// else takes the kernel-per-operation path.
+bool small_step_plan(srm_model& m, const srm_state& s, SmallPlan* P) {
+  const srm_config& c = m.cfg;
+  if (c.dtype != SRM_DTYPE_BF16 || (c.flags & (SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_HEAD_PROJ))) return false;
+  if (c.mixer != SRM_MIXER_MIXED || s.B > sb::kMaxRows || c.d_model > 1024 || c.d_model % 256 || m.F() % 1024) return false;
+  if (m.small_clusters < 0) {
+    m.small_clusters = with_small_kernel(c, [&](auto* kernel) {
+      int n = 0;
+      if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), sb::kSmemBytes) != SRM_OK) return 0;
+      SmallLaunch L(sb::kSmemBytes, nullptr);
+      L.cfg.attrs = L.attr + 1;
+      L.cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, kernel, &L.cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+      return n;
+    });
+  }
+  return m.small_clusters >= sb::kClusters &&
+         sb::smem_plan((int)s.B, c.d_model, (int)m.F(), m.state_bytes(), &P->p, &P->smem);
 }
 
 // One decode step of all B <= 64 samples of the state. SRM_ERR_UNSUPPORTED: take the ordinary path.
@@ -856,23 +867,26 @@ int decode_step_small(srm_model& m, srm_state& s, SmallPlan& P, const int32_t* t
   p.layer_bytes = c.n_layers > 1 ? (int64_t)(m.layout.layer[SRM_T_COUNT + SRM_T_LN1_G].off - m.layout.layer[SRM_T_LN1_G].off) : 0;
   p.S = s.layer_ptr(0);
   p.layer_stride = (int64_t)s.B * c.d_model * m.state_bytes();
-  p.x = w.x; p.a = reinterpret_cast<bf16*>(w.a); p.H = reinterpret_cast<bf16*>(w.H);
-  uint8_t* q = w.small;
-  p.part = reinterpret_cast<float*>(q); q += align_up((size_t)8 * sb::kMaxRows * c.d_model * 4, 256);
-  p.best = reinterpret_cast<unsigned long long*>(q); q += align_up((size_t)256 * sb::kMaxRows * 8, 256);
-  p.bar = reinterpret_cast<uint32_t*>(q);
+  p.x = w.x; p.H = reinterpret_cast<bf16*>(w.H);
+  p.best = reinterpret_cast<unsigned long long*>(w.small);
+  p.bar = reinterpret_cast<uint32_t*>(w.small + (size_t)sb::kMaxRows * 8);
   p.status = s.status;
   p.ctr = ctr;
+  p.pos = s.ragged ? s.pos_dev : nullptr;
   p.greedy = samp.mode == SRM_SELECT_GREEDY ? 1 : 0;
   p.logits = logits_out != nullptr ? logits_out : (p.greedy ? nullptr : w.logits);
   p.out = out;
-  SRM_CUDA(cudaMemsetAsync(p.bar, 0, 256, st));
+  SRM_CUDA(cudaMemsetAsync(w.small, 0, kSmallScratchBytes, st));
   int rc;
   {
     LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
-    if (c.state_dtype == SRM_DTYPE_FP16) rc = launch_step_small_t<fp16>(P, st);
-    else if (c.state_dtype == SRM_DTYPE_BF16) rc = launch_step_small_t<bf16>(P, st);
-    else rc = launch_step_small_t<float>(P, st);
+    rc = with_small_kernel(c, [&](auto* kernel) -> int {
+      int rc2 = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), sb::kSmemBytes);
+      if (rc2 != SRM_OK) return rc2;
+      SmallLaunch L(P.smem, st);
+      SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, p));
+      return SRM_OK;
+    });
   }
   if (rc != SRM_OK || p.greedy) return rc;
   return launch_select(m, s.B, p.logits, samp, samp.sample_idx_base, step, out, s.status, st);

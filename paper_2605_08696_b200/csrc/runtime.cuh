@@ -199,6 +199,7 @@ struct srm_model {
   int num_sms = 0;
   bool head_proj() const { return (cfg.flags & SRM_FLAG_HEAD_PROJ) != 0; }
   bool tc_ready = false;                 // smem attribute set for the tensor-core kernels
+  int small_clusters = -1;               // clusters of the small-batch step kernel that are resident at once (-1: not asked yet)
   int tc_clusters = 0;                   // CTA pairs of the tensor-core kernel that are resident at once
   std::vector<TmapCacheEntry> tmaps;     // weight and activation descriptors, built on first use
   std::vector<std::pair<int, tc::FfnPlan>> ffn_plans;   // work lists of the fused feed-forward kernel, by row blocks
@@ -297,11 +298,8 @@ size_t state_bytes_for(const srm_config& c, int64_t B) {
 }
 
 // ---- workspace carving ----------------------------------------------------------------------
-// Scratch of the small-batch step kernel (step_small.cuh): partial sums of the down projection
-// [8][64, d] fp32, the per-CTA results of the LM-head slabs [256][64] and the grid-barrier word.
-size_t small_scratch_bytes(const srm_config& c) {
-  return align_up((size_t)8 * sb::kMaxRows * c.d_model * 4, 256) + align_up((size_t)256 * sb::kMaxRows * 8, 256) + 256;
-}
+// Scratch of the small-batch step kernel (step_small.cuh): the best logit of every row [64] and the barrier words.
+constexpr size_t kSmallScratchBytes = (size_t)sb::kMaxRows * 8 + 256;
 
 // Partial-product planes of a small pass's down projection (GemmArgs::k_slices): up to 8 planes of the pass's rows
 // (padded to whole 256-row tiles) x d floats, never more than one 256 x 256 fp32 tile per CTA pair of the largest
@@ -324,7 +322,7 @@ struct DecodeWs {
   float* x; void* a; void* H; float* logits;
   float* part;            // kslice_bytes
   size_t part_bytes;
-  uint8_t* small;         // small_scratch_bytes
+  uint8_t* small;         // kSmallScratchBytes
   float* q;               // head projections only
   int32_t* order;         // split-K down projection: one word per (tile of x, CTA of the pair, epilogue warp)
   size_t order_bytes;
@@ -343,7 +341,7 @@ size_t decode_ws_bytes(const srm_model& m, int64_t rows) {
   const size_t d = m.cfg.d_model, F = m.F(), V = m.cfg.vocab, ab = m.act_bytes();
   return align_up(rows * d * 4, 256) + align_up(rows * d * ab, 256) + align_up(rows * F * ab, 256) +
          align_up(rows * V * 4, 256) + (m.head_proj() ? align_up(rows * d * 4, 256) : 0) +
-         (splitk_enabled(m.cfg) ? splitk_order_bytes(rows, m.cfg.d_model) : 0) + small_scratch_bytes(m.cfg) +
+         (splitk_enabled(m.cfg) ? splitk_order_bytes(rows, m.cfg.d_model) : 0) + kSmallScratchBytes +
          kslice_bytes(m.cfg, rows);
 }
 size_t prefill_ws_bytes(const srm_model& m, int64_t samples, int n) {
@@ -378,7 +376,7 @@ DecodeWs carve_decode(const srm_model& m, void* ws, int64_t rows) {
   w.order_bytes = splitk_enabled(m.cfg) ? splitk_order_bytes(rows, m.cfg.d_model) : 0;
   w.order = w.order_bytes ? reinterpret_cast<int32_t*>(p) : nullptr;
   p += w.order_bytes;
-  w.small = p; p += small_scratch_bytes(m.cfg);
+  w.small = p; p += kSmallScratchBytes;
   w.part_bytes = kslice_bytes(m.cfg, rows);
   w.part = w.part_bytes ? reinterpret_cast<float*>(p) : nullptr;
   return w;

@@ -1,36 +1,49 @@
 // One decode step of a SMALL batch (at most 64 samples) as a single persistent kernel.
 //
-// With a handful of rows the step is bound by reading the weights once (the mid model: 467 MB, 70 us at HBM
-// speed) and by the latency of its 50 dependent kernels, not by arithmetic: a 256 x 256 tensor-core tile keeps 4
-// to 16 of the 74 CTA pairs busy on a one-row GEMM, and every launch costs its ramp. Here the whole step --
-// embedding, L x (token-mixer cache update [Eq. 2, Eq. 3], feed-forward up and down), final norm, LM head,
-// greedy selection -- runs in ONE cooperative kernel of one CTA per SM. Every dense projection is cut into
-// column slabs (and, for the down projection, k-slabs), one per CTA, so that all SMs stream weights at once;
-// the few activation rows are re-read by every CTA from L2. Phases are separated by grid-wide barriers; a CTA
-// starts the bulk copy of its NEXT weight slab before it waits at a barrier (weights are constant), so the
-// weight stream continues across the barriers. The contractions run on mma.sync (m16n8k16, bf16 in, fp32
-// accumulate): with M <= 64 the kernel is HBM-bound and a tcgen05 tile would be mostly padding.
+// With a handful of rows the step is bound by reading the weights once (the mid model: 334 MB, 50 us at HBM speed)
+// and by the latency of its dependent phases, not by arithmetic. The whole step -- embedding, L x (token-mixer cache
+// update [Eq. 2, Eq. 3], feed-forward up and down), final norm, LM head, greedy selection -- runs in ONE cooperative
+// kernel of 128 CTAs, 32 clusters of four (the largest clusters that fit on that many SMs: 33 of four, 15 of eight). Two grid-wide barriers per layer remain, after the up projection (a
+// down slab reads all of its part of H) and after the down projection (a row needs all of x):
+//   - row phase: every cluster computes every row (embedding or x, LN1, cache update, residual, LN2), rank r the rows
+//     r, r + 4, ..., one warp per row, and sends the activation row to the shared memory of its four CTAs, so the
+//     rows need no grid barrier of their own; up to kAloneRows rows every CTA computes all of them for itself. The new
+//     cache row is kept in shared memory and written by one CTA of the grid after the next grid barrier, when nobody
+//     reads the old one any more;
+//   - up projection: every CTA computes F / 128 columns of H = gelu(a W1^T + b1) and stores them;
+//   - down projection: cluster c computes d / 32 columns of x, rank r over the r-th quarter of K; the four partial
+//     products meet in shared memory (each rank receives those of its quarter of the cluster's columns) and are added
+//     in rank order, so x is written once, complete.
+// W1 and W2 slabs have a region of shared memory each (up to 32 rows), refilled for the next layer by bulk copies as
+// soon as they have been used: the weight stream runs a whole layer ahead of the barriers. The small parameter
+// vectors and cache rows of the next layer are prefetched into L2 meanwhile. The contractions run on mma.sync (m16n8k16, bf16 in, fp32 accumulate): the kernel is bound by
+// latency and HBM, and a tcgen05 tile would be mostly padding. K of a tile is cut into up to eight ranges that
+// different warps take, fewer with more row tiles (batches of 1 to 16, 17 to 32, 33 to 64 rows add in different orders).
 //
-// The down projection's k-slabs leave partial sums in scratch memory; the next phase (the following layer's
-// mixer, or the final norm) adds them in slab order, so results do not depend on timing.
 // Every wait (grid barrier, mbarrier) is bounded: on a time-out the CTA raises kStatusWaitTimeout and runs through
 // the remaining phases without waiting, so the kernel always ends.
 #pragma once
 
 #include "common.cuh"
 #include "gemm_tc.cuh"      // mbarrier helpers, gelu_fast
-#include "mixer.cuh"        // row_stats, norm4
+#include "mixer.cuh"        // row_stats_full
 #include "mixer_stream.cuh" // bulk_g2s
+#include "prefill_chunk.cuh" // ld_acquire_u32
 #include "select.cuh"       // SelectOut, write_token
 
 namespace srm {
 namespace sb {
 
-constexpr int kThreads = 256, kWarps = 8;
+constexpr int kThreads = 512, kWarps = 16;
+constexpr int kCluster = 4, kClusters = 32, kGrid = kCluster * kClusters;
 constexpr int kMaxRows = 64;                 // samples per launch
+constexpr int kAloneRows = 4;                // up to this many rows every CTA computes all rows for itself
 constexpr int kPadBytes = 16;                // row padding in shared memory: ldmatrix rows land in distinct banks
 constexpr int kLmChunkCols = 16;             // LM-head weight rows per pipeline stage
-constexpr int kSmemBytes = 220 * 1024;
+constexpr int kLmMaxStages = 6;
+constexpr int kHeadBytes = 128 + 512;        // mbarriers and flags, row-phase sums
+constexpr int kMaxGroups = 8;                // ranges that K of a tile is cut into
+constexpr int kSmemBytes = 227 * 1024;
 constexpr long long kBarrierLimitCycles = 1ll << 27;
 
 struct LayerW {
@@ -50,21 +63,52 @@ struct Params {
   void* S;                     // cache of layer 0; layer l at S + l * layer_stride (bytes)
   int64_t layer_stride;
   float* x;                    // [B, d] residual stream
-  bf16* a;                     // [B, d] activations (GEMM input)
   bf16* H;                     // [B, F]
-  float* part;                 // [ks][B, d] partial sums of the down projection
   float* logits;               // [B, V] or nullptr (then only the greedy selection leaves the kernel)
-  unsigned long long* best;    // [gridDim][B] per-CTA (sortable logit, ~column) of the LM-head slab
-  uint32_t* bar;               // grid barrier counter, zero on entry
+  unsigned long long* best;    // [B] (sortable logit, ~column) maxima, zero on entry
+  uint32_t* bar;               // [0] grid barrier, [1] CTAs done with the LM head; zero on entry
   uint32_t* status;
   const int32_t* ctr;          // device-side step counters or nullptr
+  const int32_t* pos;          // [B] per-row positions or nullptr
   int greedy;                  // select inside the kernel
   SelectOut out;
-  // slab plan (host): columns per CTA and CTAs used, per projection
-  int up_cols, up_ctas;        // multiple of 8
-  int dn_cols, dn_nslabs, dn_kslabs, dn_klen;   // dn_cols = 64; k-slab length a multiple of 16
-  int lm_cols, lm_ctas;        // multiple of kLmChunkCols
+  // shared-memory plan (host): byte offsets
+  int off_w1, off_w2, off_part, off_recv, off_xo, off_s;
+  int lm_stages;               // stages of LM-head rows from off_w1 on
+  int lm_stages_w1;            // ... of which lie inside the W1 region
 };
+
+// Sizes of the slabs a CTA works on.
+__host__ __device__ inline int up_cols(int F) { return F / kGrid; }
+__host__ __device__ inline int dn_cols(int d) { return d / kClusters; }
+__host__ __device__ inline int dn_klen(int F) { return F / kCluster; }
+
+// The shared-memory plan for B rows; false when it does not fit. Fills the off_* / lm_* fields of p.
+inline bool smem_plan(int B, int d, int F, int state_elem, Params* p, size_t* bytes) {
+  const int mp = (B + 15) / 16 * 16, ld_d = 2 * d + kPadBytes, ld_k = 2 * dn_klen(F) + kPadBytes;
+  const int act = mp * (ld_d > ld_k ? ld_d : ld_k);
+  const int w1 = (up_cols(F) + 15) / 16 * 16 * ld_d, w2 = (dn_cols(d) + 15) / 16 * 16 * ld_k, stage = kLmChunkCols * ld_d;
+  const int part = kWarps * 1024, recv = kCluster * mp * (dn_cols(d) / kCluster) * 4, xo = mp * (dn_cols(d) / kCluster) * 4;
+  const int srow = d * state_elem;
+  for (int two = 1; two >= 0; --two) {                   // a region each for W1 and W2, or one for both
+    int w = two ? w1 + w2 : (w1 > w2 ? w1 : w2);
+    if (w < 2 * stage) w = 2 * stage;
+    const int fixed = kHeadBytes + act + part + recv + (xo + 15) / 16 * 16 + srow;
+    if (fixed + w > kSmemBytes) continue;
+    while (w + stage <= kLmMaxStages * stage && fixed + w + stage <= kSmemBytes) w += stage;     // a deeper LM-head ring
+    p->off_w1 = kHeadBytes + act;
+    p->off_w2 = two ? p->off_w1 + w1 : p->off_w1;
+    p->lm_stages = w / stage < kLmMaxStages ? w / stage : kLmMaxStages;
+    p->lm_stages_w1 = two ? w1 / stage : 0;
+    p->off_part = p->off_w1 + w;
+    p->off_recv = p->off_part + part;
+    p->off_xo = p->off_recv + recv;
+    p->off_s = p->off_xo + (xo + 15) / 16 * 16;
+    *bytes = (size_t)(fixed + w);
+    return true;
+  }
+  return false;
+}
 
 __device__ __forceinline__ LayerW layer_w(const Params& p, int l) {
   const int64_t o = (int64_t)l * p.layer_bytes;
@@ -74,38 +118,50 @@ __device__ __forceinline__ LayerW layer_w(const Params& p, int l) {
   return LayerW{f(w.ln1_g), f(w.ln1_b), f(w.ln2_g), f(w.ln2_b), f(w.alpha), f(w.beta), f(w.lam), f(w.b1), f(w.b2), b(w.W1), b(w.W2)};
 }
 
+__device__ __forceinline__ void red_release_inc(uint32_t* p) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v));
+}
+__device__ __forceinline__ void st_cluster_v2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
+// shared memory of this CTA -> shared memory of a CTA of the cluster, bytes counted on a barrier over there
+__device__ __forceinline__ void bulk_s2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(tc::smem_u32(src)), "r"(bytes), "r"(bar) : "memory");
+}
+
 // ---- grid-wide barrier ------------------------------------------------------------------------
 // Arrive / wait on a monotonically increasing counter: barrier number n (1, 2, ...) is passed when the counter
 // has reached n * gridDim.x. All CTAs are resident (cooperative launch), so the wait ends; it is bounded anyway.
+// `between` runs in all threads between arriving and waiting.
 struct GridBarrier {
   uint32_t* ctr;
   uint32_t n;          // barriers passed so far
   bool dead;           // a wait timed out: stop waiting (the same value in every thread of the CTA)
   uint32_t* status;
   int* shared_dead;    // a word of shared memory through which thread 0 tells the others
-  __device__ void sync() {
-    // what this CTA wrote is read after the barrier by other CTAs, partly by bulk copies (the async proxy)
-    __threadfence();
-    asm volatile("fence.proxy.async.global;" ::: "memory");
+  template <typename F>
+  __device__ __forceinline__ void sync(F&& between) {
     __syncthreads();
     ++n;
+    if (threadIdx.x == 0) red_release_inc(ctr);
+    between();
     if (threadIdx.x == 0) {
-      __threadfence();
-      atomicAdd(ctr, 1u);
       if (!dead) {
         const uint32_t want = n * gridDim.x;
         const long long t0 = clock64();
-        while (*reinterpret_cast<volatile uint32_t*>(ctr) < want) {
-          __nanosleep(64);
+        while (ld_acquire_u32(ctr) < want) {
           if (clock64() - t0 > kBarrierLimitCycles) { dead = true; raise_status(status, kStatusWaitTimeout); break; }
         }
-        __threadfence();
       }
       *shared_dead = dead ? 1 : 0;
     }
     __syncthreads();
     dead = *shared_dead != 0;
-    asm volatile("fence.proxy.async.global;" ::: "memory");
   }
 };
 
@@ -114,58 +170,89 @@ __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
-__device__ __forceinline__ void ldsm_x2(uint32_t (&r)[2], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+__device__ __forceinline__ void mma_bf16(float (&c)[8], int o, const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+               : "+f"(c[o]), "+f"(c[o + 1]), "+f"(c[o + 2]), "+f"(c[o + 3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// One 16 x 16 output tile over K (a multiple of 32): rows m0.. of A (row-major, lda bytes per row) times rows
-// n0 .. n0 + 15 of W (row-major [n][k], ldw bytes per row), both in shared memory. c0 holds columns n0 .. n0 + 7, c1
-// columns n0 + 8 .. n0 + 15; fragment layout: lane l holds c[0], c[1] = (row m0 + l / 4, columns 2 (l % 4), + 1 of its
-// eight) and c[2], c[3] = the same columns of row + 8. Even and odd k-steps accumulate separately (four independent
-// chains of dependent mma instructions instead of one: with a few rows the tile is latency-bound) and are added at
-// the end.
-__device__ __forceinline__ void tile_16x16(float (&c0)[4], float (&c1)[4], const uint8_t* A, int lda, int m0, const uint8_t* W,
-                                           int ldw, int n0, int K, int lane) {
-  float e0[4] = {0.f, 0.f, 0.f, 0.f}, e1[4] = {0.f, 0.f, 0.f, 0.f}, o0[4] = {0.f, 0.f, 0.f, 0.f}, o1[4] = {0.f, 0.f, 0.f, 0.f};
-  // A: matrices (rows 0-7, k 0-7), (rows 8-15, k 0-7), (rows 0-7, k 8-15), (rows 8-15, k 8-15): lane l points at
-  // row (l % 16), k offset 8 (l / 16). W: (n 0-7, k 0-7), (n 0-7, k 8-15), (n 8-15, k 0-7), (n 8-15, k 8-15): lane l
-  // points at row (l % 8) + 8 (l / 16), k offset 8 ((l / 8) % 2).
-  const uint32_t a_addr = tc::smem_u32(A + (size_t)(m0 + (lane & 15)) * lda + (lane >> 4) * 16);
-  const uint32_t b_addr = tc::smem_u32(W + (size_t)(n0 + (lane & 7) + ((lane >> 4) << 3)) * ldw + ((lane >> 3) & 1) * 16);
-#pragma unroll 2
-  for (int k = 0; k < K; k += 32) {
+// One 16 x 16 output tile over a part of K (klen, a multiple of 32): rows m0.. of A (row-major, lda bytes per row) times
+// rows n0 .. n0 + 15 of W (row-major [n][k], ldw bytes per row), both in shared memory from the part's first column on.
+// Fragment layout of c: lane l holds c[0], c[1] = (row m0 + l / 4, columns n0 + 2 (l % 4), + 1), c[2], c[3] = the same
+// columns of row + 8, c[4..7] = the same eight columns further. Even and odd k-steps accumulate separately (four
+// independent chains of dependent mma instructions: with a few rows the tile is latency-bound) and are added at the end.
+__device__ __forceinline__ void tile_part(float (&c)[8], uint32_t a_addr, uint32_t b_addr, int klen) {
+  float o[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { c[i] = 0.f; o[i] = 0.f; }
+#pragma unroll 4
+  for (int k = 0; k < klen; k += 32) {
     uint32_t a[4], b[4], a2[4], b2[4];
     ldsm_x4(a, a_addr + k * 2);
     ldsm_x4(b, b_addr + k * 2);
     ldsm_x4(a2, a_addr + k * 2 + 32);
     ldsm_x4(b2, b_addr + k * 2 + 32);
-    const uint32_t bl[2] = {b[0], b[1]}, bh[2] = {b[2], b[3]}, bl2[2] = {b2[0], b2[1]}, bh2[2] = {b2[2], b2[3]};
-    mma_bf16(e0, a, bl);
-    mma_bf16(e1, a, bh);
-    mma_bf16(o0, a2, bl2);
-    mma_bf16(o1, a2, bh2);
+    mma_bf16(c, 0, a, b[0], b[1]);
+    mma_bf16(c, 4, a, b[2], b[3]);
+    mma_bf16(o, 0, a2, b2[0], b2[1]);
+    mma_bf16(o, 4, a2, b2[2], b2[3]);
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) { c0[i] = e0[i] + o0[i]; c1[i] = e1[i] + o1[i]; }
+  for (int i = 0; i < 8; ++i) c[i] += o[i];
+}
+
+// How the tiles of a product are shared out between the warps: `groups` warps take a tile, a range of klen columns of K
+// each.
+struct Share { int tiles, groups, klen; };
+__device__ __forceinline__ Share share_of(int tiles, int K) {
+  int groups = kMaxGroups;
+  while (groups > 1 && (groups * tiles > kWarps || groups * 32 > K)) groups >>= 1;
+  return Share{tiles, groups, K / groups};
+}
+// Range g of tile (mt, nt).
+__device__ __forceinline__ void tile_group(float (&c)[8], const Share& sh, int g, const uint8_t* A, int lda, int mt, const uint8_t* W,
+                                           int ldw, int nt, int lane) {
+  // A: matrices (rows 0-7, k 0-7), (rows 8-15, k 0-7), (rows 0-7, k 8-15), (rows 8-15, k 8-15): lane l points at
+  // row (l % 16), k offset 8 (l / 16). W: (n 0-7, k 0-7), (n 0-7, k 8-15), (n 8-15, k 0-7), (n 8-15, k 8-15): lane l
+  // points at row (l % 8) + 8 (l / 16), k offset 8 ((l / 8) % 2).
+  const uint32_t k0 = (uint32_t)(g * sh.klen) * 2;
+  const uint32_t a_addr = tc::smem_u32(A + (size_t)(mt * 16 + (lane & 15)) * lda + (lane >> 4) * 16) + k0;
+  const uint32_t b_addr = tc::smem_u32(W + (size_t)(nt * 16 + (lane & 7) + ((lane >> 4) << 3)) * ldw + ((lane >> 3) & 1) * 16) + k0;
+  tile_part(c, a_addr, b_addr, sh.klen);
+}
+// Partial sums of the groups: element e = 32 j + lane of (group g, tile) at ((g * tiles + tile) * 256 + e).
+__device__ __forceinline__ void put_part(float* part, const Share& sh, int g, int tile, int lane, const float (&c)[8]) {
+  float* o = part + (g * sh.tiles + tile) * 256 + lane;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) o[32 * j] = c[j];
+}
+__device__ __forceinline__ float sum_groups(const float* q, int stride, int groups) {
+  if (groups == 1) return q[0];
+  if (groups == 2) return q[0] + q[stride];
+  if (groups == 4) return (q[0] + q[stride]) + (q[2 * stride] + q[3 * stride]);
+  return ((q[0] + q[stride]) + (q[2 * stride] + q[3 * stride])) + ((q[4 * stride] + q[5 * stride]) + (q[6 * stride] + q[7 * stride]));
+}
+// Item i (0 .. 128 tiles - 1) of a reduced product: the pair of adjacent columns (row, col), (row, col + 1) of a tile.
+struct Pair { int row, col; float a, b; };
+__device__ __forceinline__ Pair take_pair(const float* part, const Share& sh, int i, int m_tiles) {
+  const int tile = i >> 7, q = (i >> 5) & 3, l = i & 31;
+  const float* e = part + tile * 256 + q * 64 + l;           // j = 2 q: columns 8 (q / 2) .., rows 8 (q % 2) ..
+  return Pair{(tile % m_tiles) * 16 + (l >> 2) + (q & 1) * 8, (tile / m_tiles) * 16 + (q >> 1) * 8 + 2 * (l & 3),
+              sum_groups(e, sh.tiles * 256, sh.groups), sum_groups(e + 32, sh.tiles * 256, sh.groups)};
 }
 
 // ---- shared-memory staging --------------------------------------------------------------------
 // `rows` rows of `row_bytes` bytes (a multiple of 16), `src_stride` bytes apart in global memory, to rows
-// `row_bytes + kPadBytes` apart in shared memory; completion is counted on `bar`. Called by all lanes of warp 0:
-// lane 0 announces the bytes, then the lanes issue one bulk copy per row.
-__device__ __forceinline__ void stage_rows(uint8_t* dst, const void* src, int rows, int row_bytes, int64_t src_stride,
-                                           uint64_t* bar, int lane) {
-  tc::fence_async_smem();          // earlier reads of the region (ordered by a barrier) come before the copies into it
-  if (lane == 0) tc::mbar_expect_tx(bar, (uint32_t)rows * (uint32_t)row_bytes);
-  __syncwarp();
-  const uint8_t* s = static_cast<const uint8_t*>(src);
-  for (int r = lane; r < rows; r += 32)
-    bulk_g2s(dst + (size_t)r * (row_bytes + kPadBytes), s + (int64_t)r * src_stride, (uint32_t)row_bytes, bar);
+// `row_bytes + kPadBytes` apart in shared memory; completion is counted on `bar`. All threads of the CTA call it: one
+// announces the bytes, and the bulk copies, one per row, are spread over the warps (a warp issues its lanes' copies one
+// after the other: 32 of them from one warp took 0.8 us).
+__device__ __forceinline__ void stage_rows(uint8_t* dst, const void* src, int rows, int row_bytes, int64_t src_stride, uint64_t* bar) {
+  const int r = (threadIdx.x & 31) * kWarps + (threadIdx.x >> 5);
+  if (r < rows) {
+    tc::fence_async_smem();        // earlier reads of the region (ordered by a barrier) come before the copies into it
+    if (r == 0) tc::mbar_expect_tx(bar, (uint32_t)rows * (uint32_t)row_bytes);
+    bulk_g2s(dst + (size_t)r * (row_bytes + kPadBytes), static_cast<const uint8_t*>(src) + (int64_t)r * src_stride, (uint32_t)row_bytes, bar);
+  }
 }
 
 // Bounded wait on a phase of `bar`; all threads of the CTA call it. False after a time-out.
@@ -174,328 +261,419 @@ __device__ __forceinline__ bool wait_stage(uint64_t* bar, uint32_t parity, uint3
   return tc::mbar_wait(bar, parity, status);
 }
 
-// ---- row phase: one CTA per sample row -------------------------------------------------------------
-// Sum over the CTA of one value per thread (all threads call it; `red` holds one float per warp).
-__device__ __forceinline__ float cta_sum(float v, float* red) {
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float t = 0.f;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) t += red[w];
-  __syncthreads();                         // red may be written again
-  return t;
-}
-
-// x_in = E[tok] (layer 0) or x + b2 of the previous layer + the partial sums of its down projection in slab order.
-// layer < L: the fused mixer step (LN1, Eq. 2 / Eq. 3 update of the cache, residual, LN2), leaving x and the
-// activation a. layer == L: a = LN_f(x_in). Thread i owns channels 4 i .. 4 i + 3 (d <= 1024): every global load
-// of the row is issued before the first reduction, so the phase costs a few memory latencies, not one per vector.
-template <typename ST>
-__device__ __forceinline__ void row_phase(const Params& p, int layer, int64_t row, int t, float* red) {
-  const int d = p.d, c = threadIdx.x * 4;
-  const bool on = c < d;
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 v = zero;
-  if (layer == 0) {
-    int tk = p.tok_in[row];
-    if (tk < 0 || tk >= p.V) {
-      if (threadIdx.x == 0) raise_status(p.status, kStatusTokenRange);
-      tk = tk < 0 ? 0 : p.V - 1;
-    }
-    if (on) v = ldg4(p.E + (int64_t)tk * d + c);
-  } else if (on) {
-    // written by other CTAs in this kernel: not through L1
-    float4 q[8];
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks)
-      q[ks] = ks < p.dn_kslabs ? __ldcg(reinterpret_cast<const float4*>(p.part + ((int64_t)ks * p.B + row) * d + c)) : zero;
-    v = __ldcg(reinterpret_cast<const float4*>(p.x + row * d + c));
-    const float4 bb = ldg4(layer_w(p, layer - 1).b2 + c);
-    v = make_float4(v.x + bb.x, v.y + bb.y, v.z + bb.z, v.w + bb.w);
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) v = make_float4(v.x + q[ks].x, v.y + q[ks].y, v.z + q[ks].z, v.w + q[ks].w);
-  }
-  const bool last = layer == p.L;
-  const LayerW w = layer_w(p, last ? 0 : layer);
-  // parameters and the cache row: independent of the statistics, so their loads overlap the reductions
-  float4 g1 = zero, b1 = zero, g2 = zero, b2n = zero, bt = zero, s = zero;
-  float al = 0.f, lm = 0.f;
-  int g = 0;
-  ST* Sr = nullptr;
-  if (on) {
-    if (last) {
-      g2 = ldg4(p.lnf_g + c); b2n = ldg4(p.lnf_b + c);
-    } else {
-      g = c / (d / p.h);
-      g1 = ldg4(w.ln1_g + c); b1 = ldg4(w.ln1_b + c); g2 = ldg4(w.ln2_g + c); b2n = ldg4(w.ln2_b + c);
-      bt = ldg4(w.beta + (int64_t)t * d + c);
-      al = __ldg(w.alpha + (int64_t)g * p.n_ctx + t); lm = __ldg(w.lam + g);
-      Sr = reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)layer * p.layer_stride) + row * d + c;
-      s = ld4(Sr);
-    }
-  }
-  const float inv_d = 1.0f / (float)d;
-  if (!last) {
-    const float mean = cta_sum((v.x + v.y) + (v.z + v.w), red) * inv_d;
-    const float4 cd = on ? make_float4(v.x - mean, v.y - mean, v.z - mean, v.w - mean) : zero;
-    const float rstd = rsqrtf(cta_sum((cd.x * cd.x + cd.y * cd.y) + (cd.z * cd.z + cd.w * cd.w), red) * inv_d + p.eps);
-    if (on) {
-      const float4 z = norm4(v, mean, rstd, g1, b1);
-      float4 y, sn;
-      if (g < (p.h >> 1)) {       // row-repeat head, Eq. 2: y = a z + b + S ; S' = l (S + a z)
-        const float4 u = make_float4(al * z.x, al * z.y, al * z.z, al * z.w);
-        y = make_float4(u.x + bt.x + s.x, u.y + bt.y + s.y, u.z + bt.z + s.z, u.w + bt.w + s.w);
-        sn = make_float4(lm * (s.x + u.x), lm * (s.y + u.y), lm * (s.z + u.z), lm * (s.w + u.w));
-      } else {                    // column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
-        const float4 q = make_float4(z.x + s.x, z.y + s.y, z.z + s.z, z.w + s.w);
-        y = make_float4(al * q.x + bt.x, al * q.y + bt.y, al * q.z + bt.z, al * q.w + bt.w);
-        sn = make_float4(lm * q.x, lm * q.y, lm * q.z, lm * q.w);
-      }
-      st4(Sr, sn);
-      v = make_float4(v.x + y.x, v.y + y.y, v.z + y.z, v.w + y.w);
-      st4(p.x + row * d + c, v);
-    }
-  }
-  const float mean = cta_sum((v.x + v.y) + (v.z + v.w), red) * inv_d;
-  const float4 cd = on ? make_float4(v.x - mean, v.y - mean, v.z - mean, v.w - mean) : zero;
-  const float rstd = rsqrtf(cta_sum((cd.x * cd.x + cd.y * cd.y) + (cd.z * cd.z + cd.w * cd.w), red) * inv_d + p.eps);
-  if (on) st4(p.a + row * d + c, norm4(v, mean, rstd, g2, b2n));
-}
-
-// Shared memory: 128 bytes of mbarriers | activation rows (kMaxRows padded rows) | weight rows.
-__host__ __device__ inline int act_region_bytes(int d, int klen) {
-  const int k = d > klen ? d : klen;
-  return (kMaxRows * (2 * k + kPadBytes) + 127) / 128 * 128;
-}
-__host__ __device__ inline int weight_region_bytes(int d, int up_cols, int dn_cols, int klen) {
-  int b = up_cols * (2 * d + kPadBytes);
-  const int dn = dn_cols * (2 * klen + kPadBytes), lm = 2 * kLmChunkCols * (2 * d + kPadBytes) + 4096;   // + partial sums
-  b = b > dn ? b : dn;
-  return b > lm ? b : lm;
-}
-
 __device__ __forceinline__ unsigned long long pack_best(float v, int col) {
   return ((unsigned long long)order_key(v) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)col);
 }
 
-template <typename ST>
-__global__ void __launch_bounds__(kThreads, 1) step_small_kernel(const Params p) {
+// ---- row phase: four warps per row ---------------------------------------------------------------
+// LayerNorm statistics of the row that the four warps of a group hold, 4 NT values per thread (`on`: how many of its NT
+// vectors are inside the row): mean and sum of squared deviations per thread, merged pairwise (Chan et al.) over lanes
+// and warps in one pass of shuffles and one barrier. `slot`: eight floats that this group uses for these statistics
+// only (they are written again a whole row later).
+template <int d, int NT>
+__device__ __forceinline__ void group_stats(const float4 (&v)[NT], float eps, float* slot, int group, float& mean, float& rstd) {
+  constexpr bool full = d == NT * 512;                   // every thread holds NT whole vectors
+  float m, q = 0.f, n = 0.f;
+  if (full) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < NT; ++i) s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+    n = 4.f * NT;
+    m = s * (1.0f / (4.f * NT));
+  } else {                                               // (d = 256, 768: the last vector of a thread may be outside)
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < NT; ++i)
+      if ((threadIdx.x & 127) * 4 + 512 * i < d) { s += (v[i].x + v[i].y) + (v[i].z + v[i].w); n += 4.f; }
+    m = n > 0.f ? s / n : 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    if (full || (threadIdx.x & 127) * 4 + 512 * i < d) {
+      const float a = v[i].x - m, b = v[i].y - m, c = v[i].z - m, e = v[i].w - m;
+      q += (a * a + b * b) + (c * c + e * e);
+    }
+  }
+  auto merge = [](float& m, float& q, float& n, float m2, float q2, float n2) {
+    const float dm = m2 - m, nn = n + n2;
+    if (full) { q += q2 + dm * dm * (0.5f * n); m = 0.5f * (m + m2); }
+    else if (nn > 0.f) { const float f = n2 / nn; q += q2 + dm * dm * n * f; m = fmaf(dm, f, m); }
+    n = nn;
+  };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, m, o), q2 = __shfl_xor_sync(0xffffffffu, q, o);
+    const float n2 = full ? n : __shfl_xor_sync(0xffffffffu, n, o);
+    merge(m, q, n, m2, q2, n2);
+  }
+  if ((threadIdx.x & 31) == 0) {                         // (the lanes may differ in the last bit: lane 0's values count)
+    const int w = (threadIdx.x >> 5) & 3;
+    slot[w] = m;
+    slot[4 + w] = q;
+    if (!full) slot[8 + w] = n;
+  }
+  asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
+  float n0 = full ? n : slot[8], n1 = full ? n : slot[9], n2 = full ? n : slot[10], n3 = full ? n : slot[11];
+  float ma = slot[0], qa = slot[4], mb = slot[2], qb = slot[6];
+  merge(ma, qa, n0, slot[1], slot[5], n1);
+  merge(mb, qb, n2, slot[3], slot[7], n3);
+  merge(ma, qa, n0, mb, qb, n2);
+  mean = ma;
+  rstd = rsqrtf(qa * (1.0f / (float)d) + eps);
+}
+
+// Thread i of a group owns channels 4 i .. 4 i + 3 (and 512 further) of every row. What a layer asks of the parameters
+// for these channels is fetched once for all rows, while the CTA waits at the grid barrier before the row phase.
+template <int NT>
+struct RowParams {
+  float4 g1[NT], b1[NT], g2[NT], b2[NT];
+  float4 bt[NT];       // beta_t, and the head scalars as the multipliers of z before and of the sum after (one is 1)
+  float a1[NT], a2[NT], lm[NT];
+};
+template <int d, int NT>
+__device__ __forceinline__ void load_position(const Params& p, const LayerW& w, int t, RowParams<NT>& r) {
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const int c = (threadIdx.x & 127) * 4 + 512 * i;
+    if (c < d) {
+      const int g = c / (d / p.h);
+      r.bt[i] = ldg4(w.beta + (int64_t)t * d + c);
+      const float al = __ldg(w.alpha + (int64_t)g * p.n_ctx + t);
+      const bool is_row = g < (p.h >> 1);
+      r.a1[i] = is_row ? al : 1.0f;
+      r.a2[i] = is_row ? 1.0f : al;
+      r.lm[i] = __ldg(w.lam + g);
+    }
+  }
+}
+// Parameters of layer l (l == L: of the final norm).
+template <int d, int NT>
+__device__ __forceinline__ void load_row_params(const Params& p, int l, int t, RowParams<NT>& r) {
+  const bool last = l == p.L;
+  const LayerW w = layer_w(p, last ? 0 : l);
+  const float *g2 = last ? p.lnf_g : w.ln2_g, *b2 = last ? p.lnf_b : w.ln2_b;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const int c = (threadIdx.x & 127) * 4 + 512 * i;
+    if (c < d) {
+      r.g2[i] = ldg4(g2 + c); r.b2[i] = ldg4(b2 + c);
+      if (!last) { r.g1[i] = ldg4(w.ln1_g + c); r.b1[i] = ldg4(w.ln1_b + c); }
+    }
+  }
+  if (!last && p.pos == nullptr) load_position<d, NT>(p, w, t, r);
+}
+
+template <int d, typename ST>
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) step_small_kernel(const Params p) {
   extern __shared__ __align__(128) uint8_t sm[];
-  uint64_t* barA = reinterpret_cast<uint64_t*>(sm);
-  uint64_t* barW = barA + 1;                             // two stages
-  float* red32 = reinterpret_cast<float*>(sm + 96);     // one float per warp for the row-phase reductions
-  uint8_t* sA = sm + 128;
-  uint8_t* sW = sA + act_region_bytes(p.d, p.dn_klen);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cta = blockIdx.x, G = gridDim.x;
-  const int d = p.d, F = p.F, B = p.B;
-  if (threadIdx.x == 0) {
-    tc::mbar_init(barA, 1); tc::mbar_init(&barW[0], 1); tc::mbar_init(&barW[1], 1);
+  uint64_t* bar1 = reinterpret_cast<uint64_t*>(sm);      // W1 slab
+  uint64_t* bar2 = bar1 + 1;                             // W2 slab
+  uint64_t* barA = bar1 + 2;                             // rows of H
+  uint64_t* barR = bar1 + 3;                             // activation rows from the other CTAs of the cluster
+  uint64_t* barL = bar1 + 4;                             // LM-head stages
+  float* red = reinterpret_cast<float*>(sm + 128);       // row-phase sums: four groups x 32
+  uint8_t* sA = sm + kHeadBytes;
+  uint8_t* sW1 = sm + p.off_w1;
+  uint8_t* sW2 = sm + p.off_w2;
+  float* part = reinterpret_cast<float*>(sm + p.off_part);
+  uint8_t* recv = sm + p.off_recv;
+  uint8_t* xo = sm + p.off_xo;
+  ST* sS = reinterpret_cast<ST*>(sm + p.off_s);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int cta = blockIdx.x, cl = cta / kCluster, rank = (int)tc::cluster_ctarank();
+  const int F = p.F, B = p.B, mp = (B + 15) / 16 * 16, m_tiles = mp / 16;
+  constexpr int ld_d = 2 * d + kPadBytes, ncols = d / kClusters, gw = ncols / kCluster;
+  const int klen = dn_klen(F), ld_k = 2 * klen + kPadBytes;
+  const int ucols = up_cols(F), u0 = (cl * kCluster + rank) * ucols;
+  const int n0 = cl * ncols, k0 = rank * klen;
+  const int chunks_all = (p.V + kLmChunkCols - 1) / kLmChunkCols;
+  const int lm_c0 = (int)((int64_t)cta * chunks_all / kGrid), lm_chunks = (int)((int64_t)(cta + 1) * chunks_all / kGrid) - lm_c0;
+  constexpr int lm_stage = kLmChunkCols * ld_d;
+  const bool alone = B <= kAloneRows, one_region = p.off_w1 == p.off_w2;
+
+  if (tid == 0) {
+    for (int i = 0; i < 4 + kLmMaxStages; ++i) tc::mbar_init(bar1 + i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
-  uint32_t parA = 0, parW0 = 0, parW1 = 0;
-  GridBarrier gb{p.bar, 0u, false, p.status, reinterpret_cast<int*>(sm + 64)};
-  const int t = p.ctr != nullptr ? p.ctr[kCtrPos] : p.t;
-  const int m_tiles = (B + 15) >> 4;
-  const int ld_d = 2 * d + kPadBytes;
+  tc::cluster_sync();                                    // every CTA of the cluster is up before anyone writes into its memory
+  uint32_t par1 = 0, par2 = 0;
+  GridBarrier gb{p.bar, 0u, false, p.status, reinterpret_cast<int*>(sm + 112)};
+  const int t_all = p.ctr != nullptr ? p.ctr[kCtrPos] : p.t;
+  auto t_of = [&](int row) { return p.pos != nullptr ? min(max(p.pos[row], 0), p.n_ctx - 1) : t_all; };
 
-  // this CTA's slabs
-  const bool up_on = cta < p.up_ctas;
-  const int up_n0 = cta * p.up_cols;
-  const int up_n = up_on ? (F - up_n0 < p.up_cols ? F - up_n0 : p.up_cols) : 0;
-  const bool dn_on = cta < p.dn_nslabs * p.dn_kslabs;
-  const int dn_ns = cta % p.dn_nslabs, dn_ks = cta / p.dn_nslabs;
-  const int dn_k0 = dn_ks * p.dn_klen;
-  const int dn_k = dn_on ? (F - dn_k0 < p.dn_klen ? F - dn_k0 : p.dn_klen) : 0;
-  const int ld_k = 2 * dn_k + kPadBytes;
-  const bool lm_on = cta < p.lm_ctas;
-  const int lm_n0 = cta * p.lm_cols;
-  const int lm_n = lm_on ? (p.V - lm_n0 < p.lm_cols ? p.V - lm_n0 : p.lm_cols) : 0;
-  const int lm_chunks = (lm_n + kLmChunkCols - 1) / kLmChunkCols;
-  const int lm_stage = kLmChunkCols * ld_d;
-
-  auto stage_up = [&](int l) {            // warp 0: W1 rows of this CTA's columns
-    if (up_on && warp == 0) stage_rows(sW, layer_w(p, l).W1 + (int64_t)up_n0 * d, up_n, 2 * d, 2 * (int64_t)d, &barW[0], lane);
+  auto stage_up = [&](int l) {            // W1 rows of this CTA's columns
+    stage_rows(sW1, layer_w(p, l).W1 + (int64_t)u0 * d, ucols, 2 * d, 2 * (int64_t)d, bar1);
   };
-  auto stage_dn = [&](int l) {            // warp 0: W2 rows of the n-slab, columns of the k-slab
-    if (dn_on && warp == 0)
-      stage_rows(sW, layer_w(p, l).W2 + (int64_t)dn_ns * p.dn_cols * F + dn_k0, p.dn_cols, 2 * dn_k, 2 * (int64_t)F, &barW[0], lane);
+  auto stage_dn = [&](int l) {            // W2 rows of the cluster's columns, this rank's part of K
+    stage_rows(sW2, layer_w(p, l).W2 + (int64_t)n0 * F + k0, ncols, 2 * klen, 2 * (int64_t)F, bar2);
   };
-  auto stage_lm = [&](int ch) {           // warp 0: one chunk of LM-head rows into stage ch % 2
-    if (lm_on && warp == 0 && ch < lm_chunks) {
-      const int rows = lm_n - ch * kLmChunkCols < kLmChunkCols ? lm_n - ch * kLmChunkCols : kLmChunkCols;
-      stage_rows(sW + (ch & 1) * lm_stage, p.W_lm + (int64_t)(lm_n0 + ch * kLmChunkCols) * d, rows, 2 * d, 2 * (int64_t)d,
-                 &barW[ch & 1], lane);
+  auto stage_lm = [&](int ch) {           // one chunk of LM-head rows into stage ch % lm_stages
+    if (ch < lm_chunks) {
+      const int r0 = (lm_c0 + ch) * kLmChunkCols, rows = min(kLmChunkCols, p.V - r0), s = ch % p.lm_stages;
+      stage_rows(sW1 + s * lm_stage, p.W_lm + (int64_t)r0 * d, rows, 2 * d, 2 * (int64_t)d, barL + s);
+    }
+  };
+  // the row this CTA writes the cache of, and the L2 prefetch of what layer l will ask for
+  const int own_row = cl * kCluster + rank;
+  auto prefetch_layer = [&](int l) {
+    const LayerW w = layer_w(p, l);
+    if (warp == 1 && own_row < B) {
+      const uint8_t* r = static_cast<const uint8_t*>(p.S) + (int64_t)l * p.layer_stride + (int64_t)own_row * d * sizeof(ST);
+      for (int i = lane * 128; i < d * (int)sizeof(ST); i += 32 * 128) prefetch_l2(r + i);
+      if (p.pos != nullptr || own_row == 0) {
+        const int t = t_of(own_row);
+        const float* bt = w.beta + (int64_t)t * d;
+        for (int i = lane * 32; i < d; i += 32 * 32) prefetch_l2(bt + i);
+        if (lane < p.h) { prefetch_l2(w.alpha + (int64_t)lane * p.n_ctx + t); prefetch_l2(w.lam + lane); }
+      }
+    }
+    if (warp == 2) {                      // CTA i takes one of the vectors, every CTA its part of the bias
+      constexpr int lines = d * 4 / 128;
+      if (cta < 4 && lane < lines) {
+        const float* q = cta == 0 ? w.ln1_g : cta == 1 ? w.ln1_b : cta == 2 ? w.ln2_g : w.ln2_b;
+        prefetch_l2(q + lane * 32);
+      }
+      if (cta == 4 && lane < lines) prefetch_l2(w.b2 + lane * 32);
+      if (lane == 0) for (int i = 0; i < ucols; i += 32) prefetch_l2(w.b1 + u0 + i);
     }
   };
 
+  constexpr int NT = (d + 511) / 512;
+  const int group = warp >> 2, c0 = (tid & 127) * 4;
+  RowParams<NT> rp;
+  load_row_params<d, NT>(p, 0, t_all, rp);
+  // bytes of the rows that the other CTAs of the cluster send per row phase
+  const uint32_t peer_bytes = (uint32_t)(B - (B - rank + kCluster - 1) / kCluster) * (2 * d);
+  if (tid == 0 && !alone) tc::mbar_expect_tx(barR, peer_bytes);
   stage_up(0);
-  for (int l = 0; l < p.L; ++l) {
-    // ---- token mixer: one warp per row ----
-    for (int64_t r = cta; r < B; r += G) row_phase<ST>(p, l, r, t, red32);
-    gb.sync();
+  if (!one_region) stage_dn(0);
+  prefetch_layer(0);
+  const Share up = share_of(m_tiles * ((ucols + 15) / 16), d), dn = share_of(m_tiles * ((ncols + 15) / 16), klen);
+  for (int l = 0;; ++l) {
+    const bool last = l == p.L;
+    const LayerW w = layer_w(p, last ? 0 : l);
+    if (l + 1 < p.L) prefetch_layer(l + 1);
+    // ---- rows (after the last layer: the final norm). The activation row goes to its place here or in all CTAs of the
+    //      cluster, x + y of the cluster's own columns to the CTAs that will add the down projection to them ----
+    {
+      const ST* Sl = reinterpret_cast<const ST*>(static_cast<const uint8_t*>(p.S) + (int64_t)l * p.layer_stride);
+      float* slot = red + group * 32;
+      const int step = alone ? kMaxRows : 4 * kCluster;
+      float4 v[NT], s[NT];
+      auto load = [&](int row) {
+        int tk = 0;
+        if (l == 0) {
+          tk = p.tok_in[row];
+          if (tk < 0 || tk >= p.V) {
+            if (c0 == 0) raise_status(p.status, kStatusTokenRange);
+            tk = tk < 0 ? 0 : p.V - 1;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+          const int c = c0 + 512 * i;
+          if (c < d) {
+            if (l == 0) v[i] = ldg4(p.E + (int64_t)tk * d + c);
+            else v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c));    // other CTAs wrote it: not through L1
+            if (!last) s[i] = ld4(Sl + (int64_t)row * d + c);
+          }
+        }
+      };
+      int row = alone ? group : rank + group * kCluster;
+      if (row < B) load(row);
+      for (; row < B; row += step) {
+        float mean, rstd;
+        if (!last) {
+          if (p.pos != nullptr) load_position<d, NT>(p, w, t_of(row), rp);
+          group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
+          const float nmr = -mean * rstd;
+#pragma unroll
+          for (int i = 0; i < NT; ++i) {
+            const int c = c0 + 512 * i;
+            if (c < d) {
+              const float4 g = rp.g1[i], bb = rp.b1[i], bt = rp.bt[i];
+              const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
+                                           fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
+              // row-repeat head, Eq. 2: y = (a z + S) + b ; S' = l (S + a z).  column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
+              const float a1 = rp.a1[i], a2 = rp.a2[i], lm = rp.lm[i];
+              const float4 u = make_float4(fmaf(a1, z.x, s[i].x), fmaf(a1, z.y, s[i].y), fmaf(a1, z.z, s[i].z), fmaf(a1, z.w, s[i].w));
+              if (row == own_row) st4(sS + c, make_float4(lm * u.x, lm * u.y, lm * u.z, lm * u.w));
+              v[i] = make_float4(v[i].x + fmaf(a2, u.x, bt.x), v[i].y + fmaf(a2, u.y, bt.y), v[i].z + fmaf(a2, u.z, bt.z),
+                                 v[i].w + fmaf(a2, u.w, bt.w));
+              const int o = c - n0;                                // column inside the cluster's slab
+              if (o >= 0 && o < ncols) {
+                const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  const int q = (o + k) / gw;                      // the rank that owns this column
+                  const uint32_t at = tc::smem_u32(xo) + (uint32_t)(row * gw + (o + k) % gw) * 4;
+                  if (!alone || q == rank) st_cluster_f32(tc::mapa(at, (uint32_t)q), e[k]);
+                }
+              }
+            }
+          }
+        }
+        group_stats<d, NT>(v, p.eps, slot + 16, group, mean, rstd);
+        const float nmr2 = -mean * rstd;
+        uint2 u[NT];
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+          const float4 g = rp.g2[i], bb = rp.b2[i];
+          const __nv_bfloat162 lo = __floats2bfloat162_rn(fmaf(fmaf(v[i].x, rstd, nmr2), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr2), g.y, bb.y));
+          const __nv_bfloat162 hi = __floats2bfloat162_rn(fmaf(fmaf(v[i].z, rstd, nmr2), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr2), g.w, bb.w));
+          u[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        }
+        if (row + step < B) load(row + step);
+        uint8_t* at = sA + (size_t)row * ld_d;
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+          if (c0 + 512 * i < d) *reinterpret_cast<uint2*>(at + (c0 + 512 * i) * 2) = u[i];
+        if (!alone) {
+          // (one bulk copy per peer: eight-byte stores into the peers' memory took 1.7 us per sixteen rows)
+          tc::fence_async_smem();
+          asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
+          const int r = tid & 127;
+          if (r < kCluster && r != rank)
+            bulk_s2s(tc::mapa(tc::smem_u32(at), (uint32_t)r), at, 2 * d, tc::mapa(tc::smem_u32(barR), (uint32_t)r));
+        }
+      }
+      __syncthreads();                     // this CTA's rows
+      if (!alone) {                        // the others'
+        if (!wait_stage(barR, (uint32_t)l & 1u, p.status, gb.dead)) gb.dead = true;
+      }
+    }
+    if (last) break;
 
     // ---- up projection: H[:, slab] = gelu(a W1[slab]^T + b1) ----
-    if (up_on) {
-      if (warp == 0) stage_rows(sA, p.a, B, 2 * d, 2 * (int64_t)d, barA, lane);
-      bool ok = wait_stage(barA, parA, p.status, gb.dead);
-      ok = wait_stage(&barW[0], parW0, p.status, gb.dead) && ok;
-      parA ^= 1u; parW0 ^= 1u;
-      if (!ok) gb.dead = true;
-      const float* b1 = layer_w(p, l).b1;
-      const int n16 = (up_n + 15) >> 4, tiles = m_tiles * n16;
-      for (int tile = warp; ok && tile < tiles; tile += kWarps) {
-        const int mt = tile % m_tiles, nt = tile / m_tiles;
-        float c0[4], c1[4];
-        tile_16x16(c0, c1, sA, ld_d, mt * 16, sW, ld_d, nt * 16, d, lane);
-        const int r0 = mt * 16 + (lane >> 2);
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          const float (&c)[4] = hf ? c1 : c0;
-          const int cl = nt * 16 + hf * 8 + 2 * (lane & 3);          // column inside the slab
-          if (cl < up_n) {
-            const int col = up_n0 + cl;
-            const float2 bb = __ldg(reinterpret_cast<const float2*>(b1 + col));
-            if (r0 < B)
-              *reinterpret_cast<__nv_bfloat162*>(p.H + (int64_t)r0 * F + col) =
-                  __floats2bfloat162_rn(tc::gelu_fast(c[0] + bb.x), tc::gelu_fast(c[1] + bb.y));
-            if (r0 + 8 < B)
-              *reinterpret_cast<__nv_bfloat162*>(p.H + (int64_t)(r0 + 8) * F + col) =
-                  __floats2bfloat162_rn(tc::gelu_fast(c[2] + bb.x), tc::gelu_fast(c[3] + bb.y));
-          }
-        }
+    if (!wait_stage(bar1, par1, p.status, gb.dead)) gb.dead = true;
+    par1 ^= 1u;
+    if (!one_region && l > 0) stage_dn(l); // (W2's place is free since the previous layer; issued while a barrier is waited
+                                           //  for, the weight stream made the barrier itself slower, 1.3 -> 2.6 us)
+    if (warp < up.tiles * up.groups) {
+      const int tile = warp % up.tiles, g = warp / up.tiles;
+      float c[8];
+      tile_group(c, up, g, sA, ld_d, tile % m_tiles, sW1, ld_d, tile / m_tiles, lane);
+      put_part(part, up, g, tile, lane, c);
+    }
+    __syncthreads();                       // partial sums are visible, the weight rows have been read
+    for (int i = tid; i < up.tiles * 128; i += kThreads) {
+      const Pair q = take_pair(part, up, i, m_tiles);
+      if (q.row < B && q.col < ucols) {
+        const float2 bb = __ldg(reinterpret_cast<const float2*>(w.b1 + u0 + q.col));
+        *reinterpret_cast<__nv_bfloat162*>(p.H + (int64_t)q.row * F + u0 + q.col) =
+            __floats2bfloat162_rn(tc::gelu_fast(q.a + bb.x), tc::gelu_fast(q.b + bb.y));
       }
     }
-    __syncthreads();                       // the weight rows have been read: the region may be refilled
-    stage_dn(l);
-    gb.sync();
+    gb.sync([&] { if (one_region) stage_dn(l); });
 
-    // ---- down projection: part[ks][:, n-slab] = H[:, k-slab] W2[n-slab, k-slab]^T ----
-    if (dn_on) {
-      if (warp == 0) stage_rows(sA, p.H + dn_k0, B, 2 * dn_k, 2 * (int64_t)F, barA, lane);
-      bool ok = wait_stage(barA, parA, p.status, gb.dead);
-      ok = wait_stage(&barW[0], parW0, p.status, gb.dead) && ok;
-      parA ^= 1u; parW0 ^= 1u;
-      if (!ok) gb.dead = true;
-      float* out = p.part + (int64_t)dn_ks * B * d;
-      const int tiles = m_tiles * (p.dn_cols >> 4);
-      for (int tile = warp; ok && tile < tiles; tile += kWarps) {
-        const int mt = tile % m_tiles, nt = tile / m_tiles;
-        float c0[4], c1[4];
-        tile_16x16(c0, c1, sA, ld_k, mt * 16, sW, ld_k, nt * 16, dn_k, lane);
-        const int col = dn_ns * p.dn_cols + nt * 16 + 2 * (lane & 3), r0 = mt * 16 + (lane >> 2);
-        if (r0 < B) {
-          *reinterpret_cast<float2*>(out + (int64_t)r0 * d + col) = make_float2(c0[0], c0[1]);
-          *reinterpret_cast<float2*>(out + (int64_t)r0 * d + col + 8) = make_float2(c1[0], c1[1]);
-        }
-        if (r0 + 8 < B) {
-          *reinterpret_cast<float2*>(out + (int64_t)(r0 + 8) * d + col) = make_float2(c0[2], c0[3]);
-          *reinterpret_cast<float2*>(out + (int64_t)(r0 + 8) * d + col + 8) = make_float2(c1[2], c1[3]);
-        }
-      }
+    // ---- down projection: this rank's part of K for the cluster's columns ----
+    asm volatile("fence.proxy.async.global;" ::: "memory");     // H was written through the generic proxy
+    stage_rows(sA, p.H + k0, B, 2 * klen, 2 * (int64_t)F, barA);
+    if (own_row < B) {                     // nobody reads the old cache row any more
+      ST* Sg = reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + (int64_t)own_row * d;
+      const uint4* src = reinterpret_cast<const uint4*>(sS);
+      if (tid < d * (int)sizeof(ST) / 16) reinterpret_cast<uint4*>(Sg)[tid] = src[tid];
     }
-    __syncthreads();
-    if (l + 1 < p.L) stage_up(l + 1);
-    else { stage_lm(0); stage_lm(1); }
-    gb.sync();
-  }
-
-  // ---- final norm ----
-  for (int64_t r = cta; r < B; r += G) row_phase<ST>(p, p.L, r, t, red32);
-  gb.sync();
-
-  // ---- LM head over this CTA's vocabulary slab, chunk by chunk through two stages ----
-  if (lm_on) {
-    if (warp == 0) stage_rows(sA, p.a, B, 2 * d, 2 * (int64_t)d, barA, lane);
-    bool ok = wait_stage(barA, parA, p.status, gb.dead);
-    parA ^= 1u;
-    // Every chunk is one 16-column tile per 16 rows. Warp w takes row tile w % 4 and half w / 4 of K; the upper
-    // halves' partial sums go through shared memory to the lower warps, which own the results.
-    const int mt = warp & 3, kh = warp >> 2;
-    const int k_half = d >> 1;
-    float* xch = reinterpret_cast<float*>(sW + 2 * lm_stage);   // [4 row tiles][32 lanes][8] partial sums
-    float bv0 = -INFINITY, bv1 = -INFINITY;
-    int bi0 = 0x7fffffff, bi1 = 0x7fffffff;
-    bool bad = false;
-    for (int ch = 0; ch < lm_chunks; ++ch) {
-      const int s = ch & 1;
-      ok = wait_stage(&barW[s], s ? parW1 : parW0, p.status, gb.dead || !ok) && ok;
-      if (s) parW1 ^= 1u; else parW0 ^= 1u;
-      const int rows = lm_n - ch * kLmChunkCols < kLmChunkCols ? lm_n - ch * kLmChunkCols : kLmChunkCols;
-      float c0[4], c1[4];
-      const bool work = ok && mt < m_tiles;
-      if (work) {
-        tile_16x16(c0, c1, sA + kh * k_half * 2, ld_d, mt * 16, sW + s * lm_stage + kh * k_half * 2, ld_d, 0, k_half, lane);
-        if (kh == 1) {
-          float4* o = reinterpret_cast<float4*>(xch + (mt * 32 + lane) * 8);
-          o[0] = make_float4(c0[0], c0[1], c0[2], c0[3]);
-          o[1] = make_float4(c1[0], c1[1], c1[2], c1[3]);
-        }
-      }
-      __syncthreads();                                           // partial sums are visible; stage s has been read
-      stage_lm(ch + 2);
-      if (work && kh == 0) {
-        const float4* o = reinterpret_cast<const float4*>(xch + (mt * 32 + lane) * 8);
-        const float4 q0 = o[0], q1 = o[1];
-        c0[0] += q0.x; c0[1] += q0.y; c0[2] += q0.z; c0[3] += q0.w;
-        c1[0] += q1.x; c1[1] += q1.y; c1[2] += q1.z; c1[3] += q1.w;
-        const int col = lm_n0 + ch * kLmChunkCols + 2 * (lane & 3), r0 = mt * 16 + (lane >> 2);
-        const bool second = rows > 8;                            // V is a multiple of 8: a last chunk may hold 8 columns
-        if (p.logits != nullptr) {
-          if (r0 < B) {
-            *reinterpret_cast<float2*>(p.logits + (int64_t)r0 * p.V + col) = make_float2(c0[0], c0[1]);
-            if (second) *reinterpret_cast<float2*>(p.logits + (int64_t)r0 * p.V + col + 8) = make_float2(c1[0], c1[1]);
-          }
-          if (r0 + 8 < B) {
-            *reinterpret_cast<float2*>(p.logits + (int64_t)(r0 + 8) * p.V + col) = make_float2(c0[2], c0[3]);
-            if (second) *reinterpret_cast<float2*>(p.logits + (int64_t)(r0 + 8) * p.V + col + 8) = make_float2(c1[2], c1[3]);
-          }
-        }
-        // (rows past B of a partly filled tile hold whatever the shared memory held: not looked at)
-        if (r0 < B) bad |= !(c0[0] == c0[0]) | !(c0[1] == c0[1]) | (second & (!(c1[0] == c1[0]) | !(c1[1] == c1[1])));
-        if (r0 + 8 < B) bad |= !(c0[2] == c0[2]) | !(c0[3] == c0[3]) | (second & (!(c1[2] == c1[2]) | !(c1[3] == c1[3])));
-        if (c0[0] > bv0) { bv0 = c0[0]; bi0 = col; }            // ascending columns: the lowest among equals is kept
-        if (c0[1] > bv0) { bv0 = c0[1]; bi0 = col + 1; }
-        if (c0[2] > bv1) { bv1 = c0[2]; bi1 = col; }
-        if (c0[3] > bv1) { bv1 = c0[3]; bi1 = col + 1; }
-        if (second) {
-          if (c1[0] > bv0) { bv0 = c1[0]; bi0 = col + 8; }
-          if (c1[1] > bv0) { bv0 = c1[1]; bi0 = col + 9; }
-          if (c1[2] > bv1) { bv1 = c1[2]; bi1 = col + 8; }
-          if (c1[3] > bv1) { bv1 = c1[3]; bi1 = col + 9; }
-        }
-      }
-      __syncthreads();                                           // the partial sums have been taken
+    if (!wait_stage(bar2, par2, p.status, gb.dead)) gb.dead = true;
+    if (!wait_stage(barA, par2, p.status, gb.dead)) gb.dead = true;
+    par2 ^= 1u;
+    if (!one_region) {                     // the next weights for W1's place (used up): while this phase asks for nothing else
+      if (l + 1 < p.L) stage_up(l + 1);
+      else for (int ch = 0; ch < p.lm_stages_w1; ++ch) stage_lm(ch);
     }
-    if (!ok) gb.dead = true;
-    if (p.greedy) {
-      // per row: over the four lanes of a quad (their columns interleave, so the packed (value, lowest column) decides)
-      unsigned long long k0 = bi0 == 0x7fffffff ? 0ull : pack_best(bv0, bi0), k1 = bi1 == 0x7fffffff ? 0ull : pack_best(bv1, bi1);
-#pragma unroll
-      for (int o = 1; o <= 2; o <<= 1) {
-        const unsigned long long q0 = __shfl_xor_sync(0xffffffffu, k0, o), q1 = __shfl_xor_sync(0xffffffffu, k1, o);
-        k0 = q0 > k0 ? q0 : k0; k1 = q1 > k1 ? q1 : k1;
-      }
-      unsigned long long* red = reinterpret_cast<unsigned long long*>(sW);      // the weight stages are free now
-      if (kh == 0 && (lane & 3) == 0) { red[mt * 16 + (lane >> 2)] = k0; red[mt * 16 + 8 + (lane >> 2)] = k1; }
+    auto send = [&](int row, int col, float a, float b) {      // to the rank that owns these columns (gw is even)
+      if (row < B && col < ncols) st_cluster_v2(tc::mapa(tc::smem_u32(recv + ((size_t)(rank * mp + row) * gw + col % gw) * 4), (uint32_t)(col / gw)), a, b);
+    };
+    {
+      const int tile = warp % dn.tiles, g = warp / dn.tiles;
+      float c[8];
+      if (warp < dn.tiles * dn.groups) tile_group(c, dn, g, sA, ld_k, tile % m_tiles, sW2, ld_k, tile / m_tiles, lane);
+      if (warp < dn.tiles * dn.groups) put_part(part, dn, g, tile, lane, c);
       __syncthreads();
-      if (threadIdx.x < B) p.best[(int64_t)cta * B + threadIdx.x] = red[threadIdx.x];
-      if (bad) raise_status(p.status, kStatusNonFinite);
+      for (int i = tid; i < dn.tiles * 128; i += kThreads) {
+        const Pair q = take_pair(part, dn, i, m_tiles);
+        send(q.row, q.col, q.a, q.b);
+      }
     }
+    __syncwarp();
+    tc::cluster_sync();                    // the four partial products are here; the weight rows have been read
+    for (int i = tid; i < B * gw; i += kThreads) {
+      const int row = i / gw, c = i % gw;
+      const float* r = reinterpret_cast<const float*>(recv) + (size_t)row * gw + c;
+      float v = reinterpret_cast<const float*>(xo)[i] + __ldg(w.b2 + n0 + rank * gw + c);
+#pragma unroll
+      for (int s = 0; s < kCluster; ++s) v += r[(size_t)s * mp * gw];
+      p.x[(int64_t)row * d + n0 + rank * gw + c] = v;
+    }
+    gb.sync([&] {
+      if (tid == 0 && !alone) tc::mbar_expect_tx(barR, peer_bytes);
+      if (one_region) {
+        if (l + 1 < p.L) stage_up(l + 1);
+        else for (int ch = 0; ch < p.lm_stages; ++ch) stage_lm(ch);
+      }
+      load_row_params<d, NT>(p, l + 1, t_all, rp);
+    });
+  }
+  if (!one_region) for (int ch = p.lm_stages_w1; ch < p.lm_stages; ++ch) stage_lm(ch);
+
+  // ---- LM head over this CTA's vocabulary slab, chunk by chunk through the ring ----
+  const Share lm = share_of(m_tiles, d);
+  float bv = -INFINITY;
+  int bi = 0x7fffffff;
+  bool bad = false;
+  int my_row = kMaxRows;                                 // every thread keeps one pair of columns of one row
+  for (int ch = 0; ch < lm_chunks; ++ch) {
+    const int s = ch % p.lm_stages;
+    if (!wait_stage(barL + s, (uint32_t)(ch / p.lm_stages) & 1u, p.status, gb.dead)) gb.dead = true;
+    if (warp < lm.tiles * lm.groups) {
+      const int tile = warp % lm.tiles, g = warp / lm.tiles;
+      float c[8];
+      tile_group(c, lm, g, sA, ld_d, tile, sW1 + s * lm_stage, ld_d, 0, lane);
+      put_part(part, lm, g, tile, lane, c);
+    }
+    __syncthreads();                                     // partial sums are visible; stage s has been read
+    stage_lm(ch + p.lm_stages);
+    if (tid < lm.tiles * 128) {
+      const Pair q = take_pair(part, lm, tid, m_tiles);
+      const int col = (lm_c0 + ch) * kLmChunkCols + q.col;
+      my_row = q.row;
+      if (q.row < B && col < p.V && !gb.dead) {          // (V is a multiple of 8: pairs are whole)
+        if (p.logits != nullptr) *reinterpret_cast<float2*>(p.logits + (int64_t)q.row * p.V + col) = make_float2(q.a, q.b);
+        bad |= !(q.a == q.a) | !(q.b == q.b);
+        if (q.a > bv) { bv = q.a; bi = col; }            // ascending columns: the lowest among equals is kept
+        if (q.b > bv) { bv = q.b; bi = col + 1; }
+      }
+    }
+    __syncthreads();                                     // the partial sums have been taken
+  }
+  tc::cluster_sync();                      // the copies out of this CTA's shared memory have arrived
+  if (gb.dead) {
+    // a copy or a CTA never came: give whatever is still in flight time to land before shared memory goes away
+    const long long t0 = clock64();
+    while (clock64() - t0 < (1ll << 21)) { }
   }
   if (!p.greedy) return;                   // the caller selects from the logits
-  gb.sync();
-  if (cta == 0 && threadIdx.x < B) {
-    unsigned long long best = 0ull;
-    for (int c = 0; c < p.lm_ctas; ++c) {
-      const unsigned long long k = __ldcg(p.best + (int64_t)c * B + threadIdx.x);
-      best = k > best ? k : best;
-    }
+  if (bad) raise_status(p.status, kStatusNonFinite);
+  unsigned long long* best_s = reinterpret_cast<unsigned long long*>(part);
+  if (tid < kMaxRows) best_s[tid] = 0ull;
+  __syncthreads();
+  if (my_row < B && bi != 0x7fffffff) atomicMax(best_s + my_row, pack_best(bv, bi));
+  __syncthreads();
+  if (tid < B && best_s[tid] != 0ull) atomicMax(p.best + tid, best_s[tid]);
+  // ---- the CTA that comes last writes the tokens ----
+  __threadfence();
+  __syncthreads();
+  uint32_t* am_last = reinterpret_cast<uint32_t*>(sm + 116);
+  if (tid == 0) {
+    *am_last = atomicAdd(p.bar + 1, 1u) + 1u == gridDim.x ? 1u : 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (*am_last != 0u && tid < B) {
+    const unsigned long long best = __ldcg(p.best + tid);
     int tok = best == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)(best & 0xFFFFFFFFull));
     if (tok < 0 || tok >= p.V) tok = 0;
-    write_token(p.out, threadIdx.x, tok);
+    write_token(p.out, tid, tok);
   }
 }
 
