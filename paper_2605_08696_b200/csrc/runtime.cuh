@@ -299,7 +299,7 @@ size_t state_bytes_for(const srm_config& c, int64_t B) {
 
 // ---- workspace carving ----------------------------------------------------------------------
 // Scratch of the small-batch step kernel (step_small.cuh): the best logit of every row [64] and the barrier words.
-constexpr size_t kSmallScratchBytes = (size_t)sb::kMaxRows * 8 + 256;
+constexpr size_t kSmallScratchBytes = (size_t)sb::kMaxRows * 8 + (size_t)sb::kGrid * 4 + 256;
 
 // Partial-product planes of a small pass's down projection (GemmArgs::k_slices): up to 8 planes of the pass's rows
 // (padded to whole 256-row tiles) x d floats, never more than one 256 x 256 fp32 tile per CTA pair of the largest

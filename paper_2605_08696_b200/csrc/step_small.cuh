@@ -41,7 +41,8 @@ constexpr int kAloneRows = 4;                // up to this many rows every CTA c
 constexpr int kPadBytes = 16;                // row padding in shared memory: ldmatrix rows land in distinct banks
 constexpr int kLmChunkCols = 16;             // LM-head weight rows per pipeline stage
 constexpr int kLmMaxStages = 6;
-constexpr int kHeadBytes = 128 + 512;        // mbarriers and flags, row-phase sums
+constexpr int kHeadBytes = 128 + 256;        // mbarriers and flags, row-phase sums
+constexpr int kRowParamVecs = 5;              // parameter vectors of the row phase kept in shared memory
 constexpr int kMaxGroups = 8;                // ranges that K of a tile is cut into
 constexpr int kSmemBytes = 227 * 1024;
 constexpr long long kBarrierLimitCycles = 1ll << 27;
@@ -66,7 +67,7 @@ struct Params {
   bf16* H;                     // [B, F]
   float* logits;               // [B, V] or nullptr (then only the greedy selection leaves the kernel)
   unsigned long long* best;    // [B] (sortable logit, ~column) maxima, zero on entry
-  uint32_t* bar;               // [0] grid barrier, [1] CTAs done with the LM head; zero on entry
+  uint32_t* bar;               // [kGrid] words of the grid barrier, then the count of CTAs done with the LM head; zero on entry
   uint32_t* status;
   const int32_t* ctr;          // device-side step counters or nullptr
   const int32_t* pos;          // [B] per-row positions or nullptr
@@ -88,8 +89,10 @@ inline bool smem_plan(int B, int d, int F, int state_elem, Params* p, size_t* by
   const int mp = (B + 15) / 16 * 16, ld_d = 2 * d + kPadBytes, ld_k = 2 * dn_klen(F) + kPadBytes;
   const int act = mp * (ld_d > ld_k ? ld_d : ld_k);
   const int w1 = (up_cols(F) + 15) / 16 * 16 * ld_d, w2 = (dn_cols(d) + 15) / 16 * 16 * ld_k, stage = kLmChunkCols * ld_d;
-  const int part = kWarps * 1024, recv = kCluster * mp * (dn_cols(d) / kCluster) * 4, xo = mp * (dn_cols(d) / kCluster) * 4;
+  int recv = kCluster * mp * (dn_cols(d) / kCluster) * 4;
+  const int part = kWarps * 1024, xo = mp * (dn_cols(d) / kCluster) * 4;
   const int srow = d * state_elem;
+  if (part + recv < kRowParamVecs * d * 4) recv = kRowParamVecs * d * 4 - part;      // the row phase's parameters lie there
   for (int two = 1; two >= 0; --two) {                   // a region each for W1 and W2, or one for both
     int w = two ? w1 + w2 : (w1 > w2 ? w1 : w2);
     if (w < 2 * stage) w = 2 * stage;
@@ -121,12 +124,19 @@ __device__ __forceinline__ LayerW layer_w(const Params& p, int l) {
 __device__ __forceinline__ void red_release_inc(uint32_t* p) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v));
+__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
-__device__ __forceinline__ void st_cluster_v2(uint32_t addr, float a, float b) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+// eight bytes into the shared memory of a CTA of the cluster, counted on a barrier over there
+__device__ __forceinline__ void st_async_v2(uint32_t addr, float a, float b, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
+               ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
 }
 // shared memory of this CTA -> shared memory of a CTA of the cluster, bytes counted on a barrier over there
 __device__ __forceinline__ void bulk_s2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -137,31 +147,31 @@ __device__ __forceinline__ void bulk_s2s(uint32_t dst, const void* src, uint32_t
 // ---- grid-wide barrier ------------------------------------------------------------------------
 // Arrive / wait on a monotonically increasing counter: barrier number n (1, 2, ...) is passed when the counter
 // has reached n * gridDim.x. All CTAs are resident (cooperative launch), so the wait ends; it is bounded anyway.
-// `between` runs in all threads between arriving and waiting.
+// One thread polls, with relaxed loads and one acquire at the end (an acquiring poll drops the L1 cache every time; a
+// word per CTA polled by 128 threads that way took 4 us instead of 1.2). `between` runs in all threads between arriving
+// and waiting.
 struct GridBarrier {
   uint32_t* ctr;
   uint32_t n;          // barriers passed so far
   bool dead;           // a wait timed out: stop waiting (the same value in every thread of the CTA)
   uint32_t* status;
-  int* shared_dead;    // a word of shared memory through which thread 0 tells the others
   template <typename F>
   __device__ __forceinline__ void sync(F&& between) {
     __syncthreads();
     ++n;
     if (threadIdx.x == 0) red_release_inc(ctr);
     between();
-    if (threadIdx.x == 0) {
-      if (!dead) {
-        const uint32_t want = n * gridDim.x;
-        const long long t0 = clock64();
-        while (ld_acquire_u32(ctr) < want) {
-          if (clock64() - t0 > kBarrierLimitCycles) { dead = true; raise_status(status, kStatusWaitTimeout); break; }
-        }
+    bool late = false;
+    if (threadIdx.x == 0 && !dead) {
+      const uint32_t want = n * gridDim.x;
+      const long long t0 = clock64();
+      while (ld_relaxed_u32(ctr) < want) {
+        if (clock64() - t0 > kBarrierLimitCycles) { late = true; raise_status(status, kStatusWaitTimeout); break; }
       }
-      *shared_dead = dead ? 1 : 0;
+      ld_acquire_u32(ctr);
     }
-    __syncthreads();
-    dead = *shared_dead != 0;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");      // what `between` has fetched
+    dead = __syncthreads_or(late || dead) != 0;
   }
 };
 
@@ -265,102 +275,78 @@ __device__ __forceinline__ unsigned long long pack_best(float v, int col) {
   return ((unsigned long long)order_key(v) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)col);
 }
 
-// ---- row phase: four warps per row ---------------------------------------------------------------
-// LayerNorm statistics of the row that the four warps of a group hold, 4 NT values per thread (`on`: how many of its NT
-// vectors are inside the row): mean and sum of squared deviations per thread, merged pairwise (Chan et al.) over lanes
-// and warps in one pass of shuffles and one barrier. `slot`: eight floats that this group uses for these statistics
-// only (they are written again a whole row later).
+// ---- row phase: two warps per row ---------------------------------------------------------------
+// (one warp per row spills, and takes 12 us per layer at d = 1024; four warps do a row in the same time as two, but with
+// 64 rows the CTA then needs four rounds instead of two, 6.8 us instead of 3.6)
+constexpr int kGroups = kWarps / 2;
+
+// LayerNorm statistics of the row that the two warps of a group hold, 4 NT channels per thread: mean and sum of squared
+// deviations per thread, merged pairwise (Chan et al.; all counts are equal) over lanes and warps in one pass of shuffles
+// and one barrier. `slot`: four floats that this group uses for these statistics only.
 template <int d, int NT>
 __device__ __forceinline__ void group_stats(const float4 (&v)[NT], float eps, float* slot, int group, float& mean, float& rstd) {
-  constexpr bool full = d == NT * 512;                   // every thread holds NT whole vectors
-  float m, q = 0.f, n = 0.f;
-  if (full) {
-    float s = 0.f;
+  float m = 0.f, q = 0.f, half_n = 2.f * NT;
 #pragma unroll
-    for (int i = 0; i < NT; ++i) s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
-    n = 4.f * NT;
-    m = s * (1.0f / (4.f * NT));
-  } else {                                               // (d = 256, 768: the last vector of a thread may be outside)
-    float s = 0.f;
-#pragma unroll
-    for (int i = 0; i < NT; ++i)
-      if ((threadIdx.x & 127) * 4 + 512 * i < d) { s += (v[i].x + v[i].y) + (v[i].z + v[i].w); n += 4.f; }
-    m = n > 0.f ? s / n : 0.f;
-  }
+  for (int i = 0; i < NT; ++i) m += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+  m *= 1.0f / (4.f * NT);
 #pragma unroll
   for (int i = 0; i < NT; ++i) {
-    if (full || (threadIdx.x & 127) * 4 + 512 * i < d) {
-      const float a = v[i].x - m, b = v[i].y - m, c = v[i].z - m, e = v[i].w - m;
-      q += (a * a + b * b) + (c * c + e * e);
-    }
+    const float a = v[i].x - m, b = v[i].y - m, c = v[i].z - m, e = v[i].w - m;
+    q += (a * a + b * b) + (c * c + e * e);
   }
-  auto merge = [](float& m, float& q, float& n, float m2, float q2, float n2) {
-    const float dm = m2 - m, nn = n + n2;
-    if (full) { q += q2 + dm * dm * (0.5f * n); m = 0.5f * (m + m2); }
-    else if (nn > 0.f) { const float f = n2 / nn; q += q2 + dm * dm * n * f; m = fmaf(dm, f, m); }
-    n = nn;
+  auto merge = [&half_n](float& m, float& q, float m2, float q2) {
+    const float dm = m2 - m;
+    q += fmaf(dm * dm, half_n, q2);
+    m = 0.5f * (m + m2);
+    half_n += half_n;
   };
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float m2 = __shfl_xor_sync(0xffffffffu, m, o), q2 = __shfl_xor_sync(0xffffffffu, q, o);
-    const float n2 = full ? n : __shfl_xor_sync(0xffffffffu, n, o);
-    merge(m, q, n, m2, q2, n2);
+    merge(m, q, m2, q2);
   }
   if ((threadIdx.x & 31) == 0) {                         // (the lanes may differ in the last bit: lane 0's values count)
-    const int w = (threadIdx.x >> 5) & 3;
+    const int w = (threadIdx.x >> 5) & 1;
     slot[w] = m;
-    slot[4 + w] = q;
-    if (!full) slot[8 + w] = n;
+    slot[2 + w] = q;
   }
-  asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
-  float n0 = full ? n : slot[8], n1 = full ? n : slot[9], n2 = full ? n : slot[10], n3 = full ? n : slot[11];
-  float ma = slot[0], qa = slot[4], mb = slot[2], qb = slot[6];
-  merge(ma, qa, n0, slot[1], slot[5], n1);
-  merge(mb, qb, n2, slot[3], slot[7], n3);
-  merge(ma, qa, n0, mb, qb, n2);
-  mean = ma;
-  rstd = rsqrtf(qa * (1.0f / (float)d) + eps);
+  asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
+  m = slot[0];
+  q = slot[2];
+  merge(m, q, slot[1], slot[3]);
+  mean = m;
+  rstd = rsqrtf(q * (1.0f / (float)d) + eps);
 }
 
-// Thread i of a group owns channels 4 i .. 4 i + 3 (and 512 further) of every row. What a layer asks of the parameters
-// for these channels is fetched once for all rows, while the CTA waits at the grid barrier before the row phase.
-template <int NT>
-struct RowParams {
-  float4 g1[NT], b1[NT], g2[NT], b2[NT];
-  float4 bt[NT];       // beta_t, and the head scalars as the multipliers of z before and of the sum after (one is 1)
-  float a1[NT], a2[NT], lm[NT];
-};
-template <int d, int NT>
-__device__ __forceinline__ void load_position(const Params& p, const LayerW& w, int t, RowParams<NT>& r) {
-#pragma unroll
-  for (int i = 0; i < NT; ++i) {
-    const int c = (threadIdx.x & 127) * 4 + 512 * i;
-    if (c < d) {
-      const int g = c / (d / p.h);
-      r.bt[i] = ldg4(w.beta + (int64_t)t * d + c);
-      const float al = __ldg(w.alpha + (int64_t)g * p.n_ctx + t);
-      const bool is_row = g < (p.h >> 1);
-      r.a1[i] = is_row ? al : 1.0f;
-      r.a2[i] = is_row ? 1.0f : al;
-      r.lm[i] = __ldg(w.lam + g);
-    }
-  }
-}
-// Parameters of layer l (l == L: of the final norm).
-template <int d, int NT>
-__device__ __forceinline__ void load_row_params(const Params& p, int l, int t, RowParams<NT>& r) {
+// The parameters of a layer's row phase (l == L: of the final norm) in shared memory: ln1_g | ln1_b | beta_t | ln2_g |
+// ln2_b, fetched while the CTA waits at the grid barrier before the row phase (kRowParamVecs * d floats in the place of the
+// partial sums and the exchange buffer, which are free then).
+template <int d>
+__device__ __forceinline__ void fetch_row_params(const Params& p, int l, int t, float* dst) {
   const bool last = l == p.L;
   const LayerW w = layer_w(p, last ? 0 : l);
-  const float *g2 = last ? p.lnf_g : w.ln2_g, *b2 = last ? p.lnf_b : w.ln2_b;
+  for (int i = threadIdx.x; i < kRowParamVecs * d / 4; i += kThreads) {
+    const int k = i / (d / 4), c = i % (d / 4) * 4;
+    const float* q = k == 0 ? w.ln1_g : k == 1 ? w.ln1_b : k == 2 ? w.beta + (int64_t)t * d : k == 3 ? (last ? p.lnf_g : w.ln2_g)
+                                                                                                    : (last ? p.lnf_b : w.ln2_b);
+    cp_async16(dst + i * 4, q + c);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// The head scalars of a thread's channels at position t: the multipliers of z before and of the sum after (one of them is
+// 1), and lambda. Thread i of a group owns channels 4 i .. 4 i + 3 (and 256, 512, ... further) of every row.
+template <int d, int NT>
+__device__ __forceinline__ void head_scalars(const Params& p, const LayerW& w, int t, float (&a1)[NT], float (&a2)[NT], float (&lm)[NT]) {
+  const int dh = d / p.h;
 #pragma unroll
   for (int i = 0; i < NT; ++i) {
-    const int c = (threadIdx.x & 127) * 4 + 512 * i;
-    if (c < d) {
-      r.g2[i] = ldg4(g2 + c); r.b2[i] = ldg4(b2 + c);
-      if (!last) { r.g1[i] = ldg4(w.ln1_g + c); r.b1[i] = ldg4(w.ln1_b + c); }
-    }
+    const int g = ((threadIdx.x & 63) * 4 + 256 * i) / dh;
+    const float al = __ldg(w.alpha + (int64_t)g * p.n_ctx + t);
+    const bool is_row = g < (p.h >> 1);
+    a1[i] = is_row ? al : 1.0f;
+    a2[i] = is_row ? 1.0f : al;
+    lm[i] = __ldg(w.lam + g);
   }
-  if (!last && p.pos == nullptr) load_position<d, NT>(p, w, t, r);
 }
 
 template <int d, typename ST>
@@ -370,8 +356,9 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
   uint64_t* bar2 = bar1 + 1;                             // W2 slab
   uint64_t* barA = bar1 + 2;                             // rows of H
   uint64_t* barR = bar1 + 3;                             // activation rows from the other CTAs of the cluster
-  uint64_t* barL = bar1 + 4;                             // LM-head stages
-  float* red = reinterpret_cast<float*>(sm + 128);       // row-phase sums: four groups x 32
+  uint64_t* barP = bar1 + 4;                             // x + y and the partial products of the owned columns
+  uint64_t* barL = bar1 + 5;                             // LM-head stages
+  float* red = reinterpret_cast<float*>(sm + 128);       // row-phase sums: eight groups x 8 floats
   uint8_t* sA = sm + kHeadBytes;
   uint8_t* sW1 = sm + p.off_w1;
   uint8_t* sW2 = sm + p.off_w2;
@@ -392,12 +379,12 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
   const bool alone = B <= kAloneRows, one_region = p.off_w1 == p.off_w2;
 
   if (tid == 0) {
-    for (int i = 0; i < 4 + kLmMaxStages; ++i) tc::mbar_init(bar1 + i, 1);
+    for (int i = 0; i < 5 + kLmMaxStages; ++i) tc::mbar_init(bar1 + i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc::cluster_sync();                                    // every CTA of the cluster is up before anyone writes into its memory
   uint32_t par1 = 0, par2 = 0;
-  GridBarrier gb{p.bar, 0u, false, p.status, reinterpret_cast<int*>(sm + 112)};
+  GridBarrier gb{p.bar, 0u, false, p.status};
   const int t_all = p.ctr != nullptr ? p.ctr[kCtrPos] : p.t;
   auto t_of = [&](int row) { return p.pos != nullptr ? min(max(p.pos[row], 0), p.n_ctx - 1) : t_all; };
 
@@ -438,103 +425,101 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
     }
   };
 
-  constexpr int NT = (d + 511) / 512;
-  const int group = warp >> 2, c0 = (tid & 127) * 4;
-  RowParams<NT> rp;
-  load_row_params<d, NT>(p, 0, t_all, rp);
+  constexpr int NT = d / 256;
+  const int group = warp >> 1, c0 = (tid & 63) * 4;
+  float a1[NT], a2[NT], lm[NT];
+  float* prm = part;                                     // (with the exchange buffer behind it)
+  fetch_row_params<d>(p, 0, p.pos != nullptr ? 0 : t_all, prm);
+  head_scalars<d, NT>(p, layer_w(p, 0), p.pos != nullptr ? 0 : t_all, a1, a2, lm);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
   // bytes of the rows that the other CTAs of the cluster send per row phase
   const uint32_t peer_bytes = (uint32_t)(B - (B - rank + kCluster - 1) / kCluster) * (2 * d);
-  if (tid == 0 && !alone) tc::mbar_expect_tx(barR, peer_bytes);
+  const uint32_t part_bytes = (uint32_t)((kCluster + 1) * B * gw * 4);       // partial products, and x + y of the owned columns
+  if (tid == 0) {
+    if (!alone) tc::mbar_expect_tx(barR, peer_bytes);
+    tc::mbar_expect_tx(barP, part_bytes);
+  }
   stage_up(0);
   if (!one_region) stage_dn(0);
   prefetch_layer(0);
+  if (p.L > 1) prefetch_layer(1);
   const Share up = share_of(m_tiles * ((ucols + 15) / 16), d), dn = share_of(m_tiles * ((ncols + 15) / 16), klen);
   for (int l = 0;; ++l) {
     const bool last = l == p.L;
     const LayerW w = layer_w(p, last ? 0 : l);
-    if (l + 1 < p.L) prefetch_layer(l + 1);
-    // ---- rows (after the last layer: the final norm). The activation row goes to its place here or in all CTAs of the
-    //      cluster, x + y of the cluster's own columns to the CTAs that will add the down projection to them ----
+    // ---- rows (after the last layer: the final norm). The activation row goes to its place here and in the other CTAs of
+    //      the cluster, x + y of the cluster's own columns to the CTAs that will add the down projection to them ----
     {
-      const ST* Sl = reinterpret_cast<const ST*>(static_cast<const uint8_t*>(p.S) + (int64_t)l * p.layer_stride);
-      float* slot = red + group * 32;
-      const int step = alone ? kMaxRows : 4 * kCluster;
-      float4 v[NT], s[NT];
-      auto load = [&](int row) {
-        int tk = 0;
+      const ST* Sl = reinterpret_cast<const ST*>(static_cast<const uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + c0;
+      float* slot = red + group * 8;
+      const int step = alone ? kMaxRows : kGroups * kCluster;
+      for (int row = alone ? group : rank + group * kCluster; row < B; row += step) {
+        float4 v[NT], s[NT];
         if (l == 0) {
-          tk = p.tok_in[row];
+          int tk = p.tok_in[row];
           if (tk < 0 || tk >= p.V) {
             if (c0 == 0) raise_status(p.status, kStatusTokenRange);
             tk = tk < 0 ? 0 : p.V - 1;
           }
-        }
 #pragma unroll
-        for (int i = 0; i < NT; ++i) {
-          const int c = c0 + 512 * i;
-          if (c < d) {
-            if (l == 0) v[i] = ldg4(p.E + (int64_t)tk * d + c);
-            else v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c));    // other CTAs wrote it: not through L1
-            if (!last) s[i] = ld4(Sl + (int64_t)row * d + c);
-          }
+          for (int i = 0; i < NT; ++i) v[i] = ldg4(p.E + (int64_t)tk * d + c0 + 256 * i);
+        } else {                                         // other CTAs wrote it: not through L1
+#pragma unroll
+          for (int i = 0; i < NT; ++i) v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c0 + 256 * i));
         }
-      };
-      int row = alone ? group : rank + group * kCluster;
-      if (row < B) load(row);
-      for (; row < B; row += step) {
         float mean, rstd;
         if (!last) {
-          if (p.pos != nullptr) load_position<d, NT>(p, w, t_of(row), rp);
+#pragma unroll
+          for (int i = 0; i < NT; ++i) s[i] = ld4(Sl + (int64_t)row * d + 256 * i);
+          const float* bt_p = prm + 2 * d + c0;
+          if (p.pos != nullptr) {                        // a position per row: its own beta row and head scalars
+            const int t = t_of(row);
+            bt_p = w.beta + (int64_t)t * d + c0;
+            head_scalars<d, NT>(p, w, t, a1, a2, lm);
+          }
           group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
           const float nmr = -mean * rstd;
 #pragma unroll
           for (int i = 0; i < NT; ++i) {
-            const int c = c0 + 512 * i;
-            if (c < d) {
-              const float4 g = rp.g1[i], bb = rp.b1[i], bt = rp.bt[i];
-              const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
-                                           fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
-              // row-repeat head, Eq. 2: y = (a z + S) + b ; S' = l (S + a z).  column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
-              const float a1 = rp.a1[i], a2 = rp.a2[i], lm = rp.lm[i];
-              const float4 u = make_float4(fmaf(a1, z.x, s[i].x), fmaf(a1, z.y, s[i].y), fmaf(a1, z.z, s[i].z), fmaf(a1, z.w, s[i].w));
-              if (row == own_row) st4(sS + c, make_float4(lm * u.x, lm * u.y, lm * u.z, lm * u.w));
-              v[i] = make_float4(v[i].x + fmaf(a2, u.x, bt.x), v[i].y + fmaf(a2, u.y, bt.y), v[i].z + fmaf(a2, u.z, bt.z),
-                                 v[i].w + fmaf(a2, u.w, bt.w));
-              const int o = c - n0;                                // column inside the cluster's slab
-              if (o >= 0 && o < ncols) {
-                const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+            const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i), bt = ld4(bt_p + 256 * i);
+            const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
+                                         fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
+            // row-repeat head, Eq. 2: y = (a z + S) + b ; S' = l (S + a z).  column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
+            const float4 u = make_float4(fmaf(a1[i], z.x, s[i].x), fmaf(a1[i], z.y, s[i].y), fmaf(a1[i], z.z, s[i].z), fmaf(a1[i], z.w, s[i].w));
+            if (row == own_row) st4(sS + c0 + 256 * i, make_float4(lm[i] * u.x, lm[i] * u.y, lm[i] * u.z, lm[i] * u.w));
+            v[i] = make_float4(v[i].x + fmaf(a2[i], u.x, bt.x), v[i].y + fmaf(a2[i], u.y, bt.y), v[i].z + fmaf(a2[i], u.z, bt.z),
+                               v[i].w + fmaf(a2[i], u.w, bt.w));
+            const int o = c0 + 256 * i - n0;             // column inside the cluster's slab
+            if (o >= 0 && o < ncols) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const int q = (o + k) / gw;                      // the rank that owns this column
-                  const uint32_t at = tc::smem_u32(xo) + (uint32_t)(row * gw + (o + k) % gw) * 4;
-                  if (!alone || q == rank) st_cluster_f32(tc::mapa(at, (uint32_t)q), e[k]);
-                }
+              for (int k = 0; k < 4; k += 2) {           // (gw is even: two adjacent columns have one owner)
+                const int q = (o + k) / gw;
+                if (!alone || q == rank)
+                  st_async_v2(tc::mapa(tc::smem_u32(xo) + (uint32_t)(row * gw + (o + k) % gw) * 4, (uint32_t)q), k ? v[i].z : v[i].x,
+                              k ? v[i].w : v[i].y, tc::mapa(tc::smem_u32(barP), (uint32_t)q));
               }
             }
           }
         }
-        group_stats<d, NT>(v, p.eps, slot + 16, group, mean, rstd);
+        group_stats<d, NT>(v, p.eps, slot + 4, group, mean, rstd);
         const float nmr2 = -mean * rstd;
-        uint2 u[NT];
-#pragma unroll
-        for (int i = 0; i < NT; ++i) {
-          const float4 g = rp.g2[i], bb = rp.b2[i];
-          const __nv_bfloat162 lo = __floats2bfloat162_rn(fmaf(fmaf(v[i].x, rstd, nmr2), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr2), g.y, bb.y));
-          const __nv_bfloat162 hi = __floats2bfloat162_rn(fmaf(fmaf(v[i].z, rstd, nmr2), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr2), g.w, bb.w));
-          u[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-        }
-        if (row + step < B) load(row + step);
         uint8_t* at = sA + (size_t)row * ld_d;
 #pragma unroll
-        for (int i = 0; i < NT; ++i)
-          if (c0 + 512 * i < d) *reinterpret_cast<uint2*>(at + (c0 + 512 * i) * 2) = u[i];
+        for (int i = 0; i < NT; ++i) {
+          const float4 g = ld4(prm + 3 * d + c0 + 256 * i), bb = ld4(prm + 4 * d + c0 + 256 * i);
+          st4(reinterpret_cast<bf16*>(at) + c0 + 256 * i,
+              make_float4(fmaf(fmaf(v[i].x, rstd, nmr2), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr2), g.y, bb.y),
+                          fmaf(fmaf(v[i].z, rstd, nmr2), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr2), g.w, bb.w)));
+        }
         if (!alone) {
           // (one bulk copy per peer: eight-byte stores into the peers' memory took 1.7 us per sixteen rows)
           tc::fence_async_smem();
-          asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
-          const int r = tid & 127;
-          if (r < kCluster && r != rank)
-            bulk_s2s(tc::mapa(tc::smem_u32(at), (uint32_t)r), at, 2 * d, tc::mapa(tc::smem_u32(barR), (uint32_t)r));
+          asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
+          const int r = tid & 63;                        // threads 0, 1 of the group's first warp, 32, 33 of its second
+          const int peer = (r & 31) < 2 ? (r & 31) + 2 * (r >> 5) : rank;
+          if (peer != rank)
+            bulk_s2s(tc::mapa(tc::smem_u32(at), (uint32_t)peer), at, 2 * d, tc::mapa(tc::smem_u32(barR), (uint32_t)peer));
         }
       }
       __syncthreads();                     // this CTA's rows
@@ -581,8 +566,11 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
       if (l + 1 < p.L) stage_up(l + 1);
       else for (int ch = 0; ch < p.lm_stages_w1; ++ch) stage_lm(ch);
     }
+    if (l + 2 < p.L) prefetch_layer(l + 2);
     auto send = [&](int row, int col, float a, float b) {      // to the rank that owns these columns (gw is even)
-      if (row < B && col < ncols) st_cluster_v2(tc::mapa(tc::smem_u32(recv + ((size_t)(rank * mp + row) * gw + col % gw) * 4), (uint32_t)(col / gw)), a, b);
+      if (row < B && col < ncols)
+        st_async_v2(tc::mapa(tc::smem_u32(recv + ((size_t)(rank * mp + row) * gw + col % gw) * 4), (uint32_t)(col / gw)), a, b,
+                    tc::mapa(tc::smem_u32(barP), (uint32_t)(col / gw)));
     };
     {
       const int tile = warp % dn.tiles, g = warp / dn.tiles;
@@ -595,8 +583,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
         send(q.row, q.col, q.a, q.b);
       }
     }
-    __syncwarp();
-    tc::cluster_sync();                    // the four partial products are here; the weight rows have been read
+    if (!wait_stage(barP, (uint32_t)l & 1u, p.status, gb.dead)) gb.dead = true;      // the four partial products are here
     for (int i = tid; i < B * gw; i += kThreads) {
       const int row = i / gw, c = i % gw;
       const float* r = reinterpret_cast<const float*>(recv) + (size_t)row * gw + c;
@@ -606,18 +593,23 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
       p.x[(int64_t)row * d + n0 + rank * gw + c] = v;
     }
     gb.sync([&] {
-      if (tid == 0 && !alone) tc::mbar_expect_tx(barR, peer_bytes);
+      if (tid == 0) {
+        if (!alone) tc::mbar_expect_tx(barR, peer_bytes);
+        if (l + 1 < p.L) tc::mbar_expect_tx(barP, part_bytes);
+      }
       if (one_region) {
         if (l + 1 < p.L) stage_up(l + 1);
         else for (int ch = 0; ch < p.lm_stages; ++ch) stage_lm(ch);
       }
-      load_row_params<d, NT>(p, l + 1, t_all, rp);
+      const int t = p.pos != nullptr ? 0 : t_all;
+      fetch_row_params<d>(p, l + 1, t, prm);
+      if (l + 1 < p.L) head_scalars<d, NT>(p, layer_w(p, l + 1), t, a1, a2, lm);
     });
   }
   if (!one_region) for (int ch = p.lm_stages_w1; ch < p.lm_stages; ++ch) stage_lm(ch);
 
   // ---- LM head over this CTA's vocabulary slab, chunk by chunk through the ring ----
-  const Share lm = share_of(m_tiles, d);
+  const Share hd = share_of(m_tiles, d);
   float bv = -INFINITY;
   int bi = 0x7fffffff;
   bool bad = false;
@@ -625,16 +617,16 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
   for (int ch = 0; ch < lm_chunks; ++ch) {
     const int s = ch % p.lm_stages;
     if (!wait_stage(barL + s, (uint32_t)(ch / p.lm_stages) & 1u, p.status, gb.dead)) gb.dead = true;
-    if (warp < lm.tiles * lm.groups) {
-      const int tile = warp % lm.tiles, g = warp / lm.tiles;
+    if (warp < hd.tiles * hd.groups) {
+      const int tile = warp % hd.tiles, g = warp / hd.tiles;
       float c[8];
-      tile_group(c, lm, g, sA, ld_d, tile, sW1 + s * lm_stage, ld_d, 0, lane);
-      put_part(part, lm, g, tile, lane, c);
+      tile_group(c, hd, g, sA, ld_d, tile, sW1 + s * lm_stage, ld_d, 0, lane);
+      put_part(part, hd, g, tile, lane, c);
     }
     __syncthreads();                                     // partial sums are visible; stage s has been read
     stage_lm(ch + p.lm_stages);
-    if (tid < lm.tiles * 128) {
-      const Pair q = take_pair(part, lm, tid, m_tiles);
+    if (tid < hd.tiles * 128) {
+      const Pair q = take_pair(part, hd, tid, m_tiles);
       const int col = (lm_c0 + ch) * kLmChunkCols + q.col;
       my_row = q.row;
       if (q.row < B && col < p.V && !gb.dead) {          // (V is a multiple of 8: pairs are whole)
@@ -665,7 +657,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
   __syncthreads();
   uint32_t* am_last = reinterpret_cast<uint32_t*>(sm + 116);
   if (tid == 0) {
-    *am_last = atomicAdd(p.bar + 1, 1u) + 1u == gridDim.x ? 1u : 0u;
+    *am_last = atomicAdd(p.bar + kGrid, 1u) + 1u == gridDim.x ? 1u : 0u;
     __threadfence();
   }
   __syncthreads();
