@@ -608,28 +608,30 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
   }
   if (!one_region) for (int ch = p.lm_stages_w1; ch < p.lm_stages; ++ch) stage_lm(ch);
 
-  // ---- LM head over this CTA's vocabulary slab, chunk by chunk through the ring ----
-  const Share hd = share_of(m_tiles, d);
+  // ---- LM head over this CTA's vocabulary slab through the ring, two chunks at a time where it is deep enough ----
+  const int cpi = p.lm_stages >= 4 && m_tiles <= 2 ? 2 : 1;      // (every thread takes one pair of columns)
+  const Share hd = share_of(m_tiles * cpi, d);
+  const int lm_end = min(p.V, (lm_c0 + lm_chunks) * kLmChunkCols);
   float bv = -INFINITY;
   int bi = 0x7fffffff;
   bool bad = false;
   int my_row = kMaxRows;                                 // every thread keeps one pair of columns of one row
-  for (int ch = 0; ch < lm_chunks; ++ch) {
-    const int s = ch % p.lm_stages;
-    if (!wait_stage(barL + s, (uint32_t)(ch / p.lm_stages) & 1u, p.status, gb.dead)) gb.dead = true;
+  for (int ch = 0; ch < lm_chunks; ch += cpi) {
+    for (int c = ch; c < ch + cpi && c < lm_chunks; ++c)
+      if (!wait_stage(barL + c % p.lm_stages, (uint32_t)(c / p.lm_stages) & 1u, p.status, gb.dead)) gb.dead = true;
     if (warp < hd.tiles * hd.groups) {
       const int tile = warp % hd.tiles, g = warp / hd.tiles;
       float c[8];
-      tile_group(c, hd, g, sA, ld_d, tile, sW1 + s * lm_stage, ld_d, 0, lane);
+      tile_group(c, hd, g, sA, ld_d, tile % m_tiles, sW1 + (ch + tile / m_tiles) % p.lm_stages * lm_stage, ld_d, 0, lane);
       put_part(part, hd, g, tile, lane, c);
     }
-    __syncthreads();                                     // partial sums are visible; stage s has been read
-    stage_lm(ch + p.lm_stages);
+    __syncthreads();                                     // partial sums are visible, the stages have been read
+    for (int c = ch; c < ch + cpi; ++c) stage_lm(c + p.lm_stages);
     if (tid < hd.tiles * 128) {
       const Pair q = take_pair(part, hd, tid, m_tiles);
       const int col = (lm_c0 + ch) * kLmChunkCols + q.col;
       my_row = q.row;
-      if (q.row < B && col < p.V && !gb.dead) {          // (V is a multiple of 8: pairs are whole)
+      if (q.row < B && col < lm_end && !gb.dead) {       // (V is a multiple of 8: pairs are whole)
         if (p.logits != nullptr) *reinterpret_cast<float2*>(p.logits + (int64_t)q.row * p.V + col) = make_float2(q.a, q.b);
         bad |= !(q.a == q.a) | !(q.b == q.b);
         if (q.a > bv) { bv = q.a; bi = col; }            // ascending columns: the lowest among equals is kept
