@@ -697,6 +697,82 @@ int launch_mixer_block_proj(srm_model& m, int layer, int t, int64_t rows, int64_
   return launch_norm(m, x, rows, 1, 0, m.fptr(layer, SRM_T_LN2_G), m.fptr(layer, SRM_T_LN2_B), a, st);
 }
 
+sb::LayerW layer0_weights(const srm_model& m) {
+  return sb::LayerW{m.fptr(0, SRM_T_LN1_G), m.fptr(0, SRM_T_LN1_B), m.fptr(0, SRM_T_LN2_G), m.fptr(0, SRM_T_LN2_B),
+                    m.fptr(0, SRM_T_ALPHA), m.fptr(0, SRM_T_BETA), m.fptr(0, SRM_T_LAMBDA), m.fptr(0, SRM_T_B1),
+                    m.fptr(0, SRM_T_B2), reinterpret_cast<const bf16*>(m.ptr(0, SRM_T_W1)),
+                    reinterpret_cast<const bf16*>(m.ptr(0, SRM_T_W2))};
+}
+int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor from the same tensor of the next layer
+  return m.cfg.n_layers > 1 ? (int64_t)(m.layout.layer[SRM_T_COUNT + SRM_T_LN1_G].off - m.layout.layer[SRM_T_LN1_G].off) : 0;
+}
+
+// ---- passes of a hundred to a thousand rows: all layers in one kernel (layers_mid.cuh) -------------------
+// From this many rows: up to 64 the whole step is one kernel of another design (step_small.cuh).
+constexpr int64_t kMidMinRows = 97;
+
+// Whether a decode pass of R rows takes it, and its tile plan. bf16 mixed-head models of the widths it is built for,
+// as many rows as leave every CTA pair one tile of each projection.
+bool mid_plan(srm_model& m, int64_t R, const DecodeWs& w, mid::Params* p) {
+  const srm_config& c = m.cfg;
+  constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
+  if (R < kMidMinRows || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || c.mixer != SRM_MIXER_MIXED || w.part == nullptr) return false;
+  if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536) return false;
+  if (ensure_tc_ready(m) != SRM_OK || R > (int64_t)2 * m.tc_clusters * mid::kGroups || m.F() > (1 << 20)) return false;
+  if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, p)) return false;
+  return (size_t)p->ks * p->rb * tc::BM * c.d_model * 4 <= w.part_bytes;
+}
+
+template <int NT, typename ST>
+int launch_layers_t(srm_model& m, const CUtensorMap& ta, const CUtensorMap& th, const CUtensorMap& tw1, const CUtensorMap& tw2,
+                    const mid::Params& p, cudaStream_t st) {
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(mid::layers_kernel<NT, ST>), mid::kSmemBytes);
+  if (rc != SRM_OK) return rc;
+  const size_t smem = mid::smem_bytes(p.d, p.n, p.w_slots, p.a_slots);
+  SRM_CUDA(launch_kernel(mid::layers_kernel<NT, ST>, dim3(2u * (unsigned)m.tc_clusters), dim3(mid::kThreads), smem, st, ta, th, tw1, tw2, p));
+  SRM_CUDA(cudaGetLastError());
+  return SRM_OK;
+}
+template <int NT>
+int launch_layers_nt(srm_model& m, const CUtensorMap& ta, const CUtensorMap& th, const CUtensorMap& tw1, const CUtensorMap& tw2,
+                     const mid::Params& p, cudaStream_t st) {
+  if (m.cfg.state_dtype == SRM_DTYPE_FP16) return launch_layers_t<NT, fp16>(m, ta, th, tw1, tw2, p, st);
+  if (m.cfg.state_dtype == SRM_DTYPE_BF16) return launch_layers_t<NT, bf16>(m, ta, th, tw1, tw2, p, st);
+  return launch_layers_t<NT, float>(m, ta, th, tw1, tw2, p, st);
+}
+
+// All layers for rows [b0, b0 + R) of the state; leaves x and, in w.part, the last down projection's partial products.
+// p: from mid_plan.
+int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w, mid::Params& p,
+                      cudaStream_t st, const int32_t* ctr, const int32_t* pos) {
+  const srm_config& c = m.cfg;
+  const int d = c.d_model, F = (int)m.F();
+  p.R = (int)R; p.d = d; p.F = F; p.V = c.vocab; p.h = c.n_heads; p.n_ctx = c.n_ctx; p.L = c.n_layers; p.t = t;
+  p.eps = c.ln_eps;
+  p.tok_in = tok_in;
+  p.E = reinterpret_cast<const bf16*>(m.ptr(-1, SRM_T_E));
+  p.layer0 = layer0_weights(m);
+  p.layer_bytes = layer_stride_bytes(m);
+  p.S = static_cast<uint8_t*>(s.layer_ptr(0)) + (size_t)b0 * d * m.state_bytes();
+  p.layer_stride = (int64_t)s.B * d * m.state_bytes();
+  p.x = w.x; p.a = reinterpret_cast<bf16*>(w.a); p.H = reinterpret_cast<bf16*>(w.H);
+  p.part = w.part;
+  p.plane = (int64_t)p.rb * tc::BM * d;
+  p.cnt = reinterpret_cast<uint32_t*>(w.logits);      // (nothing uses the logits area before the LM head)
+  p.status = s.status; p.ctr = ctr; p.pos = pos;
+  SRM_CUDA(cudaMemsetAsync(p.cnt, 0, mid::kCntWords * 4, st));
+  LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
+  CUtensorMap ta, th, tw1, tw2;
+  int rc;
+  if ((rc = m.tmap(w.a, R, d, tc::kRowsPerCta, 2, &ta)) != SRM_OK) return rc;
+  if ((rc = m.tmap(w.H, R, F, tc::kRowsPerCta, 2, &th)) != SRM_OK) return rc;
+  if ((rc = make_tmap_layers(&tw1, m.ptr(0, SRM_T_W1), F, d, c.n_layers, p.layer_bytes, p.n / 2)) != SRM_OK) return rc;
+  if ((rc = make_tmap_layers(&tw2, m.ptr(0, SRM_T_W2), d, F, c.n_layers, p.layer_bytes, p.n / 2)) != SRM_OK) return rc;
+  if (d == 512) return launch_layers_nt<2>(m, ta, th, tw1, tw2, p, st);
+  if (d == 1024) return launch_layers_nt<4>(m, ta, th, tw1, tw2, p, st);
+  return launch_layers_nt<6>(m, ta, th, tw1, tw2, p, st);
+}
+
 // One decode step for rows [b0, b0 + R) of the state.
 int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_t* tok_in, const srm_sampling& samp,
                  int step, const SelectOut& out_all, float* logits_out, const DecodeWs& w, cudaStream_t st,
@@ -707,9 +783,18 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   const int t = (int)(s.pos < c.n_ctx ? s.pos : c.n_ctx - 1);
   const int32_t* pos = s.ragged ? s.pos_dev + b0 : nullptr;       // samples of different lengths: a position per row
   int rc;
+  PartialSum ps_none, ps;
+  int k_slices = 1;
+  mid::Params mp;
+  const bool one_kernel = mid_plan(m, R, w, &mp);
+  if (one_kernel) {
+    if ((rc = launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
+    k_slices = mp.ks;
+    ps = PartialSum{w.part, mp.ks, mp.plane, m.fptr(c.n_layers - 1, SRM_T_B2)};
+  }
   // the down projection shares K out between CTA pairs where that is the faster kernel for R rows
   bool split = false;
-  if (w.order != nullptr && F % tc::BK == 0) {
+  if (!one_kernel && w.order != nullptr && F % tc::BK == 0) {
     if ((rc = ensure_tc_ready(m))) return rc;
     tc::SplitPlan P;
     const int64_t tiles = ((R + tc::BM - 1) / tc::BM) * ((d + tc::BN - 1) / tc::BN);
@@ -718,7 +803,7 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   // the feed-forward block as one kernel: its per-layer counters sit in the logits area, which nothing uses before
   // the LM head
   const size_t ready_layer = ffn_ready_bytes(R, F);
-  bool fused_ffn = !(c.flags & SRM_FLAG_NO_FUSED_FFN) && ffn_fused_shape_ok(m, R) &&
+  bool fused_ffn = !one_kernel && !(c.flags & SRM_FLAG_NO_FUSED_FFN) && ffn_fused_shape_ok(m, R) &&
                    ready_layer * c.n_layers <= align_up((size_t)w.rows * c.vocab * 4, 256);
   if (fused_ffn) {
     if ((rc = ensure_tc_ready(m))) return rc;
@@ -729,16 +814,14 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   // A small pass (the down projection has less than half as many tiles as there are CTA pairs): its K dimension is
   // cut into ranges so that all pairs work on it; the partial products go to planes of their own in the workspace
   // and the next consumer of x (the next layer's mixer, the final norm) adds them in a fixed order.
-  PartialSum ps_none, ps;
-  int k_slices = 1;
   const int64_t plane_rows = (R + tc::BM - 1) / tc::BM * tc::BM;
-  if (!fused_ffn && !split && w.part != nullptr) {
+  if (!one_kernel && !fused_ffn && !split && w.part != nullptr) {
     if ((rc = ensure_tc_ready(m))) return rc;
     k_slices = down_k_slices(plane_rows / tc::BM * ((d + tc::BN - 1) / tc::BN), (int)(F / tc::BK), m.tc_clusters);
     while (k_slices > 1 && (size_t)k_slices * plane_rows * d * 4 > w.part_bytes) k_slices /= 2;
   }
-  if (k_slices > 1) ps = PartialSum{w.part, k_slices, plane_rows * (int64_t)d, nullptr};
-  for (int l = 0; l < c.n_layers; ++l) {
+  if (!one_kernel && k_slices > 1) ps = PartialSum{w.part, k_slices, plane_rows * (int64_t)d, nullptr};
+  for (int l = 0; !one_kernel && l < c.n_layers; ++l) {
     uint8_t* Sl = static_cast<uint8_t*>(s.layer_ptr(l)) + (size_t)b0 * d * m.state_bytes();
     if (c.mixer != SRM_MIXER_MIXED) {
       if ((rc = launch_mixer_variant(m, l, t, R, l == 0 ? tok_in + b0 : nullptr, 1, w.x, w.a, d, Sl, s.plane_elems(), s.status,
@@ -771,8 +854,8 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
     }
     if (rc) return rc;
   }
-  if (k_slices > 1) ps.bias = m.fptr(c.n_layers - 1, SRM_T_B2);
-  if ((rc = launch_final_norm(m, w.x, R, 1, 0, w.a, st, nullptr, k_slices > 1 ? ps : ps_none))) return rc;
+  if (ps.part != nullptr) ps.bias = m.fptr(c.n_layers - 1, SRM_T_B2);
+  if ((rc = launch_final_norm(m, w.x, R, 1, 0, w.a, st, nullptr, ps))) return rc;
   SelectOut o = out_all;
   o.last_tok += b0;
   if (o.tok_out) o.tok_out += b0;
@@ -860,11 +943,8 @@ int decode_step_small(srm_model& m, srm_state& s, SmallPlan& P, const int32_t* t
   p.E = reinterpret_cast<const bf16*>(m.ptr(-1, SRM_T_E));
   p.W_lm = reinterpret_cast<const bf16*>(m.ptr(-1, SRM_T_W_LM));
   p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
-  p.layer0 = sb::LayerW{m.fptr(0, SRM_T_LN1_G), m.fptr(0, SRM_T_LN1_B), m.fptr(0, SRM_T_LN2_G), m.fptr(0, SRM_T_LN2_B),
-                        m.fptr(0, SRM_T_ALPHA), m.fptr(0, SRM_T_BETA), m.fptr(0, SRM_T_LAMBDA), m.fptr(0, SRM_T_B1),
-                        m.fptr(0, SRM_T_B2), reinterpret_cast<const bf16*>(m.ptr(0, SRM_T_W1)),
-                        reinterpret_cast<const bf16*>(m.ptr(0, SRM_T_W2))};
-  p.layer_bytes = c.n_layers > 1 ? (int64_t)(m.layout.layer[SRM_T_COUNT + SRM_T_LN1_G].off - m.layout.layer[SRM_T_LN1_G].off) : 0;
+  p.layer0 = layer0_weights(m);
+  p.layer_bytes = layer_stride_bytes(m);
   p.S = s.layer_ptr(0);
   p.layer_stride = (int64_t)s.B * c.d_model * m.state_bytes();
   p.x = w.x; p.H = reinterpret_cast<bf16*>(w.H);

@@ -1,0 +1,410 @@
+// All layers of a decode pass of a hundred to a thousand rows as ONE persistent kernel.
+//
+// With so few rows a layer is a chain of three short kernels (token mixer, up projection, down projection over ranges of
+// K), and launch, ramp, first loads and drain of each cost more than its work: 25 us per layer at 256 rows of the mid
+// model, of which the operands need 5. Here one CTA pair per SM pair stays for the whole pass:
+//   - weights are constant, so a producer thread of their own streams every CTA's W1 and W2 tiles through a ring that
+//     runs ahead of everything else: a projection finds its first k-blocks in shared memory when its input is ready;
+//   - a pair computes at most one 256 x N tile of the up projection and one of the down projection per layer (the down
+//     projection's K cut into ranges), N the smallest of 64, 128, 256 with which the tiles fit on the pairs;
+//   - row phases (x + partial products of the previous down projection, LN1, cache update, residual, LN2) are done by two
+//     warps per row, the rows dealt to all CTAs;
+//   - the phases are ordered by counters in global memory, one per 256-row block (and range of K): rows done -> up tiles
+//     of the block start; up tiles of a range done -> down tiles of that range start; down tiles done -> rows of the
+//     block start. Nothing waits for a block it does not read.
+// Projections run as in gemm_tc_kernel: TMA loads (128-byte swizzle), tcgen05.mma.cta_group::2 issued by one thread of
+// the leader CTA, accumulator in tensor memory, 16 epilogue warps.
+//
+// Every piece of work waits for pieces of an earlier phase only, all CTAs are resident (the grid is the number of pairs
+// the device holds), and every wait is bounded: a waiter that gives up raises kStatusWaitTimeout and leaves its loops;
+// the others time out in turn, both CTAs of a pair meet at the final cluster barrier and the kernel ends.
+#pragma once
+
+#include <cuda.h>
+
+#include "common.cuh"
+#include "gemm_tc.cuh"
+#include "gemm_tc_splitk.cuh"   // fence_async_global
+#include "prefill_chunk.cuh"    // ld_acquire_u32
+#include "step_small.cuh"       // LayerW, group_stats, head_scalars, cp_async16, ld_relaxed_u32
+
+namespace srm {
+namespace mid {
+
+constexpr int kEpiWarp0 = 3;                                      // warp 0: A producer, 1: MMA, 2: W producer
+constexpr int kThreads = (kEpiWarp0 + tc::kEpiWarps) * 32;
+constexpr int kWorkers = tc::kEpiWarps * 32;                      // threads of the epilogue / row warps
+constexpr int kGroups = tc::kEpiWarps / 2;                        // rows a CTA works on at a time
+constexpr int kMaxWSlots = 16, kMaxASlots = 8;
+constexpr int kABytes = tc::kRowsPerCta * tc::BK * 2;             // one k-block of A per CTA
+constexpr int kTmemCols = 256;
+constexpr int kBarrierBytes = 512;
+constexpr int kMaxRowBlocks = 8, kMaxKSlices = 4;
+constexpr int kSmemBytes = 227 * 1024;
+constexpr long long kWaitLimitCycles = 1ll << 28;
+
+struct Params {
+  int R, d, F, V, h, n_ctx, L, t;
+  float eps;
+  int rb, n, cu, cd, ks;         // row blocks, tile width, column tiles of the up / down projection, ranges of K
+  int w_slots, a_slots;
+  const int32_t* tok_in;         // [R]
+  const bf16* E;
+  sb::LayerW layer0;             // as in sb::Params
+  int64_t layer_bytes;
+  void* S;                       // cache rows of layer 0; layer l at S + l * layer_stride (bytes)
+  int64_t layer_stride;
+  float* x;                      // [R, d]
+  bf16* a;                       // [R, d]
+  bf16* H;                       // [R, F]
+  float* part;                   // [ks] planes of plane_rows x d
+  int64_t plane;                 // elements per plane
+  uint32_t* cnt;                 // rows done [8] | up pieces done [8][4] | down pieces done [8]; zero on entry
+  uint32_t* status;
+  const int32_t* ctr;            // device-side step counters or nullptr
+  const int32_t* pos;            // [R] per-row positions or nullptr
+};
+constexpr int kCntWords = kMaxRowBlocks * (2 + kMaxKSlices);
+
+// Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers.
+__host__ __device__ inline size_t smem_bytes(int d, int n, int w_slots, int a_slots) {
+  return 1024 + (size_t)w_slots * (n / 2) * 128 + (size_t)a_slots * kABytes + (size_t)sb::kRowParamVecs * d * 4 + kGroups * 32 + kBarrierBytes;
+}
+
+// Tile widths and ranges of K for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit.
+inline bool plan(int64_t R, int d, int F, int pairs, Params* p) {
+  const int rb = (int)((R + tc::BM - 1) / tc::BM);
+  if (rb < 1 || rb > kMaxRowBlocks) return false;
+  for (int n = 64; n <= 256; n *= 2) {
+    if (F % n || d % n || rb * (F / n) > pairs) continue;
+    int ks = kMaxKSlices;
+    while (ks > 1 && (rb * (d / n) * ks > pairs || (F / 64) % ks || (F / ks) % n)) ks >>= 1;
+    if (rb * (d / n) * ks > pairs) continue;
+    p->rb = rb; p->n = n; p->cu = F / n; p->cd = d / n; p->ks = ks;
+    // the weight ring runs a phase ahead; the activation ring hides the latency of L2
+    p->w_slots = n == 64 ? 16 : n == 128 ? 10 : 6;
+    p->a_slots = n == 64 ? 8 : n == 128 ? 7 : 6;
+    while (smem_bytes(d, n, p->w_slots, p->a_slots) > (size_t)kSmemBytes) {
+      if (p->w_slots * (n / 2) * 128 > p->a_slots * kABytes) --p->w_slots; else --p->a_slots;
+      if (p->w_slots < 2 || p->a_slots < 2) return false;
+    }
+    return true;
+  }
+  return false;
+}
+
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr, int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(tc::smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_cluster_addr), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+__device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// One thread waits until the counter has reached `want`.
+__device__ __forceinline__ bool count_wait(const uint32_t* p, uint32_t want, uint32_t* status) {
+  if (sb::ld_relaxed_u32(p) < want) {
+    const long long t0 = clock64();
+    while (sb::ld_relaxed_u32(p) < want) {
+      if (clock64() - t0 > kWaitLimitCycles) { raise_status(status, kStatusWaitTimeout); return false; }
+    }
+  }
+  ld_acquire_u32(p);
+  return true;
+}
+__device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 9, %0;" ::"n"(kWorkers) : "memory"); }
+
+template <int NT, typename ST>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmW1,
+              const __grid_constant__ CUtensorMap tmW2, const Params p) {
+  pdl_trigger();
+  constexpr int d = NT * 256;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int n = p.n, w_rows = n >> 1, w_bytes = w_rows * 128;
+  uint8_t* sW = smem;
+  uint8_t* sA = sW + p.w_slots * w_bytes;
+  float* prm = reinterpret_cast<float*>(sA + p.a_slots * kABytes);
+  float* red = prm + sb::kRowParamVecs * d;
+  uint64_t* fullW = reinterpret_cast<uint64_t*>(red + kGroups * 8);      // used in the leader CTA
+  uint64_t* emptyW = fullW + kMaxWSlots;
+  uint64_t* fullA = emptyW + kMaxWSlots;                                 // used in the leader CTA
+  uint64_t* emptyA = fullA + kMaxASlots;
+  uint64_t* tfull = emptyA + kMaxASlots;
+  uint64_t* tempty = tfull + 1;                                          // leader: accumulator drained by both CTAs
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = tc::cluster_ctarank();
+  const int pair = blockIdx.x >> 1;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kMaxWSlots; ++i) { tc::mbar_init(&fullW[i], 2); tc::mbar_init(&emptyW[i], 1); }
+    for (int i = 0; i < kMaxASlots; ++i) { tc::mbar_init(&fullA[i], 2); tc::mbar_init(&emptyA[i], 1); }
+    tc::mbar_init(tfull, 1);
+    tc::mbar_init(tempty, 2 * tc::kEpiWarps);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(tmem_slot, kTmemCols);
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  tc::cluster_sync();
+  tc::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  // this pair's pieces
+  const int up_rb = pair % p.rb, up_col = pair / p.rb;
+  const bool up_on = up_col < p.cu;
+  const int dn_rb = up_rb, dn_col = up_col % p.cd, dn_slice = up_col / p.cd;
+  const bool dn_on = dn_slice < p.ks;
+  const int kb_up = d / tc::BK, kb_dn = p.F / tc::BK / p.ks;
+  const int slice_cols = p.F / p.ks;                                     // columns of H per range of K
+  uint32_t* cnt_rows = p.cnt;
+  uint32_t* cnt_up = p.cnt + kMaxRowBlocks;
+  uint32_t* cnt_dn = cnt_up + kMaxRowBlocks * kMaxKSlices;
+
+  if (warp == 2) {
+    // ---------------- weight stream (both CTAs): constant data, it waits for nothing but its ring ----------------
+    if (lane == 0) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW1)) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW2)) : "memory");
+      int slot = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int l = 0; ok && l < p.L; ++l) {
+        for (int ph = 0; ok && ph < 2; ++ph) {
+          if (!(ph ? dn_on : up_on)) continue;
+          const CUtensorMap* map = ph ? &tmW2 : &tmW1;
+          const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * kb_dn : 0;
+          const int row = (ph ? dn_col : up_col) * n + (int)rank * w_rows;
+          for (int kb = 0; kb < kbs; ++kb) {
+            if (!tc::mbar_wait(&emptyW[slot], phase ^ 1u, p.status)) { ok = false; break; }
+            const uint32_t full = tc::mapa(tc::smem_u32(&fullW[slot]), 0);
+            tc::mbar_expect_tx_cluster(full, (uint32_t)w_bytes);
+            tma_load_3d(sW + slot * w_bytes, map, full, (kb0 + kb) * tc::BK, row, l);
+            if (++slot == p.w_slots) { slot = 0; phase ^= 1u; }
+          }
+        }
+      }
+      if (!ok) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < (1ll << 21)) { }
+      }
+    }
+  } else if (warp == 0) {
+    // ---------------- activations (both CTAs) ----------------
+    if (lane == 0) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmH)) : "memory");
+      pdl_wait();
+      int slot = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      const int block_rows = min(tc::BM, p.R - up_rb * tc::BM);
+      for (int l = 0; ok && l < p.L; ++l) {
+        for (int ph = 0; ok && ph < 2; ++ph) {
+          if (!(ph ? dn_on : up_on)) continue;
+          // rows of the block done / the up tiles of this range of K done
+          if (!(ph ? count_wait(cnt_up + dn_rb * kMaxKSlices + dn_slice, (uint32_t)(l + 1) * 2u * (uint32_t)(slice_cols / n), p.status)
+                   : count_wait(cnt_rows + up_rb, (uint32_t)(l + 1) * (uint32_t)block_rows, p.status))) { ok = false; break; }
+          tc::fence_async_global();
+          const CUtensorMap* map = ph ? &tmH : &tmA;
+          const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * kb_dn : 0;
+          const int row = up_rb * tc::BM + (int)rank * tc::kRowsPerCta;
+          for (int kb = 0; kb < kbs; ++kb) {
+            if (!tc::mbar_wait(&emptyA[slot], phase ^ 1u, p.status)) { ok = false; break; }
+            const uint32_t full = tc::mapa(tc::smem_u32(&fullA[slot]), 0);
+            tc::mbar_expect_tx_cluster(full, kABytes);
+            tc::tma_load_2d(sA + slot * kABytes, map, full, (kb0 + kb) * tc::BK, row);
+            if (++slot == p.a_slots) { slot = 0; phase ^= 1u; }
+          }
+        }
+      }
+      if (!ok) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < (1ll << 21)) { }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer (leader CTA only) ----------------
+    if (rank == 0 && lane == 0) {
+      const uint32_t idesc = tc::instr_desc(n);
+      int sw = 0, sa = 0, piece = 0;
+      uint32_t pw = 0, pa = 0;
+      bool ok = true;
+      for (int l = 0; ok && l < p.L; ++l) {
+        for (int ph = 0; ok && ph < 2; ++ph) {
+          if (!(ph ? dn_on : up_on)) continue;
+          if (!tc::mbar_wait(tempty, (uint32_t)(piece & 1) ^ 1u, p.status)) { ok = false; break; }
+          tc::tc_fence_after();
+          const int kbs = ph ? kb_dn : kb_up;
+          for (int kb = 0; kb < kbs; ++kb) {
+            if (!tc::mbar_wait(&fullW[sw], pw, p.status) || !tc::mbar_wait(&fullA[sa], pa, p.status)) { ok = false; break; }
+            tc::tc_fence_after();
+            const uint64_t da = tc::make_smem_desc(tc::smem_u32(sA + sa * kABytes));
+            const uint64_t db = tc::make_smem_desc(tc::smem_u32(sW + sw * w_bytes));
+#pragma unroll
+            for (int k = 0; k < tc::BK / 16; ++k) tc::umma_bf16(tmem, da + 2u * k, db + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            tc::umma_commit_pair(&emptyW[sw]);
+            tc::umma_commit_pair(&emptyA[sa]);
+            if (++sw == p.w_slots) { sw = 0; pw ^= 1u; }
+            if (++sa == p.a_slots) { sa = 0; pa ^= 1u; }
+          }
+          if (ok) tc::umma_commit_pair(tfull);
+          ++piece;
+        }
+      }
+    }
+  } else {
+    // ---------------- rows and epilogues (both CTAs) ----------------
+    const int wid = threadIdx.x - kEpiWarp0 * 32;                // 0 .. kWorkers - 1
+    const int group = wid >> 6, c0 = (wid & 63) * 4;
+    const int quad = warp & 3, cgrp = (warp - kEpiWarp0) >> 2;
+    const int cols = n >> 2;                                     // accumulator columns per warp: 16, 32 or 64
+    pdl_wait();
+    const int t_all = p.ctr != nullptr ? p.ctr[kCtrPos] : p.t;
+    float* slot = red + group * 8;
+    int piece = 0;
+    bool ok = true;
+    for (int l = 0; l < p.L; ++l) {
+      const sb::LayerW w = sb::layer_w(p, l);
+      // ---- rows: row blockIdx.x + grid * group. Parameters first (constant data), then the wait ----
+      workers_sync();                     // the previous layer's parameters have been read
+      for (int i = wid; i < sb::kRowParamVecs * d / 4; i += kWorkers) {
+        const int k = i / (d / 4), c = i % (d / 4) * 4;
+        const float* q = k == 0 ? w.ln1_g : k == 1 ? w.ln1_b : k == 2 ? w.beta + (int64_t)t_all * d : k == 3 ? w.ln2_g : w.ln2_b;
+        sb::cp_async16(prm + i * 4, q + c);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      const int row = (int)blockIdx.x + (int)gridDim.x * group;
+      const bool mine = row < p.R;
+      const int t = mine && p.pos != nullptr ? min(max(p.pos[row], 0), p.n_ctx - 1) : t_all;
+      float a1[NT], a2[NT], lm[NT];
+      float4 s[NT], v[NT];
+      ST* Sr = reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + (int64_t)row * d + c0;
+      if (mine) {
+        sb::head_scalars<d, NT>(p, w, t, wid & 63, a1, a2, lm);
+#pragma unroll
+        for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + 256 * i);
+        if (l > 0 && (wid & 63) == 0 && ok)       // the down tiles of the row's block
+          ok = count_wait(cnt_dn + row / tc::BM, (uint32_t)l * 2u * (uint32_t)(p.cd * p.ks), p.status);
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      workers_sync();
+      if (mine) {
+        if (l == 0) {
+          int tk = p.tok_in[row];
+          if (tk < 0 || tk >= p.V) {
+            if ((wid & 63) == 0) raise_status(p.status, kStatusTokenRange);
+            tk = tk < 0 ? 0 : p.V - 1;
+          }
+#pragma unroll
+          for (int i = 0; i < NT; ++i) v[i] = ldg4(p.E + (int64_t)tk * d + c0 + 256 * i);
+        } else {                          // x + b2 + plane 0 + plane 1 + ... (other CTAs wrote the planes: not through L1)
+          const float* b2 = sb::layer_w(p, l - 1).b2 + c0;
+#pragma unroll
+          for (int i = 0; i < NT; ++i) {
+            v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c0 + 256 * i));
+            const float4 bb = ldg4(b2 + 256 * i);
+            v[i] = make_float4(v[i].x + bb.x, v[i].y + bb.y, v[i].z + bb.z, v[i].w + bb.w);
+          }
+#pragma unroll 2
+          for (int k = 0; k < p.ks; ++k) {
+            const float* q = p.part + (int64_t)k * p.plane + (int64_t)row * d + c0;
+#pragma unroll
+            for (int i = 0; i < NT; ++i) {
+              const float4 e = __ldcg(reinterpret_cast<const float4*>(q + 256 * i));
+              v[i] = make_float4(v[i].x + e.x, v[i].y + e.y, v[i].z + e.z, v[i].w + e.w);
+            }
+          }
+        }
+        const float* bt_p = p.pos != nullptr ? w.beta + (int64_t)t * d + c0 : prm + 2 * d + c0;
+        float mean, rstd;
+        sb::group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
+        const float nmr = -mean * rstd;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+          const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i), bt = ld4(bt_p + 256 * i);
+          const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
+                                       fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
+          // row-repeat head, Eq. 2: y = (a z + S) + b ; S' = l (S + a z).  column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
+          const float4 u = make_float4(fmaf(a1[i], z.x, s[i].x), fmaf(a1[i], z.y, s[i].y), fmaf(a1[i], z.z, s[i].z), fmaf(a1[i], z.w, s[i].w));
+          st4(Sr + 256 * i, make_float4(lm[i] * u.x, lm[i] * u.y, lm[i] * u.z, lm[i] * u.w));
+          v[i] = make_float4(v[i].x + fmaf(a2[i], u.x, bt.x), v[i].y + fmaf(a2[i], u.y, bt.y), v[i].z + fmaf(a2[i], u.z, bt.z),
+                             v[i].w + fmaf(a2[i], u.w, bt.w));
+          st4(p.x + (int64_t)row * d + c0 + 256 * i, v[i]);
+        }
+        sb::group_stats<d, NT>(v, p.eps, slot + 4, group, mean, rstd);
+        const float nmr2 = -mean * rstd;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+          const float4 g = ld4(prm + 3 * d + c0 + 256 * i), bb = ld4(prm + 4 * d + c0 + 256 * i);
+          st4(p.a + (int64_t)row * d + c0 + 256 * i,
+              make_float4(fmaf(fmaf(v[i].x, rstd, nmr2), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr2), g.y, bb.y),
+                          fmaf(fmaf(v[i].z, rstd, nmr2), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr2), g.w, bb.w)));
+        }
+        tc::fence_async_global();         // read by bulk tensor copies of other CTAs
+        asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
+        if ((wid & 63) == 0) red_release_add(cnt_rows + row / tc::BM, 1u);
+      }
+
+      // ---- epilogues ----
+      for (int ph = 0; ph < 2; ++ph) {
+        if (!(ph ? dn_on : up_on)) continue;
+        if (ok && !tc::mbar_wait(tfull, (uint32_t)(piece & 1), p.status)) ok = false;
+        ++piece;
+        tc::tc_fence_after();
+        const int r = up_rb * tc::BM + (int)rank * tc::kRowsPerCta + quad * 32 + lane;
+        const int col0 = (ph ? dn_col : up_col) * n + cgrp * cols;
+        const uint32_t taddr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(cgrp * cols);
+        for (int c = 0; c < cols; c += 16) {
+          uint32_t acc[16];
+          tc::tmem_ld16(taddr + c, acc);
+          tc::tmem_ld_wait();
+          if (ph == 0) {
+            uint32_t o[8];
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+              const float4 b = __ldg(reinterpret_cast<const float4*>(w.b1 + col0 + c + j));
+              const __nv_bfloat162 lo = __floats2bfloat162_rn(tc::gelu_fast(__uint_as_float(acc[j]) + b.x), tc::gelu_fast(__uint_as_float(acc[j + 1]) + b.y));
+              const __nv_bfloat162 hi = __floats2bfloat162_rn(tc::gelu_fast(__uint_as_float(acc[j + 2]) + b.z), tc::gelu_fast(__uint_as_float(acc[j + 3]) + b.w));
+              o[j / 2] = *reinterpret_cast<const uint32_t*>(&lo);
+              o[j / 2 + 1] = *reinterpret_cast<const uint32_t*>(&hi);
+            }
+            if (r < p.R) {
+              uint4* dst = reinterpret_cast<uint4*>(p.H + (int64_t)r * p.F + col0 + c);
+              dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+              dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+            }
+          } else if (r < p.R) {
+            uint4* dst = reinterpret_cast<uint4*>(p.part + (int64_t)dn_slice * p.plane + (int64_t)r * d + col0 + c);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dst[j] = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+          }
+        }
+        tc::tc_fence_before();
+        if (ph == 0) tc::fence_async_global();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive_cluster(tc::mapa(tc::smem_u32(tempty), 0));
+        workers_sync();
+        if (wid == 0)
+          red_release_add(ph ? cnt_dn + dn_rb : cnt_up + up_rb * kMaxKSlices + up_col * n / slice_cols, 1u);
+      }
+    }
+  }
+
+  // Both CTAs stay until the pair is done (see gemm_tc_kernel)
+  tc::tc_fence_before();
+  __syncwarp();
+  tc::cluster_sync();
+  if (warp == 1) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, kTmemCols);
+  }
+}
+
+}  // namespace mid
+}  // namespace srm

@@ -113,7 +113,8 @@ inline bool smem_plan(int B, int d, int F, int state_elem, Params* p, size_t* by
   return false;
 }
 
-__device__ __forceinline__ LayerW layer_w(const Params& p, int l) {
+template <typename P>
+__device__ __forceinline__ LayerW layer_w(const P& p, int l) {
   const int64_t o = (int64_t)l * p.layer_bytes;
   auto f = [o](const float* q) { return reinterpret_cast<const float*>(reinterpret_cast<const uint8_t*>(q) + o); };
   auto b = [o](const bf16* q) { return reinterpret_cast<const bf16*>(reinterpret_cast<const uint8_t*>(q) + o); };
@@ -334,13 +335,13 @@ __device__ __forceinline__ void fetch_row_params(const Params& p, int l, int t, 
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 // The head scalars of a thread's channels at position t: the multipliers of z before and of the sum after (one of them is
-// 1), and lambda. Thread i of a group owns channels 4 i .. 4 i + 3 (and 256, 512, ... further) of every row.
-template <int d, int NT>
-__device__ __forceinline__ void head_scalars(const Params& p, const LayerW& w, int t, float (&a1)[NT], float (&a2)[NT], float (&lm)[NT]) {
+// 1), and lambda. Thread `th` of a group owns channels 4 th .. 4 th + 3 (and 256, 512, ... further) of every row.
+template <int d, int NT, typename P>
+__device__ __forceinline__ void head_scalars(const P& p, const LayerW& w, int t, int th, float (&a1)[NT], float (&a2)[NT], float (&lm)[NT]) {
   const int dh = d / p.h;
 #pragma unroll
   for (int i = 0; i < NT; ++i) {
-    const int g = ((threadIdx.x & 63) * 4 + 256 * i) / dh;
+    const int g = (th * 4 + 256 * i) / dh;
     const float al = __ldg(w.alpha + (int64_t)g * p.n_ctx + t);
     const bool is_row = g < (p.h >> 1);
     a1[i] = is_row ? al : 1.0f;
@@ -430,7 +431,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
   float a1[NT], a2[NT], lm[NT];
   float* prm = part;                                     // (with the exchange buffer behind it)
   fetch_row_params<d>(p, 0, p.pos != nullptr ? 0 : t_all, prm);
-  head_scalars<d, NT>(p, layer_w(p, 0), p.pos != nullptr ? 0 : t_all, a1, a2, lm);
+  head_scalars<d, NT>(p, layer_w(p, 0), p.pos != nullptr ? 0 : t_all, tid & 63, a1, a2, lm);
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   // bytes of the rows that the other CTAs of the cluster send per row phase
@@ -476,7 +477,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
           if (p.pos != nullptr) {                        // a position per row: its own beta row and head scalars
             const int t = t_of(row);
             bt_p = w.beta + (int64_t)t * d + c0;
-            head_scalars<d, NT>(p, w, t, a1, a2, lm);
+            head_scalars<d, NT>(p, w, t, tid & 63, a1, a2, lm);
           }
           group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
           const float nmr = -mean * rstd;
@@ -603,7 +604,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
       }
       const int t = p.pos != nullptr ? 0 : t_all;
       fetch_row_params<d>(p, l + 1, t, prm);
-      if (l + 1 < p.L) head_scalars<d, NT>(p, layer_w(p, l + 1), t, a1, a2, lm);
+      if (l + 1 < p.L) head_scalars<d, NT>(p, layer_w(p, l + 1), t, tid & 63, a1, a2, lm);
     });
   }
   if (!one_region) for (int ch = p.lm_stages_w1; ch < p.lm_stages; ++ch) stage_lm(ch);

@@ -1,0 +1,84 @@
+"""Decode passes whose layers run as one kernel (layers_mid.cuh), at the edges of its tile widths and row blocks: logits,
+tokens and cache against the kernel-per-operation path fed the same tokens (same products, sums in another order: the
+bound is the one the paths with and without ranges of K are held to), a row of the batch against the oracle, equal and
+per-sample positions, and the captured step."""
+import numpy as np
+import pytest
+import torch
+
+import srm_inputs as I
+from helpers import custom_shape, oracle_for, rel_err_rows, top2_margin
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _launches(P, f):
+    n0 = P.SRM.kernel_launches()
+    f()
+    return P.SRM.kernel_launches() - n0
+
+
+@pytest.mark.parametrize("B,d,state_dtype,ragged", [(97, 512, "fp32", False), (256, 1024, "fp16", False), (257, 1024, "fp32", True),
+                                                    (512, 1024, "bf16", False), (1024, 1024, "fp32", False), (130, 1536, "fp32", True),
+                                                    (768, 1536, "fp16", False), (1000, 512, "fp32", False)])
+def test_layers_in_one_kernel_agree_with_the_kernel_per_operation_path(B, d, state_dtype, ragged):
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=3, d_model=d, vocab=2048, n_ctx=24, dtype="bf16", seed=11)
+    W = I.make_weights(shape)
+    rng = np.random.default_rng(B)
+    n = 5
+    prompts_np = rng.integers(0, shape.vocab, size=(B, n)).astype(np.int32)
+    lens_np = rng.integers(1, n + 1, size=B).astype(np.int32) if ragged else np.full(B, n, np.int32)
+    prompts, lens = torch.from_numpy(prompts_np).to(DEV), torch.from_numpy(lens_np).to(DEV)
+    g = P.Sampling("greedy")
+    outs, fed = [], None
+    for flags in (P.FLAG_NO_SMALL_BATCH, 0):                   # the second run consumes the first run's tokens
+        m = P.SRM(shape, W, device=DEV, flags=flags, state_dtype=state_dtype)
+        st, ws = m.new_state(B), m.new_workspace(B, n, prefill_samples=B)
+        tok = m.prefill_ragged(st, prompts, lens, g, ws) if ragged else m.prefill(st, prompts, g, ws)
+        lgs, toks = [], [tok.clone()]
+        for k in range(3):
+            res = []
+            launches = _launches(P, lambda: res.append(m.decode_step(st, tok if fed is None else fed[k], g, k + 1, ws, want_logits=True)))
+            tok, lg = res[0]
+            lgs.append(lg.cpu().numpy())
+            toks.append(tok.clone())
+        assert (launches <= 4) == (flags == 0)                 # layers, norm, LM head, selection
+        assert st.status() == 0
+        fed = fed if fed is not None else toks
+        outs.append((np.stack(lgs), torch.stack(toks).cpu().numpy(), st.cache().cpu().numpy()))
+    (lg_a, tok_a, S_a), (lg_b, tok_b, S_b) = outs
+    # Sums in another order flip roundings of bf16 activations, 2^-8 of the value each. Were half of them flipped, a
+    # layer would move its output by 2^-9 of its scale, three layers by 2^-9 sqrt(3); five standard deviations of that:
+    tol = 5 * 2.0 ** -9 * 3 ** 0.5
+    assert rel_err_rows(lg_b, lg_a) < tol and rel_err_rows(S_b, S_a) < tol
+    differ = tok_a[1:] != tok_b[1:]
+    assert np.all(top2_margin(lg_a)[differ] < 2e-2)
+    orc = oracle_for(shape, W)
+    for b in (0, B // 2, B - 1):
+        lo, state = orc.forward_parallel(prompts_np[b:b + 1, :lens_np[b]])
+        for k in range(3):
+            lo, state = orc.decode_step(state, tok_a[k][b:b + 1], int(lens_np[b]) + k)
+            assert rel_err_rows(lg_b[k][b:b + 1], lo) < 3e-2
+
+
+def test_captured_step_and_passes_of_one_kernel_equal_launch_by_launch():
+    """300 rows in one pass; the same steps replayed from a graph; and 300 rows as passes of 150 (same tile width)."""
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=3, d_model=512, vocab=1024, n_ctx=24, dtype="bf16", seed=12)
+    W = I.make_weights(shape)
+    B = 300
+    prompts = torch.from_numpy(np.random.default_rng(3).integers(0, shape.vocab, size=(B, 4)).astype(np.int32)).to(DEV)
+    samp = P.Sampling("topk", 50, 0.8, seed=5, sample_idx_base=7)
+    res = []
+    for flags, chunk in ((P.FLAG_NO_GRAPH, B), (P.FLAG_GRAPH, B), (P.FLAG_NO_GRAPH, 150)):
+        m = P.SRM(shape, W, device=DEV, flags=flags)
+        st, ws = m.new_state(B), m.new_workspace(chunk, 4, prefill_samples=chunk)
+        first = m.prefill(st, prompts, samp, ws)
+        out = m.generate(st, 8, 1, samp, ws)
+        assert st.status() == 0
+        res.append((first.clone(), out.clone(), st.cache().clone()))
+    for r in res[1:]:
+        for x, y in zip(res[0], r):
+            assert torch.equal(x, y)
