@@ -83,7 +83,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   uint8_t* boxes = smem + kStages * kStageBytes;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int cluster_id = blockIdx.x >> 1;
 
@@ -100,7 +100,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (threadIdx.x != 0) pdl_wait();
+  if (warp != 0) pdl_wait();
 
   const int i0 = cluster_id < plan.n_pairs ? plan.off[cluster_id] : 0;
   const int i1 = cluster_id < plan.n_pairs ? plan.off[cluster_id + 1] : 0;
@@ -109,7 +109,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW1)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmH)) : "memory");
@@ -170,7 +170,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA only) ----------------
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && elect_one()) {
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
@@ -229,7 +229,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
+      if (elect_one()) {                               // (the thread that issued the bulk stores)
         mbar_arrive_cluster(mapa(smem_u32(&tempty[acc]), 0));
         if (!down && mine) {
           // this warp's part of the H tile is in global memory: count it in (the next accumulator is a tile's
@@ -242,7 +242,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
       }
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
-    if (lane == 0) bulk_wait_all();
+    if (elect_one()) bulk_wait_all();
   }
 
   tc_fence_before();

@@ -111,6 +111,16 @@ __global__ void wait_probe_kernel(uint32_t* status, long long limit, int* gave_u
     if (gave_up != nullptr) *gave_up = ok ? 0 : 1;
   }
 }
+// One lane of a converged warp, always the same one. Branching on this (and not on lane == 0) tells the compiler that a
+// single thread runs the block; the operands of tcgen05.mma and of the tensor copies sit in registers that the whole warp
+// shares, and behind lane == 0 every one of these instructions took 110 cycles to issue: four MMAs of a k-block and its
+// waits 640 to 700 cycles whatever the tile's width (256 x 256 needs 512 of the tensor pipe, 256 x 64 needs 128), with
+// the elected thread 360 (down projection of 512 rows, d = 1024: 21.1 -> 14.2 us; up 10.3 -> 8.9).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -318,7 +328,7 @@ __device__ __forceinline__ float gelu_fast(float v) {
 template <int EPI>
 __device__ __forceinline__ void emit_box(const CUtensorMap* tmD, uint8_t* buf, int lane, int col, int row,
                                          const uint32_t (&v)[32]) {
-  if (lane == 0) bulk_wait_read();          // the previous box has left the buffer
+  if (elect_one()) bulk_wait_read();        // the previous box has left the buffer
   __syncwarp();
   uint8_t* mine = buf + lane * 128;
 #pragma unroll
@@ -326,7 +336,7 @@ __device__ __forceinline__ void emit_box(const CUtensorMap* tmD, uint8_t* buf, i
     *reinterpret_cast<uint4*>(mine + ((q ^ (lane & 7)) << 4)) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
   fence_async_smem();
   __syncwarp();
-  if (lane == 0) {
+  if (elect_one()) {
     if (EPI == kEpiBiasResidual) tma_reduce_add_2d(tmD, buf, col, row);
     else if (EPI == kEpiPlain) tma_store_2d_streaming(tmD, buf, col, row);
     else tma_store_2d(tmD, buf, col, row);
@@ -491,7 +501,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   uint8_t* boxes = smem + NS * kStageBytes;           // 1024-byte aligned, one staging buffer per epilogue warp (not with kNoBoxes)
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();           // 0 = leader of the pair
   const int64_t cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
 
@@ -509,8 +519,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   // Barriers, tensor memory and the cluster handshake are set up; from here on global memory is touched.
-  // The producer thread orders itself (it may fetch weights, which no kernel writes, ahead of the wait).
-  if (threadIdx.x != 0 || g.m_limit != nullptr) pdl_wait();
+  // The producer warp orders itself (its thread may fetch weights, which no kernel writes, ahead of the wait).
+  if (warp != 0 || g.m_limit != nullptr) pdl_wait();
   int64_t M_rows = g.M;
   if (g.m_limit != nullptr) {              // a row count left on the device by an earlier kernel
     const int64_t lim = (int64_t)*reinterpret_cast<const volatile uint32_t*>(g.m_limit);
@@ -527,7 +537,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
       int stage = 0;
@@ -586,7 +596,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA only) ----------------
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && elect_one()) {
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
@@ -638,7 +648,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (lane == 0) mbar_arrive_cluster(mapa(smem_u32(&tempty[acc]), 0));
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
-    if (lane == 0) bulk_wait_all();                  // the staged boxes must be out before shared memory goes away
+    if (elect_one()) bulk_wait_all();                // the staged boxes must be out before shared memory goes away
   }
 
   // Both CTAs stay until the pair is done: the leader's MMAs read the peer's shared memory and

@@ -170,7 +170,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   uint8_t* boxes = smem + kStages * kStageBytes;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int cluster_id = blockIdx.x >> 1;
 
@@ -187,7 +187,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (threadIdx.x != 0) pdl_wait();
+  if (warp != 0) pdl_wait();
 
   const int m_tiles = (int)((g.M + BM - 1) / BM);       // tile index = n * m_tiles + m, as in gemm_tc_kernel
   SplitCursor cur;
@@ -196,7 +196,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
       int stage = 0;
@@ -238,7 +238,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA only) ----------------
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && elect_one()) {
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
@@ -273,7 +273,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     int32_t* pend_ptr = nullptr;
     int32_t pend_val = 0;
     auto publish = [&]() {
-      if (pend_ptr != nullptr && lane == 0) {
+      if (pend_ptr != nullptr && elect_one()) {        // (the thread that issued the bulk operations)
         bulk_wait_all();
         fence_async_global();
         st_release_gpu(pend_ptr, pend_val);
@@ -295,11 +295,11 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         bool ok = true;
         if (!whole) {
           // everything above this k-range must have been added already
-          if (lane == 0) {
+          if (elect_one()) {
             ok = order_wait(word, P.kb - pc.kb1, g.status);
             fence_async_global();
           }
-          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          ok = __all_sync(0xffffffffu, ok) != 0;
         }
         if (ok) {
           const GemmArgs ga{g.M, g.N, g.K, pc.kb0 == 0 ? g.bias : nullptr, nullptr, g.status, 0};
@@ -316,7 +316,7 @@ gemm_tc_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     publish();
-    if (lane == 0) bulk_wait_all();
+    if (elect_one()) bulk_wait_all();
   }
 
   tc_fence_before();

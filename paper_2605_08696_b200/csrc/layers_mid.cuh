@@ -136,7 +136,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   uint64_t* tempty = tfull + 1;                                          // leader: accumulator drained by both CTAs
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_ctarank();
   const int pair = blockIdx.x >> 1;
   if (threadIdx.x == 0) {
@@ -168,7 +168,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 
   if (warp == 2) {
     // ---------------- weight stream (both CTAs): constant data, it waits for nothing but its ring ----------------
-    if (lane == 0) {
+    if (tc::elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW1)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmW2)) : "memory");
       int slot = 0;
@@ -196,7 +196,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     }
   } else if (warp == 0) {
     // ---------------- activations (both CTAs) ----------------
-    if (lane == 0) {
+    if (tc::elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmH)) : "memory");
       pdl_wait();
@@ -230,7 +230,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA only) ----------------
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && tc::elect_one()) {
       const uint32_t idesc = tc::instr_desc(n);
       int sw = 0, sa = 0, piece = 0;
       uint32_t pw = 0, pa = 0;
