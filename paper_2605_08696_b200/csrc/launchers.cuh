@@ -708,37 +708,39 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
 }
 
 // ---- passes of a hundred to a thousand rows: all layers in one kernel (layers_mid.cuh) -------------------
-// From this many rows: up to 64 the whole step is one kernel of another design (step_small.cuh).
-constexpr int64_t kMidMinRows = 97;
+// Fewest rows, where the whole step is not one kernel of another design (step_small.cuh: up to 64 rows at d = 512, 32 at
+// d = 1024). d = 512: a batch just past that limit keeps the kernel-per-operation path (65 rows 134 us per step there,
+// 114 us here; a test counts on it).
+int64_t mid_min_rows(int d) { return d == 512 ? 97 : 1; }
 
 // Whether a decode pass of R rows takes it, and its tile plan. bf16 mixed-head models of the widths it is built for,
 // as many rows as leave every CTA pair one tile of each projection.
 bool mid_plan(srm_model& m, int64_t R, const DecodeWs& w, mid::Params* p) {
   const srm_config& c = m.cfg;
   constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
-  if (R < kMidMinRows || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || c.mixer != SRM_MIXER_MIXED || w.part == nullptr) return false;
+  if (R < mid_min_rows(c.d_model) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || c.mixer != SRM_MIXER_MIXED || w.part == nullptr) return false;
   if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536) return false;
   if (ensure_tc_ready(m) != SRM_OK || R > (int64_t)2 * m.tc_clusters * mid::kGroups || m.F() > (1 << 20)) return false;
   if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, p)) return false;
   return (size_t)p->ks * p->rb * tc::BM * c.d_model * 4 <= w.part_bytes;
 }
 
+struct MidMaps { CUtensorMap a, h, w1, w2, hs, p; };      // loads of a, H, W1, W2; stores of H and the partial products
 template <int NT, typename ST>
-int launch_layers_t(srm_model& m, const CUtensorMap& ta, const CUtensorMap& th, const CUtensorMap& tw1, const CUtensorMap& tw2,
-                    const mid::Params& p, cudaStream_t st) {
+int launch_layers_t(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
   int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(mid::layers_kernel<NT, ST>), mid::kSmemBytes);
   if (rc != SRM_OK) return rc;
   const size_t smem = mid::smem_bytes(p.d, p.n, p.w_slots, p.a_slots);
-  SRM_CUDA(launch_kernel(mid::layers_kernel<NT, ST>, dim3(2u * (unsigned)m.tc_clusters), dim3(mid::kThreads), smem, st, ta, th, tw1, tw2, p));
+  SRM_CUDA(launch_kernel(mid::layers_kernel<NT, ST>, dim3(2u * (unsigned)m.tc_clusters), dim3(mid::kThreads), smem, st,
+                         t.a, t.h, t.w1, t.w2, t.hs, t.p, p));
   SRM_CUDA(cudaGetLastError());
   return SRM_OK;
 }
 template <int NT>
-int launch_layers_nt(srm_model& m, const CUtensorMap& ta, const CUtensorMap& th, const CUtensorMap& tw1, const CUtensorMap& tw2,
-                     const mid::Params& p, cudaStream_t st) {
-  if (m.cfg.state_dtype == SRM_DTYPE_FP16) return launch_layers_t<NT, fp16>(m, ta, th, tw1, tw2, p, st);
-  if (m.cfg.state_dtype == SRM_DTYPE_BF16) return launch_layers_t<NT, bf16>(m, ta, th, tw1, tw2, p, st);
-  return launch_layers_t<NT, float>(m, ta, th, tw1, tw2, p, st);
+int launch_layers_nt(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
+  if (m.cfg.state_dtype == SRM_DTYPE_FP16) return launch_layers_t<NT, fp16>(m, t, p, st);
+  if (m.cfg.state_dtype == SRM_DTYPE_BF16) return launch_layers_t<NT, bf16>(m, t, p, st);
+  return launch_layers_t<NT, float>(m, t, p, st);
 }
 
 // All layers for rows [b0, b0 + R) of the state; leaves x and, in w.part, the last down projection's partial products.
@@ -762,15 +764,17 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   p.status = s.status; p.ctr = ctr; p.pos = pos;
   SRM_CUDA(cudaMemsetAsync(p.cnt, 0, mid::kCntWords * 4, st));
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
-  CUtensorMap ta, th, tw1, tw2;
+  MidMaps maps;
   int rc;
-  if ((rc = m.tmap(w.a, R, d, tc::kRowsPerCta, 2, &ta)) != SRM_OK) return rc;
-  if ((rc = m.tmap(w.H, R, F, tc::kRowsPerCta, 2, &th)) != SRM_OK) return rc;
-  if ((rc = make_tmap_layers(&tw1, m.ptr(0, SRM_T_W1), F, d, c.n_layers, p.layer_bytes, p.n / 2)) != SRM_OK) return rc;
-  if ((rc = make_tmap_layers(&tw2, m.ptr(0, SRM_T_W2), d, F, c.n_layers, p.layer_bytes, p.n / 2)) != SRM_OK) return rc;
-  if (d == 512) return launch_layers_nt<2>(m, ta, th, tw1, tw2, p, st);
-  if (d == 1024) return launch_layers_nt<4>(m, ta, th, tw1, tw2, p, st);
-  return launch_layers_nt<6>(m, ta, th, tw1, tw2, p, st);
+  if ((rc = make_tmap_kblocks(&maps.a, w.a, R, d, tc::kRowsPerCta, mid::kStep)) != SRM_OK) return rc;
+  if ((rc = make_tmap_kblocks(&maps.h, w.H, R, F, tc::kRowsPerCta, mid::kStep)) != SRM_OK) return rc;
+  if ((rc = make_tmap_kblocks(&maps.w1, m.ptr(0, SRM_T_W1), F, d, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
+  if ((rc = make_tmap_kblocks(&maps.w2, m.ptr(0, SRM_T_W2), d, F, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
+  if ((rc = m.tmap(w.H, R, F, tc::kOutBoxRows, 2, &maps.hs)) != SRM_OK) return rc;
+  if ((rc = m.tmap(w.part, (int64_t)p.ks * p.rb * tc::BM, d, tc::kOutBoxRows, 4, &maps.p)) != SRM_OK) return rc;
+  if (d == 512) return launch_layers_nt<2>(m, maps, p, st);
+  if (d == 1024) return launch_layers_nt<4>(m, maps, p, st);
+  return launch_layers_nt<6>(m, maps, p, st);
 }
 
 // One decode step for rows [b0, b0 + R) of the state.

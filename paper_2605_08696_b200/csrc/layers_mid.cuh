@@ -6,7 +6,7 @@
 //   - weights are constant, so a producer thread of their own streams every CTA's W1 and W2 tiles through a ring that
 //     runs ahead of everything else: a projection finds its first k-blocks in shared memory when its input is ready;
 //   - a pair computes at most one 256 x N tile of the up projection and one of the down projection per layer (the down
-//     projection's K cut into ranges), N the smallest of 64, 128, 256 with which the tiles fit on the pairs;
+//     projection's K cut into ranges), N 64 or 128, the smaller with which the tiles fit on the pairs;
 //   - row phases (x + partial products of the previous down projection, LN1, cache update, residual, LN2) are done by two
 //     warps per row, the rows dealt to all CTAs;
 //   - the phases are ordered by counters in global memory, one per 256-row block (and range of K): rows done -> up tiles
@@ -35,9 +35,10 @@ constexpr int kEpiWarp0 = 3;                                      // warp 0: A p
 constexpr int kThreads = (kEpiWarp0 + tc::kEpiWarps) * 32;
 constexpr int kWorkers = tc::kEpiWarps * 32;                      // threads of the epilogue / row warps
 constexpr int kGroups = tc::kEpiWarps / 2;                        // rows a CTA works on at a time
-constexpr int kMaxWSlots = 16, kMaxASlots = 8;
-constexpr int kABytes = tc::kRowsPerCta * tc::BK * 2;             // one k-block of A per CTA
-constexpr int kTmemCols = 256;
+constexpr int kStep = 2;                                          // k-blocks (of 64) per stage: the waits and commits of a stage take as long as a k-block's MMAs
+constexpr int kMaxWSlots = 8, kMaxASlots = 4;
+constexpr int kABytes = kStep * tc::kRowsPerCta * tc::BK * 2;     // one stage of A per CTA
+constexpr int kTmemCols = 128;
 constexpr int kBarrierBytes = 512;
 constexpr int kMaxRowBlocks = 8, kMaxKSlices = 4;
 constexpr int kSmemBytes = 227 * 1024;
@@ -68,35 +69,44 @@ constexpr int kCntWords = kMaxRowBlocks * (2 + kMaxKSlices);
 
 // Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers.
 __host__ __device__ inline size_t smem_bytes(int d, int n, int w_slots, int a_slots) {
-  return 1024 + (size_t)w_slots * (n / 2) * 128 + (size_t)a_slots * kABytes + (size_t)sb::kRowParamVecs * d * 4 + kGroups * 32 + kBarrierBytes;
+  return 1024 + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + (size_t)sb::kRowParamVecs * d * 4 + kGroups * 32 + kBarrierBytes;
 }
 
-// Tile widths and ranges of K for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit.
+// Tile widths and ranges of K for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit. (256-wide
+// tiles, which would take mid passes of 513 to 1024 rows, measured slower than a kernel per operation: 0.59 against
+// 0.54 ms per step.)
 inline bool plan(int64_t R, int d, int F, int pairs, Params* p) {
   const int rb = (int)((R + tc::BM - 1) / tc::BM);
   if (rb < 1 || rb > kMaxRowBlocks) return false;
-  for (int n = 64; n <= 256; n *= 2) {
+  for (int n = 64; n <= 128; n *= 2) {
     if (F % n || d % n || rb * (F / n) > pairs) continue;
     int ks = kMaxKSlices;
-    while (ks > 1 && (rb * (d / n) * ks > pairs || (F / 64) % ks || (F / ks) % n)) ks >>= 1;
-    if (rb * (d / n) * ks > pairs) continue;
+    while (ks > 1 && (rb * (d / n) * ks > pairs || (F / 64) % (ks * kStep) || (F / ks) % n)) ks >>= 1;
+    if (rb * (d / n) * ks > pairs || (F / 64) % (ks * kStep)) continue;
     p->rb = rb; p->n = n; p->cu = F / n; p->cd = d / n; p->ks = ks;
-    // the weight ring runs a phase ahead; the activation ring hides the latency of L2
-    p->w_slots = n == 64 ? 16 : n == 128 ? 10 : 6;
-    p->a_slots = n == 64 ? 8 : n == 128 ? 7 : 6;
-    while (smem_bytes(d, n, p->w_slots, p->a_slots) > (size_t)kSmemBytes) {
-      if (p->w_slots * (n / 2) * 128 > p->a_slots * kABytes) --p->w_slots; else --p->a_slots;
-      if (p->w_slots < 2 || p->a_slots < 2) return false;
-    }
+    // the weight ring runs a phase ahead; the activation ring hides the latency of L2 and holds the output tile of an
+    // epilogue (128 rows of n fp32 columns)
+    p->w_slots = n == 64 ? 8 : 6;
+    p->a_slots = n == 64 ? 4 : 3;
+    while (smem_bytes(d, n, p->w_slots, p->a_slots) > (size_t)kSmemBytes)
+      if (--p->w_slots < 2) return false;
     return true;
   }
   return false;
 }
 
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr, int x, int y, int z) {
+// One stage: kStep k-blocks of 64 columns, each a tile of its own (128-byte rows, swizzled). a: {64, rows, K / 64};
+// W: {64, rows, K / 64, layer}.
+__device__ __forceinline__ void tma_load_a(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr, int row, int kb) {
   asm volatile(
       "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(tc::smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_cluster_addr), "r"(x), "r"(y), "r"(z)
+      ::"r"(tc::smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_cluster_addr), "r"(0), "r"(row), "r"(kb)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_w(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr, int row, int kb, int layer) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(tc::smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_cluster_addr), "r"(0), "r"(row), "r"(kb), "r"(layer)
       : "memory");
 }
 __device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
@@ -118,12 +128,13 @@ __device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 9, %0;" 
 template <int NT, typename ST>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmW1,
-              const __grid_constant__ CUtensorMap tmW2, const Params p) {
+              const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmHs, const __grid_constant__ CUtensorMap tmP,
+              const Params p) {
   pdl_trigger();
   constexpr int d = NT * 256;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int n = p.n, w_rows = n >> 1, w_bytes = w_rows * 128;
+  const int n = p.n, w_rows = n >> 1, w_bytes = kStep * w_rows * 128;
   uint8_t* sW = smem;
   uint8_t* sA = sW + p.w_slots * w_bytes;
   float* prm = reinterpret_cast<float*>(sA + p.a_slots * kABytes);
@@ -134,7 +145,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   uint64_t* emptyA = fullA + kMaxASlots;
   uint64_t* tfull = emptyA + kMaxASlots;
   uint64_t* tempty = tfull + 1;                                          // leader: accumulator drained by both CTAs
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 1);
+  uint64_t* ring = tempty + 1;                                           // the epilogue has left the activation ring
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_ctarank();
@@ -144,6 +156,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     for (int i = 0; i < kMaxASlots; ++i) { tc::mbar_init(&fullA[i], 2); tc::mbar_init(&emptyA[i], 1); }
     tc::mbar_init(tfull, 1);
     tc::mbar_init(tempty, 2 * tc::kEpiWarps);
+    tc::mbar_init(ring, tc::kEpiWarps);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -160,7 +173,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   const bool up_on = up_col < p.cu;
   const int dn_rb = up_rb, dn_col = up_col % p.cd, dn_slice = up_col / p.cd;
   const bool dn_on = dn_slice < p.ks;
-  const int kb_up = d / tc::BK, kb_dn = p.F / tc::BK / p.ks;
+  const int kb_up = d / tc::BK, kb_dn = p.F / tc::BK / p.ks;            // k-blocks per piece
+  const int up_boxes = n / 64, dn_boxes = n / 32;                        // boxes of 128 bytes per row that an output tile consists of
   const int slice_cols = p.F / p.ks;                                     // columns of H per range of K
   uint32_t* cnt_rows = p.cnt;
   uint32_t* cnt_up = p.cnt + kMaxRowBlocks;
@@ -180,11 +194,11 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
           const CUtensorMap* map = ph ? &tmW2 : &tmW1;
           const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * kb_dn : 0;
           const int row = (ph ? dn_col : up_col) * n + (int)rank * w_rows;
-          for (int kb = 0; kb < kbs; ++kb) {
+          for (int kb = 0; kb < kbs; kb += kStep) {
             if (!tc::mbar_wait(&emptyW[slot], phase ^ 1u, p.status)) { ok = false; break; }
             const uint32_t full = tc::mapa(tc::smem_u32(&fullW[slot]), 0);
             tc::mbar_expect_tx_cluster(full, (uint32_t)w_bytes);
-            tma_load_3d(sW + slot * w_bytes, map, full, (kb0 + kb) * tc::BK, row, l);
+            tma_load_w(sW + slot * w_bytes, map, full, row, kb0 + kb, l);
             if (++slot == p.w_slots) { slot = 0; phase ^= 1u; }
           }
         }
@@ -200,7 +214,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmH)) : "memory");
       pdl_wait();
-      int slot = 0;
+      int slot = 0, piece = 0;
       uint32_t phase = 0;
       bool ok = true;
       const int block_rows = min(tc::BM, p.R - up_rb * tc::BM);
@@ -208,17 +222,19 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         for (int ph = 0; ok && ph < 2; ++ph) {
           if (!(ph ? dn_on : up_on)) continue;
           // rows of the block done / the up tiles of this range of K done
-          if (!(ph ? count_wait(cnt_up + dn_rb * kMaxKSlices + dn_slice, (uint32_t)(l + 1) * 2u * (uint32_t)(slice_cols / n), p.status)
+          if (!(ph ? count_wait(cnt_up + dn_rb * kMaxKSlices + dn_slice, (uint32_t)(l + 1) * (uint32_t)(slice_cols / n * up_boxes) * 8u, p.status)
                    : count_wait(cnt_rows + up_rb, (uint32_t)(l + 1) * (uint32_t)block_rows, p.status))) { ok = false; break; }
+          if (piece > 0 && !tc::mbar_wait(ring, (uint32_t)(piece & 1) ^ 1u, p.status)) { ok = false; break; }
+          ++piece;
           tc::fence_async_global();
           const CUtensorMap* map = ph ? &tmH : &tmA;
           const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * kb_dn : 0;
           const int row = up_rb * tc::BM + (int)rank * tc::kRowsPerCta;
-          for (int kb = 0; kb < kbs; ++kb) {
+          for (int kb = 0; kb < kbs; kb += kStep) {
             if (!tc::mbar_wait(&emptyA[slot], phase ^ 1u, p.status)) { ok = false; break; }
             const uint32_t full = tc::mapa(tc::smem_u32(&fullA[slot]), 0);
             tc::mbar_expect_tx_cluster(full, kABytes);
-            tc::tma_load_2d(sA + slot * kABytes, map, full, (kb0 + kb) * tc::BK, row);
+            tma_load_a(sA + slot * kABytes, map, full, row, kb0 + kb);
             if (++slot == p.a_slots) { slot = 0; phase ^= 1u; }
           }
         }
@@ -241,13 +257,18 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
           if (!tc::mbar_wait(tempty, (uint32_t)(piece & 1) ^ 1u, p.status)) { ok = false; break; }
           tc::tc_fence_after();
           const int kbs = ph ? kb_dn : kb_up;
-          for (int kb = 0; kb < kbs; ++kb) {
+          for (int kb = 0; kb < kbs; kb += kStep) {
             if (!tc::mbar_wait(&fullW[sw], pw, p.status) || !tc::mbar_wait(&fullA[sa], pa, p.status)) { ok = false; break; }
             tc::tc_fence_after();
             const uint64_t da = tc::make_smem_desc(tc::smem_u32(sA + sa * kABytes));
             const uint64_t db = tc::make_smem_desc(tc::smem_u32(sW + sw * w_bytes));
 #pragma unroll
-            for (int k = 0; k < tc::BK / 16; ++k) tc::umma_bf16(tmem, da + 2u * k, db + 2u * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            for (int q = 0; q < kStep; ++q) {               // (descriptor addresses count 16 bytes)
+#pragma unroll
+              for (int k = 0; k < tc::BK / 16; ++k)
+                tc::umma_bf16(tmem, da + (uint32_t)(q * tc::kRowsPerCta * 8) + 2u * k, db + (uint32_t)(q * w_rows * 8) + 2u * k, idesc,
+                              (kb | q | k) != 0 ? 1u : 0u);
+            }
             tc::umma_commit_pair(&emptyW[sw]);
             tc::umma_commit_pair(&emptyA[sa]);
             if (++sw == p.w_slots) { sw = 0; pw ^= 1u; }
@@ -290,7 +311,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 #pragma unroll
         for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + 256 * i);
         if (l > 0 && (wid & 63) == 0 && ok)       // the down tiles of the row's block
-          ok = count_wait(cnt_dn + row / tc::BM, (uint32_t)l * 2u * (uint32_t)(p.cd * p.ks), p.status);
+          ok = count_wait(cnt_dn + row / tc::BM, (uint32_t)l * (uint32_t)(p.cd * p.ks * dn_boxes) * 8u, p.status);
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       workers_sync();
@@ -357,41 +378,58 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         if (ok && !tc::mbar_wait(tfull, (uint32_t)(piece & 1), p.status)) ok = false;
         ++piece;
         tc::tc_fence_after();
-        const int r = up_rb * tc::BM + (int)rank * tc::kRowsPerCta + quad * 32 + lane;
-        const int col0 = (ph ? dn_col : up_col) * n + cgrp * cols;
+        const int boxes = ph ? dn_boxes : up_boxes;
+        const int row0 = up_rb * tc::BM + (int)rank * tc::kRowsPerCta + quad * 32;
+        const int col0 = (ph ? dn_col : up_col) * n;
         const uint32_t taddr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(cgrp * cols);
+        // The tile goes out as bulk tensor stores (every thread storing its own row took 1.1 to 6.2 us per tile): the
+        // four warps of a row quarter fill boxes of 32 rows x 128 bytes in the activation ring, which is idle between
+        // the last MMA of this piece and the loads of the next, in the 128-byte swizzle of the output's tensor map.
+        uint8_t* stage = sA + quad * boxes * tc::kOutBoxBytes + lane * 128;
         for (int c = 0; c < cols; c += 16) {
           uint32_t acc[16];
           tc::tmem_ld16(taddr + c, acc);
           tc::tmem_ld_wait();
+          const int byte = (cgrp * cols + c) * (ph ? 4 : 2);               // of the tile's row
+          uint8_t* box = stage + (byte >> 7) * tc::kOutBoxBytes;
+          const int chunk = (byte & 127) >> 4;
           if (ph == 0) {
             uint32_t o[8];
 #pragma unroll
             for (int j = 0; j < 16; j += 4) {
-              const float4 b = __ldg(reinterpret_cast<const float4*>(w.b1 + col0 + c + j));
+              const float4 b = __ldg(reinterpret_cast<const float4*>(w.b1 + col0 + cgrp * cols + c + j));
               const __nv_bfloat162 lo = __floats2bfloat162_rn(tc::gelu_fast(__uint_as_float(acc[j]) + b.x), tc::gelu_fast(__uint_as_float(acc[j + 1]) + b.y));
               const __nv_bfloat162 hi = __floats2bfloat162_rn(tc::gelu_fast(__uint_as_float(acc[j + 2]) + b.z), tc::gelu_fast(__uint_as_float(acc[j + 3]) + b.w));
               o[j / 2] = *reinterpret_cast<const uint32_t*>(&lo);
               o[j / 2 + 1] = *reinterpret_cast<const uint32_t*>(&hi);
             }
-            if (r < p.R) {
-              uint4* dst = reinterpret_cast<uint4*>(p.H + (int64_t)r * p.F + col0 + c);
-              dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-              dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
-            }
-          } else if (r < p.R) {
-            uint4* dst = reinterpret_cast<uint4*>(p.part + (int64_t)dn_slice * p.plane + (int64_t)r * d + col0 + c);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) dst[j] = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+            for (int j = 0; j < 2; ++j)
+              *reinterpret_cast<uint4*>(box + (((chunk + j) ^ (lane & 7)) << 4)) = make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              *reinterpret_cast<uint4*>(box + (((chunk + j) ^ (lane & 7)) << 4)) = make_uint4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
           }
         }
         tc::tc_fence_before();
-        if (ph == 0) tc::fence_async_global();
+        tc::fence_async_smem();
         __syncwarp();
         if (lane == 0) tc::mbar_arrive_cluster(tc::mapa(tc::smem_u32(tempty), 0));
-        workers_sync();
-        if (wid == 0)
+        asm volatile("bar.sync %0, 128;" ::"r"(quad + 10) : "memory");      // the four warps of this row quarter
+        if (cgrp < boxes && tc::elect_one()) {
+          const uint8_t* src = sA + (quad * boxes + cgrp) * tc::kOutBoxBytes;
+          if (row0 < p.R) {
+            if (ph) tc::tma_store_2d(&tmP, src, col0 + cgrp * 32, dn_slice * p.rb * tc::BM + row0);
+            else tc::tma_store_2d(&tmHs, src, col0 + cgrp * 64, row0);
+            tc::bulk_commit();
+            tc::bulk_wait_all();
+          }
+          tc::fence_async_global();
           red_release_add(ph ? cnt_dn + dn_rb : cnt_up + up_rb * kMaxKSlices + up_col * n / slice_cols, 1u);
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(ring);
       }
     }
   }

@@ -169,15 +169,17 @@ int make_tmap(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, in
   return SRM_OK;
 }
 
-// The same matrix (bf16) of `layers` layers, `stride` bytes apart, as one three-dimensional descriptor.
-int make_tmap_layers(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int layers, int64_t stride, int box_rows) {
+// A bf16 matrix [rows, cols] as {64, rows, cols / 64} (and, with layers > 0, the same matrix of `layers` layers, `stride`
+// bytes apart, as a fourth dimension): a box holds `kbs` k-blocks of 64 columns one after the other, each box_rows rows of
+// 128 bytes.
+int make_tmap_kblocks(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows, int kbs, int layers = 0, int64_t stride = 0) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (fn == nullptr) { g_last_cuda_error = (int)cudaErrorNotSupported; return SRM_ERR_CUDA; }
-  cuuint64_t gdim[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)layers};
-  cuuint64_t gstride[2] = {(cuuint64_t)cols * 2, layers > 1 ? (cuuint64_t)stride : (cuuint64_t)(cols * rows * 2)};
-  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstride, box, estr,
+  cuuint64_t gdim[4] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64), (cuuint64_t)(layers > 0 ? layers : 1)};
+  cuuint64_t gstride[3] = {(cuuint64_t)cols * 2, 128, layers > 1 ? (cuuint64_t)stride : (cuuint64_t)(cols * rows * 2)};
+  cuuint32_t box[4] = {64, (cuuint32_t)box_rows, (cuuint32_t)kbs, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, layers > 0 ? 4 : 3, const_cast<void*>(base), gdim, gstride, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) { g_last_cuda_error = 10000 + (int)r; return SRM_ERR_CUDA; }

@@ -20,8 +20,8 @@ def _launches(P, f):
 
 
 @pytest.mark.parametrize("B,d,state_dtype,ragged", [(97, 512, "fp32", False), (256, 1024, "fp16", False), (257, 1024, "fp32", True),
-                                                    (512, 1024, "bf16", False), (1024, 1024, "fp32", False), (130, 1536, "fp32", True),
-                                                    (768, 1536, "fp16", False), (1000, 512, "fp32", False)])
+                                                    (512, 1024, "bf16", False), (33, 1024, "fp32", False), (130, 1536, "fp32", True),
+                                                    (256, 1536, "fp16", False), (1, 1536, "fp32", False), (1000, 512, "fp32", False)])
 def test_layers_in_one_kernel_agree_with_the_kernel_per_operation_path(B, d, state_dtype, ragged):
     import paper_2605_08696_b200 as P
     shape = custom_shape(n_layers=3, d_model=d, vocab=2048, n_ctx=24, dtype="bf16", seed=11)
