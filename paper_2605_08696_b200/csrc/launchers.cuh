@@ -743,7 +743,7 @@ int launch_layers_nt(srm_model& m, const MidMaps& t, const mid::Params& p, cudaS
   return launch_layers_t<NT, float>(m, t, p, st);
 }
 
-// All layers for rows [b0, b0 + R) of the state; leaves x and, in w.part, the last down projection's partial products.
+// All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
 // p: from mid_plan.
 int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w, mid::Params& p,
                       cudaStream_t st, const int32_t* ctr, const int32_t* pos) {
@@ -757,6 +757,7 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   p.layer_bytes = layer_stride_bytes(m);
   p.S = static_cast<uint8_t*>(s.layer_ptr(0)) + (size_t)b0 * d * m.state_bytes();
   p.layer_stride = (int64_t)s.B * d * m.state_bytes();
+  p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
   p.x = w.x; p.a = reinterpret_cast<bf16*>(w.a); p.H = reinterpret_cast<bf16*>(w.H);
   p.part = w.part;
   p.plane = (int64_t)p.rb * tc::BM * d;
@@ -791,11 +792,7 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   int k_slices = 1;
   mid::Params mp;
   const bool one_kernel = mid_plan(m, R, w, &mp);
-  if (one_kernel) {
-    if ((rc = launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
-    k_slices = mp.ks;
-    ps = PartialSum{w.part, mp.ks, mp.plane, m.fptr(c.n_layers - 1, SRM_T_B2)};
-  }
+  if (one_kernel && (rc = launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
   // the down projection shares K out between CTA pairs where that is the faster kernel for R rows
   bool split = false;
   if (!one_kernel && w.order != nullptr && F % tc::BK == 0) {
@@ -859,7 +856,7 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
     if (rc) return rc;
   }
   if (ps.part != nullptr) ps.bias = m.fptr(c.n_layers - 1, SRM_T_B2);
-  if ((rc = launch_final_norm(m, w.x, R, 1, 0, w.a, st, nullptr, ps))) return rc;
+  if (!one_kernel && (rc = launch_final_norm(m, w.x, R, 1, 0, w.a, st, nullptr, ps))) return rc;
   SelectOut o = out_all;
   o.last_tok += b0;
   if (o.tok_out) o.tok_out += b0;

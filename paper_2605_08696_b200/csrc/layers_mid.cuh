@@ -56,7 +56,8 @@ struct Params {
   void* S;                       // cache rows of layer 0; layer l at S + l * layer_stride (bytes)
   int64_t layer_stride;
   float* x;                      // [R, d]
-  bf16* a;                       // [R, d]
+  bf16* a;                       // [R, d]: activations of the up projection, at the end of the final norm
+  const float *lnf_g, *lnf_b;
   bf16* H;                       // [R, F]
   float* part;                   // [ks] planes of plane_rows x d
   int64_t plane;                 // elements per plane
@@ -65,11 +66,14 @@ struct Params {
   const int32_t* ctr;            // device-side step counters or nullptr
   const int32_t* pos;            // [R] per-row positions or nullptr
 };
+// Row-phase parameters in shared memory: ln1_g | ln1_b | beta_t | ln2_g | ln2_b | b2 of the previous layer, then this CTA's
+// part of b1 (first touched in the epilogue it came from HBM there: 0.7 us).
+constexpr int kVecs = 6;
 constexpr int kCntWords = kMaxRowBlocks * (2 + kMaxKSlices);
 
 // Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers.
 __host__ __device__ inline size_t smem_bytes(int d, int n, int w_slots, int a_slots) {
-  return 1024 + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + (size_t)sb::kRowParamVecs * d * 4 + kGroups * 32 + kBarrierBytes;
+  return 1024 + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + ((size_t)kVecs * d + n) * 4 + kGroups * 32 + kBarrierBytes;
 }
 
 // Tile widths and ranges of K for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit. (256-wide
@@ -138,7 +142,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   uint8_t* sW = smem;
   uint8_t* sA = sW + p.w_slots * w_bytes;
   float* prm = reinterpret_cast<float*>(sA + p.a_slots * kABytes);
-  float* red = prm + sb::kRowParamVecs * d;
+  float* b1_s = prm + kVecs * d;
+  float* red = b1_s + n;
   uint64_t* fullW = reinterpret_cast<uint64_t*>(red + kGroups * 8);      // used in the leader CTA
   uint64_t* emptyW = fullW + kMaxWSlots;
   uint64_t* fullA = emptyW + kMaxWSlots;                                 // used in the leader CTA
@@ -290,13 +295,15 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     float* slot = red + group * 8;
     int piece = 0;
     bool ok = true;
-    for (int l = 0; l < p.L; ++l) {
-      const sb::LayerW w = sb::layer_w(p, l);
+    for (int l = 0;; ++l) {
+      const bool last = l == p.L;         // after the last layer: the final norm
+      const sb::LayerW w = sb::layer_w(p, last ? 0 : l);
       // ---- rows: row blockIdx.x + grid * group. Parameters first (constant data), then the wait ----
       workers_sync();                     // the previous layer's parameters have been read
-      for (int i = wid; i < sb::kRowParamVecs * d / 4; i += kWorkers) {
+      for (int i = wid; i < (kVecs * d + n) / 4; i += kWorkers) {
         const int k = i / (d / 4), c = i % (d / 4) * 4;
-        const float* q = k == 0 ? w.ln1_g : k == 1 ? w.ln1_b : k == 2 ? w.beta + (int64_t)t_all * d : k == 3 ? w.ln2_g : w.ln2_b;
+        const float* q = k == 0 ? w.ln1_g : k == 1 ? w.ln1_b : k == 2 ? w.beta + (int64_t)t_all * d : k == 3 ? (last ? p.lnf_g : w.ln2_g)
+                         : k == 4 ? (last ? p.lnf_b : w.ln2_b) : k == 5 ? sb::layer_w(p, l > 0 ? l - 1 : 0).b2 : w.b1 + (up_on ? up_col : 0) * n;
         sb::cp_async16(prm + i * 4, q + c);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -307,9 +314,11 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       float4 s[NT], v[NT];
       ST* Sr = reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + (int64_t)row * d + c0;
       if (mine) {
-        sb::head_scalars<d, NT>(p, w, t, wid & 63, a1, a2, lm);
+        if (!last) {
+          sb::head_scalars<d, NT>(p, w, t, wid & 63, a1, a2, lm);
 #pragma unroll
-        for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + 256 * i);
+          for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + 256 * i);
+        }
         if (l > 0 && (wid & 63) == 0 && ok)       // the down tiles of the row's block
           ok = count_wait(cnt_dn + row / tc::BM, (uint32_t)l * (uint32_t)(p.cd * p.ks * dn_boxes) * 8u, p.status);
       }
@@ -325,11 +334,10 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 #pragma unroll
           for (int i = 0; i < NT; ++i) v[i] = ldg4(p.E + (int64_t)tk * d + c0 + 256 * i);
         } else {                          // x + b2 + plane 0 + plane 1 + ... (other CTAs wrote the planes: not through L1)
-          const float* b2 = sb::layer_w(p, l - 1).b2 + c0;
 #pragma unroll
           for (int i = 0; i < NT; ++i) {
             v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c0 + 256 * i));
-            const float4 bb = ldg4(b2 + 256 * i);
+            const float4 bb = ld4(prm + 5 * d + c0 + 256 * i);
             v[i] = make_float4(v[i].x + bb.x, v[i].y + bb.y, v[i].z + bb.z, v[i].w + bb.w);
           }
 #pragma unroll 2
@@ -342,21 +350,23 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             }
           }
         }
-        const float* bt_p = p.pos != nullptr ? w.beta + (int64_t)t * d + c0 : prm + 2 * d + c0;
         float mean, rstd;
-        sb::group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
-        const float nmr = -mean * rstd;
+        if (!last) {
+          const float* bt_p = p.pos != nullptr ? w.beta + (int64_t)t * d + c0 : prm + 2 * d + c0;
+          sb::group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
+          const float nmr = -mean * rstd;
 #pragma unroll
-        for (int i = 0; i < NT; ++i) {
-          const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i), bt = ld4(bt_p + 256 * i);
-          const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
-                                       fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
-          // row-repeat head, Eq. 2: y = (a z + S) + b ; S' = l (S + a z).  column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
-          const float4 u = make_float4(fmaf(a1[i], z.x, s[i].x), fmaf(a1[i], z.y, s[i].y), fmaf(a1[i], z.z, s[i].z), fmaf(a1[i], z.w, s[i].w));
-          st4(Sr + 256 * i, make_float4(lm[i] * u.x, lm[i] * u.y, lm[i] * u.z, lm[i] * u.w));
-          v[i] = make_float4(v[i].x + fmaf(a2[i], u.x, bt.x), v[i].y + fmaf(a2[i], u.y, bt.y), v[i].z + fmaf(a2[i], u.z, bt.z),
-                             v[i].w + fmaf(a2[i], u.w, bt.w));
-          st4(p.x + (int64_t)row * d + c0 + 256 * i, v[i]);
+          for (int i = 0; i < NT; ++i) {
+            const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i), bt = ld4(bt_p + 256 * i);
+            const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
+                                         fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
+            // row-repeat head, Eq. 2: y = (a z + S) + b ; S' = l (S + a z).  column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
+            const float4 u = make_float4(fmaf(a1[i], z.x, s[i].x), fmaf(a1[i], z.y, s[i].y), fmaf(a1[i], z.z, s[i].z), fmaf(a1[i], z.w, s[i].w));
+            st4(Sr + 256 * i, make_float4(lm[i] * u.x, lm[i] * u.y, lm[i] * u.z, lm[i] * u.w));
+            v[i] = make_float4(v[i].x + fmaf(a2[i], u.x, bt.x), v[i].y + fmaf(a2[i], u.y, bt.y), v[i].z + fmaf(a2[i], u.z, bt.z),
+                               v[i].w + fmaf(a2[i], u.w, bt.w));
+            st4(p.x + (int64_t)row * d + c0 + 256 * i, v[i]);
+          }
         }
         sb::group_stats<d, NT>(v, p.eps, slot + 4, group, mean, rstd);
         const float nmr2 = -mean * rstd;
@@ -371,6 +381,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
         if ((wid & 63) == 0) red_release_add(cnt_rows + row / tc::BM, 1u);
       }
+      if (last) break;
 
       // ---- epilogues ----
       for (int ph = 0; ph < 2; ++ph) {
@@ -397,7 +408,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             uint32_t o[8];
 #pragma unroll
             for (int j = 0; j < 16; j += 4) {
-              const float4 b = __ldg(reinterpret_cast<const float4*>(w.b1 + col0 + cgrp * cols + c + j));
+              const float4 b = ld4(b1_s + cgrp * cols + c + j);
               const __nv_bfloat162 lo = __floats2bfloat162_rn(tc::gelu_fast(__uint_as_float(acc[j]) + b.x), tc::gelu_fast(__uint_as_float(acc[j + 1]) + b.y));
               const __nv_bfloat162 hi = __floats2bfloat162_rn(tc::gelu_fast(__uint_as_float(acc[j + 2]) + b.z), tc::gelu_fast(__uint_as_float(acc[j + 3]) + b.w));
               o[j / 2] = *reinterpret_cast<const uint32_t*>(&lo);

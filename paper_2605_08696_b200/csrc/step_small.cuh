@@ -1,4 +1,5 @@
-// One decode step of a SMALL batch (at most 64 samples) as a single persistent kernel.
+// One decode step of a SMALL batch (at most 64 samples, at d = 1024 at most 32: as many as leave room for the weights of a
+// layer beside their activations in shared memory) as a single persistent kernel.
 //
 // With a handful of rows the step is bound by reading the weights once (the mid model: 334 MB, 50 us at HBM speed)
 // and by the latency of its dependent phases, not by arithmetic. The whole step -- embedding, L x (token-mixer cache
@@ -14,7 +15,7 @@
 //   - down projection: cluster c computes d / 32 columns of x, rank r over the r-th quarter of K; the four partial
 //     products meet in shared memory (each rank receives those of its quarter of the cluster's columns) and are added
 //     in rank order, so x is written once, complete.
-// W1 and W2 slabs have a region of shared memory each (up to 32 rows), refilled for the next layer by bulk copies as
+// W1 and W2 slabs have a region of shared memory each, refilled for the next layer by bulk copies as
 // soon as they have been used: the weight stream runs a whole layer ahead of the barriers. The small parameter
 // vectors and cache rows of the next layer are prefetched into L2 meanwhile. The contractions run on mma.sync (m16n8k16, bf16 in, fp32 accumulate): the kernel is bound by
 // latency and HBM, and a tcgen05 tile would be mostly padding. K of a tile is cut into up to eight ranges that
@@ -93,24 +94,21 @@ inline bool smem_plan(int B, int d, int F, int state_elem, Params* p, size_t* by
   const int part = kWarps * 1024, xo = mp * (dn_cols(d) / kCluster) * 4;
   const int srow = d * state_elem;
   if (part + recv < kRowParamVecs * d * 4) recv = kRowParamVecs * d * 4 - part;      // the row phase's parameters lie there
-  for (int two = 1; two >= 0; --two) {                   // a region each for W1 and W2, or one for both
-    int w = two ? w1 + w2 : (w1 > w2 ? w1 : w2);
-    if (w < 2 * stage) w = 2 * stage;
-    const int fixed = kHeadBytes + act + part + recv + (xo + 15) / 16 * 16 + srow;
-    if (fixed + w > kSmemBytes) continue;
-    while (w + stage <= kLmMaxStages * stage && fixed + w + stage <= kSmemBytes) w += stage;     // a deeper LM-head ring
-    p->off_w1 = kHeadBytes + act;
-    p->off_w2 = two ? p->off_w1 + w1 : p->off_w1;
-    p->lm_stages = w / stage < kLmMaxStages ? w / stage : kLmMaxStages;
-    p->lm_stages_w1 = two ? w1 / stage : 0;
-    p->off_part = p->off_w1 + w;
-    p->off_recv = p->off_part + part;
-    p->off_xo = p->off_recv + recv;
-    p->off_s = p->off_xo + (xo + 15) / 16 * 16;
-    *bytes = (size_t)(fixed + w);
-    return true;
-  }
-  return false;
+  int w = w1 + w2;
+  if (w < 2 * stage) w = 2 * stage;
+  const int fixed = kHeadBytes + act + part + recv + (xo + 15) / 16 * 16 + srow;
+  if (fixed + w > kSmemBytes) return false;
+  while (w + stage <= kLmMaxStages * stage && fixed + w + stage <= kSmemBytes) w += stage;       // a deeper LM-head ring
+  p->off_w1 = kHeadBytes + act;
+  p->off_w2 = p->off_w1 + w1;
+  p->lm_stages = w / stage < kLmMaxStages ? w / stage : kLmMaxStages;
+  p->lm_stages_w1 = w1 / stage;
+  p->off_part = p->off_w1 + w;
+  p->off_recv = p->off_part + part;
+  p->off_xo = p->off_recv + recv;
+  p->off_s = p->off_xo + (xo + 15) / 16 * 16;
+  *bytes = (size_t)(fixed + w);
+  return true;
 }
 
 template <typename P>
@@ -377,7 +375,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
   const int chunks_all = (p.V + kLmChunkCols - 1) / kLmChunkCols;
   const int lm_c0 = (int)((int64_t)cta * chunks_all / kGrid), lm_chunks = (int)((int64_t)(cta + 1) * chunks_all / kGrid) - lm_c0;
   constexpr int lm_stage = kLmChunkCols * ld_d;
-  const bool alone = B <= kAloneRows, one_region = p.off_w1 == p.off_w2;
+  const bool alone = B <= kAloneRows;
 
   if (tid == 0) {
     for (int i = 0; i < 5 + kLmMaxStages; ++i) tc::mbar_init(bar1 + i, 1);
@@ -442,7 +440,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
     tc::mbar_expect_tx(barP, part_bytes);
   }
   stage_up(0);
-  if (!one_region) stage_dn(0);
+  stage_dn(0);
   prefetch_layer(0);
   if (p.L > 1) prefetch_layer(1);
   const Share up = share_of(m_tiles * ((ucols + 15) / 16), d), dn = share_of(m_tiles * ((ncols + 15) / 16), klen);
@@ -533,7 +531,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
     // ---- up projection: H[:, slab] = gelu(a W1[slab]^T + b1) ----
     if (!wait_stage(bar1, par1, p.status, gb.dead)) gb.dead = true;
     par1 ^= 1u;
-    if (!one_region && l > 0) stage_dn(l); // (W2's place is free since the previous layer; issued while a barrier is waited
+    if (l > 0) stage_dn(l);                // (W2's place is free since the previous layer; issued while a barrier is waited
                                            //  for, the weight stream made the barrier itself slower, 1.3 -> 2.6 us)
     if (warp < up.tiles * up.groups) {
       const int tile = warp % up.tiles, g = warp / up.tiles;
@@ -550,7 +548,7 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
             __floats2bfloat162_rn(tc::gelu_fast(q.a + bb.x), tc::gelu_fast(q.b + bb.y));
       }
     }
-    gb.sync([&] { if (one_region) stage_dn(l); });
+    gb.sync([] {});
 
     // ---- down projection: this rank's part of K for the cluster's columns ----
     asm volatile("fence.proxy.async.global;" ::: "memory");     // H was written through the generic proxy
@@ -563,10 +561,9 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
     if (!wait_stage(bar2, par2, p.status, gb.dead)) gb.dead = true;
     if (!wait_stage(barA, par2, p.status, gb.dead)) gb.dead = true;
     par2 ^= 1u;
-    if (!one_region) {                     // the next weights for W1's place (used up): while this phase asks for nothing else
-      if (l + 1 < p.L) stage_up(l + 1);
-      else for (int ch = 0; ch < p.lm_stages_w1; ++ch) stage_lm(ch);
-    }
+    // the next weights for W1's place (used up): while this phase asks for nothing else
+    if (l + 1 < p.L) stage_up(l + 1);
+    else for (int ch = 0; ch < p.lm_stages_w1; ++ch) stage_lm(ch);
     if (l + 2 < p.L) prefetch_layer(l + 2);
     auto send = [&](int row, int col, float a, float b) {      // to the rank that owns these columns (gw is even)
       if (row < B && col < ncols)
@@ -598,16 +595,12 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads, 1) 
         if (!alone) tc::mbar_expect_tx(barR, peer_bytes);
         if (l + 1 < p.L) tc::mbar_expect_tx(barP, part_bytes);
       }
-      if (one_region) {
-        if (l + 1 < p.L) stage_up(l + 1);
-        else for (int ch = 0; ch < p.lm_stages; ++ch) stage_lm(ch);
-      }
       const int t = p.pos != nullptr ? 0 : t_all;
       fetch_row_params<d>(p, l + 1, t, prm);
       if (l + 1 < p.L) head_scalars<d, NT>(p, layer_w(p, l + 1), t, tid & 63, a1, a2, lm);
     });
   }
-  if (!one_region) for (int ch = p.lm_stages_w1; ch < p.lm_stages; ++ch) stage_lm(ch);
+  for (int ch = p.lm_stages_w1; ch < p.lm_stages; ++ch) stage_lm(ch);
 
   // ---- LM head over this CTA's vocabulary slab through the ring, two chunks at a time where it is deep enough ----
   const int cpi = p.lm_stages >= 4 && m_tiles <= 2 ? 2 : 1;      // (every thread takes one pair of columns)

@@ -44,7 +44,7 @@ def test_layers_in_one_kernel_agree_with_the_kernel_per_operation_path(B, d, sta
             tok, lg = res[0]
             lgs.append(lg.cpu().numpy())
             toks.append(tok.clone())
-        assert (launches <= 4) == (flags == 0)                 # layers, norm, LM head, selection
+        assert (launches <= 3) == (flags == 0)                 # layers and norm, LM head, selection
         assert st.status() == 0
         fed = fed if fed is not None else toks
         outs.append((np.stack(lgs), torch.stack(toks).cpu().numpy(), st.cache().cpu().numpy()))
