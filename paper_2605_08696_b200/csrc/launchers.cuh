@@ -523,31 +523,29 @@ int launch_lm_head_topk(srm_model& m, int64_t R, const void* a, void* lists, voi
   return SRM_OK;
 }
 
-// From this many prompts per pass the scan kernel (one warp per prompt) is the prefill mixer; below it the chunk kernel
-// (a CTA per 16 positions of a prompt), or, for shapes neither is built for, the tile kernel (a CTA per prompt). us per
-// launch, tile / chunk / scan kernel: mid, 1 prompt of 777 positions 2061 / 23.6 / -, 45 ragged prompts of up to 301
-// 717 / 48 / -, 2048 prompts of 256 - / 1844 / 1834; rl, 16 prompts of 200: 760 / 26 / -.
-constexpr int64_t kPrefillScanMinSamples = 384;
+// From this many prompts per pass a CTA walks a prompt (prefill_walk.cuh); below it a CTA takes 16 positions of one (the
+// chunk kernel), or, for shapes neither is built for, the tile kernel (a CTA per prompt). us per launch, tile / chunk /
+// walk: mid, 1 prompt of 777 positions 2061 / 23.6 / -, 45 ragged prompts of up to 301 717 / 48 / -, 2048 prompts of 256
+// - / 1844 / 1432; rl, 16 prompts of 200: 760 / 26 / -.
+constexpr int64_t kPrefillWalkMinPrompts = 384;
 
 template <int NV, typename WT, typename ST>
-int launch_prefill_scan(const PrefillParams& p, int num_sms, cudaStream_t st) {
-  const int warps = prefill_scan_warps(p.d, p.Bp, num_sms);
-  const size_t smem = prefill_scan_smem(p.d, warps);
-  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_scan_kernel<NV, WT, ST>), kScanSmemBudget);
+int launch_prefill_walk(const PrefillParams& p, cudaStream_t st) {
+  const size_t smem = prefill_walk_smem(NV * 128);
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(prefill_walk_kernel<NV, WT, ST>), (int)smem);
   if (rc != SRM_OK) return rc;
-  const unsigned grid = (unsigned)(p.Bp < num_sms ? p.Bp : num_sms);
-  SRM_CUDA(launch_kernel(prefill_scan_kernel<NV, WT, ST>, dim3(grid), dim3(warps * 32), smem, st, p));
+  SRM_CUDA(launch_kernel(prefill_walk_kernel<NV, WT, ST>, dim3((unsigned)p.Bp), dim3(NV * 32), smem, st, p));
   SRM_CUDA(cudaGetLastError());
   return SRM_OK;
 }
 
 template <typename WT, typename ST>
-int launch_prefill_scan_nv(const PrefillParams& p, int num_sms, cudaStream_t st) {
+int launch_prefill_walk_nv(const PrefillParams& p, cudaStream_t st) {
   switch (p.d / 128) {
-    case 4: return launch_prefill_scan<4, WT, ST>(p, num_sms, st);
-    case 8: return launch_prefill_scan<8, WT, ST>(p, num_sms, st);
-    case 12: return launch_prefill_scan<12, WT, ST>(p, num_sms, st);
-    default: return launch_prefill_scan<16, WT, ST>(p, num_sms, st);
+    case 4: return launch_prefill_walk<4, WT, ST>(p, st);
+    case 8: return launch_prefill_walk<8, WT, ST>(p, st);
+    case 12: return launch_prefill_walk<12, WT, ST>(p, st);
+    default: return launch_prefill_walk<16, WT, ST>(p, st);
   }
 }
 
@@ -558,7 +556,7 @@ bool prefill_chunk_ok(const srm_model& m, int64_t np, int n) {
   const srm_config& c = m.cfg;
   if (m.head_proj()) return false;
   if (c.mixer == SRM_MIXER_MIXED) {
-    if (np >= kPrefillScanMinSamples) return false;
+    if (np >= kPrefillWalkMinPrompts) return false;
     if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536 && c.d_model != 2048) return false;
   } else if (c.dtype != SRM_DTYPE_BF16 || (c.d_model != 512 && c.d_model != 1024)) {
     return false;
@@ -607,10 +605,8 @@ int launch_prefill_mixer(const srm_model& m, int layer, int64_t Bp, int n, const
       }
     });
   }
-  const bool scan_shape = p.d % 128 == 0 && (p.d / p.h) % 128 == 0 && p.h <= 8 && (nv == 4 || nv == 8 || nv == 12 || nv == 16);
-  if (scan_shape && Bp >= kPrefillScanMinSamples) {        // many prompts: one warp walks each prompt's positions
-    return dispatch_types(m.cfg, [&](auto w, auto c) { return launch_prefill_scan_nv<decltype(w), decltype(c)>(p, m.num_sms, st); });
-  }
+  if ((p.d == 512 || p.d == 1024 || p.d == 1536 || p.d == 2048) && Bp >= kPrefillWalkMinPrompts)      // many prompts
+    return dispatch_types(m.cfg, [&](auto w, auto c) { return launch_prefill_walk_nv<decltype(w), decltype(c)>(p, st); });
   auto go = [&](auto kernel) -> int {
     SRM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));   // smem depends on d: set per launch
     SRM_CUDA(launch_kernel(kernel, dim3((unsigned)Bp), dim3(kPrefillThreads), smem, st, p));

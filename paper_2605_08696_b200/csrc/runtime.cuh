@@ -27,7 +27,7 @@
 #include "mixer_variants.cuh"
 #include "mixer_model_variants.cuh"
 #include "prefill.cuh"
-#include "prefill_scan.cuh"
+#include "prefill_walk.cuh"
 #include "prefill_chunk.cuh"
 #include "prefill_chunk_variants.cuh"
 #include "select.cuh"
