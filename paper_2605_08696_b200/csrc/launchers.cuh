@@ -392,21 +392,26 @@ int launch_select(const srm_model& m, int64_t R, const float* logits, const srm_
     SRM_CUDA(launch_kernel(select_greedy_kernel, dim3((unsigned)(R / out.row_div)), dim3(kSelThreads), 0, st, logits, R, V, out, status));
   } else if (s.mode == SRM_SELECT_TOPP) {
     const float inv_t = 1.0f / s.temperature;
-    const size_t scratch = ((sizeof(ToppScratch) + 15) & ~size_t(15)) + sizeof(ToppHist);
-    if (V <= kToppSmemFloats) {
-      const size_t smem = scratch + (size_t)V * 4;
-      int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(select_topp_kernel<true>),
-                                   (int)(scratch + (size_t)kToppSmemFloats * 4));
-      if (rc != SRM_OK) return rc;
-      SRM_CUDA(launch_kernel(select_topp_kernel<true>, dim3((unsigned)R), dim3(kToppThreads), smem, st, logits, R, V,
-                             s.top_p, inv_t, s.seed, sample_base, step, out, status));
-    } else {
-      // the scratch alone exceeds the default dynamic shared-memory limit
-      int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(select_topp_kernel<false>), (int)scratch);
-      if (rc != SRM_OK) return rc;
-      SRM_CUDA(launch_kernel(select_topp_kernel<false>, dim3((unsigned)R), dim3(kToppThreads), scratch, st, logits, R, V,
-                             s.top_p, inv_t, s.seed, sample_base, step, out, status));
+    const int few = topp_few_ok(V) ? 1 : 0;
+    if (few) {
+      SRM_CUDA(launch_kernel(select_topp_few_kernel, dim3((unsigned)R), dim3(kToppThreads), 0, st, logits, R, V, s.top_p, inv_t, s.seed,
+                             sample_base, step, out));
+      ++g_kernel_launches;
     }
+    // (the marked rows, or all: one block per SM walks them, its shared memory leaves no room for more)
+    const unsigned grid = (unsigned)(R < m.num_sms ? R : m.num_sms);
+    const size_t scratch = ((sizeof(ToppScratch) + 15) & ~size_t(15)) + sizeof(ToppHist);
+    const bool staged = V <= kToppSmemFloats;
+    const size_t smem = scratch + (staged ? (size_t)V * 4 : 0);
+    auto go = [&](auto kernel, size_t most) -> int {
+      int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)most);
+      if (rc != SRM_OK) return rc;
+      SRM_CUDA(launch_kernel(kernel, dim3(grid), dim3(kToppThreads), smem, st, logits, R, V, s.top_p, inv_t, s.seed, sample_base, step, out,
+                             status, few));
+      return SRM_OK;
+    };
+    const int rc = staged ? go(select_topp_kernel<true>, scratch + (size_t)kToppSmemFloats * 4) : go(select_topp_kernel<false>, scratch);
+    if (rc != SRM_OK) return rc;
   } else {
     const float inv_t = 1.0f / s.temperature;
     const float z0 = topk_z0(s.top_k, V);
