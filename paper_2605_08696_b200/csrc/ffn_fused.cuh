@@ -38,6 +38,8 @@ struct FfnArgs {
   uint32_t* status;
   int32_t* ready;        // [ceil(M / 256)][F / 256] counters, zero on entry
   int w_static;          // W1, W2 are constant data: the first tiles may be fetched ahead of the dependency wait
+  const uint32_t* m_limit = nullptr;     // a device word: only *m_limit - m_off rows exist, the items of later row blocks are
+  int64_t m_off = 0;                     // skipped (nothing is fetched ahead of the dependency wait then)
 };
 
 __device__ __forceinline__ void red_release_add(int32_t* p, int32_t v) {
@@ -100,7 +102,12 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (warp != 0) pdl_wait();
+  if (warp != 0 || g.m_limit != nullptr) pdl_wait();
+  int rbs = (int)((g.M + BM - 1) / BM);  // row blocks with rows
+  if (g.m_limit != nullptr) {
+    const int64_t lim = (int64_t)*reinterpret_cast<const volatile uint32_t*>(g.m_limit) - g.m_off;
+    rbs = lim <= 0 ? 0 : min(rbs, (int)((lim + BM - 1) / BM));
+  }
 
   const int i0 = cluster_id < plan.n_pairs ? plan.off[cluster_id] : 0;
   const int i1 = cluster_id < plan.n_pairs ? plan.off[cluster_id + 1] : 0;
@@ -119,7 +126,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
       bool ok = true;
       // While the predecessor kernel drains: the weight halves of the first stages of the first item.
       int pre = 0;
-      if (i0 < i1 && g.w_static) {
+      if (i0 < i1 && g.w_static && g.m_limit == nullptr) {
         const uint16_t it = plan.item[i0];
         const bool down = ffn_item_down(it), half = ffn_item_half(it);
         const int kbs = down ? kb_dn : kb_up;
@@ -137,6 +144,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
         const uint16_t it = plan.item[i];
         const bool down = ffn_item_down(it), half = ffn_item_half(it);
         const int rb = ffn_item_rb(it);
+        if (rb >= rbs) continue;
         const int kbs = down ? kb_dn : kb_up;
         const int w_rows = half ? kHalfN / 2 : kRowsPerCta;
         const uint32_t stage_bytes = kAStageBytes + (uint32_t)w_rows * BK * 2;
@@ -175,6 +183,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
       for (int i = i0; ok && i < i1; ++i) {
+        if (ffn_item_rb(plan.item[i]) >= rbs) continue;
         const int kbs = ffn_item_down(plan.item[i]) ? kb_dn : kb_up;
         const uint32_t idesc = ffn_item_half(plan.item[i]) ? instr_desc(kHalfN) : kInstrDesc;
         if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, g.status)) { ok = false; break; }
@@ -210,6 +219,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
       const uint16_t it = plan.item[i];
       const bool down = ffn_item_down(it);
       const int rb = ffn_item_rb(it), cb = ffn_item_cb(it);
+      if (rb >= rbs) continue;
       if (!mbar_wait(&tfull[acc], acc_phase, g.status)) break;
       tc_fence_after();
       const int row0 = rb * BM + (int)rank * kRowsPerCta + quad * 32;

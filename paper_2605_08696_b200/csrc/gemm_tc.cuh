@@ -279,7 +279,16 @@ struct GemmArgs {
   // order. No half-width pieces then.
   int k_slices;
   int64_t plane_rows;
+  int64_t m_off;       // with m_limit: the rows of this launch begin at row m_off of what *m_limit counts
+  int dev_tail;        // with m_limit: the tail rule (tail_tiles_of) is applied on the device, to the rows there are
 };
+
+// How many of the last tiles of a launch run as two half-width pieces: the r tiles of a last, partly filled round when
+// their 2 r halves still fit in one round (they then end after three quarters of a tile's time with nearly every pair busy).
+__host__ __device__ inline int tail_tiles_of(int64_t tiles, int64_t pairs) {
+  const int64_t r = tiles % pairs;
+  return (r > 0 && 2 * r <= pairs) ? (int)r : 0;
+}
 
 // Piece q of a launch: the tile it belongs to, its first column inside the tile and its width.
 struct Piece { int64_t tile; int noff, nw; };
@@ -523,14 +532,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (warp != 0 || g.m_limit != nullptr) pdl_wait();
   int64_t M_rows = g.M;
   if (g.m_limit != nullptr) {              // a row count left on the device by an earlier kernel
-    const int64_t lim = (int64_t)*reinterpret_cast<const volatile uint32_t*>(g.m_limit);
+    int64_t lim = (int64_t)*reinterpret_cast<const volatile uint32_t*>(g.m_limit) - g.m_off;
+    lim = lim < 0 ? 0 : lim;
     M_rows = lim < M_rows ? lim : M_rows;
   }
 
   const int64_t m_tiles = (M_rows + BM - 1) / BM, n_tiles = (g.N + BN - 1) / BN;
   const int64_t tiles = m_tiles * n_tiles;
   const int ks = (EPI == kEpiPlain && g.k_slices > 1 && g.m_limit == nullptr) ? g.k_slices : 1;   // ranges of K per tile
-  const int tail = (g.m_limit != nullptr || ks > 1) ? 0 : g.tail_tiles;
+  const int tail = ks > 1 ? 0 : g.m_limit != nullptr ? (g.dev_tail ? tail_tiles_of(tiles, n_clusters) : 0) : g.tail_tiles;
   const int64_t pieces = (tiles + tail) * ks;          // a tail tile counts as two pieces
   const int k_all = static_cast<int>(g.K / BK);
   const int k_blocks = (k_all + ks - 1) / ks;          // k-blocks per piece (the last range of a tile may be shorter)

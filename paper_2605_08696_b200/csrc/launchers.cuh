@@ -137,18 +137,19 @@ int launch_mixer_variant(const srm_model& m, int layer, int t, int64_t R, const 
 
 template <typename WT>
 int launch_norm_t(const float* x, int64_t R, int64_t stride, int64_t offset, const float* g, const float* b, float eps,
-                  int d, void* out, cudaStream_t st, const int32_t* row_len = nullptr, const PartialSum& ps = PartialSum()) {
+                  int d, void* out, cudaStream_t st, const int32_t* row_len = nullptr, const PartialSum& ps = PartialSum(),
+                  const int32_t* row_start = nullptr) {
   const int nv = (d + 127) / 128;
   const unsigned grid = (unsigned)((R + kMixerWarps - 1) / kMixerWarps);
   const dim3 blk(kMixerWarps * 32);
   WT* o = reinterpret_cast<WT*>(out);
-  if (nv <= 1) SRM_CUDA(launch_kernel(norm_rows_kernel<1, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps));
-  else if (nv <= 2) SRM_CUDA(launch_kernel(norm_rows_kernel<2, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps));
-  else if (nv <= 4) SRM_CUDA(launch_kernel(norm_rows_kernel<4, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps));
-  else if (nv <= 6) SRM_CUDA(launch_kernel(norm_rows_kernel<6, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps));
-  else if (nv <= 8) SRM_CUDA(launch_kernel(norm_rows_kernel<8, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps));
-  else if (nv <= 12) SRM_CUDA(launch_kernel(norm_rows_kernel<12, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps));
-  else SRM_CUDA(launch_kernel(norm_rows_kernel<16, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps));
+  if (nv <= 1) SRM_CUDA(launch_kernel(norm_rows_kernel<1, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps, row_start));
+  else if (nv <= 2) SRM_CUDA(launch_kernel(norm_rows_kernel<2, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps, row_start));
+  else if (nv <= 4) SRM_CUDA(launch_kernel(norm_rows_kernel<4, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps, row_start));
+  else if (nv <= 6) SRM_CUDA(launch_kernel(norm_rows_kernel<6, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps, row_start));
+  else if (nv <= 8) SRM_CUDA(launch_kernel(norm_rows_kernel<8, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps, row_start));
+  else if (nv <= 12) SRM_CUDA(launch_kernel(norm_rows_kernel<12, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps, row_start));
+  else SRM_CUDA(launch_kernel(norm_rows_kernel<16, WT>, dim3(grid), dim3(blk), 0, st, x, R, stride, offset, g, b, eps, d, o, row_len, ps, row_start));
   SRM_CUDA(cudaGetLastError());
   return SRM_OK;
 }
@@ -163,13 +164,14 @@ int launch_norm(const srm_model& m, const float* x, int64_t R, int64_t stride, i
 }
 
 int launch_final_norm(const srm_model& m, const float* x, int64_t R, int64_t stride, int64_t offset, void* out,
-                      cudaStream_t st, const int32_t* row_len = nullptr, const PartialSum& ps = PartialSum()) {
+                      cudaStream_t st, const int32_t* row_len = nullptr, const PartialSum& ps = PartialSum(),
+                      const int32_t* row_start = nullptr) {
   if (R <= 0) return SRM_OK;
   LaunchScope scope(m, SRM_KERNEL_NORM, st);
   const float* g = m.fptr(-1, SRM_T_LNF_G);
   const float* b = m.fptr(-1, SRM_T_LNF_B);
-  if (m.cfg.dtype == SRM_DTYPE_BF16) return launch_norm_t<bf16>(x, R, stride, offset, g, b, m.cfg.ln_eps, m.cfg.d_model, out, st, row_len, ps);
-  return launch_norm_t<float>(x, R, stride, offset, g, b, m.cfg.ln_eps, m.cfg.d_model, out, st, row_len, ps);
+  if (m.cfg.dtype == SRM_DTYPE_BF16) return launch_norm_t<bf16>(x, R, stride, offset, g, b, m.cfg.ln_eps, m.cfg.d_model, out, st, row_len, ps, row_start);
+  return launch_norm_t<float>(x, R, stride, offset, g, b, m.cfg.ln_eps, m.cfg.d_model, out, st, row_len, ps, row_start);
 }
 
 template <typename T>
@@ -211,19 +213,17 @@ int ensure_tc_ready(srm_model& m) {
   return SRM_OK;
 }
 
-// How many of the last tiles of a launch run as two half-width pieces (gemm_tc.cuh): the r tiles of a last, partly
-// filled round when their 2 r halves still fit in one round (they then end after three quarters of a tile's time
-// with nearly every pair busy); none with SRM_FLAG_NO_TAIL_SPLIT.
+// tail_tiles_of (gemm_tc.cuh), or none with SRM_FLAG_NO_TAIL_SPLIT.
 int gemm_tail_tiles(const srm_model& m, int64_t tiles) {
   if (m.cfg.flags & SRM_FLAG_NO_TAIL_SPLIT) return 0;
-  const int64_t r = tiles % m.tc_clusters;
-  return (r > 0 && 2 * r <= m.tc_clusters) ? (int)r : 0;
+  return tc::tail_tiles_of(tiles, m.tc_clusters);
 }
 
 // k_slices > 1 (epilogue kEpiPlain only; K / 64 a multiple of k_slices): out is k_slices planes of plane_rows x N
 // partial products (GemmArgs::k_slices).
 int launch_gemm_tc(srm_model& m, int epi, int64_t M, int64_t N, int64_t K, const void* A, const void* W,
-                   const float* bias, void* out, uint32_t* status, cudaStream_t st, int k_slices = 1, int64_t plane_rows = 0) {
+                   const float* bias, void* out, uint32_t* status, cudaStream_t st, int k_slices = 1, int64_t plane_rows = 0,
+                   const uint32_t* m_limit = nullptr, int64_t m_off = 0) {
   int rc = ensure_tc_ready(m);
   if (rc != SRM_OK) return rc;
   CUtensorMap ta, tb, td, tb64;
@@ -240,7 +240,13 @@ int launch_gemm_tc(srm_model& m, int epi, int64_t M, int64_t N, int64_t K, const
   g.tail_tiles = tail;
   g.k_slices = k_slices > 1 ? k_slices : 1;
   g.plane_rows = plane_rows;
-  const int64_t pieces = (tiles + tail) * g.k_slices;
+  int64_t pieces = (tiles + tail) * g.k_slices;
+  if (m_limit != nullptr) {                // fewer rows than M, known on the device only
+    g.m_limit = m_limit;
+    g.m_off = m_off;
+    g.dev_tail = (m.cfg.flags & SRM_FLAG_NO_TAIL_SPLIT) ? 0 : 1;
+    pieces = m.tc_clusters;
+  }
   const unsigned grid = 2u * (unsigned)(pieces < m.tc_clusters ? pieces : m.tc_clusters);
   if (epi == kEpiBiasGelu) SRM_CUDA(launch_kernel(tc::gemm_tc_kernel<kEpiBiasGelu>, dim3(grid), dim3(tc::kThreads), tc::kSmemBytes, st, ta, tb, td, tb64, g));
   else if (epi == kEpiBiasResidual) SRM_CUDA(launch_kernel(tc::gemm_tc_kernel<kEpiBiasResidual>, dim3(grid), dim3(tc::kThreads), tc::kSmemBytes, st, ta, tb, td, tb64, g));
@@ -251,14 +257,15 @@ int launch_gemm_tc(srm_model& m, int epi, int64_t M, int64_t N, int64_t K, const
 }
 
 int launch_gemm(srm_model& m, int epi, int64_t M, int64_t N, int64_t K, const void* A, const void* W,
-                const float* bias, void* out, uint32_t* status, cudaStream_t st, int cls = -1) {
+                const float* bias, void* out, uint32_t* status, cudaStream_t st, int cls = -1, const uint32_t* m_limit = nullptr,
+                int64_t m_off = 0) {
   if (M <= 0) return SRM_OK;
   if (cls < 0) cls = epi == kEpiBiasGelu ? SRM_KERNEL_GEMM_UP : epi == kEpiBiasResidual ? SRM_KERNEL_GEMM_DOWN : SRM_KERNEL_GEMM_LM;
   LaunchScope scope(m, cls, st);
   if (epi == kEpiArgmax) return launch_gemm_tc(m, epi, M, N, K, A, W, bias, out, status, st);
   if (m.cfg.dtype == SRM_DTYPE_FP32) return launch_gemm_simt<float>(epi, M, N, K, A, W, bias, out, st);
   if (m.cfg.flags & SRM_FLAG_SIMT_GEMM) return launch_gemm_simt<bf16>(epi, M, N, K, A, W, bias, out, st);
-  return launch_gemm_tc(m, epi, M, N, K, A, W, bias, out, status, st);
+  return launch_gemm_tc(m, epi, M, N, K, A, W, bias, out, status, st, 1, 0, m_limit, m_off);
 }
 
 // out[M, N] += A[M, K] W[N, K]^T + bias with K shared out between CTA pairs. `order`: zeroed words (split_order_words).
@@ -314,8 +321,9 @@ bool ffn_fused_worthwhile(const srm_model& m, int64_t M) {
 }
 
 // `ready`: ffn_ready_bytes(M, F) bytes of zeroed words. SRM_ERR_UNSUPPORTED: take the two launches.
+// m_limit, m_off: FfnArgs.
 int launch_ffn_fused(srm_model& m, int layer, int64_t M, const void* a, void* H, float* x, int32_t* ready, uint32_t* status,
-                     cudaStream_t st) {
+                     cudaStream_t st, const uint32_t* m_limit = nullptr, int64_t m_off = 0) {
   if (M <= 0) return SRM_OK;
   if (!ffn_fused_shape_ok(m, M)) return SRM_ERR_UNSUPPORTED;
   int rc = ensure_tc_ready(m);
@@ -343,7 +351,7 @@ int launch_ffn_fused(srm_model& m, int layer, int64_t M, const void* a, void* H,
   if ((rc = m.tmap(H, M, F, tc::kRowsPerCta, 2, &th)) != SRM_OK) return rc;
   if ((rc = m.tmap(W2, d, F, tc::kRowsPerCta, 2, &tw2)) != SRM_OK) return rc;
   if ((rc = m.tmap(x, M, d, tc::kOutBoxRows, 4, &tx)) != SRM_OK) return rc;
-  tc::FfnArgs g{M, d, (int)F, m.fptr(layer, SRM_T_B1), m.fptr(layer, SRM_T_B2), status, ready, 1};
+  tc::FfnArgs g{M, d, (int)F, m.fptr(layer, SRM_T_B1), m.fptr(layer, SRM_T_B2), status, ready, 1, m_limit, m_off};
   SRM_CUDA(launch_kernel(tc::ffn_fused_kernel, dim3(2u * (unsigned)m.tc_clusters), dim3(tc::kThreads), tc::kSmemBytes, st,
                          ta, tw1, tw1h, ths, th, tw2, tx, g, *plan));
   SRM_CUDA(cudaGetLastError());
@@ -534,6 +542,11 @@ int launch_lm_head_topk(srm_model& m, int64_t R, const void* a, void* lists, voi
 // - / 1844 / 1432; rl, 16 prompts of 200: 760 / 26 / -.
 constexpr int64_t kPrefillWalkMinPrompts = 384;
 
+bool prefill_walk_ok(const srm_model& m, int64_t np) {
+  const int d = m.cfg.d_model;
+  return m.cfg.mixer == SRM_MIXER_MIXED && !m.head_proj() && (d == 512 || d == 1024 || d == 1536 || d == 2048) && np >= kPrefillWalkMinPrompts;
+}
+
 template <int NV, typename WT, typename ST>
 int launch_prefill_walk(const PrefillParams& p, cudaStream_t st) {
   const size_t smem = prefill_walk_smem(NV * 128);
@@ -586,7 +599,7 @@ int launch_prefill_chunk(const PrefillParams& p, const ChunkScratch& cs, cudaStr
 // cs: scratch of the chunk kernel (prefill_chunk_ok), or nullptr: none.
 int launch_prefill_mixer(const srm_model& m, int layer, int64_t Bp, int n, const int32_t* tok, float* x, void* S,
                          void* a, uint32_t* status, cudaStream_t st, const int32_t* len = nullptr,
-                         const ChunkScratch* cs = nullptr) {
+                         const ChunkScratch* cs = nullptr, const int32_t* row_start = nullptr) {
   if (Bp <= 0) return SRM_OK;
   LaunchScope scope(m, SRM_KERNEL_PREFILL_MIXER, st);
   PrefillParams p;
@@ -595,7 +608,7 @@ int launch_prefill_mixer(const srm_model& m, int layer, int64_t Bp, int n, const
   p.ln2_g = m.fptr(layer, SRM_T_LN2_G); p.ln2_b = m.fptr(layer, SRM_T_LN2_B);
   p.alpha = m.fptr(layer, SRM_T_ALPHA); p.beta = m.fptr(layer, SRM_T_BETA); p.lam = m.fptr(layer, SRM_T_LAMBDA);
   p.Bp = Bp; p.n = n; p.d = m.cfg.d_model; p.h = m.cfg.n_heads; p.n_ctx = m.cfg.n_ctx; p.vocab = m.cfg.vocab;
-  p.eps = m.cfg.ln_eps; p.status = status; p.len = len;
+  p.eps = m.cfg.ln_eps; p.status = status; p.len = len; p.row_start = row_start;
   const size_t smem = (size_t)kPrefillTile * m.cfg.d_model * 4;
   const int nv = p.d / 128;
   if (cs != nullptr) {
@@ -610,7 +623,7 @@ int launch_prefill_mixer(const srm_model& m, int layer, int64_t Bp, int n, const
       }
     });
   }
-  if ((p.d == 512 || p.d == 1024 || p.d == 1536 || p.d == 2048) && Bp >= kPrefillWalkMinPrompts)      // many prompts
+  if (prefill_walk_ok(m, Bp))      // many prompts
     return dispatch_types(m.cfg, [&](auto w, auto c) { return launch_prefill_walk_nv<decltype(w), decltype(c)>(p, st); });
   auto go = [&](auto kernel) -> int {
     SRM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));   // smem depends on d: set per launch

@@ -172,19 +172,20 @@ __global__ void __launch_bounds__(kMixerWarps * 32) mixer_step_kernel(const Mixe
 }
 
 // out[r, :] = LN(x[r * src_stride + src_offset, :]) in the activation type; with row_len the offset of row r
-// is row_len[r] - 1 (the last position of a sample of that length).
+// is row_len[r] - 1 (the last position of a sample of that length); with row_start the row is the last before
+// row_start[r + 1].
 template <int NV, typename WT>
 __global__ void __launch_bounds__(kMixerWarps * 32)
 norm_rows_kernel(const float* __restrict__ x, int64_t R, int64_t src_stride, int64_t src_offset,
                  const float* __restrict__ g, const float* __restrict__ b, float eps, int d,
-                 WT* __restrict__ out, const int32_t* __restrict__ row_len, const PartialSum ps) {
+                 WT* __restrict__ out, const int32_t* __restrict__ row_len, const PartialSum ps, const int32_t* __restrict__ row_start) {
   pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kMixerWarps + (threadIdx.x >> 5);
   if (row >= R) return;
   if (row_len != nullptr) src_offset = min(max((int64_t)row_len[row], (int64_t)1), src_stride) - 1;
-  const float* xr = x + (row * src_stride + src_offset) * d;
+  const float* xr = x + (row_start != nullptr ? (int64_t)row_start[row + 1] - 1 : row * src_stride + src_offset) * d;
   float4 v[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {

@@ -34,7 +34,9 @@ struct PrefillParams {
   int n, d, h, n_ctx, vocab;
   float eps;
   uint32_t* status;
-  const int32_t* len;    // [Bp] prompt lengths (1 .. n; rows of a sample stay n apart), or nullptr: all prompts have n tokens
+  const int32_t* len;    // [Bp] prompt lengths (1 .. n), or nullptr: all prompts have n tokens
+  const int32_t* row_start = nullptr;    // [Bp + 1] first row of every prompt in x and a (prompts of different lengths stored one
+                                         // after the other; chunk and walk kernel), or nullptr: n rows apart (tok always is)
 };
 
 template <typename WT, typename ST>

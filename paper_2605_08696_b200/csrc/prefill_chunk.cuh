@@ -69,7 +69,8 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
   const int64_t b = blockIdx.x / (unsigned)chunks;
   const int ch = (int)(blockIdx.x - (unsigned)b * (unsigned)chunks);
   const int j0 = ch * T;
-  const int64_t row0 = b * p.n + j0;
+  const int64_t tok0 = b * p.n + j0;
+  int64_t row0 = tok0;
   const int c = tid * 4;
   const int g = c / (d / p.h);
   const bool is_row = g < (p.h >> 1);
@@ -92,7 +93,8 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
     }
   }
   const int rows = max(0, min(T, n - j0));             // rows of the prompt in this chunk
-  const int rows_all = min(T, p.n - j0);               // ... and of the padded prompt
+  if (p.row_start != nullptr) row0 = (int64_t)p.row_start[b] + j0;
+  const int rows_all = p.row_start != nullptr ? rows : min(T, p.n - j0);      // ... and of the padded prompt
   // positions beyond the prompt: defined values for the GEMMs that follow (their results are not used)
   for (int i = rows * d + c; i < rows_all * d; i += kThreads * 4) {
     st4(p.x + row0 * d + i, make_float4(0.f, 0.f, 0.f, 0.f));
@@ -113,7 +115,7 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
   for (int r = warp; r < rows; r += NV) {
     float4 v[NV];
     if (p.tok != nullptr) {
-      int tk = p.tok[row0 + r];
+      int tk = p.tok[tok0 + r];
       if (tk < 0 || tk >= p.vocab) {
         if (lane == 0) raise_status(p.status, kStatusTokenRange);
         tk = tk < 0 ? 0 : p.vocab - 1;

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(NV * 32, NV <= 4 ? 6 : NV <= 8 ? 3 : NV <= 12 
       n = n < 1 ? 1 : p.n;
     }
   }
-  const int64_t row0 = b * p.n;
+  const int64_t row0 = p.row_start != nullptr ? (int64_t)p.row_start[b] : b * p.n;
   const int chunks = (n + T - 1) / T;
   auto issue = [&](int ch) {                           // warp 0: the rows of chunk ch into slot ch % 2
     if (p.tok == nullptr && ch < chunks && tc::elect_one()) {
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(NV * 32, NV <= 4 ? 6 : NV <= 8 ? 3 : NV <= 12 
     for (int r = warp; r < rows; r += NV) {
       float4 v[NV];
       if (p.tok != nullptr) {
-        int tk = p.tok[row0 + j0 + r];
+        int tk = p.tok[b * p.n + j0 + r];
         if (tk < 0 || tk >= p.vocab) {
           if (lane == 0) raise_status(p.status, kStatusTokenRange);
           tk = tk < 0 ? 0 : p.vocab - 1;
@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(NV * 32, NV <= 4 ? 6 : NV <= 8 ? 3 : NV <= 12 
     if (warp == 0) issue(ch + kWalkSlots);
   }
   st4(reinterpret_cast<ST*>(p.S) + b * d + c, S);      // the cache the recurrent form continues from
+  if (p.row_start != nullptr) return;
   // positions beyond the prompt: defined values for the GEMMs that follow (their results are not used)
   for (int64_t i = (int64_t)n * d + c; i < (int64_t)p.n * d; i += kThreads * 4) {
     st4(p.x + row0 * d + i, make_float4(0.f, 0.f, 0.f, 0.f));

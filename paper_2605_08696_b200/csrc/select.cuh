@@ -541,6 +541,37 @@ clamp_lengths_kernel(const int32_t* __restrict__ len, int32_t* __restrict__ pos,
   if (i < B) pos[i] = min(max(len[i], lo), hi);
 }
 
+// Rows of prompts of different lengths stored one after the other: row_start[b] = sum of the lengths (clamped to [1, n_max])
+// before b, row_start[np] = all of them. One block.
+__global__ void __launch_bounds__(1024)
+pack_rows_kernel(const int32_t* __restrict__ len, int32_t* __restrict__ row_start, int64_t np, int n_max) {
+  pdl_trigger();
+  pdl_wait();
+  __shared__ int warp_sums[32];
+  __shared__ int carry;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) carry = 0;
+  __syncthreads();
+  for (int64_t b0 = 0; b0 < np; b0 += 1024) {
+    const int v = b0 + tid < np ? min(max(len[b0 + tid], 1), n_max) : 0;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) warp_sums[warp] = incl;
+    __syncthreads();
+    int before = carry;
+    for (int w = 0; w < warp; ++w) before += warp_sums[w];
+    if (b0 + tid < np) row_start[b0 + tid] = before + incl - v;
+    __syncthreads();
+    if (tid == 1023) carry = before + incl;
+    __syncthreads();
+  }
+  if (tid == 0) row_start[np] = carry;
+}
+
 // Step counters in the state header: set before a replayed generation loop, advanced after every step.
 __global__ void set_counters_kernel(int32_t* hdr, int pos, int step, int col) {
   pdl_trigger();
