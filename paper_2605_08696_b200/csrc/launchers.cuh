@@ -724,37 +724,48 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
 // ---- passes of a hundred to a thousand rows: all layers in one kernel (layers_mid.cuh) -------------------
 // Fewest rows, where the whole step is not one kernel of another design (step_small.cuh: up to 64 rows at d = 512, 32 at
 // d = 1024). d = 512: a batch just past that limit keeps the kernel-per-operation path (65 rows 134 us per step there,
-// 114 us here; a test counts on it).
-int64_t mid_min_rows(int d) { return d == 512 ? 97 : 1; }
+// 114 us here; a test counts on it). Combined heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96
+// rows, d = 1024, 16 layers, kernels of size 4: 320 us per step, as a kernel per operation 560).
+int64_t mid_min_rows(const srm_config& c) { return c.d_model == 512 && c.mixer == SRM_MIXER_MIXED ? 97 : 1; }
 
-// Whether a decode pass of R rows takes it, and its tile plan. bf16 mixed-head models of the widths it is built for,
+int mid_mix(const srm_config& c) { return c.mixer == SRM_MIXER_COMBINED ? mid::kCombined : c.mixer == SRM_MIXER_KERNEL ? mid::kKernel : mid::kMixed; }
+
+// Whether a decode pass of R rows takes it, and its tile plan. bf16 models of the widths it is built for,
 // as many rows as leave every CTA pair one tile of each projection.
 bool mid_plan(srm_model& m, int64_t R, const DecodeWs& w, mid::Params* p) {
   const srm_config& c = m.cfg;
   constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
-  if (R < mid_min_rows(c.d_model) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || c.mixer != SRM_MIXER_MIXED || w.part == nullptr) return false;
+  if (R < mid_min_rows(c) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || w.part == nullptr) return false;
+  if (c.mixer != SRM_MIXER_MIXED && !mid_variant_model(c)) return false;
   if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536) return false;
   if (ensure_tc_ready(m) != SRM_OK || R > (int64_t)2 * m.tc_clusters * mid::kGroups || m.F() > (1 << 20)) return false;
-  if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, p)) return false;
+  if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, mid_mix(c), p)) return false;
   return (size_t)p->ks * p->rb * tc::BM * c.d_model * 4 <= w.part_bytes;
 }
 
 struct MidMaps { CUtensorMap a, h, w1, w2, hs, p; };      // loads of a, H, W1, W2; stores of H and the partial products
-template <int NT, typename ST>
+template <int NT, typename ST, int MIX>
 int launch_layers_t(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
-  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(mid::layers_kernel<NT, ST>), mid::kSmemBytes);
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(mid::layers_kernel<NT, ST, MIX>), mid::kSmemBytes);
   if (rc != SRM_OK) return rc;
-  const size_t smem = mid::smem_bytes(p.d, p.n, p.w_slots, p.a_slots);
-  SRM_CUDA(launch_kernel(mid::layers_kernel<NT, ST>, dim3(2u * (unsigned)m.tc_clusters), dim3(mid::kThreads), smem, st,
+  const size_t smem = mid::smem_bytes(p.d, p.n, p.w_slots, p.a_slots, MIX);
+  SRM_CUDA(launch_kernel(mid::layers_kernel<NT, ST, MIX>, dim3(2u * (unsigned)m.tc_clusters), dim3(mid::kThreads), smem, st,
                          t.a, t.h, t.w1, t.w2, t.hs, t.p, p));
   SRM_CUDA(cudaGetLastError());
   return SRM_OK;
 }
 template <int NT>
 int launch_layers_nt(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
-  if (m.cfg.state_dtype == SRM_DTYPE_FP16) return launch_layers_t<NT, fp16>(m, t, p, st);
-  if (m.cfg.state_dtype == SRM_DTYPE_BF16) return launch_layers_t<NT, bf16>(m, t, p, st);
-  return launch_layers_t<NT, float>(m, t, p, st);
+  if (m.cfg.state_dtype == SRM_DTYPE_FP16) return launch_layers_t<NT, fp16, mid::kMixed>(m, t, p, st);
+  if (m.cfg.state_dtype == SRM_DTYPE_BF16) return launch_layers_t<NT, bf16, mid::kMixed>(m, t, p, st);
+  return launch_layers_t<NT, float, mid::kMixed>(m, t, p, st);
+}
+template <int NT>
+int launch_layers_variant(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
+  const bool half = m.cfg.state_dtype == SRM_DTYPE_FP16;
+  if (m.cfg.mixer == SRM_MIXER_COMBINED)
+    return half ? launch_layers_t<NT, fp16, mid::kCombined>(m, t, p, st) : launch_layers_t<NT, float, mid::kCombined>(m, t, p, st);
+  return half ? launch_layers_t<NT, fp16, mid::kKernel>(m, t, p, st) : launch_layers_t<NT, float, mid::kKernel>(m, t, p, st);
 }
 
 // All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
@@ -770,7 +781,10 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   p.layer0 = layer0_weights(m);
   p.layer_bytes = layer_stride_bytes(m);
   p.S = static_cast<uint8_t*>(s.layer_ptr(0)) + (size_t)b0 * d * m.state_bytes();
-  p.layer_stride = (int64_t)s.B * d * m.state_bytes();
+  p.layer_stride = (int64_t)s.planes() * s.B * d * m.state_bytes();
+  p.k = c.kernel_size;
+  p.s_plane = s.plane_elems();
+  if (c.mixer == SRM_MIXER_COMBINED) { p.alpha_col = m.fptr(0, SRM_T_ALPHA_COL); p.lam_col = m.fptr(0, SRM_T_LAMBDA_COL); p.w_comb = m.fptr(0, SRM_T_W_COMB); }
   p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
   p.x = w.x; p.a = reinterpret_cast<bf16*>(w.a); p.H = reinterpret_cast<bf16*>(w.H);
   p.part = w.part;
@@ -787,6 +801,7 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   if ((rc = make_tmap_kblocks(&maps.w2, m.ptr(0, SRM_T_W2), d, F, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = m.tmap(w.H, R, F, tc::kOutBoxRows, 2, &maps.hs)) != SRM_OK) return rc;
   if ((rc = m.tmap(w.part, (int64_t)p.ks * p.rb * tc::BM, d, tc::kOutBoxRows, 4, &maps.p)) != SRM_OK) return rc;
+  if (c.mixer != SRM_MIXER_MIXED) return d == 512 ? launch_layers_variant<2>(m, maps, p, st) : launch_layers_variant<4>(m, maps, p, st);
   if (d == 512) return launch_layers_nt<2>(m, maps, p, st);
   if (d == 1024) return launch_layers_nt<4>(m, maps, p, st);
   return launch_layers_nt<6>(m, maps, p, st);
@@ -830,7 +845,7 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   // cut into ranges so that all pairs work on it; the partial products go to planes of their own in the workspace
   // and the next consumer of x (the next layer's mixer, the final norm) adds them in a fixed order.
   const int64_t plane_rows = (R + tc::BM - 1) / tc::BM * tc::BM;
-  if (!one_kernel && !fused_ffn && !split && w.part != nullptr) {
+  if (!one_kernel && !fused_ffn && !split && w.part != nullptr && c.mixer == SRM_MIXER_MIXED) {
     if ((rc = ensure_tc_ready(m))) return rc;
     k_slices = down_k_slices(plane_rows / tc::BM * ((d + tc::BN - 1) / tc::BN), (int)(F / tc::BK), m.tc_clusters);
     while (k_slices > 1 && (size_t)k_slices * plane_rows * d * 4 > w.part_bytes) k_slices /= 2;

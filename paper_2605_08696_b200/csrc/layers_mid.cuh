@@ -12,6 +12,8 @@
 //   - the phases are ordered by counters in global memory, one per 256-row block (and range of K): rows done -> up tiles
 //     of the block start; up tiles of a range done -> down tiles of that range start; down tiles done -> rows of the
 //     block start. Nothing waits for a block it does not read.
+// Combined heads and kernels of size k (MIX) differ in the row phase only: their cache planes and scalars, and for kernels a
+// barrier of the row's two warps per filter.
 // Projections run as in gemm_tc_kernel: TMA loads (128-byte swizzle), tcgen05.mma.cta_group::2 issued by one thread of
 // the leader CTA, accumulator in tensor memory, 16 epilogue warps.
 //
@@ -64,22 +66,30 @@ struct Params {
   uint32_t* cnt;                 // rows done [8] | up pieces done [8][4] | down pieces done [8]; zero on entry
   uint32_t* status;
   const int32_t* ctr;            // device-side step counters or nullptr
-  const int32_t* pos;            // [R] per-row positions or nullptr
+  const int32_t* pos;            // [R] per-row positions or nullptr (mixed heads only)
+  // the further mixers: cache planes `s_plane` elements apart, parameters of layer 0 (as in VariantParams)
+  int k = 1;
+  int64_t s_plane = 0;
+  const float *alpha_col = nullptr, *lam_col = nullptr, *w_comb = nullptr;
 };
 // Row-phase parameters in shared memory: ln1_g | ln1_b | beta_t | ln2_g | ln2_b | b2 of the previous layer, then this CTA's
 // part of b1 (first touched in the epilogue it came from HBM there: 0.7 us).
 constexpr int kVecs = 6;
+// Token mixers: mixed heads; combined heads; kernels of size k.
+constexpr int kMixed = 0, kCombined = 1, kKernel = 2;
+constexpr int kMixScalars = 64;      // of a layer at the pass's position: combined 6 h <= 48 floats, kernel 2 k <= 32
 constexpr int kCntWords = kMaxRowBlocks * (2 + kMaxKSlices);
 
-// Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers.
-__host__ __device__ inline size_t smem_bytes(int d, int n, int w_slots, int a_slots) {
-  return 1024 + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + ((size_t)kVecs * d + n) * 4 + kGroups * 32 + kBarrierBytes;
+// Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers | for the
+// further mixers their scalars and, for kernels, the channels a warp's last lanes read of the next warp.
+__host__ __device__ inline size_t smem_bytes(int d, int n, int w_slots, int a_slots, int mix) {
+  return 1024 + (mix == kMixed ? 0 : kMixScalars * 4 + (mix == kKernel ? (size_t)kGroups * d : 0)) + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + ((size_t)kVecs * d + n) * 4 + kGroups * 32 + kBarrierBytes;
 }
 
 // Tile widths and ranges of K for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit. (256-wide
 // tiles, which would take mid passes of 513 to 1024 rows, measured slower than a kernel per operation: 0.59 against
 // 0.54 ms per step.)
-inline bool plan(int64_t R, int d, int F, int pairs, Params* p) {
+inline bool plan(int64_t R, int d, int F, int pairs, int mix, Params* p) {
   const int rb = (int)((R + tc::BM - 1) / tc::BM);
   if (rb < 1 || rb > kMaxRowBlocks) return false;
   for (int n = 64; n <= 128; n *= 2) {
@@ -92,7 +102,7 @@ inline bool plan(int64_t R, int d, int F, int pairs, Params* p) {
     // epilogue (128 rows of n fp32 columns)
     p->w_slots = n == 64 ? 8 : 6;
     p->a_slots = n == 64 ? 4 : 3;
-    while (smem_bytes(d, n, p->w_slots, p->a_slots) > (size_t)kSmemBytes)
+    while (smem_bytes(d, n, p->w_slots, p->a_slots, mix) > (size_t)kSmemBytes)
       if (--p->w_slots < 2) return false;
     return true;
   }
@@ -129,7 +139,87 @@ __device__ __forceinline__ bool count_wait(const uint32_t* p, uint32_t want, uin
 }
 __device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 9, %0;" ::"n"(kWorkers) : "memory"); }
 
-template <int NT, typename ST>
+// Combined heads and kernels of size k on the row of a group of 64 threads (thread th: channels 4 th .. 4 th + 3 and 256,
+// 512, ... further), as in mixer_variant_step_kernel: v = x in, x + y out; z = LN1(x); f = plane 0 of the cache.
+// hs: the mixer's scalars, edge: see smem_bytes.
+template <int NT, int MIX, typename ST>
+__device__ __forceinline__ void mix_row(const Params& p, float4 (&v)[NT], const float4 (&z)[NT], float4 (&f)[NT], const float4 (&f1)[NT],
+                                        const float* bt_p, ST* Sr, const float* hs, float4* edge, int group, int th) {
+  if (MIX == kCombined) {
+    const int dh = NT * 256 / p.h;
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+      const float* q = hs + 6 * ((th * 4 + 256 * i) / dh);
+      const float ar = q[0], ac = q[1], lr = q[2], lc = q[3], wr = q[4], wc = q[5];
+      const float4 bt = ld4(bt_p + 256 * i), sr = f[i], sc = f1[i];
+      const float4 u = make_float4(ar * z[i].x, ar * z[i].y, ar * z[i].z, ar * z[i].w);
+      const float4 w = make_float4(z[i].x + sc.x, z[i].y + sc.y, z[i].z + sc.z, z[i].w + sc.w);
+      v[i] = make_float4(v[i].x + (wr * (u.x + sr.x) + wc * (ac * w.x) + bt.x), v[i].y + (wr * (u.y + sr.y) + wc * (ac * w.y) + bt.y),
+                         v[i].z + (wr * (u.z + sr.z) + wc * (ac * w.z) + bt.z), v[i].w + (wr * (u.w + sr.w) + wc * (ac * w.w) + bt.w));
+      st4(Sr + 256 * i, make_float4(lr * (sr.x + u.x), lr * (sr.y + u.y), lr * (sr.z + u.z), lr * (sr.w + u.w)));
+      st4(Sr + p.s_plane + 256 * i, make_float4(lc * w.x, lc * w.y, lc * w.z, lc * w.w));
+    }
+  } else {
+    // v_i = z + P_i ;  y[c] = beta_t[c] + sum_i alpha_i[t] v_i[c + i] ;  P_i <- lam_i v_i. A shifted read reaches at most four
+    // lanes ahead: by shuffle inside the warp, the warp's last lanes from what the next 128 channels' first lanes left in
+    // `edge` (two buffers, filters in turn: one barrier of the group per filter).
+    const int lane = threadIdx.x & 31, half = th >> 5;
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+      const float4 bt = ld4(bt_p + 256 * i);
+      v[i] = make_float4(v[i].x + bt.x, v[i].y + bt.y, v[i].z + bt.z, v[i].w + bt.w);
+    }
+    for (int fi = 0; fi < p.k; ++fi) {
+      const float al = hs[2 * fi], lm = hs[2 * fi + 1];
+      ST* Pf = Sr + (int64_t)fi * p.s_plane;
+      float4 nx[NT];
+#pragma unroll
+      for (int i = 0; i < NT; ++i) nx[i] = fi + 1 < p.k ? ld4(Pf + p.s_plane + 256 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < NT; ++i) {
+        const float4 w = make_float4(z[i].x + f[i].x, z[i].y + f[i].y, z[i].z + f[i].z, z[i].w + f[i].w);
+        st4(Pf + 256 * i, make_float4(lm * w.x, lm * w.y, lm * w.z, lm * w.w));
+        f[i] = make_float4(al * w.x, al * w.y, al * w.z, al * w.w);
+      }
+      if (fi > 0) {
+        float4* e = edge + (fi & 1) * (NT * 8);             // [128-channel vector][4 lanes]
+        if (lane < 4) {
+#pragma unroll
+          for (int i = 0; i < NT; ++i) e[(2 * i + half) * 4 + lane] = f[i];
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
+        auto ahead = [&](int i, int delta) {                // the float4 `delta` lanes ahead, 0 <= delta <= 4
+          const int src = lane + delta;
+          float4 r = make_float4(__shfl_sync(0xffffffffu, f[i].x, src & 31), __shfl_sync(0xffffffffu, f[i].y, src & 31),
+                                 __shfl_sync(0xffffffffu, f[i].z, src & 31), __shfl_sync(0xffffffffu, f[i].w, src & 31));
+          if (src >= 32) {
+            const int next = 2 * i + half + 1;
+            r = next < 2 * NT ? e[next * 4 + src - 32] : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+          return r;
+        };
+        const int q = fi >> 2, s = fi & 3;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+          const float4 A = q == 0 ? f[i] : ahead(i, q);
+          float4 r = A;
+          if (s != 0) {
+            const float4 B = ahead(i, q + 1);
+            r = s == 1 ? make_float4(A.y, A.z, A.w, B.x) : s == 2 ? make_float4(A.z, A.w, B.x, B.y) : make_float4(A.w, B.x, B.y, B.z);
+          }
+          v[i] = make_float4(v[i].x + r.x, v[i].y + r.y, v[i].z + r.z, v[i].w + r.w);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < NT; ++i) v[i] = make_float4(v[i].x + f[i].x, v[i].y + f[i].y, v[i].z + f[i].z, v[i].w + f[i].w);
+      }
+#pragma unroll
+      for (int i = 0; i < NT; ++i) f[i] = nx[i];
+    }
+  }
+}
+
+template <int NT, typename ST, int MIX>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmW1,
               const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmHs, const __grid_constant__ CUtensorMap tmP,
@@ -152,6 +242,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   uint64_t* tempty = tfull + 1;                                          // leader: accumulator drained by both CTAs
   uint64_t* ring = tempty + 1;                                           // the epilogue has left the activation ring
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring + 1);
+  float* hs = red + kGroups * 8 + kBarrierBytes / 4;                     // MIX != kMixed
+  float4* edge = reinterpret_cast<float4*>(hs + kMixScalars);            // MIX == kKernel: d bytes per group
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = tc::cluster_ctarank();
@@ -310,17 +402,32 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       const int row = (int)blockIdx.x + (int)gridDim.x * group;
       const bool mine = row < p.R;
       const int t = mine && p.pos != nullptr ? min(max(p.pos[row], 0), p.n_ctx - 1) : t_all;
-      float a1[NT], a2[NT], lm[NT];
-      float4 s[NT], v[NT];
+      float a1[NT], a2[NT], lm[NT];                  // (mixed heads)
+      float4 s[NT], s1[NT], v[NT];                   // (s1: combined heads)
       ST* Sr = reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + (int64_t)row * d + c0;
       if (mine) {
         if (!last) {
-          sb::head_scalars<d, NT>(p, w, t, wid & 63, a1, a2, lm);
+          if (MIX == kMixed) sb::head_scalars<d, NT>(p, w, t, wid & 63, a1, a2, lm);
 #pragma unroll
           for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + 256 * i);
+          if (MIX == kCombined) {
+#pragma unroll
+            for (int i = 0; i < NT; ++i) s1[i] = ld4(Sr + p.s_plane + 256 * i);
+          }
         }
         if (l > 0 && (wid & 63) == 0 && ok)       // the down tiles of the row's block
           ok = count_wait(cnt_dn + row / tc::BM, (uint32_t)l * (uint32_t)(p.cd * p.ks * dn_boxes) * 8u, p.status);
+      }
+      if (MIX != kMixed && !last) {         // scalar wid of the layer
+        const int64_t o = (int64_t)l * p.layer_bytes;
+        auto at = [o](const float* q, int64_t i) { return __ldg(reinterpret_cast<const float*>(reinterpret_cast<const uint8_t*>(q) + o) + i); };
+        if (MIX == kCombined && wid < 6 * p.h) {
+          const int g = wid / 6, q = wid % 6;
+          const int64_t ia = (int64_t)g * p.n_ctx + t_all;
+          hs[wid] = q == 0 ? __ldg(w.alpha + ia) : q == 1 ? at(p.alpha_col, ia) : q == 2 ? __ldg(w.lam + g) : q == 3 ? at(p.lam_col, g)
+                                                                                          : at(p.w_comb, 2 * g + q - 4);
+        }
+        if (MIX == kKernel && wid < 2 * p.k) hs[wid] = wid & 1 ? __ldg(w.lam + (wid >> 1)) : __ldg(w.alpha + (int64_t)(wid >> 1) * p.n_ctx + t_all);
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       workers_sync();
@@ -355,8 +462,20 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
           const float* bt_p = p.pos != nullptr ? w.beta + (int64_t)t * d + c0 : prm + 2 * d + c0;
           sb::group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
           const float nmr = -mean * rstd;
+          if (MIX != kMixed) {
+            float4 z[NT];
 #pragma unroll
-          for (int i = 0; i < NT; ++i) {
+            for (int i = 0; i < NT; ++i) {
+              const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i);
+              z[i] = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
+                                 fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
+            }
+            mix_row<NT, MIX>(p, v, z, s, s1, bt_p, Sr, hs, edge + group * (d / 16), group, wid & 63);
+#pragma unroll
+            for (int i = 0; i < NT; ++i) st4(p.x + (int64_t)row * d + c0 + 256 * i, v[i]);
+          }
+#pragma unroll
+          for (int i = 0; MIX == kMixed && i < NT; ++i) {
             const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i), bt = ld4(bt_p + 256 * i);
             const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
                                          fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));

@@ -82,3 +82,37 @@ def test_captured_step_and_passes_of_one_kernel_equal_launch_by_launch():
     for r in res[1:]:
         for x, y in zip(res[0], r):
             assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("mixer,k,B,d,state_dtype", [("combined", 1, 1, 1024, "fp32"), ("combined", 1, 300, 512, "fp16"),
+                                                     ("kernel", 1, 40, 512, "fp32"), ("kernel", 4, 257, 1024, "fp32"),
+                                                     ("kernel", 5, 97, 512, "fp16"), ("kernel", 16, 130, 1024, "fp16"),
+                                                     ("kernel", 13, 1000, 512, "fp32")])
+def test_further_mixers_in_one_kernel_agree_with_the_kernel_per_operation_path(mixer, k, B, d, state_dtype):
+    import dataclasses
+
+    import paper_2605_08696_b200 as P
+    base = custom_shape(n_layers=3, d_model=d, vocab=2048, n_ctx=24, dtype="bf16", seed=13)
+    shape = dataclasses.replace(base, mixer=mixer, kernel_size=k)
+    W = I.make_weights(shape)
+    n = 4
+    toks = torch.from_numpy(np.random.default_rng(B).integers(0, shape.vocab, size=(n + 3, B)).astype(np.int32)).to(DEV)
+    g = P.Sampling("greedy")
+    outs = []
+    for flags in (P.FLAG_NO_SMALL_BATCH, 0):
+        m = P.SRM(shape, W, device=DEV, flags=flags, state_dtype=state_dtype)
+        st, ws = m.new_state(B), m.new_workspace(B, n, prefill_samples=B)
+        m.prefill(st, toks[:n].t().contiguous(), g, ws)
+        lgs = []
+        for i in range(3):
+            launches = _launches(P, lambda: lgs.append(m.decode_step(st, toks[n + i], g, i + 1, ws, want_logits=True)[1].cpu().numpy()))
+        assert (launches <= 3) == (flags == 0) and st.status() == 0
+        outs.append((np.stack(lgs), st.cache().cpu().numpy()))
+    tol = 5 * 2.0 ** -9 * 3 ** 0.5                             # as above
+    assert rel_err_rows(outs[1][0], outs[0][0]) < tol and rel_err_rows(outs[1][1], outs[0][1]) < tol
+    orc = oracle_for(shape, W)
+    for b in (0, B - 1):
+        lo, state = orc.forward_parallel(toks[:n, b:b + 1].t().cpu().numpy())
+        for i in range(3):
+            lo, state = orc.decode_step(state, toks[n + i, b:b + 1].cpu().numpy(), n + i)
+            assert rel_err_rows(outs[1][0][i][b:b + 1], lo) < 3e-2
