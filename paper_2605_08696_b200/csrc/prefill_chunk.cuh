@@ -43,12 +43,16 @@ struct ChunkScratch {
 };
 
 inline int64_t prefill_chunks(int n) { return (n + kChunkRows - 1) / kChunkRows; }
-inline size_t prefill_chunk_smem(int d) { return (size_t)kChunkRows * d * 4 + 2 * kChunkRows * 4 + 16; }
+inline size_t prefill_chunk_smem(int d) { return (size_t)(kChunkRows + 2) * d * 4 + 2 * kChunkRows * 4 + 16; }
 
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+// Rows of a parameter on their way into L2 (bytes: a multiple of 16).
+__device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -61,7 +65,8 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
   constexpr int T = kChunkRows, d = NV * 128, kThreads = NV * 32;
   extern __shared__ __align__(128) uint8_t sm[];
   float* xs = reinterpret_cast<float*>(sm);                          // [T][d]
-  float* rs = xs + T * d;                                            // rstd of the rows
+  float* ln2 = xs + T * d;                                           // ln2_g | ln2_b (every row of a warp waited for them otherwise)
+  float* rs = ln2 + 2 * d;                                           // rstd of the rows
   float* nm = rs + T;                                                // -mean * rstd
   uint64_t* bar = reinterpret_cast<uint64_t*>(nm + T);
 
@@ -77,7 +82,10 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
   // parameters: constant data, fetched ahead of the dependency wait
   const float4 g1 = ldg4(p.ln1_g + c), b1 = ldg4(p.ln1_b + c);
   const float lam = __ldg(p.lam + g);
+  st4(ln2 + c, ldg4(p.ln2_g + c));
+  st4(ln2 + d + c, ldg4(p.ln2_b + c));
   if (tid == 0) {
+    bulk_prefetch_l2(p.beta + (int64_t)j0 * d, (uint32_t)(min(T, p.n - j0) * d * 4));
     tc::mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -152,11 +160,22 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
     }
     __stcg(reinterpret_cast<float4*>(cs.E + (b * (chunks - 1) + ch) * d + c), S);
     __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      st_release_u32(cs.flags + b * chunks + ch, cs.epoch);
-    }
+    if (tid == 0) st_release_u32(cs.flags + b * chunks + ch, cs.epoch);
   }
+  // beta and alpha of the second pass over the chunk, four positions ahead
+  const float* beta = p.beta + (int64_t)j0 * d + c;
+  float4 bt[4];
+  float al[4];
+  auto fetch = [&](int j0b) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (j0b + k < rows) {
+        bt[k] = ldg4(beta + (int64_t)(j0b + k) * d);
+        al[k] = __ldg(alpha + j0b + k);
+      }
+    }
+  };
+  fetch(0);
   S = make_float4(0.f, 0.f, 0.f, 0.f);
   if (ch > 0) {
     // ---- the start value: S <- lambda^T S + E over the earlier chunks, in order ----
@@ -179,29 +198,36 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
     }
   }
   // ---- y_j and the residual, in place ----
-  const float* beta = p.beta + (int64_t)j0 * d + c;
-#pragma unroll 4
-  for (int j = 0; j < rows; ++j) {
-    const float4 v = ld4(xs + j * d + c), z = z_of(v, j), bt = ldg4(beta + (int64_t)j * d);
-    const float al = __ldg(alpha + j);
-    float4 y;
-    if (is_row) {               // row-repeat head, Eq. 2
-      const float4 u = make_float4(al * z.x, al * z.y, al * z.z, al * z.w);
-      y = make_float4(u.x + bt.x + S.x, u.y + bt.y + S.y, u.z + bt.z + S.z, u.w + bt.w + S.w);
-      S = make_float4(lam * (S.x + u.x), lam * (S.y + u.y), lam * (S.z + u.z), lam * (S.w + u.w));
-    } else {                    // column-repeat head, Eq. 3
-      const float4 w = make_float4(z.x + S.x, z.y + S.y, z.z + S.z, z.w + S.w);
-      y = make_float4(al * w.x + bt.x, al * w.y + bt.y, al * w.z + bt.z, al * w.w + bt.w);
-      S = make_float4(lam * w.x, lam * w.y, lam * w.z, lam * w.w);
+  for (int jb = 0; jb < rows; jb += 4) {
+    float4 bc[4];
+    float ac[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { bc[k] = bt[k]; ac[k] = al[k]; }
+    fetch(jb + 4);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = jb + k;
+      if (j >= rows) break;
+      const float4 v = ld4(xs + j * d + c), z = z_of(v, j), b = bc[k];
+      const float a = ac[k];
+      float4 y;
+      if (is_row) {               // row-repeat head, Eq. 2
+        const float4 u = make_float4(a * z.x, a * z.y, a * z.z, a * z.w);
+        y = make_float4(u.x + b.x + S.x, u.y + b.y + S.y, u.z + b.z + S.z, u.w + b.w + S.w);
+        S = make_float4(lam * (S.x + u.x), lam * (S.y + u.y), lam * (S.z + u.z), lam * (S.w + u.w));
+      } else {                    // column-repeat head, Eq. 3
+        const float4 w = make_float4(z.x + S.x, z.y + S.y, z.z + S.z, z.w + S.w);
+        y = make_float4(a * w.x + b.x, a * w.y + b.y, a * w.z + b.z, a * w.w + b.w);
+        S = make_float4(lam * w.x, lam * w.y, lam * w.z, lam * w.w);
+      }
+      st4(xs + j * d + c, make_float4(v.x + y.x, v.y + y.y, v.z + y.z, v.w + y.w));
     }
-    st4(xs + j * d + c, make_float4(v.x + y.x, v.y + y.y, v.z + y.z, v.w + y.w));
   }
   if (j0 + rows == n) st4(reinterpret_cast<ST*>(p.S) + b * d + c, S);      // the cache the recurrent form continues from
   __syncthreads();
 
   // ---- LN2 and write-back ----
   for (int r = warp; r < rows; r += NV) {
-    asm volatile("" ::: "memory");      // the gains and shifts are fetched per row: held across rows they would not fit
     float4 v[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = ld4(xs + r * d + lane * 4 + i * 128);
@@ -213,7 +239,7 @@ prefill_chunk_kernel(const PrefillParams p, const ChunkScratch cs, int chunks) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       st4(xo + i * 128, v[i]);
-      const float4 gg = ld4(p.ln2_g + lane * 4 + i * 128), bb = ld4(p.ln2_b + lane * 4 + i * 128);
+      const float4 gg = ld4(ln2 + lane * 4 + i * 128), bb = ld4(ln2 + d + lane * 4 + i * 128);
       st4(ao + i * 128, make_float4(fmaf(fmaf(v[i].x, rstd, nmr), gg.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), gg.y, bb.y),
                                     fmaf(fmaf(v[i].z, rstd, nmr), gg.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), gg.w, bb.w)));
     }

@@ -14,6 +14,7 @@
 #pragma once
 
 #include "mixer_model_variants.cuh"   // VariantParams
+#include "mixer_variants.cuh"         // cp_async16
 #include "prefill_chunk.cuh"
 
 namespace srm {
@@ -30,7 +31,8 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
   constexpr int C = KM > 0 ? KM : 2;                                 // sum terms per channel
   extern __shared__ __align__(128) uint8_t sm[];
   float* xs = reinterpret_cast<float*>(sm);                          // [T][d]: x, from the statistics on z (KM > 0)
-  float* rs = xs + T * d;                                            // rstd of the rows
+  float* ln = xs + T * d;                                            // gains | shifts of LN1 (KM > 0), then of LN2
+  float* rs = ln + 2 * d;                                            // rstd of the rows
   float* nm = rs + T;                                                // -mean * rstd
   float* al_s = nm + T + 4;                                          // KM > 0: alpha_i at the chunk's positions [KM][T]
   uint64_t* bar = reinterpret_cast<uint64_t*>(nm + T);
@@ -59,8 +61,11 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
     }
 #pragma unroll
     for (int i = 0; i < C; ++i) lam[i] = i < p.k ? __ldg(p.lam + i) : 0.f;
+    st4(ln + c, ldg4(p.ln1_g + c));
+    st4(ln + d + c, ldg4(p.ln1_b + c));
   }
   if (tid == 0) {
+    bulk_prefetch_l2(p.beta + (int64_t)j0 * d, (uint32_t)(rows * d * 4));
     tc::mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -86,7 +91,6 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
   }
   constexpr float inv_d = 1.0f / (float)d;
   for (int r = warp; r < rows; r += NV) {
-    asm volatile("" ::: "memory");      // gains and shifts are fetched per row: held across rows they would not fit
     float4 v[NV];
     if (p.tok != nullptr) {
       const WT* e = reinterpret_cast<const WT*>(p.E) + (int64_t)token(r) * d + lane * 4;
@@ -102,7 +106,7 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
     if (KM > 0) {
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
-        const float4 gg = ld4(p.ln1_g + lane * 4 + i * 128), bb = ld4(p.ln1_b + lane * 4 + i * 128);
+        const float4 gg = ld4(ln + lane * 4 + i * 128), bb = ld4(ln + d + lane * 4 + i * 128);
         st4(xs + r * d + lane * 4 + i * 128,
             make_float4(fmaf(fmaf(v[i].x, rstd, nmr), gg.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), gg.y, bb.y),
                         fmaf(fmaf(v[i].z, rstd, nmr), gg.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), gg.w, bb.w)));
@@ -116,6 +120,9 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
     }
   }
   __syncthreads();
+  cp_async16(ln + c, p.ln2_g + c);                                   // (waited for before LN2)
+  cp_async16(ln + d + c, p.ln2_b + c);
+  asm volatile("cp.async.commit_group;" ::: "memory");
 
   // ---- one position of this thread's sum terms; returns y without beta ----
   float4 S[C];
@@ -173,10 +180,7 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
     for (int i = 0; i < C; ++i)
       if (i < planes) __stcg(reinterpret_cast<float4*>(cs.E + E0 + ((int64_t)ch * planes + i) * d), S[i]);
     __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      st_release_u32(cs.flags + b * chunks + ch, cs.epoch);
-    }
+    if (tid == 0) st_release_u32(cs.flags + b * chunks + ch, cs.epoch);
     clear();
   }
   if (ch > 0) {
@@ -252,11 +256,11 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
       }
     }
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
 
   // ---- LN2 and write-back ----
   for (int r = warp; r < rows; r += NV) {
-    asm volatile("" ::: "memory");
     float4 v[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = ld4(xs + r * d + lane * 4 + i * 128);
@@ -268,7 +272,7 @@ variant_chunk_kernel(const VariantParams p, const ChunkScratch cs, int n, int ch
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       st4(xo + i * 128, v[i]);
-      const float4 gg = ld4(p.ln2_g + lane * 4 + i * 128), bb = ld4(p.ln2_b + lane * 4 + i * 128);
+      const float4 gg = ld4(ln + lane * 4 + i * 128), bb = ld4(ln + d + lane * 4 + i * 128);
       st4(ao + i * 128, make_float4(fmaf(fmaf(v[i].x, rstd, nmr), gg.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), gg.y, bb.y),
                                     fmaf(fmaf(v[i].z, rstd, nmr), gg.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), gg.w, bb.w)));
     }
