@@ -738,21 +738,27 @@ bool mid_plan(srm_model& m, int64_t R, const DecodeWs& w, mid::Params* p) {
   if (R < mid_min_rows(c) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || w.part == nullptr) return false;
   if (c.mixer != SRM_MIXER_MIXED && !mid_variant_model(c)) return false;
   if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536) return false;
-  if (ensure_tc_ready(m) != SRM_OK || R > (int64_t)2 * m.tc_clusters * mid::kGroups || m.F() > (1 << 20)) return false;
+  if (ensure_tc_ready(m) != SRM_OK || R > (int64_t)2 * m.tc_clusters * mid::kMaxGroups || m.F() > (1 << 20)) return false;
   if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, mid_mix(c), p)) return false;
   return (size_t)p->ks * p->rb * tc::BM * c.d_model * 4 <= w.part_bytes;
 }
 
 struct MidMaps { CUtensorMap a, h, w1, w2, hs, p; };      // loads of a, H, W1, W2; stores of H and the partial products
-template <int NT, typename ST, int MIX>
-int launch_layers_t(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
-  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(mid::layers_kernel<NT, ST, MIX>), mid::kSmemBytes);
+template <int NT, int WPG, typename ST, int MIX>
+int launch_layers_w(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
+  int rc = ensure_dynamic_smem(reinterpret_cast<const void*>(mid::layers_kernel<NT, WPG, ST, MIX>), mid::kSmemBytes);
   if (rc != SRM_OK) return rc;
   const size_t smem = mid::smem_bytes(p.d, p.n, p.w_slots, p.a_slots, MIX);
-  SRM_CUDA(launch_kernel(mid::layers_kernel<NT, ST, MIX>, dim3(2u * (unsigned)m.tc_clusters), dim3(mid::kThreads), smem, st,
+  SRM_CUDA(launch_kernel(mid::layers_kernel<NT, WPG, ST, MIX>, dim3(2u * (unsigned)m.tc_clusters), dim3(mid::kThreads), smem, st,
                          t.a, t.h, t.w1, t.w2, t.hs, t.p, p));
   SRM_CUDA(cudaGetLastError());
   return SRM_OK;
+}
+// Four warps per row where all rows are then worked on at once, else two.
+template <int NT, typename ST, int MIX>
+int launch_layers_t(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
+  if (p.R <= (int64_t)2 * m.tc_clusters * (tc::kEpiWarps / 4)) return launch_layers_w<NT / 2, 4, ST, MIX>(m, t, p, st);
+  return launch_layers_w<NT, 2, ST, MIX>(m, t, p, st);
 }
 template <int NT>
 int launch_layers_nt(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
@@ -795,8 +801,8 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
   MidMaps maps;
   int rc;
-  if ((rc = make_tmap_kblocks(&maps.a, w.a, R, d, tc::kRowsPerCta, mid::kStep)) != SRM_OK) return rc;
-  if ((rc = make_tmap_kblocks(&maps.h, w.H, R, F, tc::kRowsPerCta, mid::kStep)) != SRM_OK) return rc;
+  if ((rc = make_tmap_kblocks(&maps.a, w.a, R, d, p.box, mid::kStep)) != SRM_OK) return rc;
+  if ((rc = make_tmap_kblocks(&maps.h, w.H, R, F, p.box, mid::kStep)) != SRM_OK) return rc;
   if ((rc = make_tmap_kblocks(&maps.w1, m.ptr(0, SRM_T_W1), F, d, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = make_tmap_kblocks(&maps.w2, m.ptr(0, SRM_T_W2), d, F, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = m.tmap(w.H, R, F, tc::kOutBoxRows, 2, &maps.hs)) != SRM_OK) return rc;

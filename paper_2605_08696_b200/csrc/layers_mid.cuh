@@ -7,13 +7,14 @@
 //     runs ahead of everything else: a projection finds its first k-blocks in shared memory when its input is ready;
 //   - a pair computes at most one 256 x N tile of the up projection and one of the down projection per layer (the down
 //     projection's K cut into ranges), N 64 or 128, the smaller with which the tiles fit on the pairs;
-//   - row phases (x + partial products of the previous down projection, LN1, cache update, residual, LN2) are done by two
-//     warps per row, the rows dealt to all CTAs;
+//   - row phases (x + partial products of the previous down projection, LN1, cache update, residual, LN2) are done by four
+//     warps per row (two where there are more rows than that serves at once), the rows dealt to all CTAs. With four all
+//     loads of a row are in flight at once: 2.9 -> 1.5 us per layer at 256 rows of the mid model;
 //   - the phases are ordered by counters in global memory, one per 256-row block (and range of K): rows done -> up tiles
 //     of the block start; up tiles of a range done -> down tiles of that range start; down tiles done -> rows of the
 //     block start. Nothing waits for a block it does not read.
 // Combined heads and kernels of size k (MIX) differ in the row phase only: their cache planes and scalars, and for kernels a
-// barrier of the row's two warps per filter.
+// barrier of the row's warps per filter.
 // Projections run as in gemm_tc_kernel: TMA loads (128-byte swizzle), tcgen05.mma.cta_group::2 issued by one thread of
 // the leader CTA, accumulator in tensor memory, 16 epilogue warps.
 //
@@ -23,6 +24,8 @@
 #pragma once
 
 #include <cuda.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "gemm_tc.cuh"
@@ -36,7 +39,7 @@ namespace mid {
 constexpr int kEpiWarp0 = 3;                                      // warp 0: A producer, 1: MMA, 2: W producer
 constexpr int kThreads = (kEpiWarp0 + tc::kEpiWarps) * 32;
 constexpr int kWorkers = tc::kEpiWarps * 32;                      // threads of the epilogue / row warps
-constexpr int kGroups = tc::kEpiWarps / 2;                        // rows a CTA works on at a time
+constexpr int kMaxGroups = tc::kEpiWarps / 2;                     // rows a CTA works on at a time, at most
 constexpr int kStep = 2;                                          // k-blocks (of 64) per stage: the waits and commits of a stage take as long as a k-block's MMAs
 constexpr int kMaxWSlots = 8, kMaxASlots = 4;
 constexpr int kABytes = kStep * tc::kRowsPerCta * tc::BK * 2;     // one stage of A per CTA
@@ -51,6 +54,8 @@ struct Params {
   float eps;
   int rb, n, cu, cd, ks;         // row blocks, tile width, column tiles of the up / down projection, ranges of K
   int w_slots, a_slots;
+  int box;                       // rows of an activation box: 128, or the rows there are (a multiple of 8); rows of zeros that the copy
+                                 // unit fills in for rows beyond the last cost it more than rows it reads (45 rows: 2.7 against 1.2 us per tile)
   const int32_t* tok_in;         // [R]
   const bf16* E;
   sb::LayerW layer0;             // as in sb::Params
@@ -83,7 +88,7 @@ constexpr int kCntWords = kMaxRowBlocks * (2 + kMaxKSlices);
 // Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers | for the
 // further mixers their scalars and, for kernels, the channels a warp's last lanes read of the next warp.
 __host__ __device__ inline size_t smem_bytes(int d, int n, int w_slots, int a_slots, int mix) {
-  return 1024 + (mix == kMixed ? 0 : kMixScalars * 4 + (mix == kKernel ? (size_t)kGroups * d : 0)) + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + ((size_t)kVecs * d + n) * 4 + kGroups * 32 + kBarrierBytes;
+  return 1024 + (mix == kMixed ? 0 : kMixScalars * 4 + (mix == kKernel ? (size_t)kMaxGroups * d : 0)) + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + ((size_t)kVecs * d + n) * 4 + kMaxGroups * 32 + kBarrierBytes;
 }
 
 // Tile widths and ranges of K for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit. (256-wide
@@ -97,6 +102,7 @@ inline bool plan(int64_t R, int d, int F, int pairs, int mix, Params* p) {
     int ks = kMaxKSlices;
     while (ks > 1 && (rb * (d / n) * ks > pairs || (F / 64) % (ks * kStep) || (F / ks) % n)) ks >>= 1;
     if (rb * (d / n) * ks > pairs || (F / 64) % (ks * kStep)) continue;
+    p->box = R < tc::kRowsPerCta ? (int)(R + 7) / 8 * 8 : tc::kRowsPerCta;
     p->rb = rb; p->n = n; p->cu = F / n; p->cd = d / n; p->ks = ks;
     // the weight ring runs a phase ahead; the activation ring hides the latency of L2 and holds the output tile of an
     // epilogue (128 rows of n fp32 columns)
@@ -139,34 +145,77 @@ __device__ __forceinline__ bool count_wait(const uint32_t* p, uint32_t want, uin
 }
 __device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 9, %0;" ::"n"(kWorkers) : "memory"); }
 
-// Combined heads and kernels of size k on the row of a group of 64 threads (thread th: channels 4 th .. 4 th + 3 and 256,
-// 512, ... further), as in mixer_variant_step_kernel: v = x in, x + y out; z = LN1(x); f = plane 0 of the cache.
+// LayerNorm statistics of a row held by WPG warps (thread th of them: float4s 32 WPG apart): every thread's mean and sum of
+// squares about it are merged over the warp, then over the warps in order. slot: 2 WPG floats of the group.
+template <int NT, int WPG>
+__device__ __forceinline__ void group_stats(const float4 (&v)[NT], float eps, float* slot, int group, float& mean, float& rstd) {
+  float m = 0.f, q = 0.f, cnt = 4.f * NT;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) m += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+  m *= 1.0f / (4.f * NT);
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const float a = v[i].x - m, b = v[i].y - m, c = v[i].z - m, e = v[i].w - m;
+    q += (a * a + b * b) + (c * c + e * e);
+  }
+  auto merge = [](float& m, float& q, float cnt, float m2, float q2) {        // of two sets of cnt values each
+    const float dm = m2 - m;
+    q += fmaf(dm * dm, 0.5f * cnt, q2);
+    m = 0.5f * (m + m2);
+  };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, m, o), q2 = __shfl_xor_sync(0xffffffffu, q, o);
+    merge(m, q, cnt, m2, q2);
+    cnt += cnt;
+  }
+  if ((threadIdx.x & 31) == 0) {                         // (the lanes may differ in the last bit: lane 0's values count)
+    const int w = ((threadIdx.x >> 5) - kEpiWarp0) % WPG;
+    slot[w] = m;
+    slot[WPG + w] = q;
+  }
+  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(WPG * 32) : "memory");
+  float mm[WPG], qq[WPG];
+#pragma unroll
+  for (int w = 0; w < WPG; ++w) { mm[w] = slot[w]; qq[w] = slot[WPG + w]; }
+#pragma unroll
+  for (int s = 1; s < WPG; s += s) {
+#pragma unroll
+    for (int w = 0; w < WPG; w += 2 * s) merge(mm[w], qq[w], cnt, mm[w + s], qq[w + s]);
+    cnt += cnt;
+  }
+  mean = mm[0];
+  rstd = rsqrtf(qq[0] / cnt + eps);
+}
+
+// Combined heads and kernels of size k on the row of a group of WPG warps (thread th: channels 4 th .. 4 th + 3 and 128 WPG,
+// 256 WPG, ... further), as in mixer_variant_step_kernel: v = x in, x + y out; z = LN1(x); f = plane 0 of the cache.
 // hs: the mixer's scalars, edge: see smem_bytes.
-template <int NT, int MIX, typename ST>
+template <int NT, int WPG, int MIX, typename ST>
 __device__ __forceinline__ void mix_row(const Params& p, float4 (&v)[NT], const float4 (&z)[NT], float4 (&f)[NT], const float4 (&f1)[NT],
                                         const float* bt_p, ST* Sr, const float* hs, float4* edge, int group, int th) {
   if (MIX == kCombined) {
-    const int dh = NT * 256 / p.h;
+    const int dh = NT * WPG * 128 / p.h;
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-      const float* q = hs + 6 * ((th * 4 + 256 * i) / dh);
+      const float* q = hs + 6 * ((th * 4 + 128 * WPG * i) / dh);
       const float ar = q[0], ac = q[1], lr = q[2], lc = q[3], wr = q[4], wc = q[5];
-      const float4 bt = ld4(bt_p + 256 * i), sr = f[i], sc = f1[i];
+      const float4 bt = ld4(bt_p + 128 * WPG * i), sr = f[i], sc = f1[i];
       const float4 u = make_float4(ar * z[i].x, ar * z[i].y, ar * z[i].z, ar * z[i].w);
       const float4 w = make_float4(z[i].x + sc.x, z[i].y + sc.y, z[i].z + sc.z, z[i].w + sc.w);
       v[i] = make_float4(v[i].x + (wr * (u.x + sr.x) + wc * (ac * w.x) + bt.x), v[i].y + (wr * (u.y + sr.y) + wc * (ac * w.y) + bt.y),
                          v[i].z + (wr * (u.z + sr.z) + wc * (ac * w.z) + bt.z), v[i].w + (wr * (u.w + sr.w) + wc * (ac * w.w) + bt.w));
-      st4(Sr + 256 * i, make_float4(lr * (sr.x + u.x), lr * (sr.y + u.y), lr * (sr.z + u.z), lr * (sr.w + u.w)));
-      st4(Sr + p.s_plane + 256 * i, make_float4(lc * w.x, lc * w.y, lc * w.z, lc * w.w));
+      st4(Sr + 128 * WPG * i, make_float4(lr * (sr.x + u.x), lr * (sr.y + u.y), lr * (sr.z + u.z), lr * (sr.w + u.w)));
+      st4(Sr + p.s_plane + 128 * WPG * i, make_float4(lc * w.x, lc * w.y, lc * w.z, lc * w.w));
     }
   } else {
     // v_i = z + P_i ;  y[c] = beta_t[c] + sum_i alpha_i[t] v_i[c + i] ;  P_i <- lam_i v_i. A shifted read reaches at most four
     // lanes ahead: by shuffle inside the warp, the warp's last lanes from what the next 128 channels' first lanes left in
     // `edge` (two buffers, filters in turn: one barrier of the group per filter).
-    const int lane = threadIdx.x & 31, half = th >> 5;
+    const int lane = threadIdx.x & 31, wi = th >> 5;
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-      const float4 bt = ld4(bt_p + 256 * i);
+      const float4 bt = ld4(bt_p + 128 * WPG * i);
       v[i] = make_float4(v[i].x + bt.x, v[i].y + bt.y, v[i].z + bt.z, v[i].w + bt.w);
     }
     for (int fi = 0; fi < p.k; ++fi) {
@@ -174,27 +223,27 @@ __device__ __forceinline__ void mix_row(const Params& p, float4 (&v)[NT], const 
       ST* Pf = Sr + (int64_t)fi * p.s_plane;
       float4 nx[NT];
 #pragma unroll
-      for (int i = 0; i < NT; ++i) nx[i] = fi + 1 < p.k ? ld4(Pf + p.s_plane + 256 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int i = 0; i < NT; ++i) nx[i] = fi + 1 < p.k ? ld4(Pf + p.s_plane + 128 * WPG * i) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int i = 0; i < NT; ++i) {
         const float4 w = make_float4(z[i].x + f[i].x, z[i].y + f[i].y, z[i].z + f[i].z, z[i].w + f[i].w);
-        st4(Pf + 256 * i, make_float4(lm * w.x, lm * w.y, lm * w.z, lm * w.w));
+        st4(Pf + 128 * WPG * i, make_float4(lm * w.x, lm * w.y, lm * w.z, lm * w.w));
         f[i] = make_float4(al * w.x, al * w.y, al * w.z, al * w.w);
       }
       if (fi > 0) {
-        float4* e = edge + (fi & 1) * (NT * 8);             // [128-channel vector][4 lanes]
+        float4* e = edge + (fi & 1) * (NT * WPG * 4);          // [128-channel vector][4 lanes]
         if (lane < 4) {
 #pragma unroll
-          for (int i = 0; i < NT; ++i) e[(2 * i + half) * 4 + lane] = f[i];
+          for (int i = 0; i < NT; ++i) e[(WPG * i + wi) * 4 + lane] = f[i];
         }
-        asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
+        asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(WPG * 32) : "memory");
         auto ahead = [&](int i, int delta) {                // the float4 `delta` lanes ahead, 0 <= delta <= 4
           const int src = lane + delta;
           float4 r = make_float4(__shfl_sync(0xffffffffu, f[i].x, src & 31), __shfl_sync(0xffffffffu, f[i].y, src & 31),
                                  __shfl_sync(0xffffffffu, f[i].z, src & 31), __shfl_sync(0xffffffffu, f[i].w, src & 31));
           if (src >= 32) {
-            const int next = 2 * i + half + 1;
-            r = next < 2 * NT ? e[next * 4 + src - 32] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const int next = WPG * i + wi + 1;
+            r = next < WPG * NT ? e[next * 4 + src - 32] : make_float4(0.f, 0.f, 0.f, 0.f);
           }
           return r;
         };
@@ -219,13 +268,14 @@ __device__ __forceinline__ void mix_row(const Params& p, float4 (&v)[NT], const 
   }
 }
 
-template <int NT, typename ST, int MIX>
+// WPG: warps per row; NT: float4s of a row per thread.
+template <int NT, int WPG, typename ST, int MIX>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmW1,
               const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmHs, const __grid_constant__ CUtensorMap tmP,
               const Params p) {
   pdl_trigger();
-  constexpr int d = NT * 256;
+  constexpr int kGroups = tc::kEpiWarps / WPG, kRowThreads = WPG * 32, kStride = kRowThreads * 4, d = NT * kStride;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int n = p.n, w_rows = n >> 1, w_bytes = kStep * w_rows * 128;
@@ -234,7 +284,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   float* prm = reinterpret_cast<float*>(sA + p.a_slots * kABytes);
   float* b1_s = prm + kVecs * d;
   float* red = b1_s + n;
-  uint64_t* fullW = reinterpret_cast<uint64_t*>(red + kGroups * 8);      // used in the leader CTA
+  uint64_t* fullW = reinterpret_cast<uint64_t*>(red + kMaxGroups * 8);      // used in the leader CTA
   uint64_t* emptyW = fullW + kMaxWSlots;
   uint64_t* fullA = emptyW + kMaxWSlots;                                 // used in the leader CTA
   uint64_t* emptyA = fullA + kMaxASlots;
@@ -242,7 +292,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   uint64_t* tempty = tfull + 1;                                          // leader: accumulator drained by both CTAs
   uint64_t* ring = tempty + 1;                                           // the epilogue has left the activation ring
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring + 1);
-  float* hs = red + kGroups * 8 + kBarrierBytes / 4;                     // MIX != kMixed
+  float* hs = red + kMaxGroups * 8 + kBarrierBytes / 4;                  // MIX != kMixed
   float4* edge = reinterpret_cast<float4*>(hs + kMixScalars);            // MIX == kKernel: d bytes per group
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -330,8 +380,9 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
           for (int kb = 0; kb < kbs; kb += kStep) {
             if (!tc::mbar_wait(&emptyA[slot], phase ^ 1u, p.status)) { ok = false; break; }
             const uint32_t full = tc::mapa(tc::smem_u32(&fullA[slot]), 0);
-            tc::mbar_expect_tx_cluster(full, kABytes);
-            tma_load_a(sA + slot * kABytes, map, full, row, kb0 + kb);
+            // (a CTA without rows arrives and loads nothing: its half of the accumulator is not stored)
+            tc::mbar_expect_tx_cluster(full, row < p.R ? (uint32_t)(kStep * p.box * 128) : 0u);
+            if (row < p.R) tma_load_a(sA + slot * kABytes, map, full, row, kb0 + kb);
             if (++slot == p.a_slots) { slot = 0; phase ^= 1u; }
           }
         }
@@ -363,7 +414,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             for (int q = 0; q < kStep; ++q) {               // (descriptor addresses count 16 bytes)
 #pragma unroll
               for (int k = 0; k < tc::BK / 16; ++k)
-                tc::umma_bf16(tmem, da + (uint32_t)(q * tc::kRowsPerCta * 8) + 2u * k, db + (uint32_t)(q * w_rows * 8) + 2u * k, idesc,
+                tc::umma_bf16(tmem, da + (uint32_t)(q * p.box * 8) + 2u * k, db + (uint32_t)(q * w_rows * 8) + 2u * k, idesc,
                               (kb | q | k) != 0 ? 1u : 0u);
             }
             tc::umma_commit_pair(&emptyW[sw]);
@@ -379,12 +430,12 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   } else {
     // ---------------- rows and epilogues (both CTAs) ----------------
     const int wid = threadIdx.x - kEpiWarp0 * 32;                // 0 .. kWorkers - 1
-    const int group = wid >> 6, c0 = (wid & 63) * 4;
+    const int group = wid / kRowThreads, th = wid % kRowThreads, c0 = th * 4;
     const int quad = warp & 3, cgrp = (warp - kEpiWarp0) >> 2;
     const int cols = n >> 2;                                     // accumulator columns per warp: 16, 32 or 64
     pdl_wait();
     const int t_all = p.ctr != nullptr ? p.ctr[kCtrPos] : p.t;
-    float* slot = red + group * 8;
+    float* slot = red + group * (2 * WPG);               // (a second set of sums lies kMaxGroups * 4 floats on)
     int piece = 0;
     bool ok = true;
     for (int l = 0;; ++l) {
@@ -407,15 +458,33 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
       ST* Sr = reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + (int64_t)row * d + c0;
       if (mine) {
         if (!last) {
-          if (MIX == kMixed) sb::head_scalars<d, NT>(p, w, t, wid & 63, a1, a2, lm);
+          if (MIX == kMixed) {            // the multipliers of z before and of the sum after (one of them is 1), and lambda
 #pragma unroll
-          for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + 256 * i);
+            for (int i = 0; i < NT; ++i) {
+              const int g = (c0 + kStride * i) / (d / p.h);
+              const float al = __ldg(w.alpha + (int64_t)g * p.n_ctx + t);
+              const bool is_row = g < (p.h >> 1);
+              a1[i] = is_row ? al : 1.0f;
+              a2[i] = is_row ? 1.0f : al;
+              lm[i] = __ldg(w.lam + g);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + kStride * i);
+          if (p.pos != nullptr) {
+#pragma unroll
+            for (int i = 0; i < NT; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(w.beta + (int64_t)t * d + c0 + kStride * i));
+          }
           if (MIX == kCombined) {
 #pragma unroll
-            for (int i = 0; i < NT; ++i) s1[i] = ld4(Sr + p.s_plane + 256 * i);
+            for (int i = 0; i < NT; ++i) s1[i] = ld4(Sr + p.s_plane + kStride * i);
           }
         }
-        if (l > 0 && (wid & 63) == 0 && ok)       // the down tiles of the row's block
+        if (l > 0) {                      // (this thread's part of x, from the previous layer: not through L1)
+#pragma unroll
+          for (int i = 0; i < NT; ++i) v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c0 + kStride * i));
+        }
+        if (l > 0 && th == 0 && ok)               // the down tiles of the row's block
           ok = count_wait(cnt_dn + row / tc::BM, (uint32_t)l * (uint32_t)(p.cd * p.ks * dn_boxes) * 8u, p.status);
       }
       if (MIX != kMixed && !last) {         // scalar wid of the layer
@@ -435,70 +504,76 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         if (l == 0) {
           int tk = p.tok_in[row];
           if (tk < 0 || tk >= p.V) {
-            if ((wid & 63) == 0) raise_status(p.status, kStatusTokenRange);
+            if (th == 0) raise_status(p.status, kStatusTokenRange);
             tk = tk < 0 ? 0 : p.V - 1;
           }
 #pragma unroll
-          for (int i = 0; i < NT; ++i) v[i] = ldg4(p.E + (int64_t)tk * d + c0 + 256 * i);
+          for (int i = 0; i < NT; ++i) v[i] = ldg4(p.E + (int64_t)tk * d + c0 + kStride * i);
         } else {                          // x + b2 + plane 0 + plane 1 + ... (other CTAs wrote the planes: not through L1)
 #pragma unroll
           for (int i = 0; i < NT; ++i) {
-            v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c0 + 256 * i));
-            const float4 bb = ld4(prm + 5 * d + c0 + 256 * i);
+            const float4 bb = ld4(prm + 5 * d + c0 + kStride * i);
             v[i] = make_float4(v[i].x + bb.x, v[i].y + bb.y, v[i].z + bb.z, v[i].w + bb.w);
           }
-#pragma unroll 2
-          for (int k = 0; k < p.ks; ++k) {
-            const float* q = p.part + (int64_t)k * p.plane + (int64_t)row * d + c0;
+          const float* part = p.part + (int64_t)row * d + c0;
+          auto add = [&](auto planes) {   // all planes' loads in flight
+            constexpr int K = decltype(planes)::value;
+            float4 e[K][NT];
 #pragma unroll
-            for (int i = 0; i < NT; ++i) {
-              const float4 e = __ldcg(reinterpret_cast<const float4*>(q + 256 * i));
-              v[i] = make_float4(v[i].x + e.x, v[i].y + e.y, v[i].z + e.z, v[i].w + e.w);
-            }
-          }
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+              for (int i = 0; i < NT; ++i) e[k][i] = __ldcg(reinterpret_cast<const float4*>(part + k * p.plane + kStride * i));
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+              for (int i = 0; i < NT; ++i) v[i] = make_float4(v[i].x + e[k][i].x, v[i].y + e[k][i].y, v[i].z + e[k][i].z, v[i].w + e[k][i].w);
+          };
+          if (p.ks == 4) add(std::integral_constant<int, 4>());
+          else if (p.ks == 2) add(std::integral_constant<int, 2>());
+          else add(std::integral_constant<int, 1>());
         }
         float mean, rstd;
         if (!last) {
           const float* bt_p = p.pos != nullptr ? w.beta + (int64_t)t * d + c0 : prm + 2 * d + c0;
-          sb::group_stats<d, NT>(v, p.eps, slot, group, mean, rstd);
+          group_stats<NT, WPG>(v, p.eps, slot, group, mean, rstd);
           const float nmr = -mean * rstd;
           if (MIX != kMixed) {
             float4 z[NT];
 #pragma unroll
             for (int i = 0; i < NT; ++i) {
-              const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i);
+              const float4 g = ld4(prm + c0 + kStride * i), bb = ld4(prm + d + c0 + kStride * i);
               z[i] = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
                                  fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
             }
-            mix_row<NT, MIX>(p, v, z, s, s1, bt_p, Sr, hs, edge + group * (d / 16), group, wid & 63);
+            mix_row<NT, WPG, MIX>(p, v, z, s, s1, bt_p, Sr, hs, edge + group * (d / 16), group, th);
 #pragma unroll
-            for (int i = 0; i < NT; ++i) st4(p.x + (int64_t)row * d + c0 + 256 * i, v[i]);
+            for (int i = 0; i < NT; ++i) st4(p.x + (int64_t)row * d + c0 + kStride * i, v[i]);
           }
 #pragma unroll
           for (int i = 0; MIX == kMixed && i < NT; ++i) {
-            const float4 g = ld4(prm + c0 + 256 * i), bb = ld4(prm + d + c0 + 256 * i), bt = ld4(bt_p + 256 * i);
+            const float4 g = ld4(prm + c0 + kStride * i), bb = ld4(prm + d + c0 + kStride * i), bt = ld4(bt_p + kStride * i);
             const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
                                          fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
             // row-repeat head, Eq. 2: y = (a z + S) + b ; S' = l (S + a z).  column-repeat head, Eq. 3: y = a (z + S) + b ; S' = l (z + S)
             const float4 u = make_float4(fmaf(a1[i], z.x, s[i].x), fmaf(a1[i], z.y, s[i].y), fmaf(a1[i], z.z, s[i].z), fmaf(a1[i], z.w, s[i].w));
-            st4(Sr + 256 * i, make_float4(lm[i] * u.x, lm[i] * u.y, lm[i] * u.z, lm[i] * u.w));
+            st4(Sr + kStride * i, make_float4(lm[i] * u.x, lm[i] * u.y, lm[i] * u.z, lm[i] * u.w));
             v[i] = make_float4(v[i].x + fmaf(a2[i], u.x, bt.x), v[i].y + fmaf(a2[i], u.y, bt.y), v[i].z + fmaf(a2[i], u.z, bt.z),
                                v[i].w + fmaf(a2[i], u.w, bt.w));
-            st4(p.x + (int64_t)row * d + c0 + 256 * i, v[i]);
+            st4(p.x + (int64_t)row * d + c0 + kStride * i, v[i]);
           }
         }
-        sb::group_stats<d, NT>(v, p.eps, slot + 4, group, mean, rstd);
+        group_stats<NT, WPG>(v, p.eps, slot + kMaxGroups * 4, group, mean, rstd);
         const float nmr2 = -mean * rstd;
 #pragma unroll
         for (int i = 0; i < NT; ++i) {
-          const float4 g = ld4(prm + 3 * d + c0 + 256 * i), bb = ld4(prm + 4 * d + c0 + 256 * i);
-          st4(p.a + (int64_t)row * d + c0 + 256 * i,
+          const float4 g = ld4(prm + 3 * d + c0 + kStride * i), bb = ld4(prm + 4 * d + c0 + kStride * i);
+          st4(p.a + (int64_t)row * d + c0 + kStride * i,
               make_float4(fmaf(fmaf(v[i].x, rstd, nmr2), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr2), g.y, bb.y),
                           fmaf(fmaf(v[i].z, rstd, nmr2), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr2), g.w, bb.w)));
         }
         tc::fence_async_global();         // read by bulk tensor copies of other CTAs
-        asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
-        if ((wid & 63) == 0) red_release_add(cnt_rows + row / tc::BM, 1u);
+        asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kRowThreads) : "memory");
+        if (th == 0) red_release_add(cnt_rows + row / tc::BM, 1u);
       }
       if (last) break;
 
