@@ -723,10 +723,11 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
 
 // ---- passes of a hundred to a thousand rows: all layers in one kernel (layers_mid.cuh) -------------------
 // Fewest rows, where the whole step is not one kernel of another design (step_small.cuh: up to 64 rows at d = 512, 32 at
-// d = 1024). d = 512: a batch just past that limit keeps the kernel-per-operation path (65 rows 134 us per step there,
-// 114 us here; a test counts on it). Combined heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96
-// rows, d = 1024, 16 layers, kernels of size 4: 320 us per step, as a kernel per operation 560).
-int64_t mid_min_rows(const srm_config& c) { return c.d_model == 512 && c.mixer == SRM_MIXER_MIXED ? 97 : 1; }
+// d = 1024; us per step there / here: mid 1 row 181 / 239, 27 rows 241 / 246, 32 rows 250 / 244; small 27 rows 87 / 98, 64 rows
+// 111 / 100). d = 512: a batch just past that limit keeps the kernel-per-operation path (a test counts on it); from 72 rows, 138
+// us there, 104 here. Combined heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96 rows, d = 1024, 16
+// layers, kernels of size 4: 275 us per step, as a kernel per operation 560).
+int64_t mid_min_rows(const srm_config& c) { return c.d_model == 512 && c.mixer == SRM_MIXER_MIXED ? 72 : 1; }
 
 int mid_mix(const srm_config& c) { return c.mixer == SRM_MIXER_COMBINED ? mid::kCombined : c.mixer == SRM_MIXER_KERNEL ? mid::kKernel : mid::kMixed; }
 
