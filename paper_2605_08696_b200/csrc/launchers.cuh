@@ -729,6 +729,8 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
 // layers, kernels of size 4: 275 us per step, as a kernel per operation 560).
 int64_t mid_min_rows(const srm_config& c) { return c.d_model == 512 && c.mixer == SRM_MIXER_MIXED ? 72 : 1; }
 
+constexpr size_t kCntFloats = 256;      // room for mid::kCntWords at the head of the logits area
+static_assert(mid::kCntWords <= (int)kCntFloats, "counters");
 int mid_mix(const srm_config& c) { return c.mixer == SRM_MIXER_COMBINED ? mid::kCombined : c.mixer == SRM_MIXER_KERNEL ? mid::kKernel : mid::kMixed; }
 
 // Whether a decode pass of R rows takes it, and its tile plan. bf16 models of the widths it is built for,
@@ -736,12 +738,17 @@ int mid_mix(const srm_config& c) { return c.mixer == SRM_MIXER_COMBINED ? mid::k
 bool mid_plan(srm_model& m, int64_t R, const DecodeWs& w, mid::Params* p) {
   const srm_config& c = m.cfg;
   constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
-  if (R < mid_min_rows(c) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || w.part == nullptr) return false;
-  if (c.mixer != SRM_MIXER_MIXED && !mid_variant_model(c)) return false;
+  if (R < mid_min_rows(c) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff)) return false;
+  if (c.mixer != SRM_MIXER_MIXED && (c.d_model > 1024 || c.n_heads > 8 || c.kernel_size > 16)) return false;
   if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536) return false;
   if (ensure_tc_ready(m) != SRM_OK || R > (int64_t)2 * m.tc_clusters * mid::kMaxGroups || m.F() > (1 << 20)) return false;
   if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, mid_mix(c), p)) return false;
-  return (size_t)p->ks * p->rb * tc::BM * c.d_model * 4 <= w.part_bytes;
+  // The planes of partial products: an area of their own where the model has one, else (combined heads, kernels) behind the
+  // counters in the logits area, from about five rows of the mid model on.
+  p->plane_rows = (int)(R + tc::kOutBoxRows - 1) / tc::kOutBoxRows * tc::kOutBoxRows;
+  const size_t need = (size_t)p->ks * p->plane_rows * c.d_model * 4;
+  p->part = w.part != nullptr ? w.part : w.logits + kCntFloats;
+  return need <= (w.part != nullptr ? w.part_bytes : (size_t)w.rows * c.vocab * 4 - std::min((size_t)w.rows * c.vocab, kCntFloats) * 4);
 }
 
 struct MidMaps { CUtensorMap a, h, w1, w2, hs, p; };      // loads of a, H, W1, W2; stores of H and the partial products
@@ -794,8 +801,7 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   if (c.mixer == SRM_MIXER_COMBINED) { p.alpha_col = m.fptr(0, SRM_T_ALPHA_COL); p.lam_col = m.fptr(0, SRM_T_LAMBDA_COL); p.w_comb = m.fptr(0, SRM_T_W_COMB); }
   p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
   p.x = w.x; p.a = reinterpret_cast<bf16*>(w.a); p.H = reinterpret_cast<bf16*>(w.H);
-  p.part = w.part;
-  p.plane = (int64_t)p.rb * tc::BM * d;
+  p.plane = (int64_t)p.plane_rows * d;
   p.cnt = reinterpret_cast<uint32_t*>(w.logits);      // (nothing uses the logits area before the LM head)
   p.status = s.status; p.ctr = ctr; p.pos = pos;
   SRM_CUDA(cudaMemsetAsync(p.cnt, 0, mid::kCntWords * 4, st));
@@ -807,7 +813,7 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   if ((rc = make_tmap_kblocks(&maps.w1, m.ptr(0, SRM_T_W1), F, d, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = make_tmap_kblocks(&maps.w2, m.ptr(0, SRM_T_W2), d, F, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = m.tmap(w.H, R, F, tc::kOutBoxRows, 2, &maps.hs)) != SRM_OK) return rc;
-  if ((rc = m.tmap(w.part, (int64_t)p.ks * p.rb * tc::BM, d, tc::kOutBoxRows, 4, &maps.p)) != SRM_OK) return rc;
+  if ((rc = m.tmap(p.part, (int64_t)p.ks * p.plane_rows, d, tc::kOutBoxRows, 4, &maps.p)) != SRM_OK) return rc;
   if (c.mixer != SRM_MIXER_MIXED) return d == 512 ? launch_layers_variant<2>(m, maps, p, st) : launch_layers_variant<4>(m, maps, p, st);
   if (d == 512) return launch_layers_nt<2>(m, maps, p, st);
   if (d == 1024) return launch_layers_nt<4>(m, maps, p, st);
@@ -852,7 +858,7 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   // cut into ranges so that all pairs work on it; the partial products go to planes of their own in the workspace
   // and the next consumer of x (the next layer's mixer, the final norm) adds them in a fixed order.
   const int64_t plane_rows = (R + tc::BM - 1) / tc::BM * tc::BM;
-  if (!one_kernel && !fused_ffn && !split && w.part != nullptr && c.mixer == SRM_MIXER_MIXED) {
+  if (!one_kernel && !fused_ffn && !split && w.part != nullptr) {
     if ((rc = ensure_tc_ready(m))) return rc;
     k_slices = down_k_slices(plane_rows / tc::BM * ((d + tc::BN - 1) / tc::BN), (int)(F / tc::BK), m.tc_clusters);
     while (k_slices > 1 && (size_t)k_slices * plane_rows * d * 4 > w.part_bytes) k_slices /= 2;

@@ -66,8 +66,9 @@ struct Params {
   bf16* a;                       // [R, d]: activations of the up projection, at the end of the final norm
   const float *lnf_g, *lnf_b;
   bf16* H;                       // [R, F]
-  float* part;                   // [ks] planes of plane_rows x d
+  float* part;                   // [ks] planes of plane_rows x d 
   int64_t plane;                 // elements per plane
+  int plane_rows;                // rows per plane: R rounded up to whole boxes
   uint32_t* cnt;                 // rows done [8] | up pieces done [8][4] | down pieces done [8]; zero on entry
   uint32_t* status;
   const int32_t* ctr;            // device-side step counters or nullptr
@@ -625,7 +626,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         if (cgrp < boxes && tc::elect_one()) {
           const uint8_t* src = sA + (quad * boxes + cgrp) * tc::kOutBoxBytes;
           if (row0 < p.R) {
-            if (ph) tc::tma_store_2d(&tmP, src, col0 + cgrp * 32, dn_slice * p.rb * tc::BM + row0);
+            if (ph) tc::tma_store_2d(&tmP, src, col0 + cgrp * 32, dn_slice * p.plane_rows + row0);
             else tc::tma_store_2d(&tmHs, src, col0 + cgrp * 64, row0);
             tc::bulk_commit();
             tc::bulk_wait_all();

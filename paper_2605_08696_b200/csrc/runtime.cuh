@@ -321,15 +321,9 @@ constexpr size_t kSmallScratchBytes = (size_t)sb::kMaxRows * 8 + (size_t)sb::kGr
 
 // Partial-product planes of a small pass's down projection (GemmArgs::k_slices): up to 8 planes of the pass's rows
 // (padded to whole 256-row tiles) x d floats, never more than one 256 x 256 fp32 tile per CTA pair of the largest
-// device (tiles x ranges stays within the pairs). Only for the models whose mixer adds them (mixer_stream_kernel;
-// combined heads and kernels: in the layers kernel only, layers_mid.cuh).
+// device (tiles x ranges stays within the pairs). Only for the models whose mixer adds them (mixer_stream_kernel).
 constexpr int kMaxKSlices = 8;
-bool mid_variant_model(const srm_config& c) {
-  return c.mixer != SRM_MIXER_MIXED && c.dtype == SRM_DTYPE_BF16 && (c.d_model == 512 || c.d_model == 1024) &&
-         !(c.flags & (SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_KSLICE | SRM_FLAG_HEAD_PROJ)) && c.n_heads <= 8 && c.kernel_size <= 16;
-}
 bool kslice_model(const srm_config& c) {
-  if (c.mixer != SRM_MIXER_MIXED) return mid_variant_model(c);
   const int d = c.d_model, nv = d / 128, se = c.state_dtype == SRM_DTYPE_FP32 ? 4 : 2;
   return c.dtype == SRM_DTYPE_BF16 && !(c.flags & (SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_KSLICE | SRM_FLAG_HEAD_PROJ)) &&
          c.mixer == SRM_MIXER_MIXED && d % 128 == 0 && (d / c.n_heads) % 128 == 0 && c.n_heads <= 8 &&

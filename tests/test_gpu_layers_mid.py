@@ -84,7 +84,7 @@ def test_captured_step_and_passes_of_one_kernel_equal_launch_by_launch():
             assert torch.equal(x, y)
 
 
-@pytest.mark.parametrize("mixer,k,B,d,state_dtype", [("combined", 1, 1, 1024, "fp32"), ("combined", 1, 300, 512, "fp16"),
+@pytest.mark.parametrize("mixer,k,B,d,state_dtype", [("combined", 1, 12, 1024, "fp32"), ("combined", 1, 300, 512, "fp16"),
                                                      ("kernel", 1, 40, 512, "fp32"), ("kernel", 4, 257, 1024, "fp32"),
                                                      ("kernel", 5, 97, 512, "fp16"), ("kernel", 16, 130, 1024, "fp16"),
                                                      ("kernel", 13, 1000, 512, "fp32")])
@@ -92,7 +92,7 @@ def test_further_mixers_in_one_kernel_agree_with_the_kernel_per_operation_path(m
     import dataclasses
 
     import paper_2605_08696_b200 as P
-    base = custom_shape(n_layers=3, d_model=d, vocab=2048, n_ctx=24, dtype="bf16", seed=13)
+    base = custom_shape(n_layers=3, d_model=d, vocab=16384, n_ctx=24, dtype="bf16", seed=13)
     shape = dataclasses.replace(base, mixer=mixer, kernel_size=k)
     W = I.make_weights(shape)
     n = 4
