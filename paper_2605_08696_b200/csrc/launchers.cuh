@@ -804,7 +804,10 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   p.plane = (int64_t)p.plane_rows * d;
   p.cnt = reinterpret_cast<uint32_t*>(w.logits);      // (nothing uses the logits area before the LM head)
   p.status = s.status; p.ctr = ctr; p.pos = pos;
-  SRM_CUDA(cudaMemsetAsync(p.cnt, 0, mid::kCntWords * 4, st));
+  // (cleared by a kernel: the layers kernel then sets itself up and starts on its weights while the kernels before it end,
+  // which it does not do behind a memset; 3 us per step)
+  ++g_kernel_launches;
+  SRM_CUDA(launch_kernel(mid::zero_counters_kernel, dim3(1), dim3(64), 0, st, p.cnt));
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
   MidMaps maps;
   int rc;

@@ -85,6 +85,12 @@ constexpr int kVecs = 6;
 constexpr int kMixed = 0, kCombined = 1, kKernel = 2;
 constexpr int kMixScalars = 64;      // of a layer at the pass's position: combined 6 h <= 48 floats, kernel 2 k <= 32
 constexpr int kCntWords = kMaxRowBlocks * (2 + kMaxKSlices);
+__global__ void __launch_bounds__(64) zero_counters_kernel(uint32_t* __restrict__ cnt) {
+  pdl_trigger();
+  pdl_wait();
+  if (threadIdx.x < kCntWords) cnt[threadIdx.x] = 0;
+}
+static_assert(kCntWords <= 64, "one thread per counter");
 
 // Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers | for the
 // further mixers their scalars and, for kernels, the channels a warp's last lanes read of the next warp.

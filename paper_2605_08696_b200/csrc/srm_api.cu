@@ -256,6 +256,21 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
       ++g_kernel_launches;
       SRM_CUDA(launch_kernel(pack_rows_kernel, dim3(1), dim3(1024), 0, st, d_len + p0, row_start, np, (int)n));
     }
+    // The feed-forward block over the rows of the pass: in slabs of kPrefillFfnRows rows, each as ONE kernel
+    // (ffn_fused.cuh: a slab's hidden activations are consumed from L2 as they are
+    // produced instead of crossing HBM twice), where the model's shape allows and the slab counters fit in the
+    // logits area (free until the LM head); else, and for a short last slab, up projection then down projection.
+    // Counters of all layers are cleared at once where they fit: behind a memset a kernel cannot start early (4 us per layer).
+    const int64_t slab_rows = rows < kPrefillFfnRows ? rows : kPrefillFfnRows;
+    const size_t slab_ready = ffn_ready_bytes(slab_rows, F), ready_room = logits_bytes - (packed ? start_bytes : 0);
+    const size_t ready_layer = (size_t)((rows + slab_rows - 1) / slab_rows) * slab_ready;
+    bool slabs = !(c.flags & SRM_FLAG_NO_FUSED_FFN) && ffn_fused_shape_ok(*m, slab_rows) && ready_layer <= ready_room;
+    if (slabs) {
+      if ((rc = ensure_tc_ready(*m))) return rc;
+      slabs = ffn_fused_worthwhile(*m, slab_rows);
+    }
+    const bool ready_once = ready_layer * c.n_layers <= ready_room;
+    if (slabs && ready_once) SRM_CUDA(cudaMemsetAsync(w.logits, 0, ready_layer * c.n_layers, st));
     for (int l = 0; l < c.n_layers; ++l) {
       uint8_t* Sl = replicas > 1 ? stage + (size_t)l * planes * np * row_bytes
                                  : static_cast<uint8_t*>(s->layer_ptr(l)) + (size_t)b0 * row_bytes;
@@ -281,26 +296,13 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
         if ((rc = launch_prefill_mixer(*m, l, np, n, l == 0 ? d_tokens + p0 * n : nullptr, w.x, Sl, w.a, s->status, st,
                                        d_len ? d_len + p0 : nullptr, chunked ? &cs : nullptr, row_start))) return rc;
       }
-      // The feed-forward block over the rows of the pass: in slabs of kPrefillFfnRows rows, each as ONE kernel
-      // (ffn_fused.cuh: a slab's hidden activations are consumed from L2 as they are
-      // produced instead of crossing HBM twice), where the model's shape allows and the slab counters fit in the
-      // logits area (free until the LM head); else, and for a short last slab, up projection then down projection.
-      const int64_t slab_rows = rows < kPrefillFfnRows ? rows : kPrefillFfnRows;
-      const size_t slab_ready = ffn_ready_bytes(slab_rows, F);
-      const int64_t n_slabs = (rows + slab_rows - 1) / slab_rows;
-      bool slabs = !(c.flags & SRM_FLAG_NO_FUSED_FFN) && ffn_fused_shape_ok(*m, slab_rows) &&
-                   (size_t)n_slabs * slab_ready <= logits_bytes - (packed ? start_bytes : 0);
-      if (slabs) {
-        if ((rc = ensure_tc_ready(*m))) return rc;
-        slabs = ffn_fused_worthwhile(*m, slab_rows);
-      }
-      if (slabs) SRM_CUDA(cudaMemsetAsync(w.logits, 0, (size_t)n_slabs * slab_ready, st));
+      if (slabs && !ready_once) SRM_CUDA(cudaMemsetAsync(w.logits, 0, ready_layer, st));
       for (int64_t r0 = 0; slabs && r0 < rows; r0 += slab_rows) {
         const int64_t nr = rows - r0 < slab_rows ? rows - r0 : slab_rows;
         uint8_t* a_s = static_cast<uint8_t*>(w.a) + (size_t)r0 * d * m->act_bytes();
         uint8_t* H_s = static_cast<uint8_t*>(w.H) + (size_t)r0 * F * m->act_bytes();
         float* x_s = w.x + (size_t)r0 * d;
-        int32_t* ready = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(w.logits) + (size_t)(r0 / slab_rows) * slab_ready);
+        int32_t* ready = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(w.logits) + (ready_once ? l * ready_layer : 0) + (size_t)(r0 / slab_rows) * slab_ready);
         rc = ffn_fused_worthwhile(*m, nr) ? launch_ffn_fused(*m, l, nr, a_s, H_s, x_s, ready, s->status, st, m_limit, r0)
                                          : SRM_ERR_UNSUPPORTED;
         if (rc == SRM_ERR_UNSUPPORTED) {
