@@ -521,14 +521,22 @@ topk_merge_kernel(const unsigned long long* __restrict__ lists, const uint32_t* 
 
 // Cache rows of `replicas` consecutive samples = the row of their prompt:
 // dst[(p0 + p) * replicas + j, :] = src[p, :] for p < np, j < replicas (16-byte vectors; one layer).
-__global__ void __launch_bounds__(256)
-broadcast_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int64_t np, int64_t replicas, int64_t vec_per_row) {
+// Bound by its stores. A block: 128 vectors of one prompt's row to 32 replicas; every vector is read once, and the indices
+// cost a division per block (three 64-bit divisions per vector made it instruction-bound: 16 rows of 6 KB to 1024 replicas
+// each, 100 MB: the launch took 13 us longer).
+constexpr int kBroadcastThreads = 128, kBroadcastReplicas = 32;
+__global__ void __launch_bounds__(kBroadcastThreads)
+broadcast_rows_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int replicas, int vec_per_row, unsigned chunks, unsigned groups) {
   pdl_trigger();
   pdl_wait();
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (i >= np * replicas * vec_per_row) return;
-  const int64_t row = i / vec_per_row, v = i % vec_per_row;
-  dst[i] = __ldg(src + (row / replicas) * vec_per_row + v);
+  const unsigned q = blockIdx.x / chunks, p = q / groups;
+  const int v = (int)(blockIdx.x - q * chunks) * kBroadcastThreads + threadIdx.x, j0 = (int)(q - p * groups) * kBroadcastReplicas;
+  if (v >= vec_per_row) return;
+  const uint4 x = __ldg(src + (int64_t)p * vec_per_row + v);
+  uint4* out = dst + ((int64_t)p * replicas + j0) * vec_per_row + v;
+  const int n = min(kBroadcastReplicas, replicas - j0);
+#pragma unroll 8
+  for (int j = 0; j < n; ++j) __stcs(out + (int64_t)j * vec_per_row, x);      // (more than L2 holds, and not read before the first step)
 }
 
 // Per-sample positions after a prefill of prompts of different lengths: the lengths as the prefill used them

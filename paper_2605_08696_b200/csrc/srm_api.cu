@@ -317,11 +317,13 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
       }
       for (int pl = 0; replicas > 1 && pl < planes; ++pl) {
         LaunchScope scope(*m, SRM_KERNEL_PREFILL_MIXER, st);
-        const int64_t vpr = (int64_t)row_bytes / 16, total = nb * vpr;
+        const int64_t vpr = (int64_t)row_bytes / 16, chunks = (vpr + kBroadcastThreads - 1) / kBroadcastThreads;
+        const int64_t groups = (replicas + kBroadcastReplicas - 1) / kBroadcastReplicas;
         const uint8_t* src = Sl + (size_t)pl * np * row_bytes;
         uint8_t* dst = static_cast<uint8_t*>(s->layer_ptr(l)) + ((size_t)pl * s->B + (size_t)b0) * row_bytes;
-        SRM_CUDA(launch_kernel(broadcast_rows_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st,
-                               reinterpret_cast<const uint4*>(src), reinterpret_cast<uint4*>(dst), np, replicas, vpr));
+        SRM_CUDA(launch_kernel(broadcast_rows_kernel, dim3((unsigned)(np * groups * chunks)), dim3(kBroadcastThreads), 0, st,
+                               reinterpret_cast<const uint4*>(src), reinterpret_cast<uint4*>(dst), (int)replicas, (int)vpr,
+                               (unsigned)chunks, (unsigned)groups));
       }
     }
     // LM head on the last prompt position only; selection per state row
