@@ -264,7 +264,11 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
     const int64_t slab_rows = rows < kPrefillFfnRows ? rows : kPrefillFfnRows;
     const size_t slab_ready = ffn_ready_bytes(slab_rows, F), ready_room = logits_bytes - (packed ? start_bytes : 0);
     const size_t ready_layer = (size_t)((rows + slab_rows - 1) / slab_rows) * slab_ready;
-    bool slabs = !(c.flags & SRM_FLAG_NO_FUSED_FFN) && ffn_fused_shape_ok(*m, slab_rows) && ready_layer <= ready_room;
+    // (Packed prompts in one slab: its work lists, made for all n rows of every prompt, would be cut off unevenly where the rows
+    // end; the two launches share out the tiles there are: mid, 45 prompts of up to
+    // 301, 7209 rows of 13545, 122 -> 105 us per layer; 12 prompts of up to 480, 3531 rows of 5760, equal.)
+    bool slabs = !(c.flags & SRM_FLAG_NO_FUSED_FFN) && ffn_fused_shape_ok(*m, slab_rows) && ready_layer <= ready_room &&
+                 !(packed && rows <= slab_rows);
     if (slabs) {
       if ((rc = ensure_tc_ready(*m))) return rc;
       slabs = ffn_fused_worthwhile(*m, slab_rows);
