@@ -15,10 +15,11 @@
 // and a block publishes before it waits, so the waits end whatever the number of resident blocks; they are bounded
 // all the same (status bit).
 //
-// What bounds it: with few prompts the chain load -> statistics -> E -> flags -> rows of one chunk (24 us per launch
-// for one prompt of 777 positions at d = 1024, where one CTA walking the prompt took 2061 us; 34 -> 0.91 ms for the
-// whole prefill of the mid model), with many the latency of its loads (131072 rows: 383 us, 3.5 TB/s of the 10 bytes
-// per element it moves). T = 16: the rows of a chunk (64 KB at d = 1024) leave room for three CTAs per SM.
+// What bounds it: with few prompts the chain load -> statistics -> E -> flags -> rows of one chunk (about 11 us per launch
+// for one prompt of 777 positions at d = 1024, where one CTA walking the prompt took 2061 us; 33.4 -> 0.74 ms for the
+// whole prefill of the mid model; 16.4 us while the second pass waited for beta and LN2 for its parameters), with many the
+// latency of its loads (131072 rows: 383 us, 3.5 TB/s of the 10 bytes per element it moves). T = 16: the rows of a chunk
+// (64 KB at d = 1024) and LN2's parameters leave room for three CTAs per SM.
 // Needs d = 128 NV (a thread per four channels, a warp per 128).
 #pragma once
 

@@ -9,8 +9,9 @@
 // therefore holds z = LN1(x), and takes x for the residual from global memory (L2: the same CTA has just read it).
 // KM: compiled bound of k (filters k .. KM - 1 have zero weights); 0: combined heads.
 //
-// What bounds it: the latency of a chunk's chain of phases. mid, k = 4, 96 prompts of 120 positions: 62 us per layer;
-// with one launch per position 120 launches of 8 to 9 us (prefill and four tokens: 22.3 -> 6.4 ms).
+// What bounds it: the latency of a chunk's chain of phases. mid, k = 4, 96 prompts of 120 positions: 57 us per layer
+// (62 while beta and the norms' parameters were fetched where they are used); with one launch per position 120 launches of 8
+// to 9 us (prefill and four tokens: 22.3 -> 6.4 ms).
 #pragma once
 
 #include "mixer_model_variants.cuh"   // VariantParams

@@ -7,7 +7,7 @@
 // kernel of 128 CTAs, 32 clusters of four (the largest clusters that fit on that many SMs: 33 of four, 15 of eight). Two grid-wide barriers per layer remain, after the up projection (a
 // down slab reads all of its part of H) and after the down projection (a row needs all of x):
 //   - row phase: every cluster computes every row (embedding or x, LN1, cache update, residual, LN2), rank r the rows
-//     r, r + 4, ..., one warp per row, and sends the activation row to the shared memory of its four CTAs, so the
+//     r, r + 4, ..., two warps per row, and sends the activation row to the shared memory of its four CTAs, so the
 //     rows need no grid barrier of their own; up to kAloneRows rows every CTA computes all of them for itself. The new
 //     cache row is kept in shared memory and written by one CTA of the grid after the next grid barrier, when nobody
 //     reads the old one any more;
