@@ -69,10 +69,13 @@ enum {
   SRM_FLAG_NO_FUSED_TOPK = 32,       /* top-k selection always from fp32 logits written to the workspace (default: the
                                         candidates are collected inside the LM-head epilogue and no logits are written
                                         when the caller does not ask for them); for comparison and measurement */
-  SRM_FLAG_NO_SMALL_BATCH = 64,      /* batches of at most 64 samples also run one kernel per operation (default: such a
-                                        batch, on a bf16 mixed-head model of at most 1024 channels, runs its whole
-                                        decode step in ONE cooperative kernel that streams the weights with all SMs;
-                                        results agree with the other path to rounding, not bit for bit) */
+  SRM_FLAG_NO_SMALL_BATCH = 64,      /* small and mid passes also run one kernel per operation (default: a bf16 mixed-head
+                                        model of at most 1024 channels, a multiple of 256, runs the whole decode step of
+                                        as many samples as fit beside a layer's weights in shared memory, 64 at d = 512,
+                                        32 at d = 1024, in ONE cooperative kernel; larger passes of d 512 (72 to 1024
+                                        samples), 1024 (to 512) and 1536 (to 256), and those of the further mixers at d
+                                        512 and 1024, run all their layers in one kernel; results agree with the
+                                        kernel-per-operation path to rounding, not bit for bit) */
   SRM_FLAG_NO_TAIL_SPLIT = 128,      /* tensor-core projections process every 256 x 256 tile whole (default: the tiles of a
                                         last, partly filled round run as two 256 x 128 pieces each, which keeps nearly all
                                         CTA pairs busy to the end); for comparison and measurement */
@@ -196,10 +199,10 @@ int32_t srm_cache_planes(const srm_config* cfg);
  * the given workspace requires. Decode never uses more than 12288 rows of it in one pass: a larger
  * batch runs as equal passes of at most 10240 rows (whole 256-row tiles), which keeps a layer's
  * activations in L2 between its kernels; results do not depend on the split, with two exceptions in the last bits:
- * a batch of at most 64 samples whose workspace holds it in one pass takes the single-kernel step (see
- * SRM_FLAG_NO_SMALL_BATCH), whose sums run in another order than those of the kernel-per-operation path; and a pass
- * small enough for its down projection to be cut along K (see SRM_FLAG_NO_KSLICE) adds that projection's partial
- * products in another order than a large pass, whatever batch it is part of. */
+ * a batch whose workspace holds it in one pass of the single-kernel step, and a pass whose layers run in one kernel
+ * (see SRM_FLAG_NO_SMALL_BATCH), add in another order than the kernel-per-operation path; and a pass small enough
+ * for its down projection to be cut along K (see SRM_FLAG_NO_KSLICE) adds that projection's partial products in
+ * another order than a large pass, whatever batch it is part of. */
 size_t srm_workspace_bytes(const srm_config* cfg, int64_t B_chunk, int32_t n_prefill_max);
 /* Workspace bytes with which srm_prefill (and its variants) processes `samples` prompts of up to n tokens in one
  * pass [Eq. 1, Eq. 3: the sequence-parallel form over all positions of a pass]. A workspace for both calls is the
@@ -330,7 +333,7 @@ int srm_decode_step_host(srm_model* m, srm_state* s, const int32_t* h_tok_in,
  * Same arguments and results as srm_decode_step, minus the workspace. Differences:
  *   - the whole batch must fit in one pass: if srm_workspace_bytes(cfg, B, 0) exceeds
  *     SRM_STATIC_SCRATCH_BYTES the call enqueues nothing and returns SRM_ERR_STATIC_SCRATCH
- *     (e.g. the mid model, 142 KB per row next to 10.6 MB of fixed scratch, takes up to about 160 rows; the tiny
+ *     (e.g. the mid model, 142 KB per row next to 8.4 MB of fixed scratch, takes up to about 170 rows; the tiny
  *     model about 13 000);
  *   - the device that is current must be the model's device (else SRM_ERR_INVALID_ARG);
  *   - the first call on each device looks up the array's device address (cudaGetSymbolAddress).
@@ -476,7 +479,7 @@ enum srm_kernel_class {
   SRM_KERNEL_SELECT,             /* token selection                                            */
   SRM_KERNEL_PREFILL_MIXER,      /* sequence-parallel token mixing                             */
   SRM_KERNEL_GEMM_PROJ,          /* head projections W_in, W_out (SRM_FLAG_HEAD_PROJ)          */
-  SRM_KERNEL_STEP_SMALL,         /* the single-kernel decode step of a small batch             */
+  SRM_KERNEL_STEP_SMALL,         /* decode of a small batch as one kernel; all layers of a mid pass as one */
   SRM_KERNEL_FFN,                /* feed-forward block as one kernel (up and down projection)  */
   SRM_KERNEL_CLASS_COUNT
 };
