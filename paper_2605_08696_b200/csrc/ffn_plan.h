@@ -84,6 +84,7 @@ inline double ffn_simulate(const FfnShape& s, const FfnPlan& P, const FfnCost& c
   std::vector<double> ready((size_t)s.Rb * s.Cu, -1.0);      // time H tile (rb, hc) becomes visible; -1: not known yet
   std::vector<int> seen_up((size_t)s.Rb * s.Cu, 0), seen_dn((size_t)s.Rb * s.Cd, 0);
   std::vector<double> pend((size_t)s.Rb * s.Cu, 0.0);        // end of the first half of a tile computed in halves
+  std::vector<int> known(s.Rb, 0);                           // H tiles of a row block whose time is known
   std::vector<int> pos(n, 0);
   std::vector<double> t(n, 0.0);
   int left = 0, halves = 0;
@@ -109,13 +110,13 @@ inline double ffn_simulate(const FfnShape& s, const FfnPlan& P, const FfnCost& c
           if (seen & bits) return -1.0;
           seen |= bits;
           t[p] += (ffn_item_half(it) ? kFfnHalfCost : 1.0) * s.ku * c.up_kb + c.up_tile;
-          if (seen == 3) ready[(size_t)rb * s.Cu + cb] = std::max(pend[(size_t)rb * s.Cu + cb], t[p]) + c.ready_lag;
-          else pend[(size_t)rb * s.Cu + cb] = t[p];
+          if (seen == 3) {
+            ready[(size_t)rb * s.Cu + cb] = std::max(pend[(size_t)rb * s.Cu + cb], t[p]) + c.ready_lag;
+            ++known[rb];
+          } else pend[(size_t)rb * s.Cu + cb] = t[p];
         } else {
           if (cb >= s.Cd) return -1.0;
-          bool known = true;
-          for (int hc = 0; hc < s.Cu; ++hc) known = known && ready[(size_t)rb * s.Cu + hc] >= 0.0;
-          if (!known) break;                                   // this pair waits for tiles no pair has reached yet
+          if (known[rb] < s.Cu) break;                         // this pair waits for tiles no pair has reached yet
           if (seen_dn[(size_t)rb * s.Cd + cb]++) return -1.0;
           double u = t[p] + c.dn_tile;
           for (int hc = 0; hc < s.Cu; ++hc) u = std::max(u, ready[(size_t)rb * s.Cu + hc]) + kFfnKbPerHTile * c.dn_kb;
@@ -139,124 +140,148 @@ inline double ffn_ideal(const FfnShape& s, int pairs, const FfnCost& c = FfnCost
   return std::max(((double)s.Rb * s.Cu * up + (double)s.Rb * s.Cd * dn) / pairs, up + kFfnKbPerHTile * c.dn_kb + dn);
 }
 
-// The plan in which the last `n_half` up tiles placed (the first of the forward lists) go out as halves.
-inline bool ffn_make_plan_halves(const FfnShape& s, int pairs, int n_half, FfnPlan* out, const FfnCost& c) {
-  if (!ffn_shape_ok(s, pairs)) return false;
-  const double up_cost = s.ku * c.up_kb + c.up_tile, dn_cost = s.kd * c.dn_kb + c.dn_tile;
-  const double h_tile = kFfnKbPerHTile * c.dn_kb;             // time a down tile spends on one column tile of H
-  const double rb_bytes = 256.0 * 256.0 * s.Cu * 2.0;
-  const int open_max = std::max(2, (int)(c.h_budget_bytes / rb_bytes));
-
-  // pairs by the (reversed) time they are free, the lowest index among equals first; the top is the pair that takes the next item
-  std::vector<std::pair<double, int>> heap;
-  for (int p = 0; p < pairs; ++p) heap.emplace_back(0.0, p);  // (equal times, ascending index: already a heap)
-  const auto later = std::greater<std::pair<double, int>>();
-  auto give = [&](double until) {                             // the top pair is busy until then
-    std::pop_heap(heap.begin(), heap.end(), later);
-    heap.back().first = until;
-    std::push_heap(heap.begin(), heap.end(), later);
-  };
-  std::vector<std::vector<uint16_t>> rev(pairs);              // items in reversed time order
+// A plan under construction, in reversed time. Pairs that are free at time `now` take items, lowest index first; a pair for
+// which nothing is released stays free until the next event, a release or another pair coming free.
+struct FfnBuilder {
+  FfnShape s;
+  FfnCost c;
+  double now = 0.0;
+  std::vector<int> idle;                                      // pairs free now: min-heap
+  std::vector<std::pair<double, int>> busy;                   // (time free, pair) of the others: min-heap
+  std::vector<std::pair<int, uint16_t>> rev;                  // (pair, item) placed so far
   // per row block: down tiles placed so far, the latest reversed start among them, up tiles placed so far
-  std::vector<int> dn_placed(s.Rb, 0), up_placed(s.Rb, 0);
-  std::vector<double> dn_start(s.Rb, 0.0);
-  int next_dn_rb = s.Rb - 1;                                  // down tiles go from the last row block to the first
+  std::vector<int> dn_placed, up_placed;
+  std::vector<double> dn_start;
+  int next_dn_rb;                                             // down tiles go from the last row block to the first
   int open = 0;                                               // row blocks with a down tile placed and up tiles left
-  int left = s.Rb * (s.Cu + s.Cd);
-  int ups_left = s.Rb * s.Cu, dns_left = s.Rb * s.Cd;
+  int ups_left, dns_left;
   int pending_half = -1;                                      // the second half of a tile whose first half has been placed
-  double pending_rel = 0.0;
-  const double half_cost = kFfnHalfCost * s.ku * c.up_kb + c.up_tile;
-  while (left > 0) {
-    const int p = heap.front().second;
-    const double t = heap.front().first;
-    if (pending_half >= 0) {                                  // (goes to the next pair that is free, whatever else is released)
-      rev[p].push_back((uint16_t)pending_half);
-      give(std::max(t, pending_rel) + half_cost);
-      pending_half = -1;
-      --left;
-      continue;
-    }
-    // (a) a down tile: of a row block already begun, or of the next one while the H budget allows
-    while (next_dn_rb >= 0 && dn_placed[next_dn_rb] == s.Cd) --next_dn_rb;
-    const bool dn_ok = next_dn_rb >= 0 && (dn_placed[next_dn_rb] > 0 || open < open_max);
-    if (dn_ok) {
-      const int rb = next_dn_rb;
-      if (dn_placed[rb] == 0) ++open;
-      rev[p].push_back(ffn_item(true, rb, s.Cd - 1 - dn_placed[rb]));
-      dn_start[rb] = std::max(dn_start[rb], t);
-      ++dn_placed[rb];
-      give(t + dn_cost);
-      --left;
-      --dns_left;
-      continue;
-    }
-    // (b) a released up tile: the highest row block first, within it the highest column tile (placed backwards)
-    int best_rb = -1;
-    double soonest = -1.0;                                    // earliest release among the tiles not yet released
-    for (int rb = s.Rb - 1; rb > next_dn_rb; --rb) {          // (row blocks from next_dn_rb down have down tiles left)
-      if (up_placed[rb] == s.Cu) continue;
-      const int hc = s.Cu - 1 - up_placed[rb];
-      const double rel = dn_start[rb] + (s.Cu - hc) * h_tile + c.ready_lag;
-      if (rel <= t) { best_rb = rb; break; }
-      if (soonest < 0.0 || rel < soonest) soonest = rel;
-    }
-    if (best_rb >= 0) {
-      const int rb = best_rb, hc = s.Cu - 1 - up_placed[rb];
-      // the last up tiles (in reversed time: the first of the forward lists), when they no longer fill a round of
-      // whole tiles, go out as halves to twice as many pairs
-      const bool halves = dns_left == 0 && ups_left <= n_half;
-      if (halves) {
-        rev[p].push_back((uint16_t)(ffn_item(false, rb, hc) | kFfnHalf | kFfnSecond));
-        pending_half = ffn_item(false, rb, hc) | kFfnHalf;
-        pending_rel = t;
-        ++left;                                               // one tile, two items
-        give(t + half_cost);
-      } else {
-        rev[p].push_back(ffn_item(false, rb, hc));
-        give(t + up_cost);
-      }
-      if (++up_placed[rb] == s.Cu) --open;
-      --ups_left;
-      --left;
-      continue;
-    }
-    // nothing released for this pair now: it idles until the next release (or until another pair frees up and
-    // places the down tiles that release more)
-    double wake = soonest;
-    for (const auto& q : heap) if (q.first > t && (wake < 0.0 || q.first < wake)) wake = q.first;
-    if (wake <= t) return false;                              // cannot happen: something is always pending
-    give(wake);
-  }
-  out->n_pairs = (uint16_t)pairs;
-  int o = 0;
-  for (int p = 0; p < pairs; ++p) {
-    out->off[p] = (uint16_t)o;
-    for (auto it = rev[p].rbegin(); it != rev[p].rend(); ++it) out->item[o++] = *it;
-  }
-  for (int p = pairs; p <= kFfnMaxPairs; ++p) out->off[p] = (uint16_t)o;
-  return ffn_simulate(s, *out, c) >= 0.0;
-}
 
-// The plan of the decode step: as few up tiles in halves as reach (within half a k-block time) the shortest plan any
+  FfnBuilder(const FfnShape& shape, int pairs, const FfnCost& cost)
+      : s(shape), c(cost), idle(pairs), dn_placed(shape.Rb, 0), up_placed(shape.Rb, 0), dn_start(shape.Rb, 0.0),
+        next_dn_rb(shape.Rb - 1), ups_left(shape.Rb * shape.Cu), dns_left(shape.Rb * shape.Cd) {
+    for (int p = 0; p < pairs; ++p) idle[p] = p;              // (ascending: already a heap)
+  }
+  void advance(double t) {                                    // to time t: pairs that have come free join the free ones
+    now = t;
+    while (!busy.empty() && busy.front().first <= now) {
+      idle.push_back(busy.front().second);
+      std::push_heap(idle.begin(), idle.end(), std::greater<int>());
+      std::pop_heap(busy.begin(), busy.end(), std::greater<std::pair<double, int>>());
+      busy.pop_back();
+    }
+  }
+  void place(int item, double cost) {                         // the first free pair takes the item
+    const int p = idle.front();
+    rev.emplace_back(p, (uint16_t)item);
+    std::pop_heap(idle.begin(), idle.end(), std::greater<int>());
+    idle.pop_back();
+    busy.emplace_back(now + cost, p);
+    std::push_heap(busy.begin(), busy.end(), std::greater<std::pair<double, int>>());
+  }
+  // Places items until `stop_ups` up tiles are left (0: all items). The last n_half up tiles go out as halves.
+  bool run(int n_half, int stop_ups) {
+    const double up_cost = s.ku * c.up_kb + c.up_tile, dn_cost = s.kd * c.dn_kb + c.dn_tile;
+    const double half_cost = kFfnHalfCost * s.ku * c.up_kb + c.up_tile;
+    const double h_tile = kFfnKbPerHTile * c.dn_kb;           // time a down tile spends on one column tile of H
+    const double rb_bytes = 256.0 * 256.0 * s.Cu * 2.0;
+    const int open_max = std::max(2, (int)(c.h_budget_bytes / rb_bytes));
+    while (ups_left > stop_ups || (stop_ups == 0 && (dns_left > 0 || pending_half >= 0))) {
+      if (idle.empty()) advance(busy.front().first);
+      if (pending_half >= 0) {                                // (goes to the next pair that is free, whatever else is released)
+        place(pending_half, half_cost);
+        pending_half = -1;
+        continue;
+      }
+      // (a) a down tile: of a row block already begun, or of the next one while the H budget allows
+      while (next_dn_rb >= 0 && dn_placed[next_dn_rb] == s.Cd) --next_dn_rb;
+      const bool dn_ok = next_dn_rb >= 0 && (dn_placed[next_dn_rb] > 0 || open < open_max);
+      if (dn_ok) {
+        const int rb = next_dn_rb;
+        if (dn_placed[rb] == 0) ++open;
+        dn_start[rb] = std::max(dn_start[rb], now);
+        place(ffn_item(true, rb, s.Cd - 1 - dn_placed[rb]), dn_cost);
+        ++dn_placed[rb];
+        --dns_left;
+        continue;
+      }
+      // (b) a released up tile: the highest row block first, within it the highest column tile (placed backwards)
+      int best_rb = -1;
+      double soonest = -1.0;                                  // earliest release among the tiles not yet released
+      for (int rb = s.Rb - 1; rb > next_dn_rb; --rb) {        // (row blocks from next_dn_rb down have down tiles left)
+        if (up_placed[rb] == s.Cu) continue;
+        const int hc = s.Cu - 1 - up_placed[rb];
+        const double rel = dn_start[rb] + (s.Cu - hc) * h_tile + c.ready_lag;
+        if (rel <= now) { best_rb = rb; break; }
+        if (soonest < 0.0 || rel < soonest) soonest = rel;
+      }
+      if (best_rb >= 0) {
+        const int rb = best_rb, hc = s.Cu - 1 - up_placed[rb];
+        // the last up tiles (in reversed time: the first of the forward lists), when they no longer fill a round of
+        // whole tiles, go out as halves to twice as many pairs
+        if (dns_left == 0 && ups_left <= n_half) {
+          place(ffn_item(false, rb, hc) | kFfnHalf | kFfnSecond, half_cost);
+          pending_half = ffn_item(false, rb, hc) | kFfnHalf;
+        } else {
+          place(ffn_item(false, rb, hc), up_cost);
+        }
+        if (++up_placed[rb] == s.Cu) --open;
+        --ups_left;
+        continue;
+      }
+      // nothing released now: on to the next release, or to the next pair that comes free and places the down tiles that
+      // release more
+      double wake = soonest;
+      if (!busy.empty() && (wake < 0.0 || busy.front().first < wake)) wake = busy.front().first;
+      if (wake <= now) return false;                          // cannot happen: something is always pending
+      advance(wake);
+    }
+    return true;
+  }
+  void write(FfnPlan* out) const {                            // every pair's items, turned around
+    const int pairs = (int)(idle.size() + busy.size());
+    out->n_pairs = (uint16_t)pairs;
+    std::vector<int> end(pairs, 0);                           // where pair p's list ends, filled from there backwards
+    for (const auto& r : rev) ++end[r.first];
+    int o = 0;
+    for (int p = 0; p < pairs; ++p) {
+      out->off[p] = (uint16_t)o;
+      o += end[p];
+      end[p] = o;
+    }
+    for (int p = pairs; p <= kFfnMaxPairs; ++p) out->off[p] = (uint16_t)o;
+    for (const auto& r : rev) out->item[--end[r.first]] = r.second;
+  }
+};
+
+// The plan of the feed-forward kernel: as few up tiles in halves as reach (within half a k-block time) the shortest plan any
 // number of halves up to pairs / 2 gives. A half moves three quarters of a tile's operand bytes for half its flops,
 // and the step runs at the power cap: halves that do not shorten the plan only cost clock.
+// Host time at the first pass of a size: the trials share all but their last up tiles, and idle pairs are not looked at one
+// by one (mid model, 8 / 16 / 29 / 64 row blocks: 0.39 / 0.37 / 0.65 / 0.30 ms; every trial whole, every idle pair waking for every
+// event: 4.6 / 1.1 / 2.0 / 1.1 ms, small model with 8 row blocks 6.0 against 0.3).
+// With many tiles per pair the halves decide little (under 1 % of the plan): every eighth number only.
 inline bool ffn_make_plan(const FfnShape& s, int pairs, FfnPlan* out, const FfnCost& c = FfnCost()) {
   if (!ffn_shape_ok(s, pairs)) return false;
   const int h_max = std::min(pairs / 2, s.Rb * s.Cu);
-  std::vector<double> len(h_max + 1, -1.0);
-  double best = -1.0;
-  // With many tiles per pair the halves decide little (under 1 % of the plan) and every trial costs host time at the
-  // first pass of a size (64 row blocks of the mid model: 38 trials 7.0 ms, 5 trials 1.0 ms): every eighth number only.
   const int step = s.Rb * (s.Cu + s.Cd) >= 8 * pairs ? 8 : 1;
+  FfnBuilder head(s, pairs, c);
+  if (!head.run(0, h_max)) return false;
+  std::vector<double> len(h_max + 1, -1.0);
+  auto make = [&](int h) {
+    FfnBuilder b = head;
+    if (!b.run(h, 0)) return -1.0;
+    b.write(out);
+    return ffn_simulate(s, *out, c);
+  };
+  double best = -1.0;
   for (int h = 0; h <= h_max; h += step) {
-    if (!ffn_make_plan_halves(s, pairs, h, out, c)) continue;
-    len[h] = ffn_simulate(s, *out, c);
+    len[h] = make(h);
     if (len[h] >= 0.0 && (best < 0.0 || len[h] < best)) best = len[h];
   }
   if (best < 0.0) return false;
   for (int h = 0; h <= h_max; ++h)
-    if (len[h] >= 0.0 && len[h] <= best + 0.5) return ffn_make_plan_halves(s, pairs, h, out, c);
+    if (len[h] >= 0.0 && len[h] <= best + 0.5) return make(h) >= 0.0;
   return false;
 }
 

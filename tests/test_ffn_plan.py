@@ -104,3 +104,17 @@ def test_unsupported_shapes_are_refused():
         with pytest.raises(P.SRMError) as e:
             P.k_ffn_plan(M, d, F, 74)
         assert e.value.code == P.ERR_UNSUPPORTED
+
+
+def test_plan_costs_little_host_time():
+    """A program that meets prompts of many lengths makes a plan per number of row blocks: the first pass of a size must not
+    wait longer for its plan than its kernels run. Two plans per call, 0.4 to 1.0 ms; with every trial made whole and every
+    idle pair waking for every event 3.3 to 11.2 ms. Best of 20: the machine may be busy."""
+    import time
+    for M, d in ((2048, 512), (2048, 1024), (4096, 1024), (7424, 1024)):
+        best = float("inf")
+        for _ in range(20):
+            t0 = time.perf_counter()
+            P.k_ffn_plan(M, d, 4 * d, 74)
+            best = min(best, time.perf_counter() - t0)
+        assert best < 2.5e-3, (M, d, best)
