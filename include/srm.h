@@ -20,7 +20,8 @@
  *     calls return without synchronising, except where stated.
  *   - All functions return 0 (SRM_OK) or a negative srm_error. No exceptions, no global
  *     mutable state besides the last CUDA error code and the launch counter (atomic). Handles
- *     are not thread-safe; distinct handles may be used from distinct threads.
+ *     are not thread-safe; distinct handles may be used from distinct threads, on streams of any
+ *     priority (kernels whose blocks wait for one another are cooperative launches).
  *   - Matrices are row-major [out, in]. Positions are absolute, 0-based; all samples of a
  *     state share one position counter.
  *   - The CUDA device current at srm_create is the one the handles belong to.

@@ -26,8 +26,11 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
 }
 
 // For a kernel whose CTAs wait for one another (a cooperative launch): all of them become resident together whatever else runs
-// on the device. Without it two such kernels from streams of different priority each held SMs that the other waited for.
-// Costs nothing measurable (layers kernel 111.9 / 111.3 us per step without / with).
+// on the device. Without it two such kernels from streams of different priority each held SMs that the other waited for, until
+// their bounded waits gave up. Every such kernel goes through here (or SmallLaunch), except the chunk mixers, whose blocks wait
+// for lower block indices only. What it costs: such a kernel does not start beside the end of the one before (layers kernel
+// 111.9 / 111.3 us per step without / with; feed-forward kernel in a decode
+// step of 4096 mid rows 1.438 / 1.467 ms, in a prefill of 2048 prompts of 256 143.4 / 144.9 ms).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_resident_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -308,7 +311,7 @@ int launch_gemm_splitk(srm_model& m, int64_t M, int64_t N, int64_t K, const void
   const uint8_t* wb = static_cast<const uint8_t*>(W);
   const int w_static = wb >= m.w && wb < m.w + m.layout.total;
   tc::SplitArgs g{M, N, K, bias, status, order, w_static};
-  SRM_CUDA(launch_kernel(tc::gemm_tc_splitk_kernel, dim3(2u * (unsigned)P.pairs), dim3(tc::kThreads), tc::kSmemBytes, st,
+  SRM_CUDA(launch_resident_kernel(tc::gemm_tc_splitk_kernel, dim3(2u * (unsigned)P.pairs), dim3(tc::kThreads), tc::kSmemBytes, st,
                          ta, tb, td, g, P));
   SRM_CUDA(cudaGetLastError());
   return SRM_OK;
@@ -341,10 +344,9 @@ bool ffn_fused_worthwhile(const srm_model& m, int64_t M) {
 }
 
 // `ready`: ffn_ready_bytes(M, F) bytes of zeroed words. SRM_ERR_UNSUPPORTED: take the two launches.
-// m_limit, m_off: FfnArgs. resident: launch_resident_kernel. It keeps a kernel from starting beside the end of the one before:
-// 1.7 % of a decode step of 4096 rows (5.83 -> 5.93 ms for four), so only the short slabs of a prefill ask for it.
+// m_limit, m_off: FfnArgs.
 int launch_ffn_fused(srm_model& m, int layer, int64_t M, const void* a, void* H, float* x, int32_t* ready, uint32_t* status,
-                     cudaStream_t st, const uint32_t* m_limit = nullptr, int64_t m_off = 0, bool resident = false) {
+                     cudaStream_t st, const uint32_t* m_limit = nullptr, int64_t m_off = 0) {
   if (M <= 0) return SRM_OK;
   if (!ffn_fused_shape_ok(m, M)) return SRM_ERR_UNSUPPORTED;
   int rc = ensure_tc_ready(m);
@@ -373,9 +375,7 @@ int launch_ffn_fused(srm_model& m, int layer, int64_t M, const void* a, void* H,
   if ((rc = m.tmap(W2, d, F, tc::kRowsPerCta, 2, &tw2)) != SRM_OK) return rc;
   if ((rc = m.tmap(x, M, d, tc::kOutBoxRows, 4, &tx)) != SRM_OK) return rc;
   tc::FfnArgs g{M, d, (int)F, m.fptr(layer, SRM_T_B1), m.fptr(layer, SRM_T_B2), status, ready, 1, m_limit, m_off};
-  SRM_CUDA(resident ? launch_resident_kernel(tc::ffn_fused_kernel, dim3(2u * (unsigned)m.tc_clusters), dim3(tc::kThreads), tc::kSmemBytes, st,
-                         ta, tw1, tw1h, ths, th, tw2, tx, g, *plan)
-                    : launch_kernel(tc::ffn_fused_kernel, dim3(2u * (unsigned)m.tc_clusters), dim3(tc::kThreads), tc::kSmemBytes, st,
+  SRM_CUDA(launch_resident_kernel(tc::ffn_fused_kernel, dim3(2u * (unsigned)m.tc_clusters), dim3(tc::kThreads), tc::kSmemBytes, st,
                          ta, tw1, tw1h, ths, th, tw2, tx, g, *plan));
   SRM_CUDA(cudaGetLastError());
   return SRM_OK;

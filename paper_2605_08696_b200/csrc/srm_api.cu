@@ -307,7 +307,7 @@ int prefill_impl(srm_model* m, srm_state* s, const int32_t* d_tokens, int64_t P,
         uint8_t* H_s = static_cast<uint8_t*>(w.H) + (size_t)r0 * F * m->act_bytes();
         float* x_s = w.x + (size_t)r0 * d;
         int32_t* ready = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(w.logits) + (ready_once ? l * ready_layer : 0) + (size_t)(r0 / slab_rows) * slab_ready);
-        rc = ffn_fused_worthwhile(*m, nr) ? launch_ffn_fused(*m, l, nr, a_s, H_s, x_s, ready, s->status, st, m_limit, r0, rows < kPrefillFfnRows)
+        rc = ffn_fused_worthwhile(*m, nr) ? launch_ffn_fused(*m, l, nr, a_s, H_s, x_s, ready, s->status, st, m_limit, r0)
                                          : SRM_ERR_UNSUPPORTED;
         if (rc == SRM_ERR_UNSUPPORTED) {
           if ((rc = launch_gemm(*m, kEpiBiasGelu, nr, F, d, a_s, m->ptr(l, SRM_T_W1), m->fptr(l, SRM_T_B1), H_s, s->status, st, -1, m_limit, r0))) return rc;
