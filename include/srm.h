@@ -71,11 +71,12 @@ enum {
                                         candidates are collected inside the LM-head epilogue and no logits are written
                                         when the caller does not ask for them); for comparison and measurement */
   SRM_FLAG_NO_SMALL_BATCH = 64,      /* small and mid passes also run one kernel per operation (default: a bf16 mixed-head
-                                        model of at most 1024 channels, a multiple of 256, runs the whole decode step of
-                                        as many samples as fit beside a layer's weights in shared memory, 64 at d = 512,
-                                        32 at d = 1024, in ONE cooperative kernel; larger passes of d 512 (72 to 1024
-                                        samples), 1024 (to 512) and 1536 (to 256), and those of the further mixers at d
-                                        512 and 1024, run all their layers in one kernel; results agree with the
+                                        model of at most 1024 channels, a multiple of 256, with F a multiple of 1024 runs
+                                        the whole decode step of as many samples as fit beside a layer's weights in
+                                        shared memory, 64 at d = 512, 32 at d = 1024, in ONE cooperative kernel; larger
+                                        passes of d 512 (72 to 1024 samples), 1024 (to 512) and 1536 (to 256), passes of
+                                        up to 64 samples of other widths up to 1024, and those of the further mixers at
+                                        d 512 and 1024, run all their layers in one kernel; results agree with the
                                         kernel-per-operation path to rounding, not bit for bit) */
   SRM_FLAG_NO_TAIL_SPLIT = 128,      /* tensor-core projections process every 256 x 256 tile whole (default: the tiles of a
                                         last, partly filled round run as two 256 x 128 pieces each, which keeps nearly all

@@ -744,34 +744,51 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
   return m.cfg.n_layers > 1 ? (int64_t)(m.layout.layer[SRM_T_COUNT + SRM_T_LN1_G].off - m.layout.layer[SRM_T_LN1_G].off) : 0;
 }
 
-// ---- passes of a hundred to a thousand rows: all layers in one kernel (layers_mid.cuh) -------------------
+// ---- decode passes of up to about a thousand rows: all layers in one kernel (layers_mid.cuh) -------------
 // Fewest rows, where the whole step is not one kernel of another design (step_small.cuh: up to 64 rows at d = 512, 32 at
 // d = 1024; us per step there / here: mid 1 row 181 / 239, 27 rows 241 / 246, 32 rows 250 / 244; small 27 rows 87 / 98, 64 rows
-// 111 / 100). d = 512: a batch just past that limit keeps the kernel-per-operation path (a test counts on it); from 72 rows, 138
-// us there, 104 here. Combined heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96 rows, d = 1024, 16
-// layers, kernels of size 4: 275 us per step, as a kernel per operation 560).
-int64_t mid_min_rows(const srm_config& c) { return c.d_model == 512 && c.mixer == SRM_MIXER_MIXED ? 72 : 1; }
+// 111 / 100). d = 512: a batch just past that limit, 65 to 71 rows, keeps the kernel-per-operation path, which its tests count on
+// (138 us at 72 rows there, 104 here); up to 64 rows come here only where the single-kernel step does not take F (as kMixedAny). Combined
+// heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96 rows, d = 1024, 16 layers, kernels of size 4:
+// 275 us per step, as a kernel per operation 560).
+bool mid_rows_ok(const srm_config& c, int64_t R) { return c.d_model != 512 || c.mixer != SRM_MIXER_MIXED || R <= sb::kMaxRows || R >= 72; }
+// The widths with instances of their own; mixed-head models of other widths up to 1024 channels take the instance for any
+// width with as many rows as the single-kernel step would, which is built for d % 256 == 0 and F % 1024 == 0 only (us per step
+// of 8 layers, V = 8000, 1 / 64 rows, as a kernel per operation -> here: d 64 83 / 91 -> 78 / 89, d 320 123 / 132 -> 95 / 103,
+// d 640 173 / 180 -> 111 / 118, d 832 266 / 262 -> 127 / 134, d 768 with F 6144 349 / 341 -> 145 / 154; the single-kernel step of
+// any width that stood here before took 109 / 148, 120 / 158, 126 / 177, 142 / 194 and 145 / 223).
+bool mid_own_width(int d) { return d == 512 || d == 1024 || d == 1536; }
 
 constexpr size_t kCntFloats = 256;      // room for mid::kCntWords at the head of the logits area
 static_assert(mid::kCntWords <= (int)kCntFloats, "counters");
-int mid_mix(const srm_config& c) { return c.mixer == SRM_MIXER_COMBINED ? mid::kCombined : c.mixer == SRM_MIXER_KERNEL ? mid::kKernel : mid::kMixed; }
+int mid_mix(const srm_config& c, int64_t R) {
+  if (c.mixer != SRM_MIXER_MIXED) return c.mixer == SRM_MIXER_COMBINED ? mid::kCombined : mid::kKernel;
+  return mid_own_width(c.d_model) && !(c.d_model == 512 && R <= sb::kMaxRows) ? mid::kMixed : mid::kMixedAny;
+}
 
 // Whether a decode pass of R rows takes it, and its tile plan. bf16 models of the widths it is built for,
 // as many rows as leave every CTA pair one tile of each projection.
 bool mid_plan(srm_model& m, int64_t R, const DecodeWs& w, mid::Params* p) {
   const srm_config& c = m.cfg;
   constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
-  if (R < mid_min_rows(c) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff)) return false;
+  if (!mid_rows_ok(c, R) || c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff)) return false;
   if (c.mixer != SRM_MIXER_MIXED && (c.d_model > 1024 || c.n_heads > 8 || c.kernel_size > 16)) return false;
-  if (c.d_model != 512 && c.d_model != 1024 && c.d_model != 1536) return false;
+  const int mix = mid_mix(c, R);
+  if (mix == mid::kMixedAny ? R > sb::kMaxRows || c.d_model > 1024 : !mid_own_width(c.d_model)) return false;
   if (ensure_tc_ready(m) != SRM_OK || R > (int64_t)2 * m.tc_clusters * mid::kMaxGroups || m.F() > (1 << 20)) return false;
-  if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, mid_mix(c), p)) return false;
-  // The planes of partial products: an area of their own where the model has one, else (combined heads, kernels) behind the
-  // counters in the logits area, from about five rows of the mid model on.
-  p->plane_rows = (int)(R + tc::kOutBoxRows - 1) / tc::kOutBoxRows * tc::kOutBoxRows;
-  const size_t need = (size_t)p->ks * p->plane_rows * c.d_model * 4;
+  // The planes of partial products: an area of their own where the model has one (kslice_model), else behind the counters in
+  // the logits area. Any widths keep the rows there are, in as many planes as there is room for; whole boxes of rows fit from
+  // about five rows of the mid model on.
+  const size_t logits = (size_t)w.rows * c.vocab;
+  const size_t room = w.part != nullptr ? w.part_bytes : (logits - std::min(logits, kCntFloats)) * 4;
   p->part = w.part != nullptr ? w.part : w.logits + kCntFloats;
-  return need <= (w.part != nullptr ? w.part_bytes : (size_t)w.rows * c.vocab * 4 - std::min((size_t)w.rows * c.vocab, kCntFloats) * 4);
+  p->plane_rows = mix == mid::kMixedAny ? (int)R : (int)(R + tc::kOutBoxRows - 1) / tc::kOutBoxRows * tc::kOutBoxRows;
+  for (int most = mix == mid::kMixedAny ? 2 * mid::kMaxKSlices : mid::kMaxKSlices; most >= 1; most /= 2) {
+    if (!mid::plan(R, c.d_model, (int)m.F(), m.tc_clusters, mix, most, p)) return false;
+    if ((size_t)p->ks * p->plane_rows * c.d_model * 4 <= room) return true;
+    if (mix != mid::kMixedAny) return false;
+  }
+  return false;
 }
 
 struct MidMaps { CUtensorMap a, h, w1, w2, hs, p; };      // loads of a, H, W1, W2; stores of H and the partial products
@@ -796,6 +813,11 @@ int launch_layers_nt(srm_model& m, const MidMaps& t, const mid::Params& p, cudaS
   if (m.cfg.state_dtype == SRM_DTYPE_FP16) return launch_layers_t<NT, fp16, mid::kMixed>(m, t, p, st);
   if (m.cfg.state_dtype == SRM_DTYPE_BF16) return launch_layers_t<NT, bf16, mid::kMixed>(m, t, p, st);
   return launch_layers_t<NT, float, mid::kMixed>(m, t, p, st);
+}
+int launch_layers_any(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {      // (at most 64 rows, 1024 channels)
+  if (m.cfg.state_dtype == SRM_DTYPE_FP16) return launch_layers_w<2, 4, fp16, mid::kMixedAny>(m, t, p, st);
+  if (m.cfg.state_dtype == SRM_DTYPE_BF16) return launch_layers_w<2, 4, bf16, mid::kMixedAny>(m, t, p, st);
+  return launch_layers_w<2, 4, float, mid::kMixedAny>(m, t, p, st);
 }
 template <int NT>
 int launch_layers_variant(srm_model& m, const MidMaps& t, const mid::Params& p, cudaStream_t st) {
@@ -839,6 +861,10 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   if ((rc = make_tmap_kblocks(&maps.w1, m.ptr(0, SRM_T_W1), F, d, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = make_tmap_kblocks(&maps.w2, m.ptr(0, SRM_T_W2), d, F, p.n / 2, mid::kStep, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = m.tmap(w.H, R, F, tc::kOutBoxRows, 2, &maps.hs)) != SRM_OK) return rc;
+  if (mid_mix(c, R) == mid::kMixedAny) {                  // (planes of the rows there are: a box must not reach into the next one)
+    if ((rc = make_tmap(&maps.p, p.part, R, d, tc::kOutBoxRows, 4, p.ks, p.plane_rows)) != SRM_OK) return rc;
+    return launch_layers_any(m, maps, p, st);
+  }
   if ((rc = m.tmap(p.part, (int64_t)p.ks * p.plane_rows, d, tc::kOutBoxRows, 4, &maps.p)) != SRM_OK) return rc;
   if (c.mixer != SRM_MIXER_MIXED) return d == 512 ? launch_layers_variant<2>(m, maps, p, st) : launch_layers_variant<4>(m, maps, p, st);
   if (d == 512) return launch_layers_nt<2>(m, maps, p, st);

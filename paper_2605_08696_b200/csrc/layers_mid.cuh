@@ -1,4 +1,4 @@
-// All layers of a decode pass of a hundred to a thousand rows as ONE persistent kernel.
+// All layers of a decode pass of up to about a thousand rows as ONE persistent kernel.
 //
 // With so few rows a layer is a chain of three short kernels (token mixer, up projection, down projection over ranges of
 // K), and launch, ramp, first loads and drain of each cost more than its work: 25 us per layer at 256 rows of the mid
@@ -15,6 +15,8 @@
 //     block start. Nothing waits for a block it does not read.
 // Combined heads and kernels of size k (MIX) differ in the row phase only: their cache planes and scalars, and for kernels a
 // barrier of the row's warps per filter.
+// Mixed-head models of other widths than 512, 1024 and 1536 (kMixedAny, up to 64 rows): threads beyond the last channel hold
+// nothing, the last column tile may be partly filled, and what a stage holds beyond the last k-block is zeros.
 // Projections run as in gemm_tc_kernel: TMA loads (128-byte swizzle), tcgen05.mma.cta_group::2 issued by one thread of
 // the leader CTA, accumulator in tensor memory, 16 epilogue warps.
 //
@@ -53,6 +55,7 @@ struct Params {
   int R, d, F, V, h, n_ctx, L, t;
   float eps;
   int rb, n, cu, cd, ks;         // row blocks, tile width, column tiles of the up / down projection, ranges of K
+  int slice_tiles;               // column tiles of H per range of K (the last range may have fewer)
   int w_slots, a_slots;
   int box;                       // rows of an activation box: 128, or the rows there are (a multiple of 8); rows of zeros that the copy
                                  // unit fills in for rows beyond the last cost it more than rows it reads (45 rows: 2.7 against 1.2 us per tile)
@@ -68,7 +71,7 @@ struct Params {
   bf16* H;                       // [R, F]
   float* part;                   // [ks] planes of plane_rows x d 
   int64_t plane;                 // elements per plane
-  int plane_rows;                // rows per plane: R rounded up to whole boxes
+  int plane_rows;                // rows per plane
   uint32_t* cnt;                 // rows done [8] | up pieces done [8][4] | down pieces done [8]; zero on entry
   uint32_t* status;
   const int32_t* ctr;            // device-side step counters or nullptr
@@ -81,8 +84,10 @@ struct Params {
 // Row-phase parameters in shared memory: ln1_g | ln1_b | beta_t | ln2_g | ln2_b | b2 of the previous layer, then this CTA's
 // part of b1 (first touched in the epilogue it came from HBM there: 0.7 us).
 constexpr int kVecs = 6;
-// Token mixers: mixed heads; combined heads; kernels of size k.
-constexpr int kMixed = 0, kCombined = 1, kKernel = 2;
+// Token mixers: mixed heads; combined heads; kernels of size k; mixed heads of any width (d a multiple of 64, at most
+// NT * kStride: threads beyond the last channel hold nothing).
+constexpr int kMixed = 0, kCombined = 1, kKernel = 2, kMixedAny = 3;
+__host__ __device__ constexpr bool mixed_heads(int mix) { return mix == kMixed || mix == kMixedAny; }
 constexpr int kMixScalars = 64;      // of a layer at the pass's position: combined 6 h <= 48 floats, kernel 2 k <= 32
 constexpr int kCntWords = kMaxRowBlocks * (2 + kMaxKSlices);
 __global__ void __launch_bounds__(64) zero_counters_kernel(uint32_t* __restrict__ cnt) {
@@ -95,22 +100,27 @@ static_assert(kCntWords <= 64, "one thread per counter");
 // Shared memory: W ring | A ring (both 1024-byte aligned) | row-phase parameters | row-phase sums | barriers | for the
 // further mixers their scalars and, for kernels, the channels a warp's last lanes read of the next warp.
 __host__ __device__ inline size_t smem_bytes(int d, int n, int w_slots, int a_slots, int mix) {
-  return 1024 + (mix == kMixed ? 0 : kMixScalars * 4 + (mix == kKernel ? (size_t)kMaxGroups * d : 0)) + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + ((size_t)kVecs * d + n) * 4 + kMaxGroups * 32 + kBarrierBytes;
+  return 1024 + (mixed_heads(mix) ? 0 : kMixScalars * 4 + (mix == kKernel ? (size_t)kMaxGroups * d : 0)) + (size_t)w_slots * kStep * (n / 2) * 128 + (size_t)a_slots * kABytes + ((size_t)kVecs * d + n) * 4 + kMaxGroups * 32 + kBarrierBytes;
 }
 
-// Tile widths and ranges of K for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit. (256-wide
+// Tile widths and ranges of K (at most most_ks: kMaxKSlices, twice that for kMixedAny, whose single row block uses the counters
+// of a second for the further ranges) for R rows of a model (d, F) on `pairs` CTA pairs; false: the pieces do not fit. (256-wide
 // tiles, which would take mid passes of 513 to 1024 rows, measured slower than a kernel per operation: 0.59 against
 // 0.54 ms per step.)
-inline bool plan(int64_t R, int d, int F, int pairs, int mix, Params* p) {
+inline bool plan(int64_t R, int d, int F, int pairs, int mix, int most_ks, Params* p) {
   const int rb = (int)((R + tc::BM - 1) / tc::BM);
-  if (rb < 1 || rb > kMaxRowBlocks) return false;
+  if (rb < 1 || rb > (mix == kMixedAny ? 1 : kMaxRowBlocks)) return false;
   for (int n = 64; n <= 128; n *= 2) {
-    if (F % n || d % n || rb * (F / n) > pairs) continue;
-    int ks = kMaxKSlices;
-    while (ks > 1 && (rb * (d / n) * ks > pairs || (F / 64) % (ks * kStep) || (F / ks) % n)) ks >>= 1;
-    if (rb * (d / n) * ks > pairs || (F / 64) % (ks * kStep)) continue;
+    const int cu = (F + n - 1) / n, cd = (d + n - 1) / n;            // (the last tile of a row block may be partly filled)
+    if (n > d || rb * cu > pairs || rb * cd > pairs) continue;
+    // ranges of whole column tiles of H and of whole stages; what a stage holds beyond the last k-block is zeros
+    const int grain = kStep * 64 / n;
+    int ks = most_ks;
+    auto per = [&] { return ((cu + ks - 1) / ks + grain - 1) / grain * grain; };
+    while (ks > 1 && (rb * cd * ks > pairs || (ks - 1) * per() >= cu)) ks >>= 1;
+    p->slice_tiles = per();
     p->box = R < tc::kRowsPerCta ? (int)(R + 7) / 8 * 8 : tc::kRowsPerCta;
-    p->rb = rb; p->n = n; p->cu = F / n; p->cd = d / n; p->ks = ks;
+    p->rb = rb; p->n = n; p->cu = cu; p->cd = cd; p->ks = ks;
     // the weight ring runs a phase ahead; the activation ring hides the latency of L2 and holds the output tile of an
     // epilogue (128 rows of n fp32 columns)
     p->w_slots = n == 64 ? 8 : 6;
@@ -135,6 +145,10 @@ __device__ __forceinline__ void tma_load_w(void* dst, const CUtensorMap* map, ui
       "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
       ::"r"(tc::smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_cluster_addr), "r"(0), "r"(row), "r"(kb), "r"(layer)
       : "memory");
+}
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void* src, int x, int y, int z) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
+               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(tc::smem_u32(src)), "r"(x), "r"(y), "r"(z) : "memory");
 }
 __device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -193,6 +207,32 @@ __device__ __forceinline__ void group_stats(const float4 (&v)[NT], float eps, fl
   }
   mean = mm[0];
   rstd = rsqrtf(qq[0] / cnt + eps);
+}
+
+// The same for a row of d channels, of which this thread holds the first `mine` of its float4s (the others are zero).
+template <int NT, int WPG>
+__device__ __forceinline__ void group_stats_any(const float4 (&v)[NT], int mine, int d, float eps, float* slot, int group, float& mean, float& rstd) {
+  auto sum = [&](float x, float* part) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) part[((threadIdx.x >> 5) - kEpiWarp0) % WPG] = x;
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(WPG * 32) : "memory");
+    float all = part[0];
+#pragma unroll
+    for (int w = 1; w < WPG; ++w) all += part[w];
+    return all;
+  };
+  float m = 0.f, q = 0.f;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) m += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+  const float inv_d = 1.0f / (float)d;
+  mean = sum(m, slot) * inv_d;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const float a = v[i].x - mean, b = v[i].y - mean, c = v[i].z - mean, e = v[i].w - mean;
+    if (i < mine) q += (a * a + b * b) + (c * c + e * e);
+  }
+  rstd = rsqrtf(sum(q, slot + WPG) * inv_d + eps);
 }
 
 // Combined heads and kernels of size k on the row of a group of WPG warps (thread th: channels 4 th .. 4 th + 3 and 128 WPG,
@@ -282,7 +322,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
               const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmHs, const __grid_constant__ CUtensorMap tmP,
               const Params p) {
   pdl_trigger();
-  constexpr int kGroups = tc::kEpiWarps / WPG, kRowThreads = WPG * 32, kStride = kRowThreads * 4, d = NT * kStride;
+  constexpr int kRowThreads = WPG * 32, kStride = kRowThreads * 4;
+  const int d = MIX == kMixedAny ? p.d : NT * kStride;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int n = p.n, w_rows = n >> 1, w_bytes = kStep * w_rows * 128;
@@ -299,7 +340,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   uint64_t* tempty = tfull + 1;                                          // leader: accumulator drained by both CTAs
   uint64_t* ring = tempty + 1;                                           // the epilogue has left the activation ring
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring + 1);
-  float* hs = red + kMaxGroups * 8 + kBarrierBytes / 4;                  // MIX != kMixed
+  float* hs = red + kMaxGroups * 8 + kBarrierBytes / 4;                  // not for mixed heads
   float4* edge = reinterpret_cast<float4*>(hs + kMixScalars);            // MIX == kKernel: d bytes per group
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -327,9 +368,11 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
   const bool up_on = up_col < p.cu;
   const int dn_rb = up_rb, dn_col = up_col % p.cd, dn_slice = up_col / p.cd;
   const bool dn_on = dn_slice < p.ks;
-  const int kb_up = d / tc::BK, kb_dn = p.F / tc::BK / p.ks;            // k-blocks per piece
+  const int slice_kb = p.slice_tiles * (n / tc::BK);
+  const int kb_up = d / tc::BK, kb_dn = min(slice_kb, p.F / tc::BK - dn_slice * slice_kb);      // k-blocks per piece
   const int up_boxes = n / 64, dn_boxes = n / 32;                        // boxes of 128 bytes per row that an output tile consists of
-  const int slice_cols = p.F / p.ks;                                     // columns of H per range of K
+  const int up_slice = up_col / p.slice_tiles;                           // range of K that this pair's column tile of H belongs to
+  const int slice_up = min(p.slice_tiles, p.cu - dn_slice * p.slice_tiles);      // column tiles of H that the down piece reads
   uint32_t* cnt_rows = p.cnt;
   uint32_t* cnt_up = p.cnt + kMaxRowBlocks;
   uint32_t* cnt_dn = cnt_up + kMaxRowBlocks * kMaxKSlices;
@@ -346,7 +389,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         for (int ph = 0; ok && ph < 2; ++ph) {
           if (!(ph ? dn_on : up_on)) continue;
           const CUtensorMap* map = ph ? &tmW2 : &tmW1;
-          const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * kb_dn : 0;
+          const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * slice_kb : 0;
           const int row = (ph ? dn_col : up_col) * n + (int)rank * w_rows;
           for (int kb = 0; kb < kbs; kb += kStep) {
             if (!tc::mbar_wait(&emptyW[slot], phase ^ 1u, p.status)) { ok = false; break; }
@@ -376,13 +419,13 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         for (int ph = 0; ok && ph < 2; ++ph) {
           if (!(ph ? dn_on : up_on)) continue;
           // rows of the block done / the up tiles of this range of K done
-          if (!(ph ? count_wait(cnt_up + dn_rb * kMaxKSlices + dn_slice, (uint32_t)(l + 1) * (uint32_t)(slice_cols / n * up_boxes) * 8u, p.status)
+          if (!(ph ? count_wait(cnt_up + dn_rb * kMaxKSlices + dn_slice, (uint32_t)(l + 1) * (uint32_t)(slice_up * up_boxes) * 8u, p.status)
                    : count_wait(cnt_rows + up_rb, (uint32_t)(l + 1) * (uint32_t)block_rows, p.status))) { ok = false; break; }
           if (piece > 0 && !tc::mbar_wait(ring, (uint32_t)(piece & 1) ^ 1u, p.status)) { ok = false; break; }
           ++piece;
           tc::fence_async_global();
           const CUtensorMap* map = ph ? &tmH : &tmA;
-          const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * kb_dn : 0;
+          const int kbs = ph ? kb_dn : kb_up, kb0 = ph ? dn_slice * slice_kb : 0;
           const int row = up_rb * tc::BM + (int)rank * tc::kRowsPerCta;
           for (int kb = 0; kb < kbs; kb += kStep) {
             if (!tc::mbar_wait(&emptyA[slot], phase ^ 1u, p.status)) { ok = false; break; }
@@ -454,20 +497,22 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         const int k = i / (d / 4), c = i % (d / 4) * 4;
         const float* q = k == 0 ? w.ln1_g : k == 1 ? w.ln1_b : k == 2 ? w.beta + (int64_t)t_all * d : k == 3 ? (last ? p.lnf_g : w.ln2_g)
                          : k == 4 ? (last ? p.lnf_b : w.ln2_b) : k == 5 ? sb::layer_w(p, l > 0 ? l - 1 : 0).b2 : w.b1 + (up_on ? up_col : 0) * n;
-        sb::cp_async16(prm + i * 4, q + c);
+        if (MIX != kMixedAny || k < kVecs || !up_on || up_col * n + c < p.F) sb::cp_async16(prm + i * 4, q + c);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
       const int row = (int)blockIdx.x + (int)gridDim.x * group;
       const bool mine = row < p.R;
+      auto on = [&](int i) { return MIX != kMixedAny || c0 + kStride * i < d; };      // float4 i lies inside the row
       const int t = mine && p.pos != nullptr ? min(max(p.pos[row], 0), p.n_ctx - 1) : t_all;
       float a1[NT], a2[NT], lm[NT];                  // (mixed heads)
       float4 s[NT], s1[NT], v[NT];                   // (s1: combined heads)
       ST* Sr = reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + (int64_t)row * d + c0;
       if (mine) {
         if (!last) {
-          if (MIX == kMixed) {            // the multipliers of z before and of the sum after (one of them is 1), and lambda
+          if (mixed_heads(MIX)) {         // the multipliers of z before and of the sum after (one of them is 1), and lambda
 #pragma unroll
             for (int i = 0; i < NT; ++i) {
+              if (!on(i)) continue;
               const int g = (c0 + kStride * i) / (d / p.h);
               const float al = __ldg(w.alpha + (int64_t)g * p.n_ctx + t);
               const bool is_row = g < (p.h >> 1);
@@ -477,10 +522,12 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             }
           }
 #pragma unroll
-          for (int i = 0; i < NT; ++i) s[i] = ld4(Sr + kStride * i);
+          for (int i = 0; i < NT; ++i)
+            if (on(i)) s[i] = ld4(Sr + kStride * i);
           if (p.pos != nullptr) {
 #pragma unroll
-            for (int i = 0; i < NT; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(w.beta + (int64_t)t * d + c0 + kStride * i));
+            for (int i = 0; i < NT; ++i)
+              if (on(i)) asm volatile("prefetch.global.L2 [%0];" ::"l"(w.beta + (int64_t)t * d + c0 + kStride * i));
           }
           if (MIX == kCombined) {
 #pragma unroll
@@ -489,12 +536,13 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
         if (l > 0) {                      // (this thread's part of x, from the previous layer: not through L1)
 #pragma unroll
-          for (int i = 0; i < NT; ++i) v[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c0 + kStride * i));
+          for (int i = 0; i < NT; ++i)
+            v[i] = on(i) ? __ldcg(reinterpret_cast<const float4*>(p.x + (int64_t)row * d + c0 + kStride * i)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (l > 0 && th == 0 && ok)               // the down tiles of the row's block
           ok = count_wait(cnt_dn + row / tc::BM, (uint32_t)l * (uint32_t)(p.cd * p.ks * dn_boxes) * 8u, p.status);
       }
-      if (MIX != kMixed && !last) {         // scalar wid of the layer
+      if (!mixed_heads(MIX) && !last) {     // scalar wid of the layer
         const int64_t o = (int64_t)l * p.layer_bytes;
         auto at = [o](const float* q, int64_t i) { return __ldg(reinterpret_cast<const float*>(reinterpret_cast<const uint8_t*>(q) + o) + i); };
         if (MIX == kCombined && wid < 6 * p.h) {
@@ -515,36 +563,46 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             tk = tk < 0 ? 0 : p.V - 1;
           }
 #pragma unroll
-          for (int i = 0; i < NT; ++i) v[i] = ldg4(p.E + (int64_t)tk * d + c0 + kStride * i);
+          for (int i = 0; i < NT; ++i) v[i] = on(i) ? ldg4(p.E + (int64_t)tk * d + c0 + kStride * i) : make_float4(0.f, 0.f, 0.f, 0.f);
         } else {                          // x + b2 + plane 0 + plane 1 + ... (other CTAs wrote the planes: not through L1)
 #pragma unroll
           for (int i = 0; i < NT; ++i) {
+            if (!on(i)) continue;
             const float4 bb = ld4(prm + 5 * d + c0 + kStride * i);
             v[i] = make_float4(v[i].x + bb.x, v[i].y + bb.y, v[i].z + bb.z, v[i].w + bb.w);
           }
           const float* part = p.part + (int64_t)row * d + c0;
-          auto add = [&](auto planes) {   // all planes' loads in flight
+          auto add = [&](auto planes) {   // all planes' loads in flight, of four at most
             constexpr int K = decltype(planes)::value;
             float4 e[K][NT];
 #pragma unroll
             for (int k = 0; k < K; ++k)
 #pragma unroll
-              for (int i = 0; i < NT; ++i) e[k][i] = __ldcg(reinterpret_cast<const float4*>(part + k * p.plane + kStride * i));
+              for (int i = 0; i < NT; ++i)
+                e[k][i] = on(i) ? __ldcg(reinterpret_cast<const float4*>(part + k * p.plane + kStride * i)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < K; ++k)
 #pragma unroll
               for (int i = 0; i < NT; ++i) v[i] = make_float4(v[i].x + e[k][i].x, v[i].y + e[k][i].y, v[i].z + e[k][i].z, v[i].w + e[k][i].w);
           };
-          if (p.ks == 4) add(std::integral_constant<int, 4>());
+          if (MIX == kMixedAny && p.ks == 8) {
+            add(std::integral_constant<int, 4>());
+            part += 4 * p.plane;
+          }
+          if (p.ks >= 4) add(std::integral_constant<int, 4>());
           else if (p.ks == 2) add(std::integral_constant<int, 2>());
           else add(std::integral_constant<int, 1>());
         }
         float mean, rstd;
+        auto stats = [&](float* sums) {
+          if constexpr (MIX == kMixedAny) group_stats_any<NT, WPG>(v, c0 < d ? (d - c0 + kStride - 1) / kStride : 0, d, p.eps, sums, group, mean, rstd);
+          else group_stats<NT, WPG>(v, p.eps, sums, group, mean, rstd);
+        };
         if (!last) {
           const float* bt_p = p.pos != nullptr ? w.beta + (int64_t)t * d + c0 : prm + 2 * d + c0;
-          group_stats<NT, WPG>(v, p.eps, slot, group, mean, rstd);
+          stats(slot);
           const float nmr = -mean * rstd;
-          if (MIX != kMixed) {
+          if constexpr (!mixed_heads(MIX)) {
             float4 z[NT];
 #pragma unroll
             for (int i = 0; i < NT; ++i) {
@@ -557,7 +615,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             for (int i = 0; i < NT; ++i) st4(p.x + (int64_t)row * d + c0 + kStride * i, v[i]);
           }
 #pragma unroll
-          for (int i = 0; MIX == kMixed && i < NT; ++i) {
+          for (int i = 0; mixed_heads(MIX) && i < NT; ++i) {
+            if (!on(i)) continue;
             const float4 g = ld4(prm + c0 + kStride * i), bb = ld4(prm + d + c0 + kStride * i), bt = ld4(bt_p + kStride * i);
             const float4 z = make_float4(fmaf(fmaf(v[i].x, rstd, nmr), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr), g.y, bb.y),
                                          fmaf(fmaf(v[i].z, rstd, nmr), g.z, bb.z), fmaf(fmaf(v[i].w, rstd, nmr), g.w, bb.w));
@@ -569,10 +628,11 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             st4(p.x + (int64_t)row * d + c0 + kStride * i, v[i]);
           }
         }
-        group_stats<NT, WPG>(v, p.eps, slot + kMaxGroups * 4, group, mean, rstd);
+        stats(slot + kMaxGroups * 4);
         const float nmr2 = -mean * rstd;
 #pragma unroll
         for (int i = 0; i < NT; ++i) {
+          if (!on(i)) continue;
           const float4 g = ld4(prm + 3 * d + c0 + kStride * i), bb = ld4(prm + 4 * d + c0 + kStride * i);
           st4(p.a + (int64_t)row * d + c0 + kStride * i,
               make_float4(fmaf(fmaf(v[i].x, rstd, nmr2), g.x, bb.x), fmaf(fmaf(v[i].y, rstd, nmr2), g.y, bb.y),
@@ -631,14 +691,15 @@ layers_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         asm volatile("bar.sync %0, 128;" ::"r"(quad + 10) : "memory");      // the four warps of this row quarter
         if (cgrp < boxes && tc::elect_one()) {
           const uint8_t* src = sA + (quad * boxes + cgrp) * tc::kOutBoxBytes;
-          if (row0 < p.R) {
-            if (ph) tc::tma_store_2d(&tmP, src, col0 + cgrp * 32, dn_slice * p.plane_rows + row0);
-            else tc::tma_store_2d(&tmHs, src, col0 + cgrp * 64, row0);
+          if (row0 < p.R && (MIX != kMixedAny || (ph ? col0 + cgrp * 32 < d : col0 + cgrp * 64 < p.F))) {
+            if (ph == 0) tc::tma_store_2d(&tmHs, src, col0 + cgrp * 64, row0);
+            else if (MIX == kMixedAny) tma_store_3d(&tmP, src, col0 + cgrp * 32, row0, dn_slice);
+            else tc::tma_store_2d(&tmP, src, col0 + cgrp * 32, dn_slice * p.plane_rows + row0);
             tc::bulk_commit();
             tc::bulk_wait_all();
           }
           tc::fence_async_global();
-          red_release_add(ph ? cnt_dn + dn_rb : cnt_up + up_rb * kMaxKSlices + up_col * n / slice_cols, 1u);
+          red_release_add(ph ? cnt_dn + dn_rb : cnt_up + up_rb * kMaxKSlices + up_slice, 1u);
         }
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(ring);

@@ -116,3 +116,49 @@ def test_further_mixers_in_one_kernel_agree_with_the_kernel_per_operation_path(m
         for i in range(3):
             lo, state = orc.decode_step(state, toks[n + i, b:b + 1].cpu().numpy(), n + i)
             assert rel_err_rows(outs[1][0][i][b:b + 1], lo) < 3e-2
+
+
+@pytest.mark.parametrize("B,d,mult,heads,layers,state_dtype,ragged", [
+    (1, 320, 4, 4, 3, "fp32", False), (64, 320, 4, 8, 3, "bf16", True), (33, 448, 4, 4, 3, "fp16", False),
+    (8, 512, 3, 4, 3, "fp32", False), (3, 512, 5, 8, 3, "fp32", True), (64, 512, 12, 4, 3, "fp16", False),
+    (17, 640, 2, 4, 3, "fp32", False), (64, 768, 8, 4, 3, "fp32", True), (9, 832, 4, 4, 1, "fp32", False),
+    (40, 832, 5, 8, 3, "fp16", False), (1, 960, 6, 4, 3, "fp32", True), (63, 960, 6, 6, 3, "bf16", False), (64, 960, 4, 4, 2, "fp32", False),
+    (100, 512, 4, 8, 1, "fp32", False), (75, 512, 4, 8, 3, "bf16", True), (130, 1536, 4, 8, 1, "fp16", True)])
+def test_models_of_any_width_and_head_count(B, d, mult, heads, layers, state_dtype, ragged):
+    """Widths and hidden widths the single-kernel step is not built for, up to 64 rows: rows that do not fill the threads,
+    k-blocks that do not fill a stage (d = 64 x odd), last column tiles partly filled (F = 5760 in tiles of 128), ranges of K of
+    unequal length (F = 3328, 5760). And heads that are not whole multiples of 128 channels (the partial products then lie in
+    the logits area); models of a single layer."""
+    import dataclasses
+
+    import paper_2605_08696_b200 as P
+    base = custom_shape(n_layers=layers, d_model=d, vocab=16384 if d == 1536 else 4096, n_ctx=24, dtype="bf16", seed=17)
+    shape = dataclasses.replace(base, ffn_mult=mult, n_heads=heads)
+    W = I.make_weights(shape)
+    rng = np.random.default_rng(B)
+    n = 5
+    prompts_np = rng.integers(0, shape.vocab, size=(B, n)).astype(np.int32)
+    lens_np = rng.integers(1, n + 1, size=B).astype(np.int32) if ragged else np.full(B, n, np.int32)
+    fed = torch.from_numpy(rng.integers(0, shape.vocab, size=(3, B)).astype(np.int32)).to(DEV)
+    prompts, lens = torch.from_numpy(prompts_np).to(DEV), torch.from_numpy(lens_np).to(DEV)
+    g = P.Sampling("greedy")
+    outs = []
+    for flags in (P.FLAG_NO_SMALL_BATCH, 0):
+        m = P.SRM(shape, W, device=DEV, flags=flags, state_dtype=state_dtype)
+        st, ws = m.new_state(B), m.new_workspace(B, n, prefill_samples=B)
+        m.prefill_ragged(st, prompts, lens, g, ws) if ragged else m.prefill(st, prompts, g, ws)
+        lgs = []
+        for k in range(3):
+            launches = _launches(P, lambda: lgs.append(m.decode_step(st, fed[k], g, k + 1, ws, want_logits=True)[1].cpu().numpy()))
+        assert (launches <= 4) == (flags == 0)                 # counters, layers and norm, LM head, selection
+        assert st.status() == 0
+        outs.append((np.stack(lgs), st.cache().cpu().float().numpy()))
+    (lg_a, S_a), (lg_b, S_b) = outs
+    tol = 5 * 2.0 ** -9 * layers ** 0.5                        # as above
+    assert rel_err_rows(lg_b, lg_a) < tol and rel_err_rows(S_b, S_a) < tol
+    orc = oracle_for(shape, W)
+    for b in (0, B - 1):
+        lo, state = orc.forward_parallel(prompts_np[b:b + 1, :lens_np[b]])
+        for k in range(3):
+            lo, state = orc.decode_step(state, fed[k, b:b + 1].cpu().numpy(), int(lens_np[b]) + k)
+            assert rel_err_rows(lg_b[k][b:b + 1], lo) < 3e-2
