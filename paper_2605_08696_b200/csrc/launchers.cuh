@@ -28,9 +28,11 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
 // For a kernel whose CTAs wait for one another (a cooperative launch): all of them become resident together whatever else runs
 // on the device. Without it two such kernels from streams of different priority each held SMs that the other waited for, until
 // their bounded waits gave up. Every such kernel goes through here (or SmallLaunch), except the chunk mixers, whose blocks wait
-// for lower block indices only. What it costs: such a kernel does not start beside the end of the one before (layers kernel
-// 111.9 / 111.3 us per step without / with; feed-forward kernel in a decode
-// step of 4096 mid rows 1.438 / 1.467 ms, in a prefill of 2048 prompts of 256 143.4 / 144.9 ms).
+// for lower block indices only. Not combined with programmatic serialization, which lets a kernel's blocks in while the one
+// before still runs: with both, a prefill beside decode steps of another stream came to a standstill once; and it gains nothing,
+// a cooperative kernel waits for all SMs anyway. What residency costs: the feed-forward kernel no longer starts beside the end
+// of the one before (decode step of 4096 mid rows 1.44 -> 1.47 ms, prefill of 2048 prompts of 256 143.5 -> 144.7 ms); the
+// layers kernel nothing.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_resident_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -38,13 +40,11 @@ cudaError_t launch_resident_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 blo
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeCooperative;
-  attr[1].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeCooperative;
+  attr.val.cooperative = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
@@ -748,9 +748,9 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
 // Fewest rows, where the whole step is not one kernel of another design (step_small.cuh: up to 64 rows at d = 512, 32 at
 // d = 1024; us per step there / here: mid 1 row 181 / 239, 27 rows 241 / 246, 32 rows 250 / 244; small 27 rows 87 / 98, 64 rows
 // 111 / 100). d = 512: a batch just past that limit, 65 to 71 rows, keeps the kernel-per-operation path, which its tests count on
-// (138 us at 72 rows there, 104 here); up to 64 rows come here only where the single-kernel step does not take F (as kMixedAny). Combined
-// heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96 rows, d = 1024, 16 layers, kernels of size 4:
-// 275 us per step, as a kernel per operation 560).
+// (138 us at 72 rows there, 104 here); up to 64 rows come here only where the single-kernel step does not take F (as kMixedAny).
+// Combined heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96 rows, d = 1024, 16 layers, kernels of
+// size 4: 275 us per step, as a kernel per operation 560).
 bool mid_rows_ok(const srm_config& c, int64_t R) { return c.d_model != 512 || c.mixer != SRM_MIXER_MIXED || R <= sb::kMaxRows || R >= 72; }
 // The widths with instances of their own; mixed-head models of other widths up to 1024 channels take the instance for any
 // width with as many rows as the single-kernel step would, which is built for d % 256 == 0 and F % 1024 == 0 only (us per step
@@ -849,8 +849,7 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   p.plane = (int64_t)p.plane_rows * d;
   p.cnt = reinterpret_cast<uint32_t*>(w.logits);      // (nothing uses the logits area before the LM head)
   p.status = s.status; p.ctr = ctr; p.pos = pos;
-  // (cleared by a kernel: the layers kernel then sets itself up and starts on its weights while the kernels before it end,
-  // which it does not do behind a memset; 3 us per step)
+  // (cleared by a kernel: behind a memset the step took 3 us longer)
   ++g_kernel_launches;
   SRM_CUDA(launch_kernel(mid::zero_counters_kernel, dim3(1), dim3(64), 0, st, p.cnt));
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
