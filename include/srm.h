@@ -200,11 +200,14 @@ int32_t srm_cache_planes(const srm_config* cfg);
  * workspace at least this large for B_chunk = 1 and split the batch into as many passes as
  * the given workspace requires. Decode never uses more than 12288 rows of it in one pass: a larger
  * batch runs as equal passes of at most 10240 rows (whole 256-row tiles), which keeps a layer's
- * activations in L2 between its kernels; results do not depend on the split, with two exceptions in the last bits:
+ * activations in L2 between its kernels; results do not depend on the split, with three exceptions in the last bits:
  * a batch whose workspace holds it in one pass of the single-kernel step, and a pass whose layers run in one kernel
- * (see SRM_FLAG_NO_SMALL_BATCH), add in another order than the kernel-per-operation path; and a pass small enough
- * for its down projection to be cut along K (see SRM_FLAG_NO_KSLICE) adds that projection's partial products in
- * another order than a large pass, whatever batch it is part of. */
+ * (see SRM_FLAG_NO_SMALL_BATCH), add in another order than the kernel-per-operation path; of the passes whose layers
+ * run in one kernel, those of more than four rows per SM (592) form the sums of the norms in another order than the
+ * smaller ones; and a pass small enough for its down projection to be cut along K (see SRM_FLAG_NO_KSLICE) adds that
+ * projection's partial products in another order than a large pass, whatever batch it is part of. The cache and the
+ * logits that a prefill leaves depend in the same way on how many prompts share its pass: up to 383 go in chunks of
+ * positions, more are walked one CTA per prompt. */
 size_t srm_workspace_bytes(const srm_config* cfg, int64_t B_chunk, int32_t n_prefill_max);
 /* Workspace bytes with which srm_prefill (and its variants) processes `samples` prompts of up to n tokens in one
  * pass [Eq. 1, Eq. 3: the sequence-parallel form over all positions of a pass]. A workspace for both calls is the

@@ -333,7 +333,7 @@ __device__ __forceinline__ float gelu_fast(float v) {
 // Hands this warp's 32 rows x 128 bytes (v = the 32 words of the lane's row) to the TMA unit.
 // The staging buffer uses the 128-byte swizzle of the output tensor map: the 16-byte piece q of row r
 // sits at piece q ^ (r % 8), which also makes the eight lanes of a quarter-warp hit distinct banks.
-// Lane 0 issues the bulk operation and is the only thread that tracks its completion.
+// The elected thread (always the same one) issues the bulk operation and is the only one that tracks its completion.
 template <int EPI>
 __device__ __forceinline__ void emit_box(const CUtensorMap* tmD, uint8_t* buf, int lane, int col, int row,
                                          const uint32_t (&v)[32]) {

@@ -9,7 +9,8 @@
 //     projection's K cut into ranges), N 64 or 128, the smaller with which the tiles fit on the pairs;
 //   - row phases (x + partial products of the previous down projection, LN1, cache update, residual, LN2) are done by four
 //     warps per row (two where there are more rows than that serves at once), the rows dealt to all CTAs. With four all
-//     loads of a row are in flight at once: 2.9 -> 1.5 us per layer at 256 rows of the mid model;
+//     loads of a row are in flight at once: 2.9 -> 1.5 us per layer at 256 rows of the mid model (two warps per row spill 76 to
+//     88 bytes at d = 1536 and with combined heads at d = 1024);
 //   - the phases are ordered by counters in global memory, one per 256-row block (and range of K): rows done -> up tiles
 //     of the block start; up tiles of a range done -> down tiles of that range start; down tiles done -> rows of the
 //     block start. Nothing waits for a block it does not read.

@@ -8,7 +8,9 @@
 // What bounds it: the latency of its three phases; 524288 rows of 1024 channels take 1.43 ms, 3.7 TB/s of the 10 bytes per
 // element it moves (LN2's parameters fetched through L1 instead of kept in shared memory: 1.60 ms). One warp per prompt (the design before) walks a chain of 14000 cycles
 // per position, and with 14 prompts per SM that was the limit: 1.83 ms.
-// T = 8, two slots: 72 KB per CTA at d = 1024, three CTAs per SM, 24 rows in work and 24 in flight.
+// T = 8, two slots: 72 KB per CTA at d = 1024, three CTAs per SM, 24 rows in work and 24 in flight. Eight positions of beta per
+// thread do not quite fit beside the rest at 80 registers: 52 to 56 bytes are spilled at d = 1024, 120 at d = 1536 (fp32
+// activations 156 and 220).
 // Needs d = 128 NV (a thread per four channels, a warp per 128). The waits are bounded (status bit).
 #pragma once
 

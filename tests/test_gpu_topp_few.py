@@ -1,6 +1,7 @@
 """Top-p rows with a small nucleus (select_topp_few_kernel: the row in registers, the nucleus ranked among the few tokens
-near the maximum) against the oracle's sampler, at the edges: vocabularies that fill the registers, ties at the nucleus
-edge, as many near tokens as fit and one more, a nucleus that reaches past them, rows handed to the general kernel."""
+near the maximum) against the oracle's sampler, at the edges: vocabularies that fill the registers and one that does not fit
+(the general kernel alone), ties at the nucleus edge, as many near tokens as fit and one more, a nucleus that reaches past
+them, rows handed to the general kernel. Both kernels give the same tokens, so which of them settled a row shows in the time."""
 import numpy as np
 import pytest
 import torch
@@ -48,3 +49,35 @@ def test_small_nucleus_rows_equal_the_oracle(V):
                 assert got[r] == want[r], (step, r)
                 checked += 1
     assert checked > 0.9 * 4 * R
+
+
+def test_rows_with_few_near_tokens_are_settled_by_the_first_kernel():
+    """Rows handed on are walked by one block per SM, three to five times the time per row (3000 rows of 32000: 192 us when the
+    first kernel settles all of them, 939 through the general one): 256 near tokens must be settled in the first pass, 257 and
+    flat rows must not, in a vocabulary that fits the registers; in one that does not, no row is."""
+    import paper_2605_08696_b200 as P
+    R = 2000
+    samp = P.Sampling("topp", temperature=0.7, seed=17, sample_idx_base=50, top_p=0.9)
+
+    def us(V, near):
+        shape = custom_shape(n_layers=1, d_model=64, vocab=V, n_ctx=8, dtype="fp32", seed=3)
+        model = P.SRM(shape, I.make_weights(shape), device=DEV)
+        lg = torch.randn(R, V, generator=torch.Generator(device=DEV).manual_seed(V), device=DEV)
+        if near:
+            lg[:, 7:7 + near] = 20.0
+        tok, status = torch.zeros(R, dtype=torch.int32, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            model.k_select(lg, samp, 0, tok, status)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 1e3)
+        assert int(status.item()) == 0
+        return sorted(times[2:])[2]
+
+    few, full, over, flat = us(32000, 4), us(32000, 256), us(32000, 257), us(32000, 0)
+    assert max(few, full) < 0.6 * min(over, flat), (few, full, over, flat)
+    edge, past = us(32768, 4), us(32776, 4)
+    assert edge < 0.6 * past, (edge, past)
