@@ -19,8 +19,8 @@ __device__ __forceinline__ void raise_status(uint32_t* status, uint32_t bit) {
   if (status != nullptr) atomicOr(status, bit);
 }
 
-// Programmatic dependent launch. Every kernel of this library is launched with the programmatic
-// stream-serialization attribute: it may start while its predecessor in the stream is still draining,
+// Programmatic dependent launch. Every kernel of this library but those whose CTAs wait for one another (cooperative
+// launches) is launched with the programmatic stream-serialization attribute: it may start while its predecessor in the stream is still draining,
 // runs whatever does not touch global memory, and calls pdl_wait() before its first global access
 // (the wait returns once the predecessor grid has completed and its writes are visible). pdl_trigger()
 // lets the successor start launching; it only affects when that grid is scheduled, never its ordering.

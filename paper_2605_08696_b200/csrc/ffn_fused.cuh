@@ -124,7 +124,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmA,     // a   [M, d] bf16
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      // While the predecessor kernel drains: the weight halves of the first stages of the first item.
+      // Ahead of everything else: the weight halves of the first stages of the first item.
       int pre = 0;
       if (i0 < i1 && g.w_static && g.m_limit == nullptr) {
         const uint16_t it = plan.item[i0];

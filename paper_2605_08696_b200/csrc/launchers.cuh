@@ -8,7 +8,7 @@
 namespace {
 
 // ---- kernel launchers -------------------------------------------------------------------------
-// Every kernel goes through here: programmatic stream serialization lets the next kernel's blocks be
+// Every other kernel than those of launch_resident_kernel and SmallLaunch goes through here: programmatic stream serialization lets the next kernel's blocks be
 // scheduled and run their set-up while this one drains; each kernel orders itself with pdl_wait().
 template <typename... KArgs, typename... Args>
 cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
