@@ -337,7 +337,8 @@ bool ffn_fused_shape_ok(const srm_model& m, int64_t M) {
 // and the down projection of such a pass runs over ranges of K instead (down_k_slices). Measured on the mid model
 // (74 pairs, 20 tiles per 256 rows), ms per step, one kernel / two launches / two launches with ranges of K: 512 rows
 // 0.73 / 0.64 / 0.50, 1024: 0.76 / 0.71 / 0.59, 1536: 0.80 / 0.81 / 0.75, 2048: 0.89 / 0.93 / 0.92, 2304: 0.94 / 0.99 /
-// 0.99, 3072: 1.14 / 1.24 / -, 4096: 1.47 / 1.51 / -.
+// 0.99, 3072: 1.14 / 1.24 / -, 4096: 1.47 / 1.51 / -. As a cooperative launch, one kernel / without: 2048 rows 0.86 / 0.90, 2304:
+// 0.93 / 0.97, 3072: 1.13 / 1.19.
 bool ffn_fused_worthwhile(const srm_model& m, int64_t M) {
   const tc::FfnShape s = ffn_shape(M, m.cfg.d_model, m.F());
   return m.tc_clusters >= 2 && (int64_t)s.Rb * (s.Cu + s.Cd) >= 2 * (int64_t)m.tc_clusters;
