@@ -872,6 +872,95 @@ int launch_layers_mid(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, 
   return launch_layers_nt<6>(m, maps, p, st);
 }
 
+// ---- small decode passes: rows inside clusters of 16 CTAs, all layers in one kernel (layers_cluster.cuh) -------------
+// f(kernel, shared memory) for an instance.
+template <int D, int RC, typename Fn>
+int with_cluster_kernel_t(const srm_config& c, Fn&& f) {
+  constexpr size_t smem = cl::Shape<D, RC>::kSmem;
+  if (c.state_dtype == SRM_DTYPE_FP16) return f(cl::layers_kernel<D, RC, fp16>, smem);
+  if (c.state_dtype == SRM_DTYPE_BF16) return f(cl::layers_kernel<D, RC, bf16>, smem);
+  return f(cl::layers_kernel<D, RC, float>, smem);
+}
+// The instance whose clusters hold `rows` rows or more.
+template <typename Fn>
+int with_cluster_kernel(const srm_config& c, int rows, Fn&& f) {
+  if (c.d_model == 1024) return rows <= 8 ? with_cluster_kernel_t<1024, 8>(c, f) : with_cluster_kernel_t<1024, 16>(c, f);
+  if (rows <= 16) return with_cluster_kernel_t<512, 16>(c, f);
+  if (rows <= 32) return with_cluster_kernel_t<512, 32>(c, f);
+  return rows <= 48 ? with_cluster_kernel_t<512, 48>(c, f) : with_cluster_kernel_t<512, 64>(c, f);
+}
+struct ClusterLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  ClusterLaunch(unsigned clusters, int threads, size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3(clusters * cl::kCluster);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cl::kCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+// How many clusters of `kernel` are resident at once (0: the device cannot run it).
+template <typename K>
+int resident_clusters(K* kernel, int threads, size_t smem) {
+  int n = 0;
+  ClusterLaunch L(1, threads, smem, nullptr);
+  L.cfg.numAttrs = 1;
+  if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), cl::kSmemBytes, true) != SRM_OK ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &L.cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return n;
+}
+// Whether a decode pass of R rows takes it: bf16 models with mixed heads, F = 4 d, of 512 or 1024 channels, as many rows as the
+// clusters the device holds at once (seven on 148 SMs) have room for. us per greedy step, the layers kernel over the whole grid or
+// the single-kernel step (d = 1024, up to 32 rows) / here: d = 512, 8 layers, 72 rows 104 / 55, 112 106 / 57, 224 110 / 69,
+// 256 109 / 77, 336 117 / 83, 448 118 / 100; d = 1024, 16 layers, 8 rows 191 / 206, 16 rows 201 / 202, 24 rows 236 / 204, 56 rows
+// 245 / 206, 112 rows 260 / 221 (with 17 to 32 rows per cluster the weight ring is too short: 22.9 us per layer against 14).
+bool cluster_rows_ok(srm_model& m, int64_t R) {
+  const srm_config& c = m.cfg;
+  constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
+  if (c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || c.mixer != SRM_MIXER_MIXED || c.ffn_mult != 4) return false;
+  if (c.d_model != 512 && (c.d_model != 1024 || R <= 16)) return false;
+  if (m.row_clusters < 0)
+    m.row_clusters = with_cluster_kernel(c, 1 << 20, [](auto* kernel, size_t smem) { return resident_clusters(kernel, cl::kThreads, smem); });
+  return R <= (int64_t)m.row_clusters * (c.d_model == 1024 ? 16 : 64);
+}
+// All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
+int launch_layers_cluster(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w,
+                          cudaStream_t st, const int32_t* ctr, const int32_t* pos) {
+  const srm_config& c = m.cfg;
+  const int d = c.d_model, F = (int)m.F();
+  cl::Params p;
+  p.R = (int)R; p.V = c.vocab; p.h = c.n_heads; p.n_ctx = c.n_ctx; p.L = c.n_layers; p.t = t;
+  p.eps = c.ln_eps;
+  p.rows = (int)((R + m.row_clusters - 1) / m.row_clusters);           // spread over all clusters: fewer rows to exchange in each
+  p.tok_in = tok_in;
+  p.E = reinterpret_cast<const bf16*>(m.ptr(-1, SRM_T_E));
+  p.layer0 = layer0_weights(m);
+  p.layer_bytes = layer_stride_bytes(m);
+  p.S = static_cast<uint8_t*>(s.layer_ptr(0)) + (size_t)b0 * d * m.state_bytes();
+  p.layer_stride = (int64_t)s.B * d * m.state_bytes();
+  p.a = reinterpret_cast<bf16*>(w.a);
+  p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
+  p.status = s.status; p.ctr = ctr; p.pos = pos;
+  LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
+  CUtensorMap w1, w2;
+  int rc;
+  if ((rc = make_tmap_kblocks(&w1, m.ptr(0, SRM_T_W1), F, d, cl::kTile, 1, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
+  if ((rc = make_tmap_kblocks(&w2, m.ptr(0, SRM_T_W2), d, F, cl::kTile, 1, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
+  return with_cluster_kernel(c, p.rows, [&](auto* kernel, size_t smem) -> int {
+    int rc2 = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), cl::kSmemBytes, true);
+    if (rc2 != SRM_OK) return rc2;
+    ClusterLaunch L((unsigned)((R + p.rows - 1) / p.rows), cl::kThreads, smem, st);
+    SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, w1, w2, p));
+    return SRM_OK;
+  });
+}
+
 // One decode step for rows [b0, b0 + R) of the state.
 int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_t* tok_in, const srm_sampling& samp,
                  int step, const SelectOut& out_all, float* logits_out, const DecodeWs& w, cudaStream_t st,
@@ -885,8 +974,10 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   PartialSum ps_none, ps;
   int k_slices = 1;
   mid::Params mp;
-  const bool one_kernel = mid_plan(m, R, w, &mp);
-  if (one_kernel && (rc = launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
+  const bool clusters = mid_rows_ok(c, R) && cluster_rows_ok(m, R);
+  const bool one_kernel = clusters || mid_plan(m, R, w, &mp);
+  if (one_kernel && (rc = clusters ? launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos)
+                                   : launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
   // the down projection shares K out between CTA pairs where that is the faster kernel for R rows
   bool split = false;
   if (!one_kernel && w.order != nullptr && F % tc::BK == 0) {
@@ -1100,7 +1191,8 @@ int decode_step_impl(srm_model* m, srm_state* s, const int32_t* d_tok_in, const 
   SelectOut out{s->last_tok, d_tok_out, d_store, store_stride, store_col, 1, ctr, s->ragged ? s->pos_dev : nullptr,
                 nullptr, nullptr, samp->mode == SRM_SELECT_TOPK ? s->thr : nullptr};
   SmallPlan small;
-  if (rows >= s->B && small_step_plan(*m, *s, &small)) {
+  // (d = 512: the single-kernel step up to its 64 rows, one launch in all; d = 1024: cluster_rows_ok's rule)
+  if (rows >= s->B && !(m->cfg.d_model == 1024 && cluster_rows_ok(*m, s->B)) && small_step_plan(*m, *s, &small)) {
     rc = decode_step_small(*m, *s, small, tok_in, *samp, step, out, d_logits_out, w, st, ctr);
     if (rc != SRM_ERR_UNSUPPORTED) {
       if (rc == SRM_OK) s->pos += 1;

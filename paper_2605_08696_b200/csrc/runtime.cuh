@@ -34,6 +34,7 @@
 #include "select_topp.cuh"
 #include "step_small.cuh"
 #include "layers_mid.cuh"
+#include "layers_cluster.cuh"
 
 using namespace srm;
 
@@ -189,7 +190,8 @@ int make_tmap_kblocks(CUtensorMap* map, const void* base, int64_t rows, int64_t 
 
 // cudaFuncAttributeMaxDynamicSharedMemorySize is a per-device setting: remember which (kernel, device) pairs have
 // it, so that a model on a second device of the process gets it too. Safe from several host threads.
-int ensure_dynamic_smem(const void* func, int bytes) {
+// large_clusters: also allows clusters of more than eight CTAs.
+int ensure_dynamic_smem(const void* func, int bytes, bool large_clusters = false) {
   static std::mutex mu;
   static std::vector<std::pair<const void*, int>> done;      // (kernel, device ordinal)
   int dev = -1;
@@ -198,6 +200,7 @@ int ensure_dynamic_smem(const void* func, int bytes) {
   for (const auto& e : done)
     if (e.first == func && e.second == dev) return SRM_OK;
   SRM_CUDA(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  if (large_clusters) SRM_CUDA(cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   done.emplace_back(func, dev);
   return SRM_OK;
 }
@@ -219,6 +222,7 @@ struct srm_model {
   bool head_proj() const { return (cfg.flags & SRM_FLAG_HEAD_PROJ) != 0; }
   bool tc_ready = false;                 // smem attribute set for the tensor-core kernels
   int small_clusters = -1;               // clusters of the small-batch step kernel that are resident at once (-1: not asked yet)
+  int row_clusters = -1;                 // clusters of 16 CTAs of the cluster layers kernel that are resident at once (-1: not asked yet)
   int tc_clusters = 0;                   // CTA pairs of the tensor-core kernel that are resident at once
   std::vector<TmapCacheEntry> tmaps;     // weight and activation descriptors, built on first use
   std::vector<std::pair<int, tc::FfnPlan>> ffn_plans;   // work lists of the fused feed-forward kernel, by row blocks

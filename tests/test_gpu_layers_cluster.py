@@ -1,0 +1,74 @@
+"""Decode passes in clusters of 16 CTAs. Rows inside one cluster (layers_cluster.cuh), at the edges of its rows per cluster (8, 16, 32, 48,
+64 times the seven clusters of the device): logits, tokens and cache against the kernel-per-operation path fed the
+same tokens, rows of the batch against the oracle, equal and per-sample positions, all cache types."""
+import numpy as np
+import pytest
+import torch
+
+import srm_inputs as I
+from helpers import custom_shape, oracle_for, rel_err_rows, top2_margin
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("B,d,layers,state_dtype,ragged", [
+    (17, 1024, 3, "fp16", False), (25, 1024, 2, "fp32", False), (32, 1024, 3, "fp32", True), (33, 1024, 3, "bf16", False),
+    (111, 512, 3, "fp32", False), (113, 512, 3, "fp16", True), (224, 512, 3, "bf16", False), (225, 512, 3, "fp32", True), (336, 512, 3, "fp16", False),
+    (337, 512, 3, "fp32", False), (448, 512, 3, "fp32", True), (449, 512, 3, "fp32", False), (56, 1024, 3, "fp32", True),
+    (57, 1024, 3, "fp32", False), (100, 1024, 3, "bf16", True), (112, 1024, 3, "fp16", False)])
+def test_rows_in_clusters_agree_with_the_kernel_per_operation_path(B, d, layers, state_dtype, ragged):
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=layers, d_model=d, vocab=2048, n_ctx=24, dtype="bf16", seed=19)
+    W = I.make_weights(shape)
+    rng = np.random.default_rng(B)
+    n = 5
+    prompts_np = rng.integers(0, shape.vocab, size=(B, n)).astype(np.int32)
+    lens_np = rng.integers(1, n + 1, size=B).astype(np.int32) if ragged else np.full(B, n, np.int32)
+    fed = torch.from_numpy(rng.integers(0, shape.vocab, size=(3, B)).astype(np.int32)).to(DEV)
+    prompts, lens = torch.from_numpy(prompts_np).to(DEV), torch.from_numpy(lens_np).to(DEV)
+    g = P.Sampling("greedy")
+    outs = []
+    for flags in (P.FLAG_NO_SMALL_BATCH, 0):
+        m = P.SRM(shape, W, device=DEV, flags=flags, state_dtype=state_dtype)
+        st, ws = m.new_state(B), m.new_workspace(B, n, prefill_samples=B)
+        m.prefill_ragged(st, prompts, lens, g, ws) if ragged else m.prefill(st, prompts, g, ws)
+        lgs, toks = [], []
+        for k in range(3):
+            tok, lg = m.decode_step(st, fed[k], g, k + 1, ws, want_logits=True)
+            lgs.append(lg.cpu().numpy())
+            toks.append(tok.cpu().numpy())
+        assert st.status() == 0
+        outs.append((np.stack(lgs), np.stack(toks), st.cache().cpu().float().numpy()))
+    (lg_a, tok_a, S_a), (lg_b, tok_b, S_b) = outs
+    # Sums in another order flip roundings of bf16 activations, 2^-8 of the value each. Were half of them flipped, a
+    # layer would move its output by 2^-9 of its scale, all layers by 2^-9 sqrt(layers); five standard deviations of that:
+    tol = 5 * 2.0 ** -9 * layers ** 0.5
+    assert rel_err_rows(lg_b, lg_a) < tol and rel_err_rows(S_b, S_a) < tol
+    assert np.all(top2_margin(lg_a)[tok_a != tok_b] < 2e-2)
+    orc = oracle_for(shape, W)
+    for b in (0, B // 2, B - 1):
+        lo, state = orc.forward_parallel(prompts_np[b:b + 1, :lens_np[b]])
+        for k in range(3):
+            lo, state = orc.decode_step(state, fed[k, b:b + 1].cpu().numpy(), int(lens_np[b]) + k)
+            assert rel_err_rows(lg_b[k][b:b + 1], lo) < 3e-2
+
+
+def test_a_row_has_the_same_bits_in_any_pass():
+    """300 rows at d = 512 in one pass, in passes of 100 and backwards: bit-equal (instances of the kernel for 16 and 48 rows)."""
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=2, d_model=512, vocab=1024, n_ctx=16, dtype="bf16", seed=20)
+    W = I.make_weights(shape)
+    B = 300
+    toks = torch.from_numpy(np.random.default_rng(4).integers(0, shape.vocab, size=(4, B)).astype(np.int32)).to(DEV)
+    g = P.Sampling("greedy")
+    res = []
+    for order, chunk in ((1, B), (1, 100), (-1, B)):
+        m = P.SRM(shape, W, device=DEV)
+        st, ws = m.new_state(B), m.new_workspace(chunk)
+        lgs = [m.decode_step(st, (t if order > 0 else t.flip(0)).contiguous(), g, k + 1, ws, want_logits=True)[1].clone() for k, t in enumerate(toks)]
+        assert st.status() == 0
+        res.append([lg if order > 0 else lg.flip(0) for lg in lgs] + [st.cache() if order > 0 else st.cache().flip(1)])
+    for r in res[1:]:
+        for x, y in zip(res[0], r):
+            assert torch.equal(x, y)
