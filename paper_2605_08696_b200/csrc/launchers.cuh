@@ -892,15 +892,21 @@ int with_cluster_kernel(const srm_config& c, int rows, Fn&& f) {
 struct ClusterLaunch {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
-  ClusterLaunch(unsigned clusters, int threads, size_t smem, cudaStream_t st) {
+  // resident: all CTAs at once (a cooperative launch), for kernels whose clusters wait for one another
+  ClusterLaunch(unsigned clusters, int threads, size_t smem, cudaStream_t st, bool resident) {
     cfg.gridDim = dim3(clusters * cl::kCluster);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cl::kCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    if (resident) {
+      attr[1].id = cudaLaunchAttributeCooperative;
+      attr[1].val.cooperative = 1;
+    } else {
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
+    }
     cfg.attrs = attr;
     cfg.numAttrs = 2;
   }
@@ -909,7 +915,7 @@ struct ClusterLaunch {
 template <typename K>
 int resident_clusters(K* kernel, int threads, size_t smem) {
   int n = 0;
-  ClusterLaunch L(1, threads, smem, nullptr);
+  ClusterLaunch L(1, threads, smem, nullptr, false);
   L.cfg.numAttrs = 1;
   if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), cl::kSmemBytes, true) != SRM_OK ||
       cudaOccupancyMaxActiveClusters(&n, kernel, &L.cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
@@ -955,7 +961,65 @@ int launch_layers_cluster(srm_model& m, srm_state& s, int64_t b0, int64_t R, int
   return with_cluster_kernel(c, p.rows, [&](auto* kernel, size_t smem) -> int {
     int rc2 = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), cl::kSmemBytes, true);
     if (rc2 != SRM_OK) return rc2;
-    ClusterLaunch L((unsigned)((R + p.rows - 1) / p.rows), cl::kThreads, smem, st);
+    ClusterLaunch L((unsigned)((R + p.rows - 1) / p.rows), cl::kThreads, smem, st, false);
+    SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, w1, w2, p));
+    return SRM_OK;
+  });
+}
+
+// ---- a few rows: weights split between clusters of 16 CTAs, all layers in one kernel (layers_split.cuh) -------------
+template <bool ALONE, typename Fn>
+int with_split_kernel_t(const srm_config& c, Fn&& f) {
+  constexpr size_t smem = sp::Shape<1024>::kSmem;
+  if (c.state_dtype == SRM_DTYPE_FP16) return f(sp::layers_kernel<1024, ALONE, fp16>, smem);
+  if (c.state_dtype == SRM_DTYPE_BF16) return f(sp::layers_kernel<1024, ALONE, bf16>, smem);
+  return f(sp::layers_kernel<1024, ALONE, float>, smem);
+}
+template <typename Fn>
+int with_split_kernel(const srm_config& c, int64_t R, Fn&& f) {
+  return R == 1 ? with_split_kernel_t<true>(c, f) : with_split_kernel_t<false>(c, f);
+}
+// Whether a decode pass of R rows takes it: bf16 models with mixed heads, F = 4 d, 1024 channels, up to 16 rows. us per greedy step of 16
+// layers, the single-kernel step / here: 1 row 181 / 150, 4 rows 186 / 154, 8 rows 190 / 159, 16 rows 202 / 165; with 27 rows (two
+// 16-row tiles, two rows per owner) it took 308, rows inside clusters 205. The words of the planes lie in the area of the
+// partial products.
+bool split_rows_ok(srm_model& m, int64_t R, const DecodeWs& w) {
+  const srm_config& c = m.cfg;
+  constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
+  if (c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || c.mixer != SRM_MIXER_MIXED || c.ffn_mult != 4 || c.d_model != 1024 || R > sp::kMaxRows) return false;
+  if (m.split_clusters < 0)
+    m.split_clusters = with_split_kernel(c, 32, [](auto* kernel, size_t smem) { return resident_clusters(kernel, sp::kThreads, smem); });
+  return m.split_clusters >= sp::kClusters && w.part != nullptr && sp::plane_bytes(R, c.d_model) <= w.part_bytes;
+}
+// All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
+int launch_layers_split(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w,
+                        cudaStream_t st, const int32_t* ctr, const int32_t* pos) {
+  const srm_config& c = m.cfg;
+  const int d = c.d_model, F = (int)m.F();
+  sp::Params p;
+  p.R = (int)R; p.V = c.vocab; p.h = c.n_heads; p.n_ctx = c.n_ctx; p.L = c.n_layers; p.t = t;
+  p.eps = c.ln_eps;
+  p.tok_in = tok_in;
+  p.E = reinterpret_cast<const bf16*>(m.ptr(-1, SRM_T_E));
+  p.layer0 = layer0_weights(m);
+  p.layer_bytes = layer_stride_bytes(m);
+  p.S = static_cast<uint8_t*>(s.layer_ptr(0)) + (size_t)b0 * d * m.state_bytes();
+  p.layer_stride = (int64_t)s.B * d * m.state_bytes();
+  p.a = reinterpret_cast<bf16*>(w.a);
+  p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
+  p.planes = reinterpret_cast<unsigned long long*>(w.part);
+  p.cnt = reinterpret_cast<uint32_t*>(w.small);
+  p.status = s.status; p.ctr = ctr; p.pos = pos;
+  SRM_CUDA(cudaMemsetAsync(w.small, 0, 256, st));
+  LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
+  CUtensorMap w1, w2;
+  int rc;
+  if ((rc = make_tmap_layers(&w1, m.ptr(0, SRM_T_W1), F, d, sp::Shape<1024>::kUpTiles * 8, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
+  if ((rc = make_tmap_layers(&w2, m.ptr(0, SRM_T_W2), d, F, d / sp::kCluster, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
+  return with_split_kernel(c, R, [&](auto* kernel, size_t smem) -> int {
+    int rc2 = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), sp::kSmemBytes, true);
+    if (rc2 != SRM_OK) return rc2;
+    ClusterLaunch L(sp::kClusters, sp::kThreads, smem, st, true);
     SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, w1, w2, p));
     return SRM_OK;
   });
@@ -974,10 +1038,11 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   PartialSum ps_none, ps;
   int k_slices = 1;
   mid::Params mp;
-  const bool clusters = mid_rows_ok(c, R) && cluster_rows_ok(m, R);
-  const bool one_kernel = clusters || mid_plan(m, R, w, &mp);
-  if (one_kernel && (rc = clusters ? launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos)
-                                   : launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
+  const bool splits = split_rows_ok(m, R, w), clusters = !splits && mid_rows_ok(c, R) && cluster_rows_ok(m, R);
+  const bool one_kernel = splits || clusters || mid_plan(m, R, w, &mp);
+  if (one_kernel && (rc = splits     ? launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos)
+                          : clusters ? launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos)
+                                     : launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
   // the down projection shares K out between CTA pairs where that is the faster kernel for R rows
   bool split = false;
   if (!one_kernel && w.order != nullptr && F % tc::BK == 0) {
@@ -1192,7 +1257,7 @@ int decode_step_impl(srm_model* m, srm_state* s, const int32_t* d_tok_in, const 
                 nullptr, nullptr, samp->mode == SRM_SELECT_TOPK ? s->thr : nullptr};
   SmallPlan small;
   // (d = 512: the single-kernel step up to its 64 rows, one launch in all; d = 1024: cluster_rows_ok's rule)
-  if (rows >= s->B && !(m->cfg.d_model == 1024 && cluster_rows_ok(*m, s->B)) && small_step_plan(*m, *s, &small)) {
+  if (rows >= s->B && !(m->cfg.d_model == 1024 && (split_rows_ok(*m, s->B, w) || cluster_rows_ok(*m, s->B))) && small_step_plan(*m, *s, &small)) {
     rc = decode_step_small(*m, *s, small, tok_in, *samp, step, out, d_logits_out, w, st, ctr);
     if (rc != SRM_ERR_UNSUPPORTED) {
       if (rc == SRM_OK) s->pos += 1;

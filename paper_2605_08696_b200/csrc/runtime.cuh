@@ -35,6 +35,7 @@
 #include "step_small.cuh"
 #include "layers_mid.cuh"
 #include "layers_cluster.cuh"
+#include "layers_split.cuh"
 
 using namespace srm;
 
@@ -188,6 +189,20 @@ int make_tmap_kblocks(CUtensorMap* map, const void* base, int64_t rows, int64_t 
   return SRM_OK;
 }
 
+// The bf16 matrix [rows, cols] of `layers` layers, `stride` bytes apart, as {cols, rows, layers}; the box is 64 columns x box_rows.
+int make_tmap_layers(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows, int layers, int64_t stride) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (fn == nullptr) { g_last_cuda_error = (int)cudaErrorNotSupported; return SRM_ERR_CUDA; }
+  cuuint64_t gdim[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)layers};
+  cuuint64_t gstride[2] = {(cuuint64_t)cols * 2, layers > 1 ? (cuuint64_t)stride : (cuuint64_t)(cols * rows * 2)};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) { g_last_cuda_error = 10000 + (int)r; return SRM_ERR_CUDA; }
+  return SRM_OK;
+}
+
 // cudaFuncAttributeMaxDynamicSharedMemorySize is a per-device setting: remember which (kernel, device) pairs have
 // it, so that a model on a second device of the process gets it too. Safe from several host threads.
 // large_clusters: also allows clusters of more than eight CTAs.
@@ -223,6 +238,7 @@ struct srm_model {
   bool tc_ready = false;                 // smem attribute set for the tensor-core kernels
   int small_clusters = -1;               // clusters of the small-batch step kernel that are resident at once (-1: not asked yet)
   int row_clusters = -1;                 // clusters of 16 CTAs of the cluster layers kernel that are resident at once (-1: not asked yet)
+  int split_clusters = -1;               // the same of the kernel with its weights split between clusters
   int tc_clusters = 0;                   // CTA pairs of the tensor-core kernel that are resident at once
   std::vector<TmapCacheEntry> tmaps;     // weight and activation descriptors, built on first use
   std::vector<std::pair<int, tc::FfnPlan>> ffn_plans;   // work lists of the fused feed-forward kernel, by row blocks

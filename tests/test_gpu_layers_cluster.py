@@ -1,5 +1,6 @@
 """Decode passes in clusters of 16 CTAs. Rows inside one cluster (layers_cluster.cuh), at the edges of its rows per cluster (8, 16, 32, 48,
-64 times the seven clusters of the device): logits, tokens and cache against the kernel-per-operation path fed the
+64 times the seven clusters of the device); a few rows with the weights split between the clusters (layers_split.cuh: up to
+16 and up to 32 rows, one, two and three layers): logits, tokens and cache against the kernel-per-operation path fed the
 same tokens, rows of the batch against the oracle, equal and per-sample positions, all cache types."""
 import numpy as np
 import pytest
@@ -13,6 +14,7 @@ DEV = "cuda:0"
 
 
 @pytest.mark.parametrize("B,d,layers,state_dtype,ragged", [
+    (1, 1024, 3, "fp32", False), (2, 1024, 1, "fp16", False), (8, 1024, 2, "fp32", True), (9, 1024, 3, "bf16", False), (16, 1024, 3, "fp16", True),
     (17, 1024, 3, "fp16", False), (25, 1024, 2, "fp32", False), (32, 1024, 3, "fp32", True), (33, 1024, 3, "bf16", False),
     (111, 512, 3, "fp32", False), (113, 512, 3, "fp16", True), (224, 512, 3, "bf16", False), (225, 512, 3, "fp32", True), (336, 512, 3, "fp16", False),
     (337, 512, 3, "fp32", False), (448, 512, 3, "fp32", True), (449, 512, 3, "fp32", False), (56, 1024, 3, "fp32", True),
