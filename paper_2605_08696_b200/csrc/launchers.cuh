@@ -746,10 +746,9 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
 }
 
 // ---- decode passes of up to about a thousand rows: all layers in one kernel (layers_mid.cuh) -------------
-// Fewest rows, where the whole step is not one kernel of another design (step_small.cuh: up to 64 rows at d = 512, 32 at
-// d = 1024; us per step there / here: mid 1 row 181 / 239, 27 rows 241 / 246, 32 rows 250 / 244; small 27 rows 87 / 98, 64 rows
-// 111 / 100). d = 512: a batch just past that limit, 65 to 71 rows, keeps the kernel-per-operation path, which its tests count on
-// (138 us at 72 rows there, 104 here); up to 64 rows come here only where the single-kernel step does not take F (as kMixedAny).
+// Fewest rows, where the passes are not those of another kernel (cluster_rows_ok and split_rows_ok come first; step_small.cuh where
+// F is not 4 d). d = 512: 65 to 71 rows keep the kernel-per-operation path, which tests count on (138 us at 72 rows there, 104
+// here, 52 in clusters); up to 64 rows come here only where the single-kernel step does not take F (as kMixedAny).
 // Combined heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96 rows, d = 1024, 16 layers, kernels of
 // size 4: 275 us per step, as a kernel per operation 560).
 bool mid_rows_ok(const srm_config& c, int64_t R) { return c.d_model != 512 || c.mixer != SRM_MIXER_MIXED || R <= sb::kMaxRows || R >= 72; }
@@ -923,8 +922,9 @@ int resident_clusters(K* kernel, int threads, size_t smem) {
 }
 // Whether a decode pass of R rows takes it: bf16 models with mixed heads, F = 4 d, of 512 or 1024 channels, as many rows as the
 // clusters the device holds at once (seven on 148 SMs) have room for. us per greedy step, the layers kernel over the whole grid or
-// the single-kernel step (d = 1024, up to 32 rows) / here: d = 512, 8 layers, 72 rows 104 / 55, 112 106 / 57, 224 110 / 69,
-// 256 109 / 77, 336 117 / 83, 448 118 / 100; d = 1024, 16 layers, 8 rows 191 / 206, 16 rows 201 / 202, 24 rows 236 / 204, 56 rows
+// the single-kernel step (up to 64 rows at d = 512, 32 at d = 1024) / here: d = 512, 8 layers, V = 8000, 1 row 73 / 49, 16 rows
+// 77 / 50, 64 rows 113 / 51, 72 rows 104 / 52, 112 106 / 54, 224 110 / 67, 256 109 / 77, 336 117 / 82, 448 118 / 102 (with LM head and
+// selection as kernels of their own 55, 57, 69, 77, 83, 100 from 72 rows on); d = 1024, 16 layers, 8 rows 191 / 206, 16 rows 201 / 202, 24 rows 236 / 204, 56 rows
 // 245 / 206, 112 rows 260 / 221 (with 17 to 32 rows per cluster the weight ring is too short: 22.9 us per layer against 14).
 bool cluster_rows_ok(srm_model& m, int64_t R) {
   const srm_config& c = m.cfg;
@@ -936,8 +936,9 @@ bool cluster_rows_ok(srm_model& m, int64_t R) {
   return R <= (int64_t)m.row_clusters * (c.d_model == 1024 ? 16 : 64);
 }
 // All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
+// out: LM head and greedy selection in the same kernel (d = 512), or nullptr.
 int launch_layers_cluster(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w,
-                          cudaStream_t st, const int32_t* ctr, const int32_t* pos) {
+                          cudaStream_t st, const int32_t* ctr, const int32_t* pos, const SelectOut* out) {
   const srm_config& c = m.cfg;
   const int d = c.d_model, F = (int)m.F();
   cl::Params p;
@@ -954,15 +955,17 @@ int launch_layers_cluster(srm_model& m, srm_state& s, int64_t b0, int64_t R, int
   p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
   p.status = s.status; p.ctr = ctr; p.pos = pos;
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
-  CUtensorMap w1, w2;
+  if (out != nullptr) { p.head = 1; p.out = *out; }
+  CUtensorMap w1, w2, lm;
   int rc;
   if ((rc = make_tmap_kblocks(&w1, m.ptr(0, SRM_T_W1), F, d, cl::kTile, 1, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = make_tmap_kblocks(&w2, m.ptr(0, SRM_T_W2), d, F, cl::kTile, 1, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
+  if ((rc = make_tmap_kblocks(&lm, m.ptr(-1, SRM_T_W_LM), c.vocab, d, cl::kTile, 1, 1)) != SRM_OK) return rc;
   return with_cluster_kernel(c, p.rows, [&](auto* kernel, size_t smem) -> int {
     int rc2 = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), cl::kSmemBytes, true);
     if (rc2 != SRM_OK) return rc2;
     ClusterLaunch L((unsigned)((R + p.rows - 1) / p.rows), cl::kThreads, smem, st, false);
-    SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, w1, w2, p));
+    SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, w1, w2, lm, p));
     return SRM_OK;
   });
 }
@@ -1038,11 +1041,19 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   PartialSum ps_none, ps;
   int k_slices = 1;
   mid::Params mp;
+  SelectOut o = out_all;
+  o.last_tok += b0;
+  if (o.tok_out) o.tok_out += b0;
+  if (o.store) o.store += b0 * o.store_stride;
+  if (o.pos) o.pos += b0;
+  if (o.thr_out) o.thr_out += b0;
   const bool splits = split_rows_ok(m, R, w), clusters = !splits && mid_rows_ok(c, R) && cluster_rows_ok(m, R);
+  const bool head = clusters && cl::has_head(d) && can_fuse_greedy(m, samp, logits_out);      // the selection, too
   const bool one_kernel = splits || clusters || mid_plan(m, R, w, &mp);
   if (one_kernel && (rc = splits     ? launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos)
-                          : clusters ? launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos)
+                          : clusters ? launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr)
                                      : launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
+  if (head) return SRM_OK;
   // the down projection shares K out between CTA pairs where that is the faster kernel for R rows
   bool split = false;
   if (!one_kernel && w.order != nullptr && F % tc::BK == 0) {
@@ -1107,12 +1118,6 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   }
   if (ps.part != nullptr) ps.bias = m.fptr(c.n_layers - 1, SRM_T_B2);
   if (!one_kernel && (rc = launch_final_norm(m, w.x, R, 1, 0, w.a, st, nullptr, ps))) return rc;
-  SelectOut o = out_all;
-  o.last_tok += b0;
-  if (o.tok_out) o.tok_out += b0;
-  if (o.store) o.store += b0 * o.store_stride;
-  if (o.pos) o.pos += b0;
-  if (o.thr_out) o.thr_out += b0;
   if (can_fuse_greedy(m, samp, logits_out)) return launch_lm_head_greedy(m, R, w.a, w.logits, o, s.status, st);
   if (can_fuse_topk(m, samp, logits_out))
     return launch_lm_head_topk(m, R, w.a, w.logits, w.H, s.thr + b0, samp, samp.sample_idx_base + (uint64_t)b0, step, o,
@@ -1256,8 +1261,7 @@ int decode_step_impl(srm_model* m, srm_state* s, const int32_t* d_tok_in, const 
   SelectOut out{s->last_tok, d_tok_out, d_store, store_stride, store_col, 1, ctr, s->ragged ? s->pos_dev : nullptr,
                 nullptr, nullptr, samp->mode == SRM_SELECT_TOPK ? s->thr : nullptr};
   SmallPlan small;
-  // (d = 512: the single-kernel step up to its 64 rows, one launch in all; d = 1024: cluster_rows_ok's rule)
-  if (rows >= s->B && !(m->cfg.d_model == 1024 && (split_rows_ok(*m, s->B, w) || cluster_rows_ok(*m, s->B))) && small_step_plan(*m, *s, &small)) {
+  if (rows >= s->B && !split_rows_ok(*m, s->B, w) && !cluster_rows_ok(*m, s->B) && small_step_plan(*m, *s, &small)) {
     rc = decode_step_small(*m, *s, small, tok_in, *samp, step, out, d_logits_out, w, st, ctr);
     if (rc != SRM_ERR_UNSUPPORTED) {
       if (rc == SRM_OK) s->pos += 1;

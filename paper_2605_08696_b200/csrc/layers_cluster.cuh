@@ -25,6 +25,10 @@
 // A row's bits depend on neither its place in the pass nor the number of rows: every output is one fixed sequence of
 // 16-deep tensor steps, and N columns of an instruction do not mix.
 //
+// At d = 512 the LM head and the greedy selection follow in the same kernel (where the caller wants nothing else): 128 vocabulary rows
+// per tile, every 16th tile per rank, the best logit of a row from every rank to its owner. A kernel of its own for each
+// takes longer to start than to run.
+//
 // No buffer needs a "free" signal of its own: an owner sends the next layer's activations after it has received every CTA's
 // partial products, a CTA sends those after its last tensor instruction of the layer has completed, and everything a
 // CTA sends in a layer is sent after all activations of that layer have come. For the same reason no byte of a layer can
@@ -37,7 +41,8 @@
 
 #include "common.cuh"
 #include "gemm_tc.cuh"
-#include "step_small.cuh"   // LayerW, layer_w, bulk_s2s
+#include "select.cuh"       // SelectOut, write_token
+#include "step_small.cuh"   // LayerW, layer_w, bulk_s2s, st_async_v2, pack_best
 
 namespace srm {
 namespace cl {
@@ -68,7 +73,10 @@ struct Params {
   uint32_t* status;
   const int32_t* ctr;            // device-side step counters or nullptr
   const int32_t* pos;            // [R] per-row positions or nullptr
+  int head = 0;                  // D = 512: LM head and greedy selection here, to `out`; else the final norm's rows to `a`
+  SelectOut out = {};
 };
+__host__ __device__ constexpr bool has_head(int d) { return d == 512; }
 
 // Shared memory: activations [k-block][row][128 bytes] | H of the K-group, the same | partial products received
 // [K-group][column][tile][own row][128] | weight ring | barriers | row-phase sums. The partial products sent are staged in the
@@ -182,7 +190,8 @@ __device__ __forceinline__ void row_stats(const float4& v, float eps, float* slo
 
 template <int D, int RC, typename ST>
 __global__ void __launch_bounds__(kThreads, 1)
-layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2, const Params p) {
+layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmLm,
+              const Params p) {
   pdl_trigger();
   using C = Shape<D, RC>;
   constexpr int kUp = C::kUpTiles, kDn = C::kDnTiles, kKb = C::kKb, kOwn = C::kOwn, kRowWarps = C::kRowWarps;
@@ -200,9 +209,10 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
   uint64_t* up_done = recv_full + 1;                                     // [kUp] accumulators
   uint64_t* dn_done = up_done + kUp;                                     // [kDn]
   uint64_t* h_full = dn_done + kDn;                                      // [column of the K-group][tile]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(h_full + kCols * kUp);
+  uint64_t* head_empty = h_full + kCols * kUp;                           // [2] accumulators of the LM head drained
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(head_empty + 2);
   float* sums = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(fullW) + kBarrierBytes);
-  static_assert((2 * kMaxSlots + 5 + kUp + kDn + kCols * kUp) * 8 + 4 <= kBarrierBytes, "barriers");
+  static_assert((2 * kMaxSlots + 7 + kUp + kDn + kCols * kUp) * 8 + 4 <= kBarrierBytes, "barriers");
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int rank = (int)tc::cluster_ctarank();
@@ -217,6 +227,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
     for (int i = 0; i < kUp; ++i) tc::mbar_init(&up_done[i], kIssuers);
     for (int i = 0; i < kDn; ++i) tc::mbar_init(&dn_done[i], kIssuers);
     for (int i = 0; i < kCols * kUp; ++i) tc::mbar_init(&h_full[i], 1);
+    for (int i = 0; i < 2; ++i) tc::mbar_init(&head_empty[i], kWorkerWarps);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -228,6 +239,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot;                                      // up tiles, then down tiles, an accumulator per issuer each
   bool ok = true;                                                        // no wait has given up in this thread
+  const bool head_here = has_head(D) && p.head != 0;
+  const int head_tiles = head_here ? (p.V + kTile - 1) / kTile : 0;      // tiles rank, rank + 16, ... are this CTA's
 
   if (warp == 0) {
     // ---------------- weight stream: constant data, it waits for nothing but its ring ----------------
@@ -246,6 +259,16 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
                      dn ? (ng * kDn + tile - kUp) * kTile : ((kg * kCols + ng) * kUp + tile) * kTile,
                      dn ? kg * kKb + down_kb<kUp, kKb>(kb, ng) : kb, l);
           if (++slot == C::kSlots) { slot = 0; phase ^= 1u; }
+        }
+      }
+      if constexpr (has_head(D)) {
+        for (int tile = rank; ok && tile < head_tiles; tile += kCluster) {
+          for (int kb = 0; kb < kKb; ++kb) {
+            if (!tc::mbar_wait(&emptyW[slot], phase ^ 1u, p.status)) { ok = false; break; }
+            tc::mbar_expect_tx(&fullW[slot], kSlotBytes);
+            tma_load_w(sW + slot * kSlotBytes, &tmLm, &fullW[slot], tile * kTile, kb, 0);
+            if (++slot == C::kSlots) { slot = 0; phase ^= 1u; }
+          }
         }
       }
     }
@@ -297,6 +320,22 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
             if (ok) k_block(acc, sH + kb * kRowBytes, i == mine);
           }
           if (ok) umma_commit(&dn_done[m]);
+        }
+      }
+      if constexpr (has_head(D)) {
+        if (head_here && ok) {
+          if (mine == 0)
+            for (int i = 0; i < 4; ++i) tc::mbar_expect_tx(&act_full[i], (uint32_t)(rows * D / 2));
+          for (int i = 0; ok && i < 4; ++i) ok = tc::mbar_wait(&act_full[i], (uint32_t)(p.L & 1), p.status);
+          tc::fence_async_smem();
+          int n = 0;
+          for (int tile = rank; ok && tile < head_tiles; tile += kCluster, ++n) {
+            if (n >= 2) ok = tc::mbar_wait(&head_empty[n & 1], (uint32_t)((n >> 1) - 1) & 1u, p.status);
+            tc::tc_fence_after();
+            const uint32_t acc = tmem + ((n & 1) * kIssuers + mine) * C::kN;
+            for (int kb = mine; ok && kb < kKb; kb += kIssuers) k_block(acc, sA + kb * kRowBytes, kb == mine);
+            if (ok) umma_commit(n & 1 ? &dn_done[0] : &up_done[0]);
+          }
         }
       }
     }
@@ -380,7 +419,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
         const float nmr2 = -mean * rstd;
         const float4 o = make_float4(fmaf(fmaf(v.x, rstd, nmr2), g2.x, h2.x), fmaf(fmaf(v.y, rstd, nmr2), g2.y, h2.y),
                                      fmaf(fmaf(v.z, rstd, nmr2), g2.z, h2.z), fmaf(fmaf(v.w, rstd, nmr2), g2.w, h2.w));
-        if (last) {
+        if (last && !head_here) {
           st4(p.a + (int64_t)row * D + c0, o);
         } else {
           const __nv_bfloat162 lo = __floats2bfloat162_rn(o.x, o.y), hi = __floats2bfloat162_rn(o.z, o.w);
@@ -459,6 +498,83 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
         if (n > 0 && tc::elect_one())
           sb::bulk_s2s(tc::mapa(tc::smem_u32(recv + ((kg * kCols + ng) * kDn + m) * kOwn * kTile), (uint32_t)to), stage + to * kOwn * kTile,
                        n * kTile * 4, tc::mapa(tc::smem_u32(recv_full), (uint32_t)to));
+      }
+    }
+  }
+
+  if constexpr (has_head(D)) {
+    if (head_here && warp >= kWorker0) {
+      // ---- LM head: the largest logit of each row (lowest column among equals), in a thread over its columns, then over the lanes,
+      //      the warps, and by the row's owner over the ranks ----
+      const int wid = threadIdx.x - kWorker0 * 32, ww = wid >> 5, quad = warp & 3, cgrp = ww >> 2;
+      unsigned long long* best = reinterpret_cast<unsigned long long*>(recv);                     // [RC]
+      unsigned long long* slots = best + 64;                                                      // [own row][rank]
+      const int own = rows_of(rank);
+      if (wid == 0 && own > 0) tc::mbar_expect_tx(recv_full, (uint32_t)(own * kCluster * 8));
+      float bv[kOwn][4];
+      int bi[kOwn][4];
+      bool bad = false;
+#pragma unroll
+      for (int g = 0; g < kOwn; ++g)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { bv[g][j] = -INFINITY; bi[g][j] = -1; }
+      int n = 0;
+      for (int tile = rank; tile < head_tiles; tile += kCluster, ++n) {
+        if (ok) ok = tc::mbar_wait(n & 1 ? &dn_done[0] : &up_done[0], (uint32_t)(p.L + (n >> 1)) & 1u, p.status);
+        tc::tc_fence_after();
+        if (cgrp * 4 < RC) {
+          float acc[kOwn][4];
+          take_tile<kOwn>(tmem + (static_cast<uint32_t>(quad * 32) << 16) + (uint32_t)((n & 1) * kIssuers * C::kN + cgrp * 4), C::kN, acc);
+          const int col = tile * kTile + quad * 32 + lane;
+          if (col < p.V && ok) {
+#pragma unroll
+            for (int g = 0; g < kOwn; ++g)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                bad |= g * kCluster + cgrp * 4 + j < rows && !(acc[g][j] == acc[g][j]);
+                if (acc[g][j] > bv[g][j]) { bv[g][j] = acc[g][j]; bi[g][j] = col; }              // (ascending columns)
+              }
+          }
+        }
+        tc::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&head_empty[n & 1]);
+      }
+      if (bad) raise_status(p.status, kStatusNonFinite);
+      workers_sync();                                                    // (the partial products that lay here have been read)
+      for (int i = wid; i < RC; i += kWorkers) best[i] = 0ull;
+      workers_sync();
+      if (cgrp * 4 < RC) {
+#pragma unroll
+        for (int g = 0; g < kOwn; ++g)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            unsigned long long k = bi[g][j] < 0 ? 0ull : sb::pack_best(bv[g][j] + 0.0f, bi[g][j]);      // (minus zero equals zero)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, k, o);
+              k = k2 > k ? k2 : k;
+            }
+            if (lane == 0 && k != 0ull) atomicMax(&best[g * kCluster + cgrp * 4 + j], k);
+          }
+      }
+      workers_sync();
+      if (wid < rows) {                                                  // row wid: to its owner
+        const uint32_t to = (uint32_t)(wid % kCluster);
+        const unsigned long long k = best[wid];
+        sb::st_async_v2(tc::mapa(tc::smem_u32(slots + (wid / kCluster) * kCluster + rank), to), __uint_as_float((uint32_t)k),
+                        __uint_as_float((uint32_t)(k >> 32)), tc::mapa(tc::smem_u32(recv_full), to));
+      }
+      if (wid < own) {
+        if (ok) ok = tc::mbar_wait(recv_full, (uint32_t)(p.L & 1), p.status, kWaitLimitCycles);
+        unsigned long long k = 0ull;
+        for (int r = 0; r < kCluster; ++r) {
+          const unsigned long long k2 = slots[wid * kCluster + r];
+          k = k2 > k ? k2 : k;
+        }
+        int tok = k == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)k);      // (no finite logit: 0)
+        if (tok < 0 || tok >= p.V) tok = 0;
+        write_token(p.out, row_base + wid * kCluster + rank, tok);
       }
     }
   }

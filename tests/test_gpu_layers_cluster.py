@@ -74,3 +74,28 @@ def test_a_row_has_the_same_bits_in_any_pass():
     for r in res[1:]:
         for x, y in zip(res[0], r):
             assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("B,vocab", [(1, 1000), (7, 2056), (16, 128), (64, 8000), (113, 136), (225, 1920), (337, 5000), (448, 2048)])
+def test_selection_in_the_same_kernel_equals_selection_from_the_logits(B, vocab):
+    """d = 512, greedy: vocabularies that leave ranks without a tile, end inside a tile, give ranks unequal numbers of tiles. The same
+    products in two orders of addition (512 terms, fp32): ids must agree where the two largest logits differ by more than
+    2^-20 of the largest, sixteen times the rounding of one addition."""
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=2, d_model=512, vocab=vocab, n_ctx=16, dtype="bf16", seed=21)
+    m = P.SRM(shape, I.make_weights(shape), device=DEV)
+    toks = torch.from_numpy(np.random.default_rng(B).integers(0, vocab, size=(3, B)).astype(np.int32)).to(DEV)
+    g = P.Sampling("greedy")
+    a, b, ws = m.new_state(B), m.new_state(B), m.new_workspace(B)
+    strict = 0
+    for k in range(3):
+        n0 = P.SRM.kernel_launches()
+        tok_a = m.decode_step(a, toks[k], g, k + 1, ws)
+        assert P.SRM.kernel_launches() - n0 == 1
+        tok_b, lg = m.decode_step(b, toks[k], g, k + 1, ws, want_logits=True)
+        lg = lg.cpu().numpy()
+        clear = top2_margin(lg) > 2.0 ** -20 * np.abs(lg).max(-1)
+        strict += clear.mean() / 3
+        assert np.array_equal(tok_a.cpu().numpy()[clear], tok_b.cpu().numpy()[clear])
+        assert torch.equal(a.last_token(), tok_a)
+    assert strict > 0.9 and a.status() == 0 and b.status() == 0 and torch.equal(a.cache(), b.cache())
