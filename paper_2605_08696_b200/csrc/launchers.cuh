@@ -983,7 +983,8 @@ int with_split_kernel(const srm_config& c, int64_t R, Fn&& f) {
   return R == 1 ? with_split_kernel_t<true>(c, f) : with_split_kernel_t<false>(c, f);
 }
 // Whether a decode pass of R rows takes it: bf16 models with mixed heads, F = 4 d, 1024 channels, up to 16 rows. us per greedy step of 16
-// layers, the single-kernel step / here: 1 row 181 / 150, 4 rows 186 / 154, 8 rows 190 / 159, 16 rows 202 / 165; with 27 rows (two
+// layers, the single-kernel step / here: 1 row 181 / 140, 4 rows 186 / 147, 8 rows 190 / 149, 16 rows 202 / 157 (150, 154, 159 and 165
+// with LM head and selection as kernels of their own); with 27 rows (two
 // 16-row tiles, two rows per owner) it took 308, rows inside clusters 205. The words of the planes lie in the area of the
 // partial products.
 bool split_rows_ok(srm_model& m, int64_t R, const DecodeWs& w) {
@@ -995,8 +996,9 @@ bool split_rows_ok(srm_model& m, int64_t R, const DecodeWs& w) {
   return m.split_clusters >= sp::kClusters && w.part != nullptr && sp::plane_bytes(R, c.d_model) <= w.part_bytes;
 }
 // All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
+// out: LM head and greedy selection in the same kernel, or nullptr.
 int launch_layers_split(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w,
-                        cudaStream_t st, const int32_t* ctr, const int32_t* pos) {
+                        cudaStream_t st, const int32_t* ctr, const int32_t* pos, const SelectOut* out) {
   const srm_config& c = m.cfg;
   const int d = c.d_model, F = (int)m.F();
   sp::Params p;
@@ -1012,18 +1014,22 @@ int launch_layers_split(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t
   p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
   p.planes = reinterpret_cast<unsigned long long*>(w.part);
   p.cnt = reinterpret_cast<uint32_t*>(w.small);
+  p.best = reinterpret_cast<unsigned long long*>(w.small + 64);
+  static_assert(64 + sp::kMaxRows * 8 <= 256 && kSmallScratchBytes >= 256, "counters and maxima");
   p.status = s.status; p.ctr = ctr; p.pos = pos;
+  if (out != nullptr) { p.head = 1; p.out = *out; }
   SRM_CUDA(cudaMemsetAsync(w.small, 0, 256, st));
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
-  CUtensorMap w1, w2;
+  CUtensorMap w1, w2, lm;
   int rc;
+  if ((rc = make_tmap_layers(&lm, m.ptr(-1, SRM_T_W_LM), c.vocab, d, sp::Shape<1024>::kUpTiles * 8, 1, 0)) != SRM_OK) return rc;
   if ((rc = make_tmap_layers(&w1, m.ptr(0, SRM_T_W1), F, d, sp::Shape<1024>::kUpTiles * 8, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   if ((rc = make_tmap_layers(&w2, m.ptr(0, SRM_T_W2), d, F, d / sp::kCluster, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
   return with_split_kernel(c, R, [&](auto* kernel, size_t smem) -> int {
     int rc2 = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), sp::kSmemBytes, true);
     if (rc2 != SRM_OK) return rc2;
     ClusterLaunch L(sp::kClusters, sp::kThreads, smem, st, true);
-    SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, w1, w2, p));
+    SRM_CUDA(cudaLaunchKernelEx(&L.cfg, kernel, w1, w2, lm, p));
     return SRM_OK;
   });
 }
@@ -1048,9 +1054,9 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   if (o.pos) o.pos += b0;
   if (o.thr_out) o.thr_out += b0;
   const bool splits = split_rows_ok(m, R, w), clusters = !splits && mid_rows_ok(c, R) && cluster_rows_ok(m, R);
-  const bool head = clusters && cl::has_head(d) && can_fuse_greedy(m, samp, logits_out);      // the selection, too
+  const bool head = (splits || (clusters && cl::has_head(d))) && can_fuse_greedy(m, samp, logits_out);      // the selection, too
   const bool one_kernel = splits || clusters || mid_plan(m, R, w, &mp);
-  if (one_kernel && (rc = splits     ? launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos)
+  if (one_kernel && (rc = splits     ? launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr)
                           : clusters ? launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr)
                                      : launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
   if (head) return SRM_OK;

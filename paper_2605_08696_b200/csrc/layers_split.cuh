@@ -29,6 +29,10 @@
 // shared memory, each filled for the next layer as soon as it has been used. Buffers need no "free" signals, as in
 // layers_cluster.cuh: whatever overwrites one was computed from what its last reader sent afterwards.
 //
+// The LM head and the greedy selection follow in the same kernel where the caller wants nothing else: every CTA takes its 112th
+// of the vocabulary in chunks of 40 rows through the two places of the weights, as an up projection, and keeps the best logit of
+// every row; the CTA that comes last writes the tokens. A step of one row takes 140 us so, 150 with kernels of their own.
+//
 // All CTAs must be resident (cooperative launch). Every wait is bounded: a waiter that gives up raises kStatusWaitTimeout and
 // goes on without waiting.
 #pragma once
@@ -39,7 +43,8 @@
 #include "gemm_tc.cuh"
 #include "layers_cluster.cuh"   // st_async_16
 #include "prefill_chunk.cuh"    // ld_acquire_u32
-#include "step_small.cuh"       // LayerW, layer_w, ldsm_x4, ld_relaxed_u32, red_release_inc
+#include "select.cuh"           // SelectOut, write_token
+#include "step_small.cuh"       // LayerW, layer_w, ldsm_x4, ld_relaxed_u32, red_release_inc, pack_best
 
 namespace srm {
 namespace sp {
@@ -48,7 +53,7 @@ constexpr int kCluster = 16, kClusters = 7;    // as many as 148 SMs hold
 constexpr int kWarps = 16, kThreads = kWarps * 32, kMaxRows = 16;
 constexpr int kRowWarps = 8, kMmaWarps = 8, kRowThreads = kRowWarps * 32;
 constexpr int kDnSplits = 4;                   // warps that share out K of the down projection (up: all)
-constexpr int kBarrierBytes = 512, kSumBytes = 2 * kRowWarps * 8;
+constexpr int kBarrierBytes = 1024, kSumBytes = 2 * kRowWarps * 8;
 constexpr int kSmemBytes = 227 * 1024;
 constexpr long long kWaitLimitCycles = 1ll << 28;
 
@@ -64,7 +69,10 @@ struct Params {
   bf16* a;                       // [R, d]: the final norm's rows
   const float *lnf_g, *lnf_b;
   unsigned long long* planes;    // [2][clusters][R][d] words (value, tag)
-  uint32_t* cnt;                 // CTAs that have cleared their words; zero on entry
+  uint32_t* cnt;                 // CTAs that have cleared their words | CTAs done with the LM head; zero on entry
+  int head = 0;                  // LM head and greedy selection here, to `out`; else the final norm's rows to `a`
+  unsigned long long* best = nullptr;      // [R] (sortable logit, ~column) maxima, zero on entry
+  SelectOut out = {};
   uint32_t* status;
   const int32_t* ctr;            // device-side step counters or nullptr
   const int32_t* pos;            // [R] per-row positions or nullptr
@@ -86,7 +94,7 @@ struct Shape {
   static constexpr int kBarriers = (kKb + kHKb) * kRowBytes + kKb * kUpBytes + kHKb * kDnBytes;
   static constexpr size_t kSmem = kBarriers + kBarrierBytes + kSumBytes + 1024;
   static_assert(kKb == 2 * kMmaWarps && D == 4 * kRowThreads && kHKb <= 2 * kMmaWarps && kUpTiles <= kMmaWarps && kDnTiles == kMmaWarps &&
-                kSmem <= kSmemBytes && kUpTiles * 512 <= 2 * kRowBytes && kDnSplits * kDnTiles * 512 <= kKb * kRowBytes, "shape");
+                kSmem <= kSmemBytes && kHKb * kDnBytes >= kKb * kUpBytes && kMmaWarps * kUpTiles * 512 <= kHKb * kRowBytes && kUpTiles * 512 <= 2 * kRowBytes && kDnSplits * kDnTiles * 512 <= kKb * kRowBytes, "shape");
 };
 
 __device__ __forceinline__ void tma_load_w(void* dst, const CUtensorMap* map, uint64_t* bar, int col, int row, int layer) {
@@ -162,7 +170,8 @@ __device__ __forceinline__ void row_stats(const float4& x, float eps, float2* sl
 // ALONE: the one row there is, computed by every CTA.
 template <int D, bool ALONE, typename ST>
 __global__ void __launch_bounds__(kThreads, 1)
-layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2, const Params p) {
+layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmLm,
+              const Params p) {
   pdl_trigger();
   using C = Shape<D>;
   constexpr int kRowBytes = C::kRowBytes, kKb = C::kKb;
@@ -177,8 +186,11 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
   uint64_t* act_full = full_dn + C::kHKb;                                // by quarters of the channels
   uint64_t* h_full = act_full + 4;
   uint64_t* stored = h_full + 1;                                         // this CTA's words of a layer are on their way: time to look for the others'
+  uint64_t* full_lm = stored + 1;                                        // [2][kKb] k-blocks of the LM head's chunks, in the places of W1 and of W2
+  unsigned long long* best = reinterpret_cast<unsigned long long*>(full_lm + 2 * kKb);      // [kMaxRows] of this CTA
+  uint32_t* am_last = reinterpret_cast<uint32_t*>(best + kMaxRows);
   float2* sums = reinterpret_cast<float2*>(smem + C::kBarriers + kBarrierBytes);
-  static_assert((kKb + C::kHKb + 6) * 8 <= kBarrierBytes, "barriers");
+  static_assert((kKb + C::kHKb + 6 + 2 * kKb + kMaxRows + 1) * 8 <= kBarrierBytes, "barriers");
 
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int rank = (int)tc::cluster_ctarank(), cluster = (int)(blockIdx.x / kCluster);
@@ -192,6 +204,8 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
     for (int i = 0; i < 4; ++i) tc::mbar_init(&act_full[i], ALONE ? kRowWarps / 4 : 1);
     tc::mbar_init(h_full, 1);
     tc::mbar_init(stored, kMmaWarps);
+    for (int i = 0; i < 2 * kKb; ++i) tc::mbar_init(&full_lm[i], 1);
+    for (int i = 0; i < kMaxRows; ++i) best[i] = 0ull;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -208,6 +222,15 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
     if (l >= p.L) return;
     tc::mbar_expect_tx(&full_dn[kb], C::kDnBytes);
     tma_load_w(sD + kb * C::kDnBytes, &tmW2, &full_dn[kb], h0 + kb * 64, rank * (D / kCluster), l);
+  };
+  // the LM head: chunk i of this CTA's 8-row tiles of the vocabulary, into the place of W1 (even) or of W2 (odd)
+  const int lm_all = (p.V + 7) / 8, lm0 = (int)((int64_t)blockIdx.x * lm_all / gridDim.x), lm_tiles = (int)((int64_t)(blockIdx.x + 1) * lm_all / gridDim.x) - lm0;
+  const int lm_chunks = p.head ? (lm_tiles + C::kUpTiles - 1) / C::kUpTiles : 0;
+  auto load_lm = [&](int i, int kb) {
+    if (i >= lm_chunks) return;
+    uint64_t* bar = &full_lm[(i & 1) * kKb + kb];
+    tc::mbar_expect_tx(bar, C::kUpBytes);
+    tma_load_w((i & 1 ? sD : sU) + kb * C::kUpBytes, &tmLm, bar, kb * 64, (lm0 + i * C::kUpTiles) * 8, 0);
   };
   if (tc::elect_one()) {
     load_up(0, warp);
@@ -245,7 +268,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
     const int64_t plane_step = (int64_t)p.R * D;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f), keep = v;
     for (int l = 0; row < p.R; ++l) {
-      const bool last = l == p.L;
+      const bool last = l == p.L, send = !last || p.head != 0;           // (to the LM head: the final norm's rows)
       // parameters: constant data, and this thread's part of the cache row, on their way while the projections run
       const sb::LayerW w = sb::layer_w(p, last ? 0 : l);
       auto cache_row = [&](int l) { return reinterpret_cast<ST*>(static_cast<uint8_t*>(p.S) + (int64_t)l * p.layer_stride) + (int64_t)row * D + c0; };
@@ -316,7 +339,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
       const float nmr2 = -mean * rstd;
       const float4 o = make_float4(fmaf(fmaf(v.x, rstd, nmr2), g2.x, h2.x), fmaf(fmaf(v.y, rstd, nmr2), g2.y, h2.y),
                                    fmaf(fmaf(v.z, rstd, nmr2), g2.z, h2.z), fmaf(fmaf(v.w, rstd, nmr2), g2.w, h2.w));
-      if (last) {
+      if (!send) {
         if (writes) st4(p.a + (int64_t)row * D + c0, o);
       } else if (ALONE) {                 // (row 0 of this CTA's activations: it has no swizzle)
         st4(reinterpret_cast<bf16*>(sA + (c0 >> 6) * kRowBytes) + (c0 & 63), o);
@@ -419,10 +442,12 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
         }
         __syncwarp();
         if (tc::elect_one()) {
-          load_up(l + 1, 2 * m);
-          load_up(l + 1, 2 * m + 1);
+          for (int i = 2 * m; i < 2 * m + 2; ++i) {
+            if (l + 1 < p.L) load_up(l + 1, i);
+            else load_lm(0, i);
+          }
         }
-        if (!ALONE && tid == leader && l + 1 < p.L)                      // (every phase of this layer has been waited for)
+        if (!ALONE && tid == leader && (l + 1 < p.L || p.head))          // (every phase of this layer has been waited for)
           for (int i = 0; i < 4; ++i) tc::mbar_expect_tx(&act_full[i], (uint32_t)(p.R * D / 2));
         __syncwarp();
       }
@@ -487,6 +512,89 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
         if (lane == 0) tc::mbar_arrive(stored);
         if (tid == leader && l + 1 < p.L) tc::mbar_expect_tx(h_full, (uint32_t)(p.R * hc * 2));
         __syncwarp();
+      }
+    }
+    if (p.head) {
+      // ---- LM head ----
+      if (tc::elect_one())
+        for (int i = 2 * m; i < 2 * m + 2; ++i) load_lm(1, i);           // (all warps have used W2)
+      __syncwarp();
+      float bv[2] = {-INFINITY, -INFINITY};                              // rows g and g + 8
+      int bi[2] = {-1, -1};
+      bool bad = false;
+      if (ok) ok = tc::mbar_wait(&act_full[m / 2], (uint32_t)(p.L & 1), p.status);
+      __syncwarp();
+      uint32_t a[2][4][4];                                               // this warp's two k-blocks of the rows, for all chunks
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sb::ldsm_x4(a[i][k], tc::smem_u32(sA) + (2 * m + i) * kRowBytes + a_row + (((2 * k + a_c) ^ a_sw) << 4));
+      float4* part = reinterpret_cast<float4*>(sH) + lane;
+      for (int ch = 0; ch < lm_chunks; ++ch) {
+        float c[C::kUpTiles][4] = {};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int kb = 2 * m + i;
+          if (ok) ok = tc::mbar_wait(&full_lm[(ch & 1) * kKb + kb], (uint32_t)(ch >> 1) & 1u, p.status);
+          __syncwarp();
+          const uint32_t w0 = tc::smem_u32(ch & 1 ? sD : sU) + kb * C::kUpBytes + w_row;
+#pragma unroll
+          for (int j = 0; j < C::kUpTiles; ++j) {
+            uint32_t b[2][4];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) sb::ldsm_x4(b[k], w0 + (uint32_t)(j * 1024) + (((4 * k + w_c) ^ (lane & 7)) << 4));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) mma(c[j], a[i][k], b[k >> 1][2 * (k & 1)], b[k >> 1][2 * (k & 1) + 1]);
+          }
+        }
+        mma_sync();                                                      // the partial sums of the chunk before have been taken
+#pragma unroll
+        for (int j = 0; j < C::kUpTiles; ++j) part[(m * C::kUpTiles + j) * 32] = make_float4(c[j][0], c[j][1], c[j][2], c[j][3]);
+        __syncwarp();                                                    // (only this warp uses these k-blocks)
+        if (tc::elect_one())
+          for (int i = 2 * m; i < 2 * m + 2; ++i) load_lm(ch + 2, i);
+        mma_sync();
+        const int tile = ch * C::kUpTiles + m;
+        if (m < C::kUpTiles && tile < lm_tiles && ok) {
+          float4 e = part[m * 32];
+#pragma unroll
+          for (int k = 1; k < kMmaWarps; ++k) {
+            const float4 f = part[(k * C::kUpTiles + m) * 32];
+            e = make_float4(e.x + f.x, e.y + f.y, e.z + f.z, e.w + f.w);
+          }
+          const int col = (lm0 + tile) * 8 + 2 * q;                      // (V is a multiple of 8; ascending: the lowest among equals is kept)
+          if (g < p.R) {
+            bad |= !(e.x == e.x) | !(e.y == e.y);
+            if (e.x > bv[0]) { bv[0] = e.x; bi[0] = col; }
+            if (e.y > bv[0]) { bv[0] = e.y; bi[0] = col + 1; }
+          }
+          if (g + 8 < p.R) {
+            bad |= !(e.z == e.z) | !(e.w == e.w);
+            if (e.z > bv[1]) { bv[1] = e.z; bi[1] = col; }
+            if (e.w > bv[1]) { bv[1] = e.w; bi[1] = col + 1; }
+          }
+        }
+      }
+      if (bad) raise_status(p.status, kStatusNonFinite);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (bi[i] >= 0) atomicMax(&best[g + 8 * i], sb::pack_best(bv[i] + 0.0f, bi[i]));      // (minus zero equals zero)
+      mma_sync();
+      const int r = tid - leader;
+      if (r < p.R && best[r] != 0ull) atomicMax(p.best + r, best[r]);
+      // ---- the CTA that comes last writes the tokens ----
+      __threadfence();
+      mma_sync();
+      if (r == 0) {
+        *am_last = atomicAdd(p.cnt + 1, 1u) + 1u == gridDim.x ? 1u : 0u;
+        __threadfence();
+      }
+      mma_sync();
+      if (*am_last != 0u && r < p.R) {
+        const unsigned long long k = __ldcg(p.best + r);
+        int tok = k == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)k);      // (no finite logit: 0)
+        if (tok < 0 || tok >= p.V) tok = 0;
+        write_token(p.out, r, tok);
       }
     }
   }

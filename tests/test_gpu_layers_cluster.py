@@ -76,13 +76,14 @@ def test_a_row_has_the_same_bits_in_any_pass():
             assert torch.equal(x, y)
 
 
-@pytest.mark.parametrize("B,vocab", [(1, 1000), (7, 2056), (16, 128), (64, 8000), (113, 136), (225, 1920), (337, 5000), (448, 2048)])
-def test_selection_in_the_same_kernel_equals_selection_from_the_logits(B, vocab):
-    """d = 512, greedy: vocabularies that leave ranks without a tile, end inside a tile, give ranks unequal numbers of tiles. The same
-    products in two orders of addition (512 terms, fp32): ids must agree where the two largest logits differ by more than
+@pytest.mark.parametrize("B,d,vocab", [(1, 512, 1000), (7, 512, 2056), (16, 512, 128), (64, 512, 8000), (113, 512, 136), (225, 512, 1920),
+                                       (337, 512, 5000), (448, 512, 2048), (1, 1024, 8000), (2, 1024, 136), (9, 1024, 4488), (16, 1024, 32000)])
+def test_selection_in_the_same_kernel_equals_selection_from_the_logits(B, d, vocab):
+    """Greedy steps of one launch: vocabularies that leave ranks (or CTAs) without a tile, end inside a tile, give unequal numbers of
+    tiles. The same products in two orders of addition (at most 1024 terms, fp32): ids must agree where the two largest logits differ by more than
     2^-20 of the largest, sixteen times the rounding of one addition."""
     import paper_2605_08696_b200 as P
-    shape = custom_shape(n_layers=2, d_model=512, vocab=vocab, n_ctx=16, dtype="bf16", seed=21)
+    shape = custom_shape(n_layers=2, d_model=d, vocab=vocab, n_ctx=16, dtype="bf16", seed=21)
     m = P.SRM(shape, I.make_weights(shape), device=DEV)
     toks = torch.from_numpy(np.random.default_rng(B).integers(0, vocab, size=(3, B)).astype(np.int32)).to(DEV)
     g = P.Sampling("greedy")
