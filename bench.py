@@ -546,7 +546,7 @@ def run_ours(args):
         # the step is one weight-streaming kernel: algorithmic bytes = the bf16 weights once + the cache read and written
         step_bytes = step_flops(shape) + B * 2 * L * d * sbytes
         gbs = prof_steps * step_bytes / (gemm_ms / 1e3) / 1e9 if gemm_ms > 0 else 0.0
-        roofline = {"bound": "hbm", "kernel": "step_small_kernel (the whole decode step of a batch of at most 64 samples)",
+        roofline = {"bound": "hbm", "kernel": "layers_kernel or step_small_kernel (all layers of a small pass as one kernel)",
                     "achieved": round(gbs, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": round(gbs / peaks["hbm_gbs"], 4),
                     "peak_source": f"hbm_gbs, {peak_src}", "launches": int(gemm_launches), "steps_profiled": prof_steps,
                     "traffic": None, "bytes_per_step": step_bytes}
