@@ -20,8 +20,8 @@
 //   up:    H columns [kg F / 4 + ng F / 16, + F / 16) for all rows of the cluster (D^T = W1 a^T: weights are the 128-row operand
 //          of tcgen05.mma, rows of the batch its N columns, so a few rows waste no tensor time); GELU; each finished tile is
 //          copied to the three ranks of the same K-group;
-//   down:  output features [ng d / 4, + d / 4) over K = the K-group's quarter of H; the partial product's rows go to the ranks
-//          that own them, which add the four K-groups' in rank order.
+//   down:  output features [ng d / 4, + d / 4) over K = the K-group's quarter of H; the partial product's rows go from
+//          registers to the ranks that own them, which add the four K-groups' in rank order.
 // A row's bits depend on neither its place in the pass nor the number of rows: every output is one fixed sequence of
 // 16-deep tensor steps, and N columns of an instruction do not mix.
 //
@@ -30,9 +30,15 @@
 // takes longer to start than to run.
 //
 // No buffer needs a "free" signal of its own: an owner sends the next layer's activations after it has received every CTA's
-// partial products, a CTA sends those after its last tensor instruction of the layer has completed, and everything a
-// CTA sends in a layer is sent after all activations of that layer have come. For the same reason no byte of a layer can
-// be counted in the phase of the layer before.
+// partial products for its rows, a CTA sends those after the products that they come from, and everything else a CTA sends
+// in a layer is sent after the activations of ALL owners have come. So, when bytes of layer l + 1 are written,
+//   activations: the products that read layer l's have completed (the last partial products come after all of them);
+//   H: every owner has all its partial products, so every CTA's products that read H have completed, and with them the copies of
+//      hidden columns that these products waited for;
+//   partial products received: their owner has added up layer l's, or its activations would not have come.
+// Nothing else may leave from shared memory: a copy is counted where it arrives, and that tells one receiver, nobody else, that its
+// source has been read (partial products staged over the activations could meet another owner's activations of the next layer).
+// For the same reason no byte of a layer can be counted in the phase of the layer before.
 // Every wait is bounded: a waiter that gives up raises kStatusWaitTimeout and goes on without waiting; all CTAs meet at the
 // final cluster barrier.
 #pragma once
@@ -79,8 +85,7 @@ struct Params {
 __host__ __device__ constexpr bool has_head(int d) { return d == 512; }
 
 // Shared memory: activations [k-block][row][128 bytes] | H of the K-group, the same | partial products received
-// [K-group][column][tile][own row][128] | weight ring | barriers | row-phase sums. The partial products sent are staged in the
-// place of the activations, which no copy is left to read or write by then.
+// [K-group][column][tile][own row][128] | weight ring | barriers | row-phase sums.
 template <int D, int RC>
 struct Shape {
   static constexpr int kUpTiles = D / 512, kDnTiles = D / 512;   // 128-wide tiles per CTA: F / 16, d / 4 with F = 4 d
@@ -140,6 +145,14 @@ __device__ __forceinline__ void take_tile(uint32_t taddr, int stride, float (&v)
 #pragma unroll
       for (int i = 1; i < kIssuers; ++i) v[g][j] += __uint_as_float(acc[i][g][j]);
     }
+}
+// Four values of each of four neighbouring lanes, transposed: lane i of the four gets value i of all four.
+__device__ __forceinline__ uint4 transpose4(const float (&v)[4], int lane) {
+  const bool odd = lane & 1, high = lane & 2;
+  const float a = __shfl_xor_sync(0xffffffffu, odd ? v[0] : v[1], 1), b = __shfl_xor_sync(0xffffffffu, odd ? v[2] : v[3], 1);
+  const float w0 = odd ? a : v[0], w1 = odd ? v[1] : a, w2 = odd ? b : v[2], w3 = odd ? v[3] : b;
+  const float c = __shfl_xor_sync(0xffffffffu, high ? w0 : w2, 2), e = __shfl_xor_sync(0xffffffffu, high ? w1 : w3, 2);
+  return make_uint4(__float_as_uint(high ? c : w0), __float_as_uint(high ? e : w1), __float_as_uint(high ? w2 : c), __float_as_uint(high ? w3 : e));
 }
 // The i-th k-block of the down projection: the first tile of each rank of the K-group, the own one in front, then the second
 // tiles (they come later).
@@ -481,23 +494,19 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
       for (int m = 0; m < kDn; ++m) {
         if (ok) ok = tc::mbar_wait(&dn_done[m], (uint32_t)(l & 1), p.status);
         tc::tc_fence_after();
-        float* stage = reinterpret_cast<float*>(sA) + m * (kCluster * kOwn) * kTile;      // [owner][its rows][128]
-        if (cols) {
+        if (cgrp * 4 < min(rows, RC)) {                                  // (rows 4 cgrp .. + 3, and 16, 32, 48 further, as far as there are any)
           float acc[kOwn][4];
           take_tile<kOwn>(tmem + (static_cast<uint32_t>(quad * 32) << 16) + (uint32_t)((kUp + m) * kIssuers * C::kN + cgrp * 4), C::kN, acc);
-          float* at = stage + cgrp * 4 * kOwn * kTile + quad * 32 + lane;
+          const int to = cgrp * 4 + (lane & 3);                          // four features of one row per lane, 128 bytes per row and warp
+          const uint32_t at = tc::mapa(tc::smem_u32(recv + ((kg * kCols + ng) * kDn + m) * kOwn * kTile + quad * 32 + (lane & ~3)), (uint32_t)to);
+          const uint32_t bar = tc::mapa(tc::smem_u32(recv_full), (uint32_t)to);
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int g = 0; g < kOwn; ++g) at[(j * kOwn + g) * kTile] = acc[g][j];
+          for (int g = 0; g < kOwn; ++g) {
+            const uint4 e = transpose4(acc[g], lane);
+            if (to + kCluster * g < rows) st_async_16(at + g * kTile * 4, e, bar);
+          }
         }
         tc::tc_fence_before();
-        tc::fence_async_smem();
-        workers_sync();
-        const int to = (rank + ww) % kCluster, n = rows_of(to);          // a warp per rank: one warp issues copies 43 cycles apart
-        if (n > 0 && tc::elect_one())
-          sb::bulk_s2s(tc::mapa(tc::smem_u32(recv + ((kg * kCols + ng) * kDn + m) * kOwn * kTile), (uint32_t)to), stage + to * kOwn * kTile,
-                       n * kTile * 4, tc::mapa(tc::smem_u32(recv_full), (uint32_t)to));
       }
     }
   }

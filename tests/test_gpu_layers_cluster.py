@@ -76,6 +76,25 @@ def test_a_row_has_the_same_bits_in_any_pass():
             assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("B,d,state_dtype", [(448, 512, "fp32"), (256, 512, "fp16"), (17, 1024, "fp32"), (112, 1024, "fp32")])
+def test_thousands_of_passes_give_the_same_bits(B, d, state_dtype):
+    """The kernel's exchanges through shared memory, whatever their timing: the same 500 steps again and again (4000 passes)."""
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=4, d_model=d, vocab=2048, n_ctx=504, dtype="bf16", seed=22)
+    m = P.SRM(shape, I.make_weights(shape), device=DEV, state_dtype=state_dtype)
+    tok = torch.from_numpy(np.random.default_rng(B).integers(0, shape.vocab, size=(B, 1)).astype(np.int32)).to(DEV)
+    g = P.Sampling("greedy")
+    st, ws = m.new_state(B), m.new_workspace(B, 1, prefill_samples=B)
+    first = None
+    for _ in range(8):
+        st.reset()
+        m.prefill(st, tok, g, ws)
+        out, cache = m.generate(st, 500, 1, g, ws).clone(), st.cache().clone()
+        first = first or (out, cache)
+        assert torch.equal(out, first[0]) and torch.equal(cache, first[1])
+    assert st.status() == 0
+
+
 @pytest.mark.parametrize("B,d,vocab", [(1, 512, 1000), (7, 512, 2056), (16, 512, 128), (64, 512, 8000), (113, 512, 136), (225, 512, 1920),
                                        (337, 512, 5000), (448, 512, 2048), (1, 1024, 8000), (2, 1024, 136), (9, 1024, 4488), (16, 1024, 32000)])
 def test_selection_in_the_same_kernel_equals_selection_from_the_logits(B, d, vocab):
