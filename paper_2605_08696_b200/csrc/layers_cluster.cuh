@@ -519,6 +519,11 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
       unsigned long long* best = reinterpret_cast<unsigned long long*>(recv);                     // [RC]
       unsigned long long* slots = best + 64;                                                      // [own row][rank]
       const int own = rows_of(rank);
+      // The final norm's rows have come from every owner: each has added up its partial products, and the phase that counted them is over.
+      // Without this a rank that has no tile of the vocabulary, and so waits for no product, could send its logits into that phase.
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (ok) ok = tc::mbar_wait(&act_full[i], (uint32_t)(p.L & 1), p.status);
       if (wid == 0 && own > 0) tc::mbar_expect_tx(recv_full, (uint32_t)(own * kCluster * 8));
       float bv[kOwn][4];
       int bi[kOwn][4];

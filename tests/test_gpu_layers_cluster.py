@@ -119,3 +119,28 @@ def test_selection_in_the_same_kernel_equals_selection_from_the_logits(B, d, voc
         assert np.array_equal(tok_a.cpu().numpy()[clear], tok_b.cpu().numpy()[clear])
         assert torch.equal(a.last_token(), tok_a)
     assert strict > 0.9 and a.status() == 0 and b.status() == 0 and torch.equal(a.cache(), b.cache())
+
+
+@pytest.mark.parametrize("B,vocab", [(1, 8), (1, 128), (5, 1000), (7, 1920), (40, 8), (112, 136), (113, 1912), (448, 264)])
+def test_vocabularies_that_leave_ranks_without_a_tile(B, vocab):
+    """Greedy steps of one launch at d = 512, a thousand of them: ranks of a cluster without vocabulary rows, with and without rows of the batch,
+    send their part of the selection when its receivers have done with the last layer, not before."""
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=1, d_model=512, vocab=vocab, n_ctx=1008, dtype="bf16", seed=23)
+    m = P.SRM(shape, I.make_weights(shape), device=DEV)
+    first = torch.from_numpy(np.random.default_rng(B).integers(0, vocab, size=B).astype(np.int32)).to(DEV)
+    g = P.Sampling("greedy")
+    a, b, ws = m.new_state(B), m.new_state(B), m.new_workspace(B)
+    tok, differ, clear_all = first, [], []
+    for k in range(1000):
+        n0 = P.SRM.kernel_launches()
+        got = m.decode_step(a, tok, g, k + 1, ws)
+        assert P.SRM.kernel_launches() - n0 == 1
+        want, lg = m.decode_step(b, tok, g, k + 1, ws, want_logits=True)
+        top = torch.topk(lg, 2, dim=-1).values
+        clear = top[:, 0] - top[:, 1] > 2.0 ** -20 * lg.abs().amax(-1)          # (two orders of addition, as above)
+        differ.append(((got != want) & clear).any())
+        clear_all.append(clear.float().mean())
+        tok = want.clone()
+    assert not torch.stack(differ).any() and torch.stack(clear_all).mean() > 0.9
+    assert a.status() == 0 and b.status() == 0 and torch.equal(a.cache(), b.cache())
