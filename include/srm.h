@@ -218,6 +218,16 @@ size_t srm_prefill_workspace_bytes(const srm_config* cfg, int64_t samples, int32
 /* Rows per decode pass that a batch of B samples is processed in when the workspace has room for
  * `ws_rows` rows (the rule stated above; host only, no device work). 0 if B < 1 or ws_rows < 1. */
 int64_t srm_decode_pass_rows(int64_t B, int64_t ws_rows);
+/* Which kernels the first pass of a decode step of B samples runs with a workspace of ws_bytes (an SRM_ROUTE_* value, or a
+ * negative SRM_ERR_*; nothing is launched). A step's tokens do not depend on it but for rounding. */
+enum {
+  SRM_ROUTE_KERNELS = 0,             /* a kernel per operation                                                          */
+  SRM_ROUTE_STEP = 1,                /* the whole step as one kernel on clusters of four CTAs                           */
+  SRM_ROUTE_LAYERS = 2,              /* all layers as one kernel over the whole grid                                    */
+  SRM_ROUTE_CLUSTERS = 3,            /* all layers as one kernel, rows inside clusters of 16 CTAs                       */
+  SRM_ROUTE_SPLIT = 4                /* all layers as one kernel, weights split between clusters of 16 CTAs             */
+};
+int32_t srm_decode_route(srm_model* m, int64_t B, size_t ws_bytes);
 
 /* ---- handles ------------------------------------------------------------------------------ */
 

@@ -86,6 +86,7 @@ SYMBOLS = {
     "srm_prefill_workspace_bytes": (_SZ, [C.POINTER(_Config), _I64, _I32]),
     "srm_create": (C.c_int, [C.POINTER(_Config), _P, _SZ, C.POINTER(_P)]),
     "srm_destroy": (C.c_int, [_P]),
+    "srm_decode_route": (_I32, [_P, _I64, _SZ]),
     "srm_state_create": (C.c_int, [_P, _I64, _P, _SZ, _P, C.POINTER(_P)]),
     "srm_state_destroy": (C.c_int, [_P]),
     "srm_state_reset": (C.c_int, [_P, _P]),
@@ -394,6 +395,14 @@ class SRM:
         return torch.empty(nb, dtype=torch.uint8, device=self.device)
 
     # ---- hot path ----
+    ROUTES = ("kernels", "step", "layers", "clusters", "split")
+
+    def decode_route(self, B: int, ws: torch.Tensor) -> str:
+        """Which kernels the first pass of a decode step of B samples runs with this workspace."""
+        r = _lib().srm_decode_route(self.handle, B, ws.numel() * ws.element_size())
+        _check(min(r, 0), "srm_decode_route")
+        return self.ROUTES[r]
+
     def prefill(self, state: SRMState, tokens: torch.Tensor, sampling: Sampling, ws: torch.Tensor,
                 want_logits: bool = False):
         B, n = tokens.shape

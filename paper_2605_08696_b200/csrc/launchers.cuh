@@ -1034,6 +1034,75 @@ int launch_layers_split(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t
   });
 }
 
+// ---- small batches: the whole step in one cooperative kernel (step_small.cuh) ----------------------
+struct SmallPlan { sb::Params p; size_t smem; };
+
+// f(kernel) for the instance of the step kernel that the configuration takes.
+template <int d, typename Fn>
+int with_small_kernel_d(const srm_config& c, Fn&& f) {
+  if (c.state_dtype == SRM_DTYPE_FP16) return f(sb::step_small_kernel<d, fp16>);
+  if (c.state_dtype == SRM_DTYPE_BF16) return f(sb::step_small_kernel<d, bf16>);
+  return f(sb::step_small_kernel<d, float>);
+}
+template <typename Fn>
+int with_small_kernel(const srm_config& c, Fn&& f) {
+  switch (c.d_model) {
+    case 256: return with_small_kernel_d<256>(c, f);
+    case 512: return with_small_kernel_d<512>(c, f);
+    case 768: return with_small_kernel_d<768>(c, f);
+    default: return with_small_kernel_d<1024>(c, f);
+  }
+}
+
+// Both launch attributes of the kernel: all CTAs resident at once (it has grid-wide barriers), in clusters.
+struct SmallLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  SmallLaunch(size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3(sb::kGrid);
+    cfg.blockDim = dim3(sb::kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = sb::kCluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
+// Whether a batch of B samples takes the single-kernel step, and its shared-memory plan. Mixed heads, bf16 weights, at
+// most 64 samples and 1024 channels (a multiple of 256), a device that holds all clusters at once; everything
+// else takes the kernel-per-operation path.
+bool small_step_plan(srm_model& m, int64_t B, SmallPlan* P) {
+  const srm_config& c = m.cfg;
+  if (c.dtype != SRM_DTYPE_BF16 || (c.flags & (SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_HEAD_PROJ))) return false;
+  if (c.mixer != SRM_MIXER_MIXED || B > sb::kMaxRows || c.d_model > 1024 || c.d_model % 256 || m.F() % 1024) return false;
+  if (m.small_clusters < 0) {
+    m.small_clusters = with_small_kernel(c, [&](auto* kernel) {
+      int n = 0;
+      if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), sb::kSmemBytes) != SRM_OK) return 0;
+      SmallLaunch L(sb::kSmemBytes, nullptr);
+      L.cfg.attrs = L.attr + 1;
+      L.cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, kernel, &L.cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+      return n;
+    });
+  }
+  return m.small_clusters >= sb::kClusters &&
+         sb::smem_plan((int)B, c.d_model, (int)m.F(), m.state_bytes(), &P->p, &P->smem);
+}
+
+// What a decode pass of R rows runs; `whole`: the pass is its state's whole batch. `small`, `mid`: the plan where that kernel is taken.
+enum DecodeRoute { kRouteKernels, kRouteStep, kRouteLayers, kRouteClusters, kRouteSplit };      // SRM_ROUTE_* of the C ABI
+DecodeRoute decode_route(srm_model& m, int64_t R, bool whole, const DecodeWs& w, SmallPlan* small, mid::Params* mid) {
+  if (split_rows_ok(m, R, w)) return kRouteSplit;
+  if (mid_rows_ok(m.cfg, R) && cluster_rows_ok(m, R)) return kRouteClusters;
+  if (whole && small_step_plan(m, R, small)) return kRouteStep;
+  return mid_plan(m, R, w, mid) ? kRouteLayers : kRouteKernels;
+}
+
 // One decode step for rows [b0, b0 + R) of the state.
 int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_t* tok_in, const srm_sampling& samp,
                  int step, const SelectOut& out_all, float* logits_out, const DecodeWs& w, cudaStream_t st,
@@ -1053,12 +1122,14 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   if (o.store) o.store += b0 * o.store_stride;
   if (o.pos) o.pos += b0;
   if (o.thr_out) o.thr_out += b0;
-  const bool splits = split_rows_ok(m, R, w), clusters = !splits && mid_rows_ok(c, R) && cluster_rows_ok(m, R);
-  const bool head = (splits || (clusters && cl::has_head(d))) && can_fuse_greedy(m, samp, logits_out);      // the selection, too
-  const bool one_kernel = splits || clusters || mid_plan(m, R, w, &mp);
-  if (one_kernel && (rc = splits     ? launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr)
-                          : clusters ? launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr)
-                                     : launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos))) return rc;
+  SmallPlan small;
+  const DecodeRoute route = decode_route(m, R, false, w, &small, &mp);
+  const bool one_kernel = route != kRouteKernels;
+  const bool head = (route == kRouteSplit || (route == kRouteClusters && cl::has_head(d))) && can_fuse_greedy(m, samp, logits_out);      // the selection, too
+  if (route == kRouteSplit) rc = launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr);
+  else if (route == kRouteClusters) rc = launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr);
+  else rc = one_kernel ? launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos) : SRM_OK;
+  if (rc) return rc;
   if (head) return SRM_OK;
   // the down projection shares K out between CTA pairs where that is the faster kernel for R rows
   bool split = false;
@@ -1131,66 +1202,6 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   float* lg = logits_out != nullptr ? logits_out + b0 * c.vocab : w.logits;
   if ((rc = launch_gemm(m, kEpiPlain, R, c.vocab, d, w.a, m.ptr(-1, SRM_T_W_LM), nullptr, lg, s.status, st))) return rc;
   return launch_select(m, R, lg, samp, samp.sample_idx_base + (uint64_t)b0, step, o, s.status, st);
-}
-
-// ---- small batches: the whole step in one cooperative kernel (step_small.cuh) ----------------------
-struct SmallPlan { sb::Params p; size_t smem; };
-
-// f(kernel) for the instance of the step kernel that the configuration takes.
-template <int d, typename Fn>
-int with_small_kernel_d(const srm_config& c, Fn&& f) {
-  if (c.state_dtype == SRM_DTYPE_FP16) return f(sb::step_small_kernel<d, fp16>);
-  if (c.state_dtype == SRM_DTYPE_BF16) return f(sb::step_small_kernel<d, bf16>);
-  return f(sb::step_small_kernel<d, float>);
-}
-template <typename Fn>
-int with_small_kernel(const srm_config& c, Fn&& f) {
-  switch (c.d_model) {
-    case 256: return with_small_kernel_d<256>(c, f);
-    case 512: return with_small_kernel_d<512>(c, f);
-    case 768: return with_small_kernel_d<768>(c, f);
-    default: return with_small_kernel_d<1024>(c, f);
-  }
-}
-
-// Both launch attributes of the kernel: all CTAs resident at once (it has grid-wide barriers), in clusters.
-struct SmallLaunch {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
-  SmallLaunch(size_t smem, cudaStream_t st) {
-    cfg.gridDim = dim3(sb::kGrid);
-    cfg.blockDim = dim3(sb::kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = sb::kCluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-  }
-};
-
-// Whether a batch of B samples takes the single-kernel step, and its shared-memory plan. Mixed heads, bf16 weights, at
-// most 64 samples and 1024 channels (a multiple of 256), a device that holds all clusters at once; everything
-// else takes the kernel-per-operation path.
-bool small_step_plan(srm_model& m, const srm_state& s, SmallPlan* P) {
-  const srm_config& c = m.cfg;
-  if (c.dtype != SRM_DTYPE_BF16 || (c.flags & (SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_HEAD_PROJ))) return false;
-  if (c.mixer != SRM_MIXER_MIXED || s.B > sb::kMaxRows || c.d_model > 1024 || c.d_model % 256 || m.F() % 1024) return false;
-  if (m.small_clusters < 0) {
-    m.small_clusters = with_small_kernel(c, [&](auto* kernel) {
-      int n = 0;
-      if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), sb::kSmemBytes) != SRM_OK) return 0;
-      SmallLaunch L(sb::kSmemBytes, nullptr);
-      L.cfg.attrs = L.attr + 1;
-      L.cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&n, kernel, &L.cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
-      return n;
-    });
-  }
-  return m.small_clusters >= sb::kClusters &&
-         sb::smem_plan((int)s.B, c.d_model, (int)m.F(), m.state_bytes(), &P->p, &P->smem);
 }
 
 // One decode step of all B <= 64 samples of the state. SRM_ERR_UNSUPPORTED: take the ordinary path.
@@ -1267,7 +1278,8 @@ int decode_step_impl(srm_model* m, srm_state* s, const int32_t* d_tok_in, const 
   SelectOut out{s->last_tok, d_tok_out, d_store, store_stride, store_col, 1, ctr, s->ragged ? s->pos_dev : nullptr,
                 nullptr, nullptr, samp->mode == SRM_SELECT_TOPK ? s->thr : nullptr};
   SmallPlan small;
-  if (rows >= s->B && !split_rows_ok(*m, s->B, w) && !cluster_rows_ok(*m, s->B) && small_step_plan(*m, *s, &small)) {
+  mid::Params mid;
+  if (rows >= s->B && decode_route(*m, s->B, true, w, &small, &mid) == kRouteStep) {
     rc = decode_step_small(*m, *s, small, tok_in, *samp, step, out, d_logits_out, w, st, ctr);
     if (rc != SRM_ERR_UNSUPPORTED) {
       if (rc == SRM_OK) s->pos += 1;

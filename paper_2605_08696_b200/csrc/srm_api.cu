@@ -118,6 +118,19 @@ uint64_t srm_kernel_launches(void) { return g_kernel_launches; }
 
 int64_t srm_decode_pass_rows(int64_t B, int64_t ws_rows) { return B < 1 || ws_rows < 1 ? 0 : choose_pass_rows(B, ws_rows); }
 
+int32_t srm_decode_route(srm_model* m, int64_t B, size_t ws_bytes) {
+  static_assert(kRouteKernels == SRM_ROUTE_KERNELS && kRouteStep == SRM_ROUTE_STEP && kRouteLayers == SRM_ROUTE_LAYERS &&
+                kRouteClusters == SRM_ROUTE_CLUSTERS && kRouteSplit == SRM_ROUTE_SPLIT, "routes");
+  if (m == nullptr || B < 1) return SRM_ERR_INVALID_ARG;
+  const int64_t fit = fit_rows(ws_bytes, B, decode_need, *m, 0);
+  if (fit < 1) return SRM_ERR_BUFFER_TOO_SMALL;
+  const int64_t rows = choose_pass_rows(B, fit);
+  SmallPlan small;
+  mid::Params mid;
+  // (the areas of a workspace are told apart by their sizes; an address stands in for the caller's)
+  return decode_route(*m, rows < B ? rows : B, rows >= B, carve_decode(*m, reinterpret_cast<void*>(256), rows), &small, &mid);
+}
+
 int srm_state_create(srm_model* m, int64_t B, void* d_state, size_t nbytes, void* stream, srm_state** out) {
   if (out == nullptr) return SRM_ERR_INVALID_ARG;
   *out = nullptr;
