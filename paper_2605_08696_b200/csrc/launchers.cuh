@@ -935,10 +935,11 @@ bool cluster_rows_ok(srm_model& m, int64_t R) {
     m.row_clusters = with_cluster_kernel(c, 1 << 20, [](auto* kernel, size_t smem) { return resident_clusters(kernel, cl::kThreads, smem); });
   return R <= (int64_t)m.row_clusters * (c.d_model == 1024 ? 16 : 64);
 }
-// All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
-// out: LM head and greedy selection in the same kernel (d = 512), or nullptr.
+// What of the LM head the layers kernel of a pass does, too: nothing, the logits, the greedy selection, or both.
+struct LmHead { bool here, select; float* logits; SelectOut out; };
+// All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a, or goes on to the LM head.
 int launch_layers_cluster(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w,
-                          cudaStream_t st, const int32_t* ctr, const int32_t* pos, const SelectOut* out) {
+                          cudaStream_t st, const int32_t* ctr, const int32_t* pos, const LmHead& head) {
   const srm_config& c = m.cfg;
   const int d = c.d_model, F = (int)m.F();
   cl::Params p;
@@ -954,8 +955,8 @@ int launch_layers_cluster(srm_model& m, srm_state& s, int64_t b0, int64_t R, int
   p.a = reinterpret_cast<bf16*>(w.a);
   p.lnf_g = m.fptr(-1, SRM_T_LNF_G); p.lnf_b = m.fptr(-1, SRM_T_LNF_B);
   p.status = s.status; p.ctr = ctr; p.pos = pos;
+  p.head = head.here; p.select = head.select; p.logits = head.logits; p.out = head.out;
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
-  if (out != nullptr) { p.head = 1; p.out = *out; }
   CUtensorMap w1, w2, lm;
   int rc;
   if ((rc = make_tmap_kblocks(&w1, m.ptr(0, SRM_T_W1), F, d, cl::kTile, 1, c.n_layers, p.layer_bytes)) != SRM_OK) return rc;
@@ -995,10 +996,9 @@ bool split_rows_ok(srm_model& m, int64_t R, const DecodeWs& w) {
     m.split_clusters = with_split_kernel(c, 32, [](auto* kernel, size_t smem) { return resident_clusters(kernel, sp::kThreads, smem); });
   return m.split_clusters >= sp::kClusters && w.part != nullptr && sp::plane_bytes(R, c.d_model) <= w.part_bytes;
 }
-// All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a.
-// out: LM head and greedy selection in the same kernel, or nullptr.
+// All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a, or goes on to the LM head.
 int launch_layers_split(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t, const int32_t* tok_in, const DecodeWs& w,
-                        cudaStream_t st, const int32_t* ctr, const int32_t* pos, const SelectOut* out) {
+                        cudaStream_t st, const int32_t* ctr, const int32_t* pos, const LmHead& head) {
   const srm_config& c = m.cfg;
   const int d = c.d_model, F = (int)m.F();
   sp::Params p;
@@ -1017,7 +1017,7 @@ int launch_layers_split(srm_model& m, srm_state& s, int64_t b0, int64_t R, int t
   p.best = reinterpret_cast<unsigned long long*>(w.small + 64);
   static_assert(64 + sp::kMaxRows * 8 <= 256 && kSmallScratchBytes >= 256, "counters and maxima");
   p.status = s.status; p.ctr = ctr; p.pos = pos;
-  if (out != nullptr) { p.head = 1; p.out = *out; }
+  p.head = head.here; p.select = head.select; p.logits = head.logits; p.out = head.out;
   SRM_CUDA(cudaMemsetAsync(w.small, 0, 256, st));
   LaunchScope scope(m, SRM_KERNEL_STEP_SMALL, st);
   CUtensorMap w1, w2, lm;
@@ -1103,6 +1103,25 @@ DecodeRoute decode_route(srm_model& m, int64_t R, bool whole, const DecodeWs& w,
   return mid_plan(m, R, w, mid) ? kRouteLayers : kRouteKernels;
 }
 
+// Whether the LM head runs in the layers kernel of a pass, too, and so the greedy selection or the logits for another. A separate LM head
+// starts later, but shares the vocabulary out over the device, where a cluster reads all of it by itself. us per step of 8 layers at d = 512,
+// separate / inside, greedy without logits: V = 8000 1 row 47 / 45, 224 rows 65 / 63, 448 rows 94 / 98; V = 16000 48 / 48, 66 / 67,
+// 98 / 106; V = 32000 52 / 57, 70 / 76, 105 / 125; V = 131072 84 / 103, 95 / 124, 146 / 223. Logits in memory cost the separate one tiles of 256
+// rows for a few, and greedy selection a launch more: V = 131072, 16 / 112 rows, logits 137 / 104 and 157 / 111, top-p 354 / 292
+// and 364 / 394 (the single-kernel step 145 and 329 with 16). Top-k has a selection of its own in a separate LM head, three launches more:
+// V = 8000, 16 rows 78 / 57 (one layer 48 / 26, the single-kernel step 34), V = 131072 111 / about 150.
+// Weights split between clusters: all CTAs share the vocabulary. 16 layers, d = 1024, V = 32000, 1 / 16 rows: logits 155 / 138 and 178 /
+// 157, top-p 161 / 154 and 175 / 177, top-k 167 / 152 and 193 / 172; V = 131072, 8 layers, logits 172 / 112 and 222 / 123.
+constexpr int kHeadInsideVocab = 12288, kTopkInsideVocab = 32768;
+bool head_in_layers(const srm_model& m, const srm_sampling& samp, const float* logits_out, DecodeRoute route, int64_t R) {
+  const srm_config& c = m.cfg;
+  const bool own_topk = can_fuse_topk(m, samp, logits_out);
+  if (route == kRouteSplit) return !own_topk || c.vocab <= kTopkInsideVocab;
+  if (route != kRouteClusters || !cl::has_head(c.d_model)) return false;
+  if (c.vocab <= kHeadInsideVocab) return true;
+  return !own_topk && !can_fuse_greedy(m, samp, logits_out) && R <= (int64_t)(samp.mode == SRM_SELECT_GREEDY ? 16 * m.row_clusters : 16);
+}
+
 // One decode step for rows [b0, b0 + R) of the state.
 int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_t* tok_in, const srm_sampling& samp,
                  int step, const SelectOut& out_all, float* logits_out, const DecodeWs& w, cudaStream_t st,
@@ -1125,12 +1144,16 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   SmallPlan small;
   const DecodeRoute route = decode_route(m, R, false, w, &small, &mp);
   const bool one_kernel = route != kRouteKernels;
-  const bool head = (route == kRouteSplit || (route == kRouteClusters && cl::has_head(d))) && can_fuse_greedy(m, samp, logits_out);      // the selection, too
-  if (route == kRouteSplit) rc = launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr);
-  else if (route == kRouteClusters) rc = launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head ? &o : nullptr);
+  const bool greedy = samp.mode == SRM_SELECT_GREEDY, here = head_in_layers(m, samp, logits_out, route, R);
+  const bool topk = !here && can_fuse_topk(m, samp, logits_out);
+  // logits in memory: the caller wants them, or the selection reads them there
+  float* lg = logits_out != nullptr ? logits_out + b0 * c.vocab : can_fuse_greedy(m, samp, logits_out) || topk ? nullptr : w.logits;
+  const LmHead head{here, here && greedy, here ? lg : nullptr, o};
+  if (route == kRouteSplit) rc = launch_layers_split(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head);
+  else if (route == kRouteClusters) rc = launch_layers_cluster(m, s, b0, R, t, tok_in + b0, w, st, ctr, pos, head);
   else rc = one_kernel ? launch_layers_mid(m, s, b0, R, t, tok_in + b0, w, mp, st, ctr, pos) : SRM_OK;
   if (rc) return rc;
-  if (head) return SRM_OK;
+  if (here) return greedy ? SRM_OK : launch_select(m, R, lg, samp, samp.sample_idx_base + (uint64_t)b0, step, o, s.status, st);
   // the down projection shares K out between CTA pairs where that is the faster kernel for R rows
   bool split = false;
   if (!one_kernel && w.order != nullptr && F % tc::BK == 0) {
@@ -1196,10 +1219,9 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   if (ps.part != nullptr) ps.bias = m.fptr(c.n_layers - 1, SRM_T_B2);
   if (!one_kernel && (rc = launch_final_norm(m, w.x, R, 1, 0, w.a, st, nullptr, ps))) return rc;
   if (can_fuse_greedy(m, samp, logits_out)) return launch_lm_head_greedy(m, R, w.a, w.logits, o, s.status, st);
-  if (can_fuse_topk(m, samp, logits_out))
+  if (topk)
     return launch_lm_head_topk(m, R, w.a, w.logits, w.H, s.thr + b0, samp, samp.sample_idx_base + (uint64_t)b0, step, o,
                                s.status, s.status + kCtrHandedBack, st);
-  float* lg = logits_out != nullptr ? logits_out + b0 * c.vocab : w.logits;
   if ((rc = launch_gemm(m, kEpiPlain, R, c.vocab, d, w.a, m.ptr(-1, SRM_T_W_LM), nullptr, lg, s.status, st))) return rc;
   return launch_select(m, R, lg, samp, samp.sample_idx_base + (uint64_t)b0, step, o, s.status, st);
 }

@@ -25,9 +25,9 @@
 // A row's bits depend on neither its place in the pass nor the number of rows: every output is one fixed sequence of
 // 16-deep tensor steps, and N columns of an instruction do not mix.
 //
-// At d = 512 the LM head and the greedy selection follow in the same kernel (where the caller wants nothing else): 128 vocabulary rows
-// per tile, every 16th tile per rank, the best logit of a row from every rank to its owner. A kernel of its own for each
-// takes longer to start than to run.
+// At d = 512 the LM head and the greedy selection may follow in the same kernel: 128 vocabulary rows per tile, every 16th tile per
+// rank, the logits to global memory where they are wanted, the best logit of a row from every rank to its owner. A kernel of
+// its own for each takes longer to start than to run, up to a size of the vocabulary: every cluster reads all of it.
 //
 // No buffer needs a "free" signal of its own: an owner sends the next layer's activations after it has received every CTA's
 // partial products for its rows, a CTA sends those after the products that they come from, and everything else a CTA sends
@@ -79,7 +79,9 @@ struct Params {
   uint32_t* status;
   const int32_t* ctr;            // device-side step counters or nullptr
   const int32_t* pos;            // [R] per-row positions or nullptr
-  int head = 0;                  // D = 512: LM head and greedy selection here, to `out`; else the final norm's rows to `a`
+  int head = 0;                  // D = 512: LM head here; else the final norm's rows to `a`
+  int select = 0;                // ... and the greedy selection, to `out`
+  float* logits = nullptr;       // ... and the logits, to here ([R, V])
   SelectOut out = {};
 };
 __host__ __device__ constexpr bool has_head(int d) { return d == 512; }
@@ -524,7 +526,7 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (ok) ok = tc::mbar_wait(&act_full[i], (uint32_t)(p.L & 1), p.status);
-      if (wid == 0 && own > 0) tc::mbar_expect_tx(recv_full, (uint32_t)(own * kCluster * 8));
+      if (p.select && wid == 0 && own > 0) tc::mbar_expect_tx(recv_full, (uint32_t)(own * kCluster * 8));
       float bv[kOwn][4];
       int bi[kOwn][4];
       bool bad = false;
@@ -540,6 +542,15 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
           float acc[kOwn][4];
           take_tile<kOwn>(tmem + (static_cast<uint32_t>(quad * 32) << 16) + (uint32_t)((n & 1) * kIssuers * C::kN + cgrp * 4), C::kN, acc);
           const int col = tile * kTile + quad * 32 + lane;
+          if (p.logits != nullptr && col < p.V) {
+#pragma unroll
+            for (int g = 0; g < kOwn; ++g)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const int r = g * kCluster + cgrp * 4 + j;
+                if (r < rows) p.logits[(int64_t)(row_base + r) * p.V + col] = acc[g][j];
+              }
+          }
           if (col < p.V && ok) {
 #pragma unroll
             for (int g = 0; g < kOwn; ++g)
@@ -554,41 +565,43 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&head_empty[n & 1]);
       }
-      if (bad) raise_status(p.status, kStatusNonFinite);
-      workers_sync();                                                    // (the partial products that lay here have been read)
-      for (int i = wid; i < RC; i += kWorkers) best[i] = 0ull;
-      workers_sync();
-      if (cgrp * 4 < RC) {
+      if (p.select) {
+        if (bad) raise_status(p.status, kStatusNonFinite);
+        workers_sync();                                                    // (the partial products that lay here have been read)
+        for (int i = wid; i < RC; i += kWorkers) best[i] = 0ull;
+        workers_sync();
+        if (cgrp * 4 < RC) {
 #pragma unroll
-        for (int g = 0; g < kOwn; ++g)
+          for (int g = 0; g < kOwn; ++g)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            unsigned long long k = bi[g][j] < 0 ? 0ull : sb::pack_best(bv[g][j] + 0.0f, bi[g][j]);      // (minus zero equals zero)
+            for (int j = 0; j < 4; ++j) {
+              unsigned long long k = bi[g][j] < 0 ? 0ull : sb::pack_best(bv[g][j] + 0.0f, bi[g][j]);      // (minus zero equals zero)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, k, o);
-              k = k2 > k ? k2 : k;
+              for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, k, o);
+                k = k2 > k ? k2 : k;
+              }
+              if (lane == 0 && k != 0ull) atomicMax(&best[g * kCluster + cgrp * 4 + j], k);
             }
-            if (lane == 0 && k != 0ull) atomicMax(&best[g * kCluster + cgrp * 4 + j], k);
-          }
-      }
-      workers_sync();
-      if (wid < rows) {                                                  // row wid: to its owner
-        const uint32_t to = (uint32_t)(wid % kCluster);
-        const unsigned long long k = best[wid];
-        sb::st_async_v2(tc::mapa(tc::smem_u32(slots + (wid / kCluster) * kCluster + rank), to), __uint_as_float((uint32_t)k),
-                        __uint_as_float((uint32_t)(k >> 32)), tc::mapa(tc::smem_u32(recv_full), to));
-      }
-      if (wid < own) {
-        if (ok) ok = tc::mbar_wait(recv_full, (uint32_t)(p.L & 1), p.status, kWaitLimitCycles);
-        unsigned long long k = 0ull;
-        for (int r = 0; r < kCluster; ++r) {
-          const unsigned long long k2 = slots[wid * kCluster + r];
-          k = k2 > k ? k2 : k;
         }
-        int tok = k == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)k);      // (no finite logit: 0)
-        if (tok < 0 || tok >= p.V) tok = 0;
-        write_token(p.out, row_base + wid * kCluster + rank, tok);
+        workers_sync();
+        if (wid < rows) {                                                  // row wid: to its owner
+          const uint32_t to = (uint32_t)(wid % kCluster);
+          const unsigned long long k = best[wid];
+          sb::st_async_v2(tc::mapa(tc::smem_u32(slots + (wid / kCluster) * kCluster + rank), to), __uint_as_float((uint32_t)k),
+                          __uint_as_float((uint32_t)(k >> 32)), tc::mapa(tc::smem_u32(recv_full), to));
+        }
+        if (wid < own) {
+          if (ok) ok = tc::mbar_wait(recv_full, (uint32_t)(p.L & 1), p.status, kWaitLimitCycles);
+          unsigned long long k = 0ull;
+          for (int r = 0; r < kCluster; ++r) {
+            const unsigned long long k2 = slots[wid * kCluster + r];
+            k = k2 > k ? k2 : k;
+          }
+          int tok = k == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)k);      // (no finite logit: 0)
+          if (tok < 0 || tok >= p.V) tok = 0;
+          write_token(p.out, row_base + wid * kCluster + rank, tok);
+        }
       }
     }
   }

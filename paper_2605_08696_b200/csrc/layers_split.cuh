@@ -29,9 +29,9 @@
 // shared memory, each filled for the next layer as soon as it has been used. Buffers need no "free" signals, as in
 // layers_cluster.cuh: whatever overwrites one was computed from what its last reader sent afterwards.
 //
-// The LM head and the greedy selection follow in the same kernel where the caller wants nothing else: every CTA takes its 112th
-// of the vocabulary in chunks of 40 rows through the two places of the weights, as an up projection, and keeps the best logit of
-// every row; the CTA that comes last writes the tokens. A step of one row takes 140 us so, 150 with kernels of their own.
+// The LM head and the greedy selection follow in the same kernel (but for selections that have an LM head of their own): every CTA
+// takes its 112th of the vocabulary in chunks of 40 rows through the two places of the weights, as an up projection, writes the
+// logits where they are wanted and keeps the best one of every row; the CTA that comes last writes the tokens. A step of one row takes 140 us so, 150 with kernels of their own.
 //
 // All CTAs must be resident (cooperative launch). Every wait is bounded: a waiter that gives up raises kStatusWaitTimeout and
 // goes on without waiting.
@@ -70,7 +70,9 @@ struct Params {
   const float *lnf_g, *lnf_b;
   unsigned long long* planes;    // [2][clusters][R][d] words (value, tag)
   uint32_t* cnt;                 // CTAs that have cleared their words | CTAs done with the LM head; zero on entry
-  int head = 0;                  // LM head and greedy selection here, to `out`; else the final norm's rows to `a`
+  int head = 0;                  // LM head here; else the final norm's rows to `a`
+  int select = 0;                // ... and the greedy selection, to `out`
+  float* logits = nullptr;       // ... and the logits, to here ([R, V])
   unsigned long long* best = nullptr;      // [R] (sortable logit, ~column) maxima, zero on entry
   SelectOut out = {};
   uint32_t* status;
@@ -563,6 +565,11 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
             e = make_float4(e.x + f.x, e.y + f.y, e.z + f.z, e.w + f.w);
           }
           const int col = (lm0 + tile) * 8 + 2 * q;                      // (V is a multiple of 8; ascending: the lowest among equals is kept)
+          if (p.logits != nullptr) {
+            float* to = p.logits + (int64_t)g * p.V + col;
+            if (g < p.R) *reinterpret_cast<float2*>(to) = make_float2(e.x, e.y);
+            if (g + 8 < p.R) *reinterpret_cast<float2*>(to + (int64_t)8 * p.V) = make_float2(e.z, e.w);
+          }
           if (g < p.R) {
             bad |= !(e.x == e.x) | !(e.y == e.y);
             if (e.x > bv[0]) { bv[0] = e.x; bi[0] = col; }
@@ -575,26 +582,28 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
           }
         }
       }
-      if (bad) raise_status(p.status, kStatusNonFinite);
+      if (p.select) {
+        if (bad) raise_status(p.status, kStatusNonFinite);
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-        if (bi[i] >= 0) atomicMax(&best[g + 8 * i], sb::pack_best(bv[i] + 0.0f, bi[i]));      // (minus zero equals zero)
-      mma_sync();
-      const int r = tid - leader;
-      if (r < p.R && best[r] != 0ull) atomicMax(p.best + r, best[r]);
-      // ---- the CTA that comes last writes the tokens ----
-      __threadfence();
-      mma_sync();
-      if (r == 0) {
-        *am_last = atomicAdd(p.cnt + 1, 1u) + 1u == gridDim.x ? 1u : 0u;
+        for (int i = 0; i < 2; ++i)
+          if (bi[i] >= 0) atomicMax(&best[g + 8 * i], sb::pack_best(bv[i] + 0.0f, bi[i]));      // (minus zero equals zero)
+        mma_sync();
+        const int r = tid - leader;
+        if (r < p.R && best[r] != 0ull) atomicMax(p.best + r, best[r]);
+        // ---- the CTA that comes last writes the tokens ----
         __threadfence();
-      }
-      mma_sync();
-      if (*am_last != 0u && r < p.R) {
-        const unsigned long long k = __ldcg(p.best + r);
-        int tok = k == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)k);      // (no finite logit: 0)
-        if (tok < 0 || tok >= p.V) tok = 0;
-        write_token(p.out, r, tok);
+        mma_sync();
+        if (r == 0) {
+          *am_last = atomicAdd(p.cnt + 1, 1u) + 1u == gridDim.x ? 1u : 0u;
+          __threadfence();
+        }
+        mma_sync();
+        if (*am_last != 0u && r < p.R) {
+          const unsigned long long k = __ldcg(p.best + r);
+          int tok = k == 0ull ? 0 : (int)(0xFFFFFFFFu - (uint32_t)k);      // (no finite logit: 0)
+          if (tok < 0 || tok >= p.V) tok = 0;
+          write_token(p.out, r, tok);
+        }
       }
     }
   }

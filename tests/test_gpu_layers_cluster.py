@@ -144,3 +144,41 @@ def test_vocabularies_that_leave_ranks_without_a_tile(B, vocab):
         tok = want.clone()
     assert not torch.stack(differ).any() and torch.stack(clear_all).mean() > 0.9
     assert a.status() == 0 and b.status() == 0 and torch.equal(a.cache(), b.cache())
+
+
+@pytest.mark.parametrize("B,d,vocab,mode,want_logits,inside", [
+    (448, 512, 12288, "greedy", False, True), (64, 512, 12296, "greedy", False, False), (112, 512, 12296, "greedy", True, True),
+    (113, 512, 12296, "greedy", True, False), (448, 512, 12288, "topk", False, True), (1, 512, 12296, "topk", False, False),
+    (300, 512, 5000, "topp", False, True), (16, 512, 16392, "topp", False, True), (17, 512, 16392, "topp", True, False),
+    (1, 1024, 32768, "topk", False, True), (16, 1024, 4104, "topk", True, True), (9, 1024, 32776, "topk", False, False),
+    (16, 1024, 32776, "topp", False, True), (1, 1024, 32776, "greedy", True, True)])
+def test_lm_head_inside_or_outside_the_layers_kernel(B, d, vocab, mode, want_logits, inside):
+    """Both sides of every line between them, by the number of launches; logits against the kernel-per-operation path, tokens against the selection
+    kernels run on those logits."""
+    import paper_2605_08696_b200 as P
+    shape = custom_shape(n_layers=2, d_model=d, vocab=vocab, n_ctx=8, dtype="bf16", seed=24)
+    W = I.make_weights(shape)
+    samp = {"greedy": P.Sampling("greedy"), "topk": P.Sampling("topk", 40, 0.8, seed=3, sample_idx_base=5),
+            "topp": P.Sampling("topp", temperature=0.7, seed=4, sample_idx_base=6, top_p=0.9)}[mode]
+    toks = torch.from_numpy(np.random.default_rng(B).integers(0, vocab, size=(3, B)).astype(np.int32)).to(DEV)
+    m, ref = P.SRM(shape, W, device=DEV), P.SRM(shape, W, device=DEV, flags=P.FLAG_NO_SMALL_BATCH)
+    a, b, c, ws = m.new_state(B), m.new_state(B), ref.new_state(B), ref.new_workspace(B)
+    own_head = mode == "topk" and not want_logits          # (a selection of its own where the head is outside)
+    for k in range(3):
+        got, lg = m.decode_step(a, toks[k], samp, k + 1, ws, want_logits=True)
+        n0 = P.SRM.kernel_launches()
+        want = torch.empty_like(got)
+        m.k_select(lg, samp, k + 1, want)
+        selection, n0 = P.SRM.kernel_launches() - n0, P.SRM.kernel_launches()
+        tok = m.decode_step(b, toks[k], samp, k + 1, ws, want_logits=want_logits)
+        n = P.SRM.kernel_launches() - n0
+        if inside:
+            assert n == (1 if mode == "greedy" else 1 + selection)
+        else:
+            assert n == 2 + selection or (own_head and n > 2)
+        assert torch.equal(got, want)
+        if inside or want_logits or mode != "greedy":      # (greedy without logits outside: columns of one tile in another order of addition)
+            assert torch.equal(tok[0] if want_logits else tok, got)
+        lr = ref.decode_step(c, toks[k], samp, k + 1, ws, want_logits=True)[1]
+        assert rel_err_rows(lg.cpu().numpy(), lr.cpu().numpy()) < 5 * 2.0 ** -9 * 2 ** 0.5          # (as above, two layers)
+    assert a.status() == 0 and b.status() == 0 and torch.equal(a.cache(), b.cache())
