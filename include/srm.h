@@ -219,7 +219,7 @@ size_t srm_prefill_workspace_bytes(const srm_config* cfg, int64_t samples, int32
  * `ws_rows` rows (the rule stated above; host only, no device work). 0 if B < 1 or ws_rows < 1. */
 int64_t srm_decode_pass_rows(int64_t B, int64_t ws_rows);
 /* Which kernels the first pass of a decode step of B samples runs with a workspace of ws_bytes (an SRM_ROUTE_* value, or a
- * negative SRM_ERR_*; nothing is launched). A step's tokens do not depend on it but for rounding. */
+ * negative SRM_ERR_*; nothing is launched), where the step leaves no logits in memory. A step's tokens do not depend on it but for rounding. */
 enum {
   SRM_ROUTE_KERNELS = 0,             /* a kernel per operation                                                          */
   SRM_ROUTE_STEP = 1,                /* the whole step as one kernel on clusters of four CTAs                           */

@@ -1094,11 +1094,18 @@ bool small_step_plan(srm_model& m, int64_t B, SmallPlan* P) {
          sb::smem_plan((int)B, c.d_model, (int)m.F(), m.state_bytes(), &P->p, &P->smem);
 }
 
-// What a decode pass of R rows runs; `whole`: the pass is its state's whole batch. `small`, `mid`: the plan where that kernel is taken.
+// What a decode pass of R rows runs; `whole`: the pass is its state's whole batch; `in_memory`: its step leaves logits in memory.
+// `small`, `mid`: the plan where that kernel is taken.
 enum DecodeRoute { kRouteKernels, kRouteStep, kRouteLayers, kRouteClusters, kRouteSplit };      // SRM_ROUTE_* of the C ABI
-DecodeRoute decode_route(srm_model& m, int64_t R, bool whole, const DecodeWs& w, SmallPlan* small, mid::Params* mid) {
+DecodeRoute decode_route(srm_model& m, int64_t R, bool whole, bool in_memory, const DecodeWs& w, SmallPlan* small, mid::Params* mid) {
   if (split_rows_ok(m, R, w)) return kRouteSplit;
-  if (mid_rows_ok(m.cfg, R) && cluster_rows_ok(m, R)) return kRouteClusters;
+  if (mid_rows_ok(m.cfg, R) && cluster_rows_ok(m, R)) {
+    // 17 to 32 rows at d = 1024: the clusters gain 2 to 3 us per layer on the single-kernel step, which has the LM head inside; where that
+    // writes logits, a large vocabulary makes up for it (us per step with logits and with top-p, 32 rows, single-kernel step / clusters: V = 32000,
+    // 16 layers 249 / 210 and 259 / 212, 3 layers 81 / 72 and 91 / 71; V = 131072, 8 layers 216 / 225 and 404 / 433).
+    const bool step = whole && in_memory && !cl::has_head(m.cfg.d_model) && m.cfg.vocab > 8192 * std::max(8, m.cfg.n_layers);
+    return step && small_step_plan(m, R, small) ? kRouteStep : kRouteClusters;
+  }
   if (whole && small_step_plan(m, R, small)) return kRouteStep;
   return mid_plan(m, R, w, mid) ? kRouteLayers : kRouteKernels;
 }
@@ -1142,7 +1149,7 @@ int decode_chunk(srm_model& m, srm_state& s, int64_t b0, int64_t R, const int32_
   if (o.pos) o.pos += b0;
   if (o.thr_out) o.thr_out += b0;
   SmallPlan small;
-  const DecodeRoute route = decode_route(m, R, false, w, &small, &mp);
+  const DecodeRoute route = decode_route(m, R, false, false, w, &small, &mp);
   const bool one_kernel = route != kRouteKernels;
   const bool greedy = samp.mode == SRM_SELECT_GREEDY, here = head_in_layers(m, samp, logits_out, route, R);
   const bool topk = !here && can_fuse_topk(m, samp, logits_out);
@@ -1301,7 +1308,8 @@ int decode_step_impl(srm_model* m, srm_state* s, const int32_t* d_tok_in, const 
                 nullptr, nullptr, samp->mode == SRM_SELECT_TOPK ? s->thr : nullptr};
   SmallPlan small;
   mid::Params mid;
-  if (rows >= s->B && decode_route(*m, s->B, true, w, &small, &mid) == kRouteStep) {
+  const bool in_memory = !can_fuse_greedy(*m, *samp, d_logits_out) && !can_fuse_topk(*m, *samp, d_logits_out);
+  if (rows >= s->B && decode_route(*m, s->B, true, in_memory, w, &small, &mid) == kRouteStep) {
     rc = decode_step_small(*m, *s, small, tok_in, *samp, step, out, d_logits_out, w, st, ctr);
     if (rc != SRM_ERR_UNSUPPORTED) {
       if (rc == SRM_OK) s->pos += 1;

@@ -128,7 +128,7 @@ int32_t srm_decode_route(srm_model* m, int64_t B, size_t ws_bytes) {
   SmallPlan small;
   mid::Params mid;
   // (the areas of a workspace are told apart by their sizes; an address stands in for the caller's)
-  return decode_route(*m, rows < B ? rows : B, rows >= B, carve_decode(*m, reinterpret_cast<void*>(256), rows), &small, &mid);
+  return decode_route(*m, rows < B ? rows : B, rows >= B, false, carve_decode(*m, reinterpret_cast<void*>(256), rows), &small, &mid);
 }
 
 int srm_state_create(srm_model* m, int64_t B, void* d_state, size_t nbytes, void* stream, srm_state** out) {

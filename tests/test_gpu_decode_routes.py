@@ -231,3 +231,28 @@ def test_status_of_a_step_that_selects_in_the_layers_kernel(B, d):
         assert st.status() == 4 and got[row].item() == 0
         others = [r for r in range(B) if r != row]
         assert torch.equal(got[others], clean[others]) and bool(st.cache()[:, others].isfinite().all())
+
+
+@pytest.mark.parametrize("B,vocab,layers,logits,launches", [(32, 65544, 1, True, 1), (32, 65544, 1, False, 3), (17, 65536, 1, True, 3), (33, 65544, 1, True, 3),
+                                                            (20, 73736, 9, True, 1), (20, 73728, 9, True, 3)])
+def test_logits_of_a_large_vocabulary_after_few_layers(B, vocab, layers, logits, launches):
+    """17 to 32 rows at d = 1024: the single-kernel step, LM head included, where logits are wanted and the vocabulary is large for the number of
+    layers; the same step on kernels per operation."""
+    import paper_2605_08696_b200 as P
+    shape = _shape(1024, vocab=vocab, layers=layers, n_ctx=8)
+    W = I.make_weights(shape)
+    toks, g = _tokens(B, vocab, 2, B), P.Sampling("greedy")
+    m = P.SRM(shape, W, device=DEV)
+    st, ws = m.new_state(B), m.new_workspace(B)
+    n0, out = P.SRM.kernel_launches(), None
+    for k in range(2):
+        out = m.decode_step(st, toks[k], g, k + 1, ws, want_logits=logits)
+    assert P.SRM.kernel_launches() - n0 == 2 * launches and st.status() == 0
+    ref = P.SRM(shape, W, device=DEV, flags=P.FLAG_NO_SMALL_BATCH)
+    sr = ref.new_state(B)
+    for k in range(2):
+        _, lr = ref.decode_step(sr, toks[k], g, k + 1, ws, want_logits=True)
+    tol = 5 * 2.0 ** -9 * layers ** 0.5                      # (as above)
+    assert rel_err_rows(st.cache().cpu().numpy(), sr.cache().cpu().numpy()) < tol
+    if logits:
+        assert rel_err_rows(out[1].cpu().numpy(), lr.cpu().numpy()) < tol
