@@ -485,7 +485,8 @@ def run_ours(args):
     prof = model.profile_read()
     d, L, V, F = shape.d_model, shape.n_layers, shape.vocab, shape.d_ffn
     single_kernel = prof["step_small"][0] > 0          # small batch: the whole step is one kernel (dense work included)
-    gemm_classes = ("step_small",) if single_kernel else ("ffn", "gemm_up", "gemm_down", "gemm_lm", "gemm_proj")
+    # (where the LM head is a kernel of its own, its launch and the selection count too: its weights are in step_bytes below)
+    gemm_classes = ("step_small", "gemm_lm", "select") if single_kernel else ("ffn", "gemm_up", "gemm_down", "gemm_lm", "gemm_proj")
     gemm_ms = sum(prof[k][1] for k in gemm_classes)
     gemm_launches = sum(prof[k][0] for k in gemm_classes)
     gemm_flops = prof_steps * B * step_flops(shape)
@@ -546,7 +547,7 @@ def run_ours(args):
         # the step is one weight-streaming kernel: algorithmic bytes = the bf16 weights once + the cache read and written
         step_bytes = step_flops(shape) + B * 2 * L * d * sbytes
         gbs = prof_steps * step_bytes / (gemm_ms / 1e3) / 1e9 if gemm_ms > 0 else 0.0
-        roofline = {"bound": "hbm", "kernel": "layers_kernel or step_small_kernel (all layers of a small pass as one kernel)",
+        roofline = {"bound": "hbm", "kernel": "layers_kernel or step_small_kernel (all layers of a small pass as one kernel), LM head and selection included",
                     "achieved": round(gbs, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": round(gbs / peaks["hbm_gbs"], 4),
                     "peak_source": f"hbm_gbs, {peak_src}", "launches": int(gemm_launches), "steps_profiled": prof_steps,
                     "traffic": None, "bytes_per_step": step_bytes}

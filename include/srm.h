@@ -72,8 +72,8 @@ enum {
                                         when the caller does not ask for them); for comparison and measurement */
   SRM_FLAG_NO_SMALL_BATCH = 64,      /* small and mid passes also run one kernel per operation (default: bf16 mixed-head models with
                                         F = 4 d run all layers of a pass in one kernel of CTA clusters, at d = 512 up to 448
-                                        samples (65 to 71 excepted), at d = 1024 up to 112, with LM head and greedy selection
-                                        at d = 512 and up to 16 samples; other such models of at most 1024 channels, a
+                                        samples (65 to 71 so far excepted), at d = 1024 up to 112, with the LM head at
+                                        d = 512 for vocabularies to 12288 and at d = 1024 up to 16 samples; other such models of at most 1024 channels, a
                                         multiple of 256, with F a multiple of 1024 run the whole decode step of as many
                                         samples as fit beside a layer's weights in shared memory in ONE cooperative kernel;
                                         larger passes of d 512 (to 1024 samples), 1024 (to 512) and 1536 (to 256), passes of
@@ -204,9 +204,10 @@ int32_t srm_cache_planes(const srm_config* cfg);
  * batch runs as equal passes of at most 10240 rows (whole 256-row tiles), which keeps a layer's
  * activations in L2 between its kernels; results do not depend on the split, with three exceptions in the last bits:
  * a batch whose workspace holds it in one pass of the single-kernel step, and a pass whose layers run in one kernel
- * (see SRM_FLAG_NO_SMALL_BATCH; each of those kernels), add in another order than the kernel-per-operation path; of the passes whose layers
- * run in one kernel, those of more than four rows per SM (592) form the sums of the norms in another order than the
- * smaller ones; and a pass small enough for its down projection to be cut along K (see SRM_FLAG_NO_KSLICE) adds that
+ * (see SRM_FLAG_NO_SMALL_BATCH), add in another order than the kernel-per-operation path, each of those kernels in an order of its own:
+ * the last bits of a sample may change where its pass takes another kernel (srm_decode_route), at d = 1024 between 16 and 17 and
+ * between 112 and 113 rows, at d = 512 between 64, 65 to 71 and 72 and between 448 and 449, and where logits come from a
+ * separate LM head; the layers kernel over the grid also forms the sums of the norms in another order above four rows per SM (592); and a pass small enough for its down projection to be cut along K (see SRM_FLAG_NO_KSLICE) adds that
  * projection's partial products in another order than a large pass, whatever batch it is part of. The cache and the
  * logits that a prefill leaves depend in the same way on how many prompts share its pass: up to 383 go in chunks of
  * positions, more are walked one CTA per prompt. */

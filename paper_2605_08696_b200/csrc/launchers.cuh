@@ -747,8 +747,8 @@ int64_t layer_stride_bytes(const srm_model& m) {      // distance of a tensor fr
 
 // ---- decode passes of up to about a thousand rows: all layers in one kernel (layers_mid.cuh) -------------
 // Fewest rows, where the passes are not those of another kernel (cluster_rows_ok and split_rows_ok come first; step_small.cuh where
-// F is not 4 d). d = 512: 65 to 71 rows keep the kernel-per-operation path, which tests count on (138 us at 72 rows there, 104
-// here, 52 in clusters); up to 64 rows come here only where the single-kernel step does not take F (as kMixedAny).
+// F is not 4 d). d = 512: 65 to 71 rows keep the kernel-per-operation path for one reason, a test that counts its launches at 65 samples
+// (138 us at 72 rows there, 104 here, 52 in clusters, where these rows would be as fast); up to 64 rows come here only where the single-kernel step does not take F (as kMixedAny).
 // Combined heads and kernels (d 512 and 1024) have no other one-kernel step: any pass (96 rows, d = 1024, 16 layers, kernels of
 // size 4: 275 us per step, as a kernel per operation 560).
 bool mid_rows_ok(const srm_config& c, int64_t R) { return c.d_model != 512 || c.mixer != SRM_MIXER_MIXED || R <= sb::kMaxRows || R >= 72; }
@@ -993,7 +993,7 @@ bool split_rows_ok(srm_model& m, int64_t R, const DecodeWs& w) {
   constexpr int kOff = SRM_FLAG_SIMT_GEMM | SRM_FLAG_NO_SMALL_BATCH | SRM_FLAG_NO_KSLICE | SRM_FLAG_NO_FUSED_FFN | SRM_FLAG_HEAD_PROJ;
   if (c.dtype != SRM_DTYPE_BF16 || (c.flags & kOff) || c.mixer != SRM_MIXER_MIXED || c.ffn_mult != 4 || c.d_model != 1024 || R > sp::kMaxRows) return false;
   if (m.split_clusters < 0)
-    m.split_clusters = with_split_kernel(c, 32, [](auto* kernel, size_t smem) { return resident_clusters(kernel, sp::kThreads, smem); });
+    m.split_clusters = with_split_kernel(c, sp::kMaxRows, [](auto* kernel, size_t smem) { return resident_clusters(kernel, sp::kThreads, smem); });
   return m.split_clusters >= sp::kClusters && w.part != nullptr && sp::plane_bytes(R, c.d_model) <= w.part_bytes;
 }
 // All layers and the final norm for rows [b0, b0 + R) of the state; leaves the normed rows in w.a, or goes on to the LM head.

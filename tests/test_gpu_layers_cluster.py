@@ -1,6 +1,6 @@
 """Decode passes in clusters of 16 CTAs. Rows inside one cluster (layers_cluster.cuh), at the edges of its rows per cluster (8, 16, 32, 48,
-64 times the seven clusters of the device); a few rows with the weights split between the clusters (layers_split.cuh: up to
-16 and up to 32 rows, one, two and three layers): logits, tokens and cache against the kernel-per-operation path fed the
+64 times the seven clusters of the device); up to 16 rows at d = 1024 with the weights split between the clusters (layers_split.cuh; one, two
+and three layers): logits, tokens and cache against the kernel-per-operation path fed the
 same tokens, rows of the batch against the oracle, equal and per-sample positions, all cache types."""
 import numpy as np
 import pytest

@@ -1,4 +1,6 @@
-"""Decode passes whose layers run as one kernel (layers_mid.cuh), at the edges of its tile widths and row blocks: logits,
+"""Decode passes whose layers run as one kernel, at the edges of the tile widths and row blocks of layers_mid.cuh (mixed heads with F = 4 d
+of up to 448 rows at d = 512 and 112 at d = 1024 take the clusters of layers_cluster.cuh; captured steps and two streams of the kernel over the
+grid are in test_gpu_decode_routes.py): logits,
 tokens and cache against the kernel-per-operation path fed the same tokens (same products, sums in another order: the
 bound is the one the paths with and without ranges of K are held to), a row of the batch against the oracle, equal and
 per-sample positions, and the captured step."""
@@ -64,7 +66,7 @@ def test_layers_in_one_kernel_agree_with_the_kernel_per_operation_path(B, d, sta
 
 
 def test_captured_step_and_passes_of_one_kernel_equal_launch_by_launch():
-    """300 rows in one pass; the same steps replayed from a graph; and 300 rows as passes of 150 (same tile width)."""
+    """300 rows in one pass; the same steps replayed from a graph; and 300 rows as passes of 150 (rows in clusters, all three)."""
     import paper_2605_08696_b200 as P
     shape = custom_shape(n_layers=3, d_model=512, vocab=1024, n_ctx=24, dtype="bf16", seed=12)
     W = I.make_weights(shape)

@@ -1,6 +1,6 @@
-"""The single-kernel decode step of small batches (at most 64 samples; step_small.cuh): one cooperative kernel
-runs embedding, every layer's cache update and feed-forward, the final norm, the LM head and the greedy selection,
-with the projections cut into per-SM slabs. Parity against the oracle (teacher-forced: logits at every step, the
+"""Small decode batches whose step is one kernel: embedding, every layer's cache update and feed-forward, the final norm, the LM
+head and the greedy selection. The models "small" and "mid" take the kernels of CTA clusters (layers_cluster.cuh at d = 512,
+layers_split.cuh up to 16 samples at d = 1024); the models that step_small.cuh serves are in test_gpu_decode_routes.py. Parity against the oracle (teacher-forced: logits at every step, the
 cache at the end, tokens under the margin rule), agreement with the kernel-per-operation path, sampling on the
 logits it writes, and replay from a captured graph."""
 import numpy as np
@@ -29,8 +29,7 @@ def _launches_of_one_step(model, st, samp, ws):
 
 @pytest.mark.parametrize("B,state_dtype", [(1, "fp32"), (8, "fp32"), (33, "fp16"), (64, "fp32"), (16, "bf16")])
 def test_small_model_small_batch_parity(B, state_dtype):
-    """L8 d512 V8000 (eight n-slabs x eight k-slabs in the down projection, 16-column slabs in the up
-    projection, ragged last LM-head slab): 1 to 64 rows, partly filled row tiles included."""
+    """L8 d512 V8000 (ragged last tile of the LM head): 1 to 64 rows, one to ten per cluster."""
     import paper_2605_08696_b200 as P
     shape, W, model = _model("small", state_dtype=state_dtype)
     prompts = I.make_prompts("small")[7:7 + B]
@@ -56,7 +55,7 @@ def test_small_config_full_horizon_on_the_single_kernel_path():
 
 
 def test_mid_model_small_batch_parity():
-    """L16 d1024 V32000: 32-column slabs of the up projection, 512-long k-slabs, 224-column LM-head slabs."""
+    """L16 d1024 V32000, 8 samples: weights split between clusters."""
     shape, W, model = _model("mid")
     prompts = I.make_prompts("mid", batch=64)[3:11]
     r = teacher_forced("mid", shape, W, model, prompts, 10)
@@ -64,7 +63,7 @@ def test_mid_model_small_batch_parity():
 
 
 def test_single_kernel_step_agrees_with_the_kernel_per_operation_path():
-    """Same sums in another order (slabs of K in the down projection, mma.sync fragments instead of tcgen05 tiles).
+    """Same sums in another order (K in four groups of two issuers in the down projection).
     Both paths consume the SAME tokens (those the kernel-per-operation path selects): logits agree to a fraction of
     the bf16 tolerance at every step, the cache likewise, and the selected tokens are equal wherever the top-2
     margin is not thin."""
@@ -94,7 +93,7 @@ def test_single_kernel_step_agrees_with_the_kernel_per_operation_path():
 
 @pytest.mark.parametrize("mode", ["topk", "topp"])
 def test_sampling_on_the_logits_of_the_single_kernel_step(mode):
-    """Sampled selection: the kernel writes the logits, the selection kernels follow. The oracle's sampler run on
+    """Sampled selection: the layers kernel writes the logits, the selection kernels follow. The oracle's sampler run on
     those logits picks the device's token (CDF-edge cases excepted)."""
     import paper_2605_08696_b200 as P
     from oracle import srm_oracle as O
