@@ -11,7 +11,8 @@
 // What a layer takes (device clock, 16 rows per cluster unless said otherwise): d = 512, 9000 clocks = 4.7 us (the layers kernel over
 // the whole grid 11 us): activations -> up products 2150, GELU and copies 900, down products 2300, partial products out 600
 // and in 900, row phase 1600, activations out 500. With 37 rows per cluster 14200: distributed shared memory takes 21 bytes
-// per clock out of an SM and 32 into it. d = 1024, 8 rows: 19500 = 10.1 us, of which the weight stream needs 12600.
+// per clock out of an SM and 32 into it. d = 1024, 8 rows: 19500 = 10.1 us, of which the weight stream needs 12600. (Taken when partial
+// products were staged in shared memory and copied; from registers, as now, whole calls take the same within half a percent.)
 //
 // Rank r of the cluster is (K-group kg = r / 4, column ng = r % 4) of a 4 x 4 arrangement:
 //   rows:  rank r owns rows r, r + 16, .. of the cluster, whole warps per row, a float4 of the residual stream per thread, in
@@ -496,7 +497,9 @@ layers_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ 
       for (int m = 0; m < kDn; ++m) {
         if (ok) ok = tc::mbar_wait(&dn_done[m], (uint32_t)(l & 1), p.status);
         tc::tc_fence_after();
-        if (cgrp * 4 < min(rows, RC)) {                                  // (rows 4 cgrp .. + 3, and 16, 32, 48 further, as far as there are any)
+        // (a warp whose rows do not exist reads what nobody uses; with a test of `rows` instead, the same for the whole warp, a step of 8 layers
+        // with 10 or 16 rows per cluster at d = 512 took 52.4 and 54.3 us instead of 50.8 and 52.9)
+        if (cols) {
           float acc[kOwn][4];
           take_tile<kOwn>(tmem + (static_cast<uint32_t>(quad * 32) << 16) + (uint32_t)((kUp + m) * kIssuers * C::kN + cgrp * 4), C::kN, acc);
           const int to = cgrp * 4 + (lane & 3);                          // four features of one row per lane, 128 bytes per row and warp

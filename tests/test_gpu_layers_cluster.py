@@ -34,6 +34,8 @@ def test_rows_in_clusters_agree_with_the_kernel_per_operation_path(B, d, layers,
     for flags in (P.FLAG_NO_SMALL_BATCH, 0):
         m = P.SRM(shape, W, device=DEV, flags=flags, state_dtype=state_dtype)
         st, ws = m.new_state(B), m.new_workspace(B, n, prefill_samples=B)
+        one_kernel = "split" if d == 1024 and B <= 16 else "clusters" if B <= (112 if d == 1024 else 448) else "layers"
+        assert m.decode_route(B, ws) == ("kernels" if flags else one_kernel)
         m.prefill_ragged(st, prompts, lens, g, ws) if ragged else m.prefill(st, prompts, g, ws)
         lgs, toks = [], []
         for k in range(3):
